@@ -1,7 +1,8 @@
-"""ctypes binding of the C ABI in include/wino.h.
+"""Binding of the C ABI in include/wino.h: ctypes for what a program calls once per plan,
+the native module (csrc/wino_python.c) for what it calls on every pass.
 
 Argument marshalling only: every step of the layer runs in the CUDA library.
-PyTorch is used for device memory and streams.  If the shared library is
+PyTorch is used for device memory and streams.  If a shared library is
 missing or fails to load, importing this module raises.
 """
 from __future__ import annotations
@@ -49,13 +50,6 @@ class DescC(ct.Structure):
                 ("q_M", QuantC), ("q_Y", QuantC), ("out_dtype", ct.c_int32)]
 
 
-class DirectDescC(ct.Structure):
-    _fields_ = [("N", ct.c_int32), ("C", ct.c_int32), ("H", ct.c_int32), ("W", ct.c_int32),
-                ("K", ct.c_int32), ("stride", ct.c_int32),
-                ("q_x", QuantC), ("q_w", QuantC), ("q_Y", QuantC), ("out_dtype", ct.c_int32),
-                ("s_w_K_dev", ct.c_void_p), ("s_Y_K_dev", ct.c_void_p)]
-
-
 class WinoError(RuntimeError):
     def __init__(self, code: int, what: str):
         self.code = code
@@ -78,13 +72,9 @@ def _load() -> ct.CDLL:
     lib.wino_plan_force_path.argtypes = [vp, i32]
     lib.wino_plan_set_channel_scales.argtypes = [vp, vp, vp, vp, vp]
     lib.wino_plan_multipliers.argtypes = [vp, vp]
-    lib.wino_transform_weights.argtypes = [vp, vp, vp, vp, vp]
     lib.wino_transform_weights_channel_stats.argtypes = [vp, vp, vp, vp, vp]
-    lib.wino_conv_forward.argtypes = [vp, vp, vp, vp, vp, vp, vp]
-    lib.wino_conv_forward_static.argtypes = [vp, vp, vp, vp, vp, vp]
     lib.wino_calibrate_forward.argtypes = [vp, vp, vp, vp, vp, vp, vp, vp]
     lib.wino_debug_run_stages.argtypes = [vp, i32, vp, vp, vp, vp, vp, vp]
-    lib.wino_direct_conv_forward.argtypes = [ct.POINTER(DirectDescC), vp, vp, vp, vp, vp]
     lib.wino_direct_last_status.argtypes = [vp]
     lib.wino_debug_mma_probe.argtypes = [vp, i32, vp]
     lib.wino_last_status.argtypes = [vp, vp]
@@ -102,6 +92,7 @@ def _load() -> ct.CDLL:
 
 
 _lib = _load()
+from . import _native  # noqa: E402  (after the library: its absence is what should be reported)
 
 
 def strerror(code: int) -> str:
@@ -149,12 +140,10 @@ def direct_conv_forward(N, C, H, W, K, stride, q_x, q_w, q_Y, x_dev, w_dev, bias
                         out_dtype=0, stream=None, s_w_K_dev=None, s_Y_K_dev=None) -> None:
     """wino_direct_conv_forward: direct int8 3x3 convolution, stride 1 or 2; s_w_K_dev and
     s_Y_K_dev: optional per-output-channel scales (float32 tensors of K elements on the device)."""
-    d = DirectDescC(N, C, H, W, K, stride, _quant(q_x), _quant(q_w), _quant(q_Y), out_dtype,
-                    None if s_w_K_dev is None else s_w_K_dev.data_ptr(),
-                    None if s_Y_K_dev is None else s_Y_K_dev.data_ptr())
-    _check(_lib.wino_direct_conv_forward(ct.byref(d), _dptr(x_dev), _dptr(w_dev), _dptr(bias_dev),
-                                         _dptr(y_dev), _stream_handle(stream)),
-           "wino_direct_conv_forward")
+    rc = _native.direct_conv_forward(N, C, H, W, K, stride, q_x, q_w, q_Y, x_dev, w_dev, bias_dev, y_dev,
+                                     out_dtype, stream, s_w_K_dev, s_Y_K_dev)
+    if rc != WINO_OK:
+        raise WinoError(rc, "wino_direct_conv_forward")
 
 
 class Plan:
@@ -173,6 +162,7 @@ class Plan:
                           _quant(q_V), _quant(q_U), _quant(q_M), _quant(q_Y), out_dtype)
         self._h = ct.c_void_p()
         _check(_lib.wino_plan(ct.byref(self.desc), ct.byref(self._h)), "wino_plan")
+        self._address = self._h.value      # what the native module takes
         self.N, self.C, self.H, self.W, self.K, self.m, self.t = N, C, H, W, K, m, t
         self.TH, self.TW = -(-H // m), -(-W // m)
         self.T = N * self.TH * self.TW
@@ -233,8 +223,9 @@ class Plan:
 
     # --- device entry points ---
     def transform_weights(self, w_dev, Uq_dev, absmax_dev=None, stream=None) -> None:
-        _check(_lib.wino_transform_weights(self._h, _dptr(w_dev), _dptr(Uq_dev), _dptr(absmax_dev),
-                                           _stream_handle(stream)), "wino_transform_weights")
+        rc = _native.transform_weights(self._address, w_dev, Uq_dev, absmax_dev, stream)
+        if rc != WINO_OK:
+            raise WinoError(rc, "wino_transform_weights")
 
     def transform_weights_channel_stats(self, w_dev, Uq_dev, absmax_K_dev, stream=None) -> None:
         _check(_lib.wino_transform_weights_channel_stats(
@@ -242,16 +233,16 @@ class Plan:
             "wino_transform_weights_channel_stats")
 
     def conv_forward(self, x_dev, Uq_dev, bias_dev, y_dev, workspace_dev, stream=None) -> None:
-        _check(_lib.wino_conv_forward(self._h, _dptr(x_dev), _dptr(Uq_dev), _dptr(bias_dev),
-                                      _dptr(y_dev), _dptr(workspace_dev), _stream_handle(stream)),
-               "wino_conv_forward")
+        rc = _native.conv_forward(self._address, x_dev, Uq_dev, bias_dev, y_dev, workspace_dev, stream)
+        if rc != WINO_OK:
+            raise WinoError(rc, "wino_conv_forward")
 
     def conv_forward_static(self, x_dev, Uq_dev, bias_dev, y_dev, stream=None) -> None:
         """wino_conv_forward_static: no workspace argument; the library's built-in static
         scratch (STATIC_SCRATCH_BYTES at most) is used, and nothing is allocated."""
-        _check(_lib.wino_conv_forward_static(self._h, _dptr(x_dev), _dptr(Uq_dev), _dptr(bias_dev),
-                                             _dptr(y_dev), _stream_handle(stream)),
-               "wino_conv_forward_static")
+        rc = _native.conv_forward_static(self._address, x_dev, Uq_dev, bias_dev, y_dev, stream)
+        if rc != WINO_OK:
+            raise WinoError(rc, "wino_conv_forward_static")
 
     def debug_run_stages(self, stage_mask, x_dev, Uq_dev, bias_dev, y_dev, workspace_dev,
                          stream=None) -> None:

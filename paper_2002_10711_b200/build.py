@@ -1,9 +1,11 @@
 """Builds the CUDA library (sm_100a only) in-tree with nvcc: one object per
-translation unit, compiled in parallel, linked into one shared library."""
+translation unit, compiled in parallel, linked into one shared library; and the
+CPython module with the per-pass entry points (csrc/wino_python.c), linked against it."""
 from __future__ import annotations
 
 import os
 import subprocess
+import sysconfig
 from concurrent.futures import ThreadPoolExecutor
 
 HERE = os.path.dirname(os.path.abspath(__file__))
@@ -11,6 +13,7 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 OBJ = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libwino_b200.so")
+NATIVE = os.path.join(HERE, "_native.so")
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-O3", "-lineinfo", "-std=c++17",
     "-fmad=false", "--expt-relaxed-constexpr", "-Xcompiler", "-fPIC",
@@ -50,7 +53,20 @@ def build(force: bool = False, verbose: bool = False) -> str:
         subprocess.check_call([nvcc, "-gencode", "arch=compute_100a,code=sm_100a", "-shared",
                                "-cudart", "static", *objs, "-o", tmp])
         os.replace(tmp, LIB)
+    _build_native(force)
     return LIB
+
+
+def _build_native(force: bool) -> None:
+    src, header = os.path.join(CSRC, "wino_python.c"), os.path.join(ROOT, "include", "wino.h")
+    if not force and os.path.exists(NATIVE) and os.path.getmtime(NATIVE) >= max(os.path.getmtime(src),
+                                                                               os.path.getmtime(header)):
+        return
+    tmp = NATIVE + f".tmp{os.getpid()}"
+    subprocess.check_call([os.environ.get("CC", "gcc"), "-O2", "-std=c11", "-Wall", "-Wextra", "-fPIC", "-shared",
+                           "-I", sysconfig.get_paths()["include"], "-I", os.path.join(ROOT, "include"), src,
+                           "-L", HERE, "-l:" + os.path.basename(LIB), "-Wl,-rpath,$ORIGIN", "-o", tmp])
+    os.replace(tmp, NATIVE)
 
 
 if __name__ == "__main__":

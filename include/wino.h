@@ -77,7 +77,9 @@ enum {
 
 /* Execution paths a plan can use (see wino_plan_path / wino_plan_force_path).  The automatic
  * choice is 5 where it applies, else 2 for layers of at most 16 channels in and out, else 1
- * where C and K are multiples of 16, else 2. */
+ * where C and K are multiples of 16, else 2.  wino_conv_forward on a plan whose path was not
+ * forced runs a layer of few tiles by kernel 8 instead, where that is estimated to be faster
+ * (same results, same workspace requirement). */
 enum {
   WINO_PATH_AUTO = 0,
   WINO_PATH_STAGED_TC = 1,   /* transform kernels (TMA-staged where the shape allows) + tcgen05 int8 GEMMs */
@@ -87,9 +89,12 @@ enum {
   WINO_PATH_FUSED_F2 = 5,    /* one fused tcgen05 kernel: m = 2, Cook-Toom matrices, C in {32, 64}, K <= 64 */
   WINO_PATH_STAGED_TC_MMA = 6, /* as 1, with the transforms themselves on the tensor cores where that is
                                  exact: Cook-Toom F2 / F4, channel counts multiples of 128 */
-  WINO_PATH_FUSED_LAYER = 7   /* the whole layer in one persistent launch (tensor-core transforms and
+  WINO_PATH_FUSED_LAYER = 7,  /* the whole layer in one persistent launch (tensor-core transforms and
                                  GEMMs; V_q and m_q pass through the workspace in L2): Cook-Toom F2 / F4,
                                  C and K multiples of 128, input zero point 0, Q_M on, int8 output */
+  WINO_PATH_FUSED_SMALL = 8   /* the whole layer in one launch without scratch, for layers of few tiles: any m,
+                                 matrices and options (per-channel scales among them), C a multiple of 4 (at most 512 for m = 6,
+                                 else 1024), products of Q_V below 2^15 in magnitude whatever the data */
 };
 
 /* Stages that wino_debug_dump_stage can copy out (staged paths only). */
@@ -156,8 +161,8 @@ int wino_plan_force_path(wino_plan_t* plan, int path);
  * side (x, V) is summed over its channels and keeps one scale; zero points and code ranges
  * stay per layer.  All four NULL returns the plan to per-layer scales.  Call before
  * wino_transform_weights; U_q made under other scales is stale.  The staged paths
- * (WINO_PATH_STAGED_TC, WINO_PATH_STAGED_TC_PTR, WINO_PATH_STAGED_DP4A) implement it: a
- * plan on another path moves to the staged tcgen05 path (or the staged dp4a path), forcing
+ * (WINO_PATH_STAGED_TC, WINO_PATH_STAGED_TC_PTR, WINO_PATH_STAGED_DP4A) and
+ * WINO_PATH_FUSED_SMALL implement it: a plan on another path moves to the staged tcgen05 path (or the staged dp4a path), forcing
  * another path afterwards returns WINO_ERR_UNSUPPORTED, and wino_plan_multipliers keeps
  * reporting the per-layer values.  Synchronous (one small host-to-device copy);
  * WINO_ERR_INVALID for a bad scale, WINO_ERR_CUDA without a device. */
@@ -282,7 +287,8 @@ int wino_last_status(wino_plan_t* plan, void* stream);
  * (staged paths only) into dst_dev: V_q int8 [t*t][T][C], M int32 [t*t][T][K]
  * (recomputed from V_q and U_q with the plan's GEMM kernel), m_q int8
  * [t*t][T][K].  `bytes` must equal the stage size.  Asynchronous on the stream
- * of that forward call. */
+ * of that forward call, whose x and U_q must still be in place (a one-launch call keeps its
+ * intermediates on the SMs; they are then recomputed by the staged kernels). */
 int wino_debug_dump_stage(wino_plan_t* plan, int stage, void* dst_dev, size_t bytes);
 
 /* The forward pass on a single-kernel path (WINO_PATH_SMALLC, WINO_PATH_FUSED_F2;

@@ -21,6 +21,7 @@ PATH_AUTO, PATH_STAGED_TC, PATH_STAGED_DP4A, PATH_SMALLC, PATH_STAGED_TC_PTR = 0
 PATH_FUSED_F2 = 5
 PATH_STAGED_TC_MMA = 6
 PATH_FUSED_LAYER = 7
+PATH_FUSED_SMALL = 8
 STAGE_VQ, STAGE_M_I32, STAGE_MQ = 0, 1, 2
 STATIC_SCRATCH_BYTES = 20 * 1024 * 1024
 

@@ -23,6 +23,9 @@ struct Params {
   int z_x, z_w, z_Y;
   int qM_enabled;
   int out_dtype;               // 0 int8, 1 float
+  // whatever the data, every rounded product of Q_V (of Q_M) has a magnitude below 2^15, so
+  // that its clamp can be done in 16-bit lanes
+  int v_fits_16, m_fits_16;
 };
 // Per-output-channel scales travel beside Params as a device array `chan` [5][K] (null: the
 // per-layer values of Params): row kChMultU = s_w[k]/s_U[k], kChMultM = s_U[k]*s_V/s_M[k],
@@ -183,15 +186,5 @@ struct Mat {
     else return p.AT[i * T + k];
   }
 };
-
-// One step of a fused-multiply-add chain; with a compile-time zero coefficient
-// the step disappears (the chain's value is unchanged by it).
-template <bool STD>
-__device__ __forceinline__ float chain(float coef, float x, float acc) {
-  if constexpr (STD) {
-    if (coef == 0.0f) return acc;
-  }
-  return __fmaf_rn(coef, x, acc);
-}
 
 }  // namespace wino

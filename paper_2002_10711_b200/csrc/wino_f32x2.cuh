@@ -1,0 +1,80 @@
+// Two fp32 values in one 64-bit register pair, for the packed fp32 instructions of sm_100
+// (add / fma on f32x2), and the quantizer on such pairs.
+//
+// Why: the transforms and quantizers are bound by instruction issue and by the ALU pipe.
+// Measured on B200, issue cycles per warp instruction and scheduler: packed fma / add 2.05
+// (two results), scalar fma / add 1.25, integer add 1.3 (either pipe); prmt, lop3, min, max,
+// the 16x2 integer min / max, int-to-float and the saturating pack 2.05 each, all on the ALU
+// pipe, which the packed fp32 instructions leave free (a packed fma and a prmt together: 2.3 to
+// 2.5).  So the arithmetic goes in pairs on the fp32 pipe, and the quantizer's clamp, which in
+// fp32 costs two ALU instructions a code, is done on two 16-bit codes per instruction.
+#pragma once
+#include "wino_common.cuh"
+
+namespace wino {
+
+struct F2 {
+  unsigned long long v;
+};
+__device__ __forceinline__ F2 f2_make(float lo, float hi) {
+  F2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r.v) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ F2 f2_bits(uint32_t lo, uint32_t hi) {
+  F2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r.v) : "r"(lo), "r"(hi));
+  return r;
+}
+__device__ __forceinline__ F2 f2_both(float a) { return f2_make(a, a); }
+__device__ __forceinline__ void f2_split(F2 a, uint32_t& lo, uint32_t& hi) {
+  asm("mov.b64 {%0, %1}, %2;" : "=r"(lo), "=r"(hi) : "l"(a.v));
+}
+
+// The operations of the transforms, for one value and for a pair.
+__device__ __forceinline__ float v_add(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ float v_sub(float a, float b) { return __fsub_rn(a, b); }
+__device__ __forceinline__ float v_fma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ float v_mul(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ F2 v_add(F2 a, F2 b) {
+  F2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+  return r;
+}
+__device__ __forceinline__ F2 v_fma(F2 a, F2 b, F2 c) {
+  F2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
+  return r;
+}
+__device__ __forceinline__ F2 v_fma(float a, F2 b, F2 c) { return v_fma(f2_both(a), b, c); }
+__device__ __forceinline__ F2 v_sub(F2 a, F2 b) {   // a - b, rounded once
+  return v_fma(f2_both(-1.0f), b, a);
+}
+__device__ __forceinline__ F2 v_mul(float a, F2 b) {
+  F2 r;
+  const F2 aa = f2_both(a);
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(aa.v), "l"(b.v));
+  return r;
+}
+
+// Codes of the quantizer in 16-bit lanes.  r holds kMagic + n for two rounded products n; the
+// caller has made sure that |n| < 2^15, so the low halves are the n in two's complement.
+__device__ __forceinline__ uint32_t f2_low_halves(F2 r) {
+  uint32_t lo, hi;
+  f2_split(r, lo, hi);
+  return __byte_perm(lo, hi, 0x5410u);
+}
+__device__ __forceinline__ uint32_t clamp_s16x2(uint32_t a, uint32_t lo, uint32_t hi) {
+  uint32_t t, r;
+  asm("max.s16x2 %0, %1, %2;" : "=r"(t) : "r"(a), "r"(lo));
+  asm("min.s16x2 %0, %1, %2;" : "=r"(r) : "r"(t), "r"(hi));
+  return r;
+}
+__device__ __forceinline__ uint32_t s16x2_both(int v) { return ((uint32_t)v & 0xFFFFu) * 0x00010001u; }
+
+// round_half_even(v * mult) of a pair, clamped, as 16-bit lanes (|v * mult| < 2^15).
+__device__ __forceinline__ uint32_t quant_s16x2(F2 v, F2 mult, F2 magic, uint32_t lo, uint32_t hi) {
+  return clamp_s16x2(f2_low_halves(v_fma(v, mult, magic)), lo, hi);
+}
+
+}  // namespace wino

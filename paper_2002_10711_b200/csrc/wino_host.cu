@@ -46,6 +46,9 @@ struct wino_plan {
   float s_Y;
   bool std_mats;        // BT and AT equal the built-in Cook-Toom matrices bit for bit
   int path;
+  bool forced;          // wino_plan_force_path pinned it
+  bool small_ok;        // the one-launch kernel for layers of few tiles can run this layer
+  SmallGeom small;      // its geometry and cost estimate
   int* status_dev;      // device status word (may be null when no GPU is present)
   float* chan_dev;      // per-output-channel multipliers [5][K] (null: per-layer scales)
   void* kron_dev;       // Kronecker tables of the tensor-core transforms (same allocation)
@@ -61,9 +64,10 @@ struct wino_plan {
   const void* map_uq_ptr;
   CUtensorMap mapV, mapU;
   // maps of the TMA-staged transform kernels, keyed by buffer address
-  MapCache cache_x, cache_vst, cache_mld, cache_y, cache_uf, cache_x_sw, cache_m_sw;
+  MapCache cache_x, cache_vst, cache_mld, cache_y, cache_uf, cache_x_sw, cache_m_sw, cache_x_small, cache_u_small;
   // last forward call, for wino_debug_dump_stage
   const int8_t* last_uq;
+  const int8_t* last_x;     // non-null: that call left no V_q and m_q in its workspace
   void* last_ws;
   cudaStream_t last_stream;
   long launches;
@@ -139,7 +143,7 @@ bool path_supported(const wino_plan_t* pl, int path) {
   const int C = pl->d.C, K = pl->d.K;
   // per-output-channel scales are built into the staged kernels only
   if (pl->chan_dev != nullptr && path != WINO_PATH_STAGED_TC && path != WINO_PATH_STAGED_TC_PTR &&
-      path != WINO_PATH_STAGED_DP4A)
+      path != WINO_PATH_STAGED_DP4A && path != WINO_PATH_FUSED_SMALL)
     return false;
   switch (path) {
     case WINO_PATH_STAGED_TC:
@@ -148,6 +152,7 @@ bool path_supported(const wino_plan_t* pl, int path) {
     case WINO_PATH_STAGED_DP4A: return C % 4 == 0 && K % 4 == 0;
     case WINO_PATH_SMALLC: return C % 4 == 0 && K % 4 == 0 && C <= 32 && K <= 32;
     case WINO_PATH_FUSED_F2: return fused_f2_supported(pl->p, pl->std_mats);
+    case WINO_PATH_FUSED_SMALL: return pl->small_ok;
     case WINO_PATH_FUSED_LAYER:
       return layer_fused_supported(pl->p, pl->std_mats) &&
              layer_fused_geometry(pl->p, pl->num_sms).stages >= 2;
@@ -158,6 +163,11 @@ bool path_supported(const wino_plan_t* pl, int path) {
 size_t vq_bytes(const wino_plan_t* pl) { return (size_t)pl->p.t * pl->p.t * pl->p.T * pl->p.C; }
 size_t m_elems(const wino_plan_t* pl) { return (size_t)pl->p.t * pl->p.t * pl->p.T * pl->p.K; }
 size_t mbuf_bytes(const wino_plan_t* pl) { return m_elems(pl) * (pl->p.qM_enabled ? 1 : 4); }
+
+// Every shape the library plans has a staged path.
+int staged_path_of(const wino_plan_t* pl) {
+  return path_supported(pl, WINO_PATH_STAGED_TC) ? WINO_PATH_STAGED_TC : WINO_PATH_STAGED_DP4A;
+}
 
 LaunchOpt opt_of(const wino_plan_t* pl, bool pdl) {
   LaunchOpt o;
@@ -276,6 +286,32 @@ const CUtensorMap* map_u_fused(wino_plan_t* pl, const void* Uq) {
   return m;
 }
 
+// Maps of the small-layer kernel: rows of one 64-channel chunk, no swizzle.
+const CUtensorMap* map_x_small(wino_plan_t* pl, const void* x) {
+  if (const CUtensorMap* m = pl->cache_x_small.find(x)) return m;
+  const Params& p = pl->p;
+  const uint64_t dims[4] = {(uint64_t)p.C, (uint64_t)p.W, (uint64_t)p.H, (uint64_t)p.N};
+  const uint32_t box[4] = {64, (uint32_t)p.t, (uint32_t)p.t, 1};
+  CUtensorMap* m = pl->cache_x_small.slot(x);
+  if (encode_tiled(m, x, 4, dims, box, CU_TENSOR_MAP_SWIZZLE_NONE) != WINO_OK) {
+    pl->cache_x_small.key[(pl->cache_x_small.next + MapCache::kN - 1) % MapCache::kN] = nullptr;
+    return nullptr;
+  }
+  return m;
+}
+const CUtensorMap* map_u_small(wino_plan_t* pl, const void* Uq, int KB) {
+  if (const CUtensorMap* m = pl->cache_u_small.find(Uq)) return m;
+  const Params& p = pl->p;
+  const uint64_t dims[3] = {(uint64_t)p.C, (uint64_t)p.K, (uint64_t)(p.t * p.t)};
+  const uint32_t box[3] = {64, (uint32_t)(16 * KB), (uint32_t)(p.t * p.t)};
+  CUtensorMap* m = pl->cache_u_small.slot(Uq);
+  if (encode_tiled(m, Uq, 3, dims, box, CU_TENSOR_MAP_SWIZZLE_NONE) != WINO_OK) {
+    pl->cache_u_small.key[(pl->cache_u_small.next + MapCache::kN - 1) % MapCache::kN] = nullptr;
+    return nullptr;
+  }
+  return m;
+}
+
 int launch_gemm(wino_plan_t* pl, const int8_t* Vq, const int8_t* Uq, void* out, int out_mode,
                 unsigned* absmaxM, bool pdl, cudaStream_t st) {
   const Params& p = pl->p;
@@ -298,6 +334,33 @@ int launch_gemm(wino_plan_t* pl, const int8_t* Vq, const int8_t* Uq, void* out, 
                         pl->status_dev, st);
 }
 
+// Time of the plan's own path, for the choice between it and the one-launch kernel, in ns: a
+// floor of three dependent launches (their host time alone is 6.6 us), then transforms and
+// quantizers by the number of codes.  Measured, see the table beside small_geometry.
+long staged_cost(const wino_plan_t* pl) {
+  const double codes = (double)pl->p.t * pl->p.t * pl->p.T * (pl->p.C + pl->p.K);
+  if (pl->path == WINO_PATH_FUSED_F2)   // by waves of 128 tiles per SM, full or not
+    return 28200l * (((pl->p.T + 127) / 128 + pl->num_sms - 1) / pl->num_sms);
+  const long gpu = 6500 + (long)(codes * 6.6e-4);
+  return gpu > 7500 ? gpu : 7500;
+}
+
+int forward_small(wino_plan_t* pl, const int8_t* x, const int8_t* Uq, const float* bias, void* y,
+                  cudaStream_t st) {
+  const SmallGeom& g = pl->small;
+  const CUtensorMap none = {};
+  SmallArgs a;
+  a.mapX = a.mapU = &none;
+  if (pl->p.C % 16 == 0) {
+    a.mapX = map_x_small(pl, x);
+    a.mapU = map_u_small(pl, Uq, g.KB);
+    if (a.mapX == nullptr || a.mapU == nullptr) return WINO_ERR_CUDA;
+  }
+  a.x = x; a.Uq = Uq; a.bias = bias; a.y = y; a.s_Y = pl->s_Y; a.status = pl->status_dev;
+  pl->launches++;
+  return launch_small(pl->p, opt_of(pl, pl->pdl), g, a, st);
+}
+
 // stage_mask: bit 0 input transform, bit 1 Hadamard GEMMs, bit 2 output transform.
 // dbgM (single-kernel paths only): receives the int32 Hadamard sums M[xi][tau][k].
 int forward_impl(wino_plan_t* pl, const int8_t* x, const int8_t* Uq, const float* bias, void* y,
@@ -306,6 +369,8 @@ int forward_impl(wino_plan_t* pl, const int8_t* x, const int8_t* Uq, const float
   if (pl->status_dev == nullptr) return WINO_ERR_CUDA;
   const bool calib = absmax4 != nullptr;
   const bool pdl = pl->pdl && !calib;
+  if (pl->path == WINO_PATH_FUSED_SMALL && !calib && stage_mask == 7 && dbgM == nullptr)
+    return forward_small(pl, x, Uq, bias, y, st);
   if (pl->path == WINO_PATH_SMALLC && !calib) {
     pl->launches++;
     return launch_smallc(pl->p, opt_of(pl, pdl), x, Uq, bias, y, pl->s_Y, dbgM, st);
@@ -350,6 +415,7 @@ int forward_impl(wino_plan_t* pl, const int8_t* x, const int8_t* Uq, const float
                                       pl->status_dev, st);
     if (rc != WINO_OK) return rc;
     pl->last_uq = Uq;
+    pl->last_x = nullptr;
     pl->last_ws = ws;
     pl->last_stream = st;
     return WINO_OK;
@@ -360,6 +426,7 @@ int forward_impl(wino_plan_t* pl, const int8_t* x, const int8_t* Uq, const float
   if (pl->path == WINO_PATH_SMALLC) gemm_path = WINO_PATH_STAGED_DP4A;
   if (pl->path == WINO_PATH_FUSED_F2) gemm_path = WINO_PATH_STAGED_TC_PTR;
   if (pl->path == WINO_PATH_FUSED_LAYER) gemm_path = WINO_PATH_STAGED_TC;
+  if (pl->path == WINO_PATH_FUSED_SMALL) gemm_path = staged_path_of(pl);
   const bool tma_ok = (pl->path == WINO_PATH_STAGED_TC || pl->path == WINO_PATH_STAGED_TC_MMA) && !calib;
   const bool mma_ok = pl->path == WINO_PATH_STAGED_TC_MMA && !calib;
   int rc = WINO_OK;
@@ -412,13 +479,14 @@ int forward_impl(wino_plan_t* pl, const int8_t* x, const int8_t* Uq, const float
   }
   if (rc != WINO_OK) return rc;
   pl->last_uq = Uq;
+  pl->last_x = nullptr;
   pl->last_ws = ws;
   pl->last_stream = st;
   return WINO_OK;
 }
 
 bool path_uses_scratch(const wino_plan_t* pl) {
-  return pl->path != WINO_PATH_SMALLC && pl->path != WINO_PATH_FUSED_F2;
+  return pl->path != WINO_PATH_SMALLC && pl->path != WINO_PATH_FUSED_F2 && pl->path != WINO_PATH_FUSED_SMALL;
 }
 
 DeviceOnce g_once_selftest;
@@ -481,6 +549,18 @@ int wino_plan(const wino_desc_t* desc, wino_plan_t** out) {
   p.z_x = d.q_x.zero_point; p.z_w = d.q_w.zero_point; p.z_Y = d.q_Y.zero_point;
   p.qM_enabled = d.q_M.enabled ? 1 : 0;
   p.out_dtype = d.out_dtype;
+  {
+    // largest |V|: |x - z_x| <= 127 + |z_x| + 1 through the largest absolute row sum, twice
+    double row = 0.0;
+    for (int i = 0; i < t; ++i) {
+      double r = 0.0;
+      for (int k = 0; k < t; ++k) r += std::fabs((double)p.BT[i * t + k]);
+      if (r > row) row = r;
+    }
+    const double v_max = row * row * (128.0 + std::fabs((double)p.z_x));
+    p.v_fits_16 = v_max * (double)p.mult_V < 32000.0 ? 1 : 0;
+    p.m_fits_16 = 16384.0 * d.C * (double)p.mult_M < 32000.0 ? 1 : 0;
+  }
   pl->std_mats = d.m == 2 ? is_std<2>(p.BT, p.AT) : d.m == 4 ? is_std<4>(p.BT, p.AT)
                                                                : is_std<6>(p.BT, p.AT);
   // Automatic choice, by measurement on B200: the fused F2 kernel where it applies; for
@@ -523,6 +603,8 @@ int wino_plan(const wino_desc_t* desc, wino_plan_t** out) {
     }
   }
   cudaGetLastError();
+  pl->small_ok = small_supported(p);
+  if (pl->small_ok) pl->small = small_geometry(p, pl->num_sms);
   *out = pl;
   return WINO_OK;
 }
@@ -541,9 +623,10 @@ int wino_plan_path(const wino_plan_t* pl) { return pl ? pl->path : WINO_ERR_INVA
 
 int wino_plan_force_path(wino_plan_t* pl, int path) {
   if (pl == nullptr) return WINO_ERR_INVALID;
-  if (path < WINO_PATH_STAGED_TC || path > WINO_PATH_FUSED_LAYER) return WINO_ERR_INVALID;
+  if (path < WINO_PATH_STAGED_TC || path > WINO_PATH_FUSED_SMALL) return WINO_ERR_INVALID;
   if (!path_supported(pl, path)) return WINO_ERR_UNSUPPORTED;
   pl->path = path;
+  pl->forced = true;
   return WINO_OK;
 }
 
@@ -588,9 +671,8 @@ int wino_plan_set_channel_scales(wino_plan_t* pl, const float* s_w_K, const floa
     return WINO_ERR_CUDA;
   }
   pl->chan_dev = fresh;
-  if (!path_supported(pl, pl->path)) {   // every shape the library plans has a staged path
-    if (path_supported(pl, WINO_PATH_STAGED_TC)) pl->path = WINO_PATH_STAGED_TC;
-    else pl->path = WINO_PATH_STAGED_DP4A;
+  if (!path_supported(pl, pl->path)) {
+    pl->path = staged_path_of(pl);
   }
   return WINO_OK;
 }
@@ -626,6 +708,17 @@ int wino_conv_forward(wino_plan_t* pl, const int8_t* x, const int8_t* Uq, const 
   if (pl == nullptr || x == nullptr || Uq == nullptr || y == nullptr) return WINO_ERR_INVALID;
   if (!aligned16(x) || !aligned16(Uq) || !aligned16(y) || (bias && !aligned16(bias)))
     return WINO_ERR_ALIGNMENT;
+  if (!pl->forced && pl->small_ok && pl->small.cost < staged_cost(pl)) {
+    const bool scratch = path_uses_scratch(pl);
+    if (pl->status_dev == nullptr) return WINO_ERR_CUDA;
+    if (scratch && ws == nullptr) return WINO_ERR_WORKSPACE;
+    if (scratch && !aligned16(ws)) return WINO_ERR_ALIGNMENT;
+    const int rc = forward_small(pl, x, Uq, bias, y, (cudaStream_t)stream);
+    if (rc == WINO_OK && scratch) {
+      pl->last_uq = Uq; pl->last_x = x; pl->last_ws = ws; pl->last_stream = (cudaStream_t)stream;
+    }
+    return rc;
+  }
   return forward_impl(pl, x, Uq, bias, y, ws, nullptr, (cudaStream_t)stream);
 }
 
@@ -655,7 +748,8 @@ int wino_debug_run_stages(wino_plan_t* pl, int stage_mask, const int8_t* x, cons
                           const float* bias, void* y, void* ws, void* stream) {
   if (pl == nullptr || x == nullptr || Uq == nullptr || y == nullptr) return WINO_ERR_INVALID;
   if (stage_mask < 1 || stage_mask > 7) return WINO_ERR_INVALID;
-  if ((pl->path == WINO_PATH_SMALLC || pl->path == WINO_PATH_FUSED_F2) && stage_mask != 7)
+  if ((pl->path == WINO_PATH_SMALLC || pl->path == WINO_PATH_FUSED_F2 || pl->path == WINO_PATH_FUSED_SMALL) &&
+      stage_mask != 7)
     return WINO_ERR_UNSUPPORTED;   // the fused paths have no separate stages
   if (!aligned16(x) || !aligned16(Uq) || !aligned16(y) || (bias && !aligned16(bias)))
     return WINO_ERR_ALIGNMENT;
@@ -754,7 +848,8 @@ int wino_debug_forward_accumulators(wino_plan_t* pl, const int8_t* x, const int8
                                     void* stream) {
   if (pl == nullptr || x == nullptr || Uq == nullptr || y == nullptr || M_dev == nullptr)
     return WINO_ERR_INVALID;
-  if (path_uses_scratch(pl)) return WINO_ERR_UNSUPPORTED;   // staged paths: wino_debug_dump_stage
+  if (path_uses_scratch(pl) || pl->path == WINO_PATH_FUSED_SMALL)
+    return WINO_ERR_UNSUPPORTED;   // staged paths: wino_debug_dump_stage
   if (bytes != m_elems(pl) * 4) return WINO_ERR_INVALID;
   if (!aligned16(x) || !aligned16(Uq) || !aligned16(y) || !aligned16(M_dev) ||
       (bias && !aligned16(bias)))
@@ -787,6 +882,10 @@ int wino_debug_dump_stage(wino_plan_t* pl, int stage, void* dst, size_t bytes) {
   if (!aligned16(dst)) return WINO_ERR_ALIGNMENT;
   const uint8_t* ws = reinterpret_cast<const uint8_t*>(pl->last_ws);
   cudaStream_t st = pl->last_stream;
+  if (pl->last_x != nullptr) {   // a one-launch call keeps V_q and m_q on the SMs: make them now
+    const int rc = forward_impl(pl, pl->last_x, pl->last_uq, nullptr, nullptr, pl->last_ws, nullptr, st, 3);
+    if (rc != WINO_OK) return rc;
+  }
   if (stage == WINO_STAGE_VQ) {
     if (bytes != vq_bytes(pl)) return WINO_ERR_INVALID;
     return cudaMemcpyAsync(dst, ws, bytes, cudaMemcpyDeviceToDevice, st) == cudaSuccess ? WINO_OK
@@ -804,6 +903,7 @@ int wino_debug_dump_stage(wino_plan_t* pl, int stage, void* dst, size_t bytes) {
     if (pl->path == WINO_PATH_SMALLC) pl->path = WINO_PATH_STAGED_DP4A;
     if (pl->path == WINO_PATH_FUSED_F2) pl->path = WINO_PATH_STAGED_TC_PTR;
     if (pl->path == WINO_PATH_FUSED_LAYER) pl->path = WINO_PATH_STAGED_TC;
+    if (pl->path == WINO_PATH_FUSED_SMALL) pl->path = staged_path_of(pl);
     const int rc = launch_gemm(pl, reinterpret_cast<const int8_t*>(ws), pl->last_uq, dst, kOutI32,
                                nullptr, false, st);
     pl->path = saved_path;

@@ -4,6 +4,7 @@
 #pragma once
 #include <cstdio>
 #include <mutex>
+#include <utility>
 
 #include <cuda.h>
 #include <cuda_runtime.h>
@@ -128,6 +129,24 @@ int launch_gemm_tc(const Params& p, const LaunchOpt& o, const TcGeom& g, const C
 int launch_smallc(const Params& p, const LaunchOpt& o, const int8_t* x, const int8_t* Uq,
                   const float* bias, void* y, float s_Y, int* dbgM, cudaStream_t st);
 
+// The whole layer in one launch for layers of few tiles (any m, matrices and options; C a
+// multiple of 4): a block owns 8 tiles x 16*KB output channels, the S blocks of a cluster
+// `chunks` chunks of 64 channels each.  `cost`: the launcher's estimate of the kernel's time, ns.
+// The maps (C a multiple of 16): x as [N][H][W][C] with box {64, t, t, 1}, U_q as [t*t][K][C]
+// with box {64, 16*KB, t*t}, no swizzle.
+struct SmallGeom { int KB, chunks, S, n_kblk, grid; size_t smem; long cost; };
+struct SmallArgs {
+  const CUtensorMap *mapX, *mapU;
+  const int8_t *x, *Uq;
+  const float* bias;
+  void* y;
+  float s_Y;
+  int* status;
+};
+bool small_supported(const Params& p);
+SmallGeom small_geometry(const Params& p, int num_sms);
+int launch_small(const Params& p, const LaunchOpt& o, const SmallGeom& g, const SmallArgs& s, cudaStream_t st);
+
 // Fully fused F2 kernel for narrow layers (C in {32, 64}, K <= 64, Cook-Toom matrices).
 bool fused_f2_supported(const Params& p, bool std_mats);
 int launch_fused_f2(const Params& p, const LaunchOpt& o, const CUtensorMap& mapU, const int8_t* x,
@@ -181,18 +200,26 @@ enum { kOutMq = 0, kOutI32 = 1 };
 constexpr int kBM = 128;      // tiles per GEMM block (MMA M)
 constexpr int kStageK = 128;  // channels (bytes) per shared-memory stage
 
-// Generic launcher: plain <<<>>> or cudaLaunchKernelEx with the programmatic
-// stream serialization attribute (the kernel then calls griddep_wait()).
+// Generic launcher: cudaLaunchKernelEx with, where asked for, the programmatic stream
+// serialization attribute (the kernel then calls griddep_wait()) and clusters of `cluster`
+// blocks along x.
 template <typename... KArgs, typename... Args>
-int launch_kernel(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
-                  bool pdl, Args&&... args) {
+int launch_kernel_cluster(void (*kernel)(KArgs...), dim3 grid, dim3 block, unsigned cluster, size_t smem,
+                          cudaStream_t st, bool pdl, Args&&... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchAttribute attr[2];
   cfg.attrs = attr;
-  cfg.numAttrs = pdl ? 1 : 0;
+  if (pdl) {
+    attr[cfg.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[cfg.numAttrs++].val.programmaticStreamSerializationAllowed = 1;
+  }
+  if (cluster > 1) {
+    attr[cfg.numAttrs].id = cudaLaunchAttributeClusterDimension;
+    attr[cfg.numAttrs].val.clusterDim.x = cluster;
+    attr[cfg.numAttrs].val.clusterDim.y = 1;
+    attr[cfg.numAttrs++].val.clusterDim.z = 1;
+  }
   const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
 #ifdef WINO_TRACE
   if (e != cudaSuccess)
@@ -200,6 +227,11 @@ int launch_kernel(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, 
                  block.x, smem);
 #endif
   return e == cudaSuccess ? 0 : -5;
+}
+template <typename... KArgs, typename... Args>
+int launch_kernel(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                  bool pdl, Args&&... args) {
+  return launch_kernel_cluster(kernel, grid, block, 1u, smem, st, pdl, std::forward<Args>(args)...);
 }
 
 }  // namespace wino

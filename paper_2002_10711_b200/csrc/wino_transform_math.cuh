@@ -12,7 +12,7 @@
 //             shared sub-expressions are factored out.  The F6 output stage falls
 //             back to the ordered chains.
 #pragma once
-#include "wino_common.cuh"
+#include "wino_f32x2.cuh"
 
 namespace wino {
 
@@ -64,43 +64,97 @@ __device__ __forceinline__ void bt_exact(const float (&d)[6], float (&r)[6]) {
   r[4] = __fmaf_rn(-2.0f, t1, t2);
   r[5] = __fmaf_rn(4.0f, d[1], __fmaf_rn(-5.0f, d[3], d[5]));
 }
-// 1-D A^T, factored (exact mode only: integer codes in, integers below 2^24 throughout).
-__device__ __forceinline__ void at_exact(const float (&m)[4], float (&y)[2]) {
-  y[0] = __fadd_rn(__fadd_rn(m[0], m[1]), m[2]);
-  y[1] = __fadd_rn(__fsub_rn(m[1], m[2]), m[3]);
+// The same for a pair of values, with row 1 NEGATED: packed instructions take no operand
+// negation, and every other row comes out with the same operation count.  (B^T d) B of such
+// passes has the sign pair_sign(i) * pair_sign(j) at (i, j), which the quantizer's multiplier
+// absorbs (rounding half to even is symmetric).
+template <int T_>
+__device__ __forceinline__ constexpr bool pair_negated(int i) { return T_ >= 6 && i == 1; }
+__device__ __forceinline__ void bt_exact(const F2 (&d)[4], F2 (&r)[4]) {
+  r[0] = v_sub(d[0], d[2]);
+  r[1] = v_add(d[1], d[2]);
+  r[2] = v_sub(d[2], d[1]);
+  r[3] = v_sub(d[3], d[1]);
 }
-__device__ __forceinline__ void at_exact(const float (&m)[6], float (&y)[4]) {
-  const float a = __fadd_rn(m[1], m[2]);
-  const float b = __fsub_rn(m[1], m[2]);
-  const float c = __fadd_rn(m[3], m[4]);
-  const float d = __fsub_rn(m[3], m[4]);
-  y[0] = __fadd_rn(__fadd_rn(m[0], a), c);
-  y[1] = __fmaf_rn(2.0f, d, b);
-  y[2] = __fmaf_rn(4.0f, c, a);
-  y[3] = __fadd_rn(__fmaf_rn(8.0f, d, b), m[5]);
+__device__ __forceinline__ void bt_exact(const F2 (&d)[6], F2 (&r)[6]) {
+  const F2 t1 = v_sub(d[3], d[1]);
+  const F2 t2 = v_sub(d[4], d[2]);
+  const F2 u = v_fma(-4.0f, d[2], d[4]);
+  const F2 v = v_fma(-4.0f, d[1], d[3]);
+  r[0] = v_fma(4.0f, d[0], v_fma(-5.0f, d[2], d[4]));
+  r[1] = v_add(u, v);
+  r[2] = v_sub(v, u);
+  r[3] = v_fma(2.0f, t1, t2);
+  r[4] = v_fma(-2.0f, t1, t2);
+  r[5] = v_fma(4.0f, d[1], v_fma(-5.0f, d[3], d[5]));
+}
+__device__ __forceinline__ void bt_exact(const F2 (&d)[8], F2 (&r)[8]) {
+  const F2 e1 = v_fma(-4.25f, d[4], v_add(d[2], d[6]));
+  const F2 o1 = v_fma(-4.25f, d[3], v_add(d[1], d[5]));
+  const F2 e2 = v_fma(0.25f, d[2], v_fma(-1.25f, d[4], d[6]));
+  const F2 o2 = v_fma(0.5f, d[1], v_fma(-2.5f, d[3], v_add(d[5], d[5])));
+  const F2 e3 = v_fma(4.0f, d[2], v_fma(-5.0f, d[4], d[6]));
+  const F2 o3 = v_fma(2.0f, d[1], v_fma(-2.5f, d[3], v_mul(0.5f, d[5])));
+  r[0] = v_fma(5.25f, v_sub(d[4], d[2]), v_sub(d[0], d[6]));
+  r[1] = v_add(e1, o1);
+  r[2] = v_sub(o1, e1);
+  r[3] = v_add(e2, o2);
+  r[4] = v_sub(e2, o2);
+  r[5] = v_add(e3, o3);
+  r[6] = v_sub(e3, o3);
+  r[7] = v_fma(5.25f, v_sub(d[3], d[5]), v_sub(d[7], d[1]));
+}
+// 1-D A^T, factored (exact mode only: integer codes in, integers below 2^24 throughout).
+template <typename V>
+__device__ __forceinline__ void at_exact(const V (&m)[4], V (&y)[2]) {
+  y[0] = v_add(v_add(m[0], m[1]), m[2]);
+  y[1] = v_add(v_sub(m[1], m[2]), m[3]);
+}
+template <typename V>
+__device__ __forceinline__ void at_exact(const V (&m)[6], V (&y)[4]) {
+  const V a = v_add(m[1], m[2]);
+  const V b = v_sub(m[1], m[2]);
+  const V c = v_add(m[3], m[4]);
+  const V d = v_sub(m[3], m[4]);
+  y[0] = v_add(v_add(m[0], a), c);
+  y[1] = v_fma(2.0f, d, b);
+  y[2] = v_fma(4.0f, c, a);
+  y[3] = v_add(v_fma(8.0f, d, b), m[5]);
+}
+__device__ __forceinline__ float v_zero(float) { return 0.0f; }
+__device__ __forceinline__ F2 v_zero(F2) { return f2_both(0.0f); }
+// One step of a fused-multiply-add chain; with a compile-time zero coefficient
+// the step disappears (the chain's value is unchanged by it).
+template <bool STD, typename V>
+__device__ __forceinline__ V chain(float coef, V x, V acc) {
+  if constexpr (STD) {
+    if (coef == 0.0f) return acc;
+  }
+  return v_fma(coef, x, acc);
 }
 
-// V = (B^T d) B for one channel.  d is given column-wise through `col(l, out)`.
-template <int M, int MODE, typename ColFn>
+// V = (B^T d) B for one channel, or for a pair of channels (VT = F2; kExact: with the signs of
+// pair_negated).  d is given column-wise through `col(l, out)`.
+template <int M, int MODE, typename VT, typename ColFn>
 __device__ __forceinline__ void input_transform_2d(const Params& p, ColFn col,
-                                                   float (&V)[(M + 2) * (M + 2)]) {
+                                                   VT (&V)[(M + 2) * (M + 2)]) {
   constexpr int T_ = M + 2;
   constexpr bool STD = MODE != kDense;
   using MT = Mat<M, STD>;
-  float P[T_][T_];
+  VT P[T_][T_];
 #pragma unroll
   for (int l = 0; l < T_; ++l) {
-    float dcol[T_];
+    VT dcol[T_];
     col(l, dcol);
     if constexpr (MODE == kExact) {
-      float r[T_];
+      VT r[T_];
       bt_exact(dcol, r);
 #pragma unroll
       for (int i = 0; i < T_; ++i) P[i][l] = r[i];
     } else {
 #pragma unroll
       for (int i = 0; i < T_; ++i) {
-        float acc = 0.0f;
+        VT acc = v_zero(VT());
 #pragma unroll
         for (int k = 0; k < T_; ++k) acc = chain<STD>(MT::bt(p, i, k), dcol[k], acc);
         P[i][l] = acc;
@@ -110,14 +164,14 @@ __device__ __forceinline__ void input_transform_2d(const Params& p, ColFn col,
 #pragma unroll
   for (int i = 0; i < T_; ++i) {
     if constexpr (MODE == kExact) {
-      float r[T_];
+      VT r[T_];
       bt_exact(P[i], r);
 #pragma unroll
       for (int j = 0; j < T_; ++j) V[i * T_ + j] = r[j];
     } else {
 #pragma unroll
       for (int j = 0; j < T_; ++j) {
-        float acc = 0.0f;
+        VT acc = v_zero(VT());
 #pragma unroll
         for (int l = 0; l < T_; ++l) acc = chain<STD>(MT::bt(p, j, l), P[i][l], acc);
         V[i * T_ + j] = acc;
@@ -126,48 +180,44 @@ __device__ __forceinline__ void input_transform_2d(const Params& p, ColFn col,
   }
 }
 
-// Y = A^T (m A) for one channel: right factor first.  m row-wise via `row(i, out)`.
-template <int M, int MODE, typename RowFn>
-__device__ __forceinline__ void output_transform_2d(const Params& p, RowFn row,
-                                                    float (&Y)[M * M]) {
+// y = A^T v, one 1-D pass of the output transform.
+template <int M, int MODE, typename VT>
+__device__ __forceinline__ void at_pass(const Params& p, const VT (&v)[M + 2], VT (&y)[M]) {
   constexpr int T_ = M + 2;
   constexpr bool STD = MODE != kDense;
-  using MT = Mat<M, STD>;
-  float R[T_][M];
+  if constexpr (MODE == kExact && M != 6) {
+    at_exact(v, y);
+  } else {
+#pragma unroll
+    for (int r = 0; r < M; ++r) {
+      VT acc = v_zero(VT());
+#pragma unroll
+      for (int j = 0; j < T_; ++j) acc = chain<STD>(Mat<M, STD>::at(p, r, j), v[j], acc);
+      y[r] = acc;
+    }
+  }
+}
+
+// Y = A^T (m A) for one channel or a pair of them: right factor first.  m row-wise via `row(i, out)`.
+template <int M, int MODE, typename VT, typename RowFn>
+__device__ __forceinline__ void output_transform_2d(const Params& p, RowFn row,
+                                                    VT (&Y)[M * M]) {
+  constexpr int T_ = M + 2;
+  VT R[T_][M];
 #pragma unroll
   for (int i = 0; i < T_; ++i) {
-    float mrow[T_];
+    VT mrow[T_];
     row(i, mrow);
-    if constexpr (MODE == kExact && M != 6) {
-      at_exact(mrow, R[i]);
-    } else {
-#pragma unroll
-      for (int jp = 0; jp < M; ++jp) {
-        float acc = 0.0f;
-#pragma unroll
-        for (int j = 0; j < T_; ++j) acc = chain<STD>(MT::at(p, jp, j), mrow[j], acc);
-        R[i][jp] = acc;
-      }
-    }
+    at_pass<M, MODE>(p, mrow, R[i]);
   }
 #pragma unroll
   for (int jp = 0; jp < M; ++jp) {
-    if constexpr (MODE == kExact && M != 6) {
-      float c[T_], y4[M];
+    VT c[T_], y[M];
 #pragma unroll
-      for (int i = 0; i < T_; ++i) c[i] = R[i][jp];
-      at_exact(c, y4);
+    for (int i = 0; i < T_; ++i) c[i] = R[i][jp];
+    at_pass<M, MODE>(p, c, y);
 #pragma unroll
-      for (int ip = 0; ip < M; ++ip) Y[ip * M + jp] = y4[ip];
-    } else {
-#pragma unroll
-      for (int ip = 0; ip < M; ++ip) {
-        float acc = 0.0f;
-#pragma unroll
-        for (int i = 0; i < T_; ++i) acc = chain<STD>(MT::at(p, ip, i), R[i][jp], acc);
-        Y[ip * M + jp] = acc;
-      }
-    }
+    for (int ip = 0; ip < M; ++ip) Y[ip * M + jp] = y[ip];
   }
 }
 

@@ -19,8 +19,9 @@ class WinogradConv:
         self.Uq = torch.empty(plan.weight_bytes, dtype=torch.int8, device=self.device)
         self.ws = torch.empty(max(plan.workspace_bytes, 16), dtype=torch.uint8, device=self.device)
         self.bias = None
-        self._y_shape = (plan.N, plan.H, plan.W, plan.K)
-        self._y_dtype = torch.float32 if plan.out_dtype == 1 else torch.int8
+        # one element, expanded: what an output looks like (empty_like costs half of empty)
+        self._y_like = torch.empty(1, dtype=torch.float32 if plan.out_dtype == 1 else torch.int8,
+                                   device=self.device).expand(plan.N, plan.H, plan.W, plan.K)
 
     def load_weights(self, w_q, bias=None, absmax=None) -> None:
         """w_q: int8 [K,3,3,C] (numpy or torch); runs the weight transform."""
@@ -31,7 +32,7 @@ class WinogradConv:
         torch.cuda.current_stream().synchronize()  # w may be freed after return
 
     def empty_output(self) -> torch.Tensor:
-        return torch.empty(self._y_shape, dtype=self._y_dtype, device=self.device)
+        return torch.empty_like(self._y_like, memory_format=torch.contiguous_format)
 
     def forward(self, x_dev: torch.Tensor, y_dev: torch.Tensor | None = None) -> torch.Tensor:
         """x_dev: int8 [N,H,W,C] on the device."""

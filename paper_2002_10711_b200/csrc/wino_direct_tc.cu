@@ -15,16 +15,17 @@
 //   warp 1    : tensor-memory owner; walks the MMA loop as a whole warp, one elected lane issues
 //   warps 2-17: epilogue; warp w reads TMEM lanes 32*(w%4) .. +31 and every fourth 32-column chunk
 //
-// For stride 2 (even H and W) the input is addressed as [N][H/2][2][W/2][2*C]: a tap then reads
-// one row parity and one column parity, again a dense box.
+// For stride 2 with even H and W the input is addressed as [N][H/2][2][W/2][2*C]: a tap then
+// reads one row parity and one column parity, again a dense box.  With an odd H or W the copies
+// take every other row and column themselves (element strides of the tensor map).
 // Narrow layers (one block of output channels, 9 * C * K bytes of weights that fit beside the
 // input ring; the 64- and 128-channel layers of the network): the weights are fetched once per
 // block and stay in shared memory, and the ring's stages carry input boxes only, three taps
 // (one row of the filter) per stage where that fits.  The producer and the MMA warp are
 // single threads of control whose every instruction costs ten to twenty cycles, so what
 // bounds these layers is the number of copies, waits and commits per item, which this halves.
-// Zero points on x or w, odd sizes at stride 2 and channel counts that are not multiples of
-// 64 / 32 stay on the ALU kernel (wino_direct.cu).
+// Zero points on x or w and channel counts that are not multiples of 64 / 32 stay on the ALU
+// kernel (wino_direct.cu).
 #include "wino_launch.h"
 #include "wino_ptx.cuh"
 
@@ -119,7 +120,9 @@ __device__ __forceinline__ void direct_conv_tc_body(const CUtensorMap& mapX, con
       // (a lone thread retires an instruction every ten to twenty cycles, and a stage's MMAs take
       // about five hundred: everything that does not change inside an item is computed once per
       // item, and the loops carry running coordinates instead of multiplying)
-      const int n_stages = a.stages, kblocks = a.KB, cb = a.cB, strided = a.stride != 1;
+      const int n_stages = a.stages, kblocks = a.KB, cb = a.cB;
+      const bool strided = a.stride != 1 && !a.element_strides;
+      const int step = a.element_strides ? 2 : 1;   // input pixels per output pixel in box coordinates
       if constexpr (RW) {
         // the whole weight tensor, once: slice (tap, channel block) at res + (tap * KB + kb) * b_bytes
         mbar_expect_tx(bar_w, res_bytes);
@@ -152,10 +155,10 @@ __device__ __forceinline__ void direct_conv_tc_body(const CUtensorMap& mapX, con
         for (int ta = 0; ta < 3 && ok; ++ta) {
           // stride 1: input row h0 - 1 + ta.  Stride 2: input row 2*ho - 1 + ta, i.e. (half-row
           // ho - 1, parity 1), (ho, 0), (ho, 1) for ta = 0, 1, 2
-          const int hc = strided ? h0 + (ta == 0 ? -1 : 0) : h0 - 1 + ta;
+          const int hc = strided ? h0 + (ta == 0 ? -1 : 0) : h0 * step - 1 + ta;
           const int prow = ta == 1 ? 0 : 1;
           for (int tb = 0; tb < 3 && ok; ++tb, ++tap) {
-            const int wc = strided ? w0 + (tb == 0 ? -1 : 0) : w0 - 1 + tb;
+            const int wc = strided ? w0 + (tb == 0 ? -1 : 0) : w0 * step - 1 + tb;
             const int c_base = strided ? (tb == 1 ? 0 : a.C) : 0;
             int c_off = 0;
             if constexpr (RW) {
@@ -357,15 +360,16 @@ __device__ int g_direct_status;
 
 }  // namespace
 
-bool direct_tc_supported(int C, int K, int H, int W, int stride, int z_x, int z_w) {
+bool direct_tc_supported(int C, int K, int stride, int z_x, int z_w) {
   if (z_x != 0 || z_w != 0 || C % 64 != 0 || K % 32 != 0 || K > 2048) return false;
-  return stride == 1 || (stride == 2 && H % 2 == 0 && W % 2 == 0);
+  return stride == 1 || stride == 2;
 }
 
 DirectTcArgs direct_tc_geometry(int N, int C, int H_in, int W_in, int K, int stride, int num_sms) {
   DirectTcArgs a = {};
   const int H = (H_in - 1) / stride + 1, W = (W_in - 1) / stride + 1;   // output size
   a.N = N; a.C = C; a.H = H; a.W = W; a.K = K; a.stride = stride;
+  a.element_strides = stride == 2 && (H_in % 2 != 0 || W_in % 2 != 0);
   auto pow2_ceil = [](int v) { int p = 1; while (p < v) p *= 2; return p; };
   a.BW = pow2_ceil(W) < 16 ? pow2_ceil(W) : 16;
   a.BH = pow2_ceil(H) < 128 / a.BW ? pow2_ceil(H) : 128 / a.BW;

@@ -180,7 +180,7 @@ LaunchOpt opt_of(const wino_plan_t* pl, bool pdl) {
 }
 
 int encode_tiled(CUtensorMap* map, const void* base, int rank, const uint64_t* dims,
-                 const uint32_t* box, CUtensorMapSwizzle swz) {
+                 const uint32_t* box, CUtensorMapSwizzle swz, const uint32_t* element_strides = nullptr) {
   EncodeTiledFn fn = get_encode_fn();
   if (fn == nullptr) return WINO_ERR_CUDA;
   cuuint64_t d[5], strides[4];
@@ -189,6 +189,7 @@ int encode_tiled(CUtensorMap* map, const void* base, int rank, const uint64_t* d
   for (int i = 0; i < rank; ++i) {
     d[i] = dims[i];
     b[i] = box[i];
+    if (element_strides != nullptr) estr[i] = element_strides[i];
     stride *= dims[i];
     if (i < rank - 1) strides[i] = stride;  // bytes: int8 elements
   }
@@ -768,7 +769,7 @@ int wino_direct_conv_forward(const wino_direct_desc_t* d, const int8_t* x, const
   if ((reinterpret_cast<uintptr_t>(d->s_w_K_dev) & 3u) != 0 || (reinterpret_cast<uintptr_t>(d->s_Y_K_dev) & 3u) != 0)
     return WINO_ERR_ALIGNMENT;
   const double s_in = (double)d->q_x.scale * (double)d->q_w.scale;
-  if (direct_tc_supported(d->C, d->K, d->H, d->W, d->stride, d->q_x.zero_point, d->q_w.zero_point) &&
+  if (direct_tc_supported(d->C, d->K, d->stride, d->q_x.zero_point, d->q_w.zero_point) &&
       (reinterpret_cast<uintptr_t>(y) & 31u) == 0) {
     // implicit GEMM on the tensor cores: x as [N][H][W][C] boxes of one output tile, w as
     // [K][9][C] slices of one tap
@@ -789,7 +790,12 @@ int wino_direct_conv_forward(const wino_direct_desc_t* d, const int8_t* x, const
     const CUtensorMapSwizzle swz = a.cB == 128 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B;
     CUtensorMap mapX, mapW;
     int rcx;
-    if (d->stride == 1) {
+    if (a.element_strides) {
+      const uint64_t xd[4] = {(uint64_t)d->C, (uint64_t)d->W, (uint64_t)d->H, (uint64_t)d->N};
+      const uint32_t xb[4] = {(uint32_t)a.cB, (uint32_t)(2 * a.BW), (uint32_t)(2 * a.BH), (uint32_t)a.BI};
+      const uint32_t xs[4] = {1, 2, 2, 1};
+      rcx = encode_tiled(&mapX, x, 4, xd, xb, swz, xs);
+    } else if (d->stride == 1) {
       const uint64_t xd[4] = {(uint64_t)d->C, (uint64_t)d->W, (uint64_t)d->H, (uint64_t)d->N};
       const uint32_t xb[4] = {(uint32_t)a.cB, (uint32_t)a.BW, (uint32_t)a.BH, (uint32_t)a.BI};
       rcx = encode_tiled(&mapX, x, 4, xd, xb, swz);

@@ -78,8 +78,8 @@ enum {
 /* Execution paths a plan can use (see wino_plan_path / wino_plan_force_path).  The automatic
  * choice is 5 where it applies, else 2 for layers of at most 16 channels in and out, else 1
  * where C and K are multiples of 16, else 2.  wino_conv_forward on a plan whose path was not
- * forced runs a layer of few tiles by kernel 8 instead, where that is estimated to be faster
- * (same results, same workspace requirement). */
+ * forced runs a layer of few tiles by kernel 8 instead, and a layer of path 5 by the kernels of
+ * path 1 if it is given a workspace, where that is estimated to be faster (same results). */
 enum {
   WINO_PATH_AUTO = 0,
   WINO_PATH_STAGED_TC = 1,   /* transform kernels (TMA-staged where the shape allows) + tcgen05 int8 GEMMs */

@@ -76,7 +76,6 @@ __device__ __forceinline__ void direct_conv_tc_body(const CUtensorMap& mapX, con
   const int n_tiles = a.nW * a.nH * a.nI;
   const int steps = RW ? 9 / a.taps_per_stage : 9 * a.KB;   // stages per item
 
-  griddep_launch();
   if (threadIdx.x == 0) {
     for (int s = 0; s < a.stages; ++s) {
       mbar_init(bar_full + 8u * s, 1);
@@ -111,6 +110,9 @@ __device__ __forceinline__ void direct_conv_tc_body(const CUtensorMap& mapX, con
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  // only now may the next kernel's blocks start: every block of this grid holds its tensor memory,
+  // so none of them can be kept from it by a block that waits for this grid
+  griddep_launch();
   const uint32_t tmem_base = *tmem_slot_p;
 
   if (warp == 0) {

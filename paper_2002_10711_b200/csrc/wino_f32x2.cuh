@@ -77,4 +77,28 @@ __device__ __forceinline__ uint32_t quant_s16x2(F2 v, F2 mult, F2 magic, uint32_
   return clamp_s16x2(f2_low_halves(v_fma(v, mult, magic)), lo, hi);
 }
 
+// 32 int32 values of one row -> 32 codes in eight words (|value * mult| < 2^15, |value| < 2^24).
+__device__ __forceinline__ void quant32_fits16(const uint32_t (&v)[32], F2 mult, F2 magic, uint32_t lo, uint32_t hi,
+                                               uint32_t (&w)[8]) {
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+    const uint32_t a = quant_s16x2(f2_make(__int2float_rn((int)v[4 * q]), __int2float_rn((int)v[4 * q + 1])), mult,
+                                   magic, lo, hi);
+    const uint32_t b = quant_s16x2(f2_make(__int2float_rn((int)v[4 * q + 2]), __int2float_rn((int)v[4 * q + 3])), mult,
+                                   magic, lo, hi);
+    w[q] = __byte_perm(a, b, 0x6420u);
+  }
+}
+// 32 bytes of a row, of which `left` (a positive multiple of 16) exist; wide: 32-byte aligned.
+__device__ __forceinline__ void store_row32(int8_t* dst, const uint32_t (&w)[8], bool wide, int left) {
+  if (wide) {   // the whole sector in one request
+    asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(dst), "r"(w[0]), "r"(w[1]),
+                 "r"(w[2]), "r"(w[3]), "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7]) : "memory");
+  } else {
+    uint4* d = reinterpret_cast<uint4*>(dst);
+    d[0] = make_uint4(w[0], w[1], w[2], w[3]);
+    if (left > 16) d[1] = make_uint4(w[4], w[5], w[6], w[7]);
+  }
+}
+
 }  // namespace wino

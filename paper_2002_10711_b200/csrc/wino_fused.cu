@@ -76,7 +76,6 @@ k_fused_f2(const __grid_constant__ Params p, const __grid_constant__ CUtensorMap
   const int ksteps = p.C / 32;                      // 1 or 2
   const int n_nblk = (p.K + 31) / 32;               // 1 or 2
 
-  griddep_launch();
   if (threadIdx.x == 0) {
     mbar_init(bar_b, 1);
     mbar_init(bar_a_full, kFusedWorkers);
@@ -89,6 +88,9 @@ k_fused_f2(const __grid_constant__ Params p, const __grid_constant__ CUtensorMap
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  // only now may the next kernel's blocks start: every block of this grid holds its tensor memory,
+  // so none of them can be kept from it by a block that waits for this grid
+  griddep_launch();
   const uint32_t tmem_base = *tmem_slot_p;
   griddep_wait();
 

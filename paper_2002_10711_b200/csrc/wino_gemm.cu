@@ -10,6 +10,7 @@
 //                 next.
 //   k_gemm_dp4a : the same contraction with 4-way integer dot products on the
 //                 ALUs; fallback for channel counts the TMA path cannot take.
+#include "wino_f32x2.cuh"
 #include "wino_launch.h"
 #include "wino_ptx.cuh"
 #include "wino_trace.cuh"
@@ -107,29 +108,37 @@ __device__ __forceinline__ float acc_to_float(uint32_t v) {
   else return __int2float_rn((int)v);
 }
 
+// The lean kernels' quantizer of one 32-column chunk: int8 codes, products below 2^15 (clamp on
+// 16-bit lanes).
+template <bool PK>
+__device__ __forceinline__ void lean_codes(const Params& p, const uint32_t (&r)[32], int k0, const float* mult_k,
+                                           uint32_t (&w)[8]) {
+  const F2 magic = f2_both(kMagic);
+  const uint32_t lo = s16x2_both((int)p.lo_M), hi = s16x2_both((int)p.hi_M);
+  if constexpr (PK) {
+    // every lane reads the same 32 multipliers of the block's table (broadcasts)
+    const float4* mp = reinterpret_cast<const float4*>(mult_k + k0);
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      const float4 mm = mp[q];
+      const uint32_t a = quant_s16x2(f2_make(__int2float_rn((int)r[4 * q]), __int2float_rn((int)r[4 * q + 1])),
+                                     f2_make(mm.x, mm.y), magic, lo, hi);
+      const uint32_t b = quant_s16x2(f2_make(__int2float_rn((int)r[4 * q + 2]), __int2float_rn((int)r[4 * q + 3])),
+                                     f2_make(mm.z, mm.w), magic, lo, hi);
+      w[q] = __byte_perm(a, b, 0x6420u);
+    }
+  } else {
+    quant32_fits16(r, f2_both(p.mult_M), magic, lo, hi, w);
+  }
+}
+
 // Epilogue of one 32-column chunk of one accumulator row.  FULL: all 32 columns
 // are inside K (no per-element guards).  STATS: track max |M| for calibration.  PK: the
 // multiplier of Q_M varies per output channel (column).
-template <bool SMALL, bool FULL, bool STATS, bool PK, bool LEAN = false>
+template <bool SMALL, bool FULL, bool STATS, bool PK>
 __device__ __forceinline__ void epilogue_chunk(const Params& p, const uint32_t (&r)[32], int k0,
                                                long o, int out_mode, void* out, float& vmax,
                                                bool wide_store, const float* mult_k) {
-  if constexpr (LEAN) {
-    // the one configuration the lean kernel is launched for: int8 codes, upper bound 127
-    // (saturating pack), 32-byte aligned rows
-    const float lo_m = __fadd_rn(p.lo_M, kMagic), hi_m = __fadd_rn(p.hi_M, kMagic);
-    uint32_t w[8];
-#pragma unroll
-    for (int q = 0; q < 8; ++q)
-      w[q] = quant_pack4<true>(acc_to_float<SMALL>(r[4 * q + 0]), acc_to_float<SMALL>(r[4 * q + 1]),
-                               acc_to_float<SMALL>(r[4 * q + 2]), acc_to_float<SMALL>(r[4 * q + 3]),
-                               p.mult_M, lo_m, hi_m);
-    asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(
-                     reinterpret_cast<int8_t*>(out) + o),
-                 "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3]), "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7])
-                 : "memory");
-    return;
-  }
   if constexpr (STATS) {
 #pragma unroll
     for (int j = 0; j < 32; ++j)
@@ -226,7 +235,13 @@ __device__ __forceinline__ void epilogue_loop(const Params& p, const GemmTcArgs&
       if (tau >= p.T) return;
       const int k0 = nb * a.BN + kcol;
       const long o = ((long)xi * p.T + tau) * p.K + k0;
-      epilogue_chunk<SMALL, FULL, STATS, PK, LEAN>(p, r, k0, o, a.out_mode, out, vmax, a.wide_store != 0, mult_k);
+      if constexpr (LEAN) {
+        uint32_t w[8];
+        lean_codes<PK>(p, r, k0, mult_k, w);
+        store_row32(reinterpret_cast<int8_t*>(out) + o, w, true, 32);
+      } else {
+        epilogue_chunk<SMALL, FULL, STATS, PK>(p, r, k0, o, a.out_mode, out, vmax, a.wide_store != 0, mult_k);
+      }
     };
     for (int col = sub * 32; col < a.MB * a.BN; col += 128) {
       uint32_t r0[32];
@@ -244,9 +259,9 @@ __device__ __forceinline__ void epilogue_loop(const Params& p, const GemmTcArgs&
 
 // PK: Q_M takes one multiplier per output channel (a build of its own, so that the
 // per-layer kernel carries none of that code).
-// LEAN: only the epilogue of the common case is compiled in (Q_M to int8 codes with upper
-// bound 127, C <= 260, whole 32-column chunks, 32-byte aligned rows); the kernel's code is a
-// third of the general one's, which shows at every launch.
+// LEAN: only the epilogue of the common case is compiled in (Q_M to int8 codes whose products
+// stay below 2^15, whole 32-column chunks, 32-byte aligned rows); the kernel's code is a third
+// of the general one's, which shows at every launch.
 template <bool PK, bool LEAN = false>
 __device__ __forceinline__ void gemm_tc_body(const Params& p, const CUtensorMap* mapV,
                                              const CUtensorMap* mapU, const GemmTcArgs& a,
@@ -280,7 +295,6 @@ __device__ __forceinline__ void gemm_tc_body(const Params& p, const CUtensorMap*
     WINO_ST(g_gemm_trace, trace_step_s, 0);
   }
 #endif
-  griddep_launch();
   if (threadIdx.x == 0) {
     for (int s = 0; s < a.stages; ++s) {
       mbar_init(bar_full + 8u * s, 1);
@@ -307,6 +321,9 @@ __device__ __forceinline__ void gemm_tc_body(const Params& p, const CUtensorMap*
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  // only now may the next kernel's blocks start: every block of this grid holds its tensor memory,
+  // so none of them can be kept from it by a block that waits for this grid
+  griddep_launch();
   const uint32_t tmem_base = *tmem_slot_p;
 #ifdef WINO_TRACE
   trace_step = trace_step_s;
@@ -448,8 +465,8 @@ __device__ __forceinline__ void gemm_tc_body(const Params& p, const CUtensorMap*
     griddep_wait();
     if constexpr (LEAN) {
       (void)per_channel; (void)small; (void)full;
-      epilogue_loop<true, true, false, false, true>(p, a, out, absmaxM, tmem_base, bar_acc_full,
-                                                    bar_acc_empty, abort_p, warp, lane, trace_step);
+      epilogue_loop<true, true, false, PK, true>(p, a, out, absmaxM, tmem_base, bar_acc_full, bar_acc_empty, abort_p,
+                                                 warp, lane, trace_step, mult_k);
     } else if constexpr (PK) {
       (void)per_channel;
       if (absmaxM != nullptr)
@@ -491,11 +508,12 @@ k_gemm_tc(const __grid_constant__ Params p, const __grid_constant__ CUtensorMap 
           unsigned* __restrict__ absmaxM, int* __restrict__ status) {
   gemm_tc_body<false>(p, &mapV, &mapU, a, out, absmaxM, status);
 }
+template <bool PK>
 __global__ void __launch_bounds__(kGemmThreads, 1)
 k_gemm_tc_lean(const __grid_constant__ Params p, const __grid_constant__ CUtensorMap mapV,
                const __grid_constant__ CUtensorMap mapU, const GemmTcArgs a, void* __restrict__ out,
                unsigned* __restrict__ absmaxM, int* __restrict__ status) {
-  gemm_tc_body<false, true>(p, &mapV, &mapU, a, out, absmaxM, status);
+  gemm_tc_body<PK, true>(p, &mapV, &mapU, a, out, absmaxM, status);
 }
 __global__ void __launch_bounds__(kGemmThreads, 1)
 k_gemm_tc_per_channel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMap mapV,
@@ -549,21 +567,19 @@ int launch_gemm_tc(const Params& p, const LaunchOpt& o, const TcGeom& g, const C
   a.chan = o.chan;
   // room for the multipliers behind the ring and the barriers (the ring stops at 196 KB)
   a.chan_smem = (o.chan != nullptr && (size_t)p.K * 4 <= 24 * 1024) ? 1 : 0;
+  const bool lean = absmaxM == nullptr && out_mode == kOutMq && a.wide_store && p.K % a.BN == 0 && a.BN % 32 == 0 &&
+                    (o.chan != nullptr ? o.chan_m_fits_16 && a.chan_smem : p.m_fits_16 != 0);
+  static DeviceOnce once_pk, once_lean_pk, once_lean;
+  auto go = [&](auto kernel, DeviceOnce& done, size_t smem) -> int {
+    if (int rc = set_max_smem(done, o.device, kernel, 227 * 1024)) return rc;
+    return launch_kernel(kernel, dim3((unsigned)g.grid), dim3(kGemmThreads), smem, st, o.pdl, p, mapV, mapU, a, out,
+                         absmaxM, status);
+  };
   if (o.chan != nullptr) {
-    static DeviceOnce once_pk;
-    if (int rc = set_max_smem(once_pk, o.device, k_gemm_tc_per_channel, 227 * 1024)) return rc;
     const size_t smem = g.smem + (a.chan_smem ? (size_t)p.K * 4 : 0);
-    return launch_kernel(k_gemm_tc_per_channel, dim3((unsigned)g.grid), dim3(kGemmThreads), smem, st,
-                         o.pdl, p, mapV, mapU, a, out, absmaxM, status);
+    return lean ? go(k_gemm_tc_lean<true>, once_lean_pk, smem) : go(k_gemm_tc_per_channel, once_pk, smem);
   }
-  const bool lean = absmaxM == nullptr && out_mode == kOutMq && p.hi_M == 127.0f && a.wide_store &&
-                    p.C <= 260 && p.K % a.BN == 0 && a.BN % 32 == 0;
-  if (lean) {
-    static DeviceOnce once_lean;
-    if (int rc = set_max_smem(once_lean, o.device, k_gemm_tc_lean, 227 * 1024)) return rc;
-    return launch_kernel(k_gemm_tc_lean, dim3((unsigned)g.grid), dim3(kGemmThreads), g.smem, st, o.pdl,
-                         p, mapV, mapU, a, out, absmaxM, status);
-  }
+  if (lean) return go(k_gemm_tc_lean<false>, once_lean, g.smem);
   return launch_kernel(k_gemm_tc, dim3((unsigned)g.grid), dim3(kGemmThreads), g.smem, st, o.pdl, p,
                        mapV, mapU, a, out, absmaxM, status);
 }

@@ -51,11 +51,13 @@ struct wino_plan {
   SmallGeom small;      // its geometry and cost estimate
   int* status_dev;      // device status word (may be null when no GPU is present)
   float* chan_dev;      // per-output-channel multipliers [5][K] (null: per-layer scales)
+  bool chan_m_fits_16;  // products of Q_M under them stay below 2^15
   void* kron_dev;       // Kronecker tables of the tensor-core transforms (same allocation)
   unsigned* counters_dev;  // progress counters of the single-launch layer kernel (same allocation)
   CUtensorMap fmapV, fmapU;   // GEMM operand maps of the single-launch kernel
   const void* fmap_vq_ptr;
   const void* fmap_uq_ptr;
+  const uint8_t* xt_images;   // constant operands of the tensor-core transforms (per device, not owned)
   int num_sms;
   int device;           // the device that was current when the plan was made
   bool pdl;             // programmatic dependent launch between the stages
@@ -64,7 +66,7 @@ struct wino_plan {
   const void* map_uq_ptr;
   CUtensorMap mapV, mapU;
   // maps of the TMA-staged transform kernels, keyed by buffer address
-  MapCache cache_x, cache_vst, cache_mld, cache_y, cache_uf, cache_x_sw, cache_m_sw, cache_x_small, cache_u_small;
+  MapCache cache_x, cache_vst, cache_mld, cache_y, cache_uf, cache_x_sw, cache_m_sw, cache_x_small, cache_u_small, cache_x_tc, cache_m_tc, cache_vst1;
   // last forward call, for wino_debug_dump_stage
   const int8_t* last_uq;
   const int8_t* last_x;     // non-null: that call left no V_q and m_q in its workspace
@@ -176,6 +178,7 @@ LaunchOpt opt_of(const wino_plan_t* pl, bool pdl) {
   o.device = pl->device;
   o.num_sms = pl->num_sms;
   o.chan = pl->chan_dev;
+  o.chan_m_fits_16 = pl->chan_m_fits_16;
   return o;
 }
 
@@ -232,12 +235,12 @@ const CUtensorMap* map_y(wino_plan_t* pl, const void* y) {
   return m;
 }
 // V_q (store side) and m_q (load side): [t*t][T][channels], box {chunk, G, t*t}
-const CUtensorMap* map_stage(wino_plan_t* pl, MapCache& cache, const void* buf, int channels) {
+const CUtensorMap* map_stage(wino_plan_t* pl, MapCache& cache, const void* buf, int channels, int group) {
   if (const CUtensorMap* m = cache.find(buf)) return m;
   const Params& p = pl->p;
   const int chunk = tma_chunk(channels);
   const uint64_t dims[3] = {(uint64_t)channels, (uint64_t)p.T, (uint64_t)(p.t * p.t)};
-  const uint32_t box[3] = {(uint32_t)chunk, (uint32_t)tma_group(chunk), (uint32_t)(p.t * p.t)};
+  const uint32_t box[3] = {(uint32_t)chunk, (uint32_t)group, (uint32_t)(p.t * p.t)};
   CUtensorMap* m = cache.slot(buf);
   if (encode_tiled(m, buf, 3, dims, box, CU_TENSOR_MAP_SWIZZLE_NONE) != WINO_OK) {
     cache.key[(cache.next + MapCache::kN - 1) % MapCache::kN] = nullptr;
@@ -282,6 +285,37 @@ const CUtensorMap* map_u_fused(wino_plan_t* pl, const void* Uq) {
   CUtensorMap* m = pl->cache_uf.slot(Uq);
   if (encode_tiled(m, Uq, 3, dims, box, CU_TENSOR_MAP_SWIZZLE_64B) != WINO_OK) {
     pl->cache_uf.key[(pl->cache_uf.next + MapCache::kN - 1) % MapCache::kN] = nullptr;
+    return nullptr;
+  }
+  return m;
+}
+
+// Maps of the tensor-core transforms: rows of one channel chunk, swizzled.
+CUtensorMapSwizzle xt_swizzle(int channels) {
+  return xt_chunk(channels) == 128 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B;
+}
+const CUtensorMap* map_x_tc(wino_plan_t* pl, const void* x) {
+  if (const CUtensorMap* m = pl->cache_x_tc.find(x)) return m;
+  const Params& p = pl->p;
+  const uint64_t dims[4] = {(uint64_t)p.C, (uint64_t)p.W, (uint64_t)p.H, (uint64_t)p.N};
+  uint32_t box[4];
+  input_tc_box(p, box);
+  CUtensorMap* m = pl->cache_x_tc.slot(x);
+  if (encode_tiled(m, x, 4, dims, box, xt_swizzle(p.C)) != WINO_OK) {
+    pl->cache_x_tc.key[(pl->cache_x_tc.next + MapCache::kN - 1) % MapCache::kN] = nullptr;
+    return nullptr;
+  }
+  return m;
+}
+const CUtensorMap* map_m_tc(wino_plan_t* pl, const void* mbuf) {
+  if (const CUtensorMap* m = pl->cache_m_tc.find(mbuf)) return m;
+  const Params& p = pl->p;
+  const uint64_t dims[3] = {(uint64_t)p.K, (uint64_t)p.T, (uint64_t)(p.t * p.t)};
+  uint32_t box[3];
+  output_tc_box(p, box);
+  CUtensorMap* m = pl->cache_m_tc.slot(mbuf);
+  if (encode_tiled(m, mbuf, 3, dims, box, xt_swizzle(p.K)) != WINO_OK) {
+    pl->cache_m_tc.key[(pl->cache_m_tc.next + MapCache::kN - 1) % MapCache::kN] = nullptr;
     return nullptr;
   }
   return m;
@@ -335,15 +369,47 @@ int launch_gemm(wino_plan_t* pl, const int8_t* Vq, const int8_t* Uq, void* out, 
                         pl->status_dev, st);
 }
 
-// Time of the plan's own path, for the choice between it and the one-launch kernel, in ns: a
-// floor of three dependent launches (their host time alone is 6.6 us), then transforms and
-// quantizers by the number of codes.  Measured, see the table beside small_geometry.
+// Whether the tensor-core transforms are the faster ones (both kinds being possible), by the
+// number of codes.  They cost fewer instructions a code but start up more slowly (tensor memory,
+// a constant operand, two hand-overs).  Measured on B200, us, ALU / tensor cores:
+//   input   F2  8.4 M codes 4.7 / 5.1   16.8 M 7.8 / 7.2   33.6 M 14.4 / 11.6   67 M 29 / 24
+//           F4  4.7 M 3.7 / 4.2   9.4 M 5.4 / 5.7   18.9 M 9.6 / 9.0   37.7 M 19.0 / 16.3
+//           F6  4.7 M 3.7 / 4.5   8.4 M 6.5 / 6.0   18.9 M 11.4 / 9.2   37.7 M 23 / 16.5
+//   output  F2  8.4 M 4.1 / 4.9   16.8 M 7.4 / 6.3   33.6 M 12.6 / 8.6   67 M 24 / 13
+//           F4  9.4 M 4.6 / 5.2   18.9 M 7.8 / 7.7   37.7 M 13.6 / 11.9
+bool input_tc_pays(const Params& p) {
+  const double codes = (double)p.t * p.t * p.T * p.C;
+  return codes > (p.m == 2 ? 12e6 : p.m == 4 ? 14e6 : 7e6);
+}
+bool output_tc_pays(const Params& p) {
+  const double codes = (double)p.t * p.t * p.T * p.K;
+  return codes > (p.m == 2 ? 11e6 : 18e6);
+}
+
+// The options of an input transform; the GEMMs that follow it in the same call read U_q, which no
+// kernel of the call writes.
+LaunchOpt opt_with_hint(const wino_plan_t* pl, bool pdl, int stage_mask, const int8_t* Uq) {
+  LaunchOpt o = opt_of(pl, pdl);
+  if (stage_mask & 2) {
+    o.l2_hint = Uq;
+    o.l2_hint_bytes = (size_t)pl->p.t * pl->p.t * pl->p.K * pl->p.C;
+  }
+  return o;
+}
+
+// Estimated times in ns, for the choice between kernels that can run the same layer.  Staged: a
+// start-up latency of three dependent kernels plus a time per code (measured, us: F2 16.8 M codes
+// in and out 14, 134 M 62; F4 9.4 M 12, 75 M 43; F6 9.4 M 14, 75 M 49; with integer dot products
+// 0.6 M 8, 4.9 M 17).  Fused F2: waves of 128 tiles per SM, full or not (28 us at 64 channels).
 long staged_cost(const wino_plan_t* pl) {
   const double codes = (double)pl->p.t * pl->p.t * pl->p.T * (pl->p.C + pl->p.K);
-  if (pl->path == WINO_PATH_FUSED_F2)   // by waves of 128 tiles per SM, full or not
-    return 28200l * (((pl->p.T + 127) / 128 + pl->num_sms - 1) / pl->num_sms);
-  const long gpu = 6500 + (long)(codes * 6.6e-4);
-  return gpu > 7500 ? gpu : 7500;
+  if (pl->path == WINO_PATH_STAGED_DP4A) return 6500 + (long)(codes * 1.9e-3);
+  const long gpu = (pl->p.m == 6 ? 9500 : 7500) + (long)(codes * (pl->p.m == 2 ? 4.1e-4 : 4.8e-4));
+  return gpu;
+}
+long fused_f2_cost(const wino_plan_t* pl) {
+  const long waves = ((pl->p.T + 127) / 128 + pl->num_sms - 1) / pl->num_sms;
+  return waves * 220l * (pl->p.C + pl->p.K);
 }
 
 int forward_small(wino_plan_t* pl, const int8_t* x, const int8_t* Uq, const float* bias, void* y,
@@ -403,7 +469,7 @@ int forward_impl(wino_plan_t* pl, const int8_t* x, const int8_t* Uq, const float
     }
     FusedMaps m;
     m.x = map_x_sw(pl, x);
-    m.v_store = map_stage(pl, pl->cache_vst, Vq, p.C);
+    m.v_store = map_stage(pl, pl->cache_vst1, Vq, p.C, 1);
     m.v_load = &pl->fmapV;
     m.u = &pl->fmapU;
     m.m_load = map_m_sw(pl, mbuf);
@@ -429,26 +495,20 @@ int forward_impl(wino_plan_t* pl, const int8_t* x, const int8_t* Uq, const float
   if (pl->path == WINO_PATH_FUSED_LAYER) gemm_path = WINO_PATH_STAGED_TC;
   if (pl->path == WINO_PATH_FUSED_SMALL) gemm_path = staged_path_of(pl);
   const bool tma_ok = (pl->path == WINO_PATH_STAGED_TC || pl->path == WINO_PATH_STAGED_TC_MMA) && !calib;
-  const bool mma_ok = pl->path == WINO_PATH_STAGED_TC_MMA && !calib;
+  const bool mma = pl->path == WINO_PATH_STAGED_TC_MMA;
   int rc = WINO_OK;
   if (!(stage_mask & 1)) {
-  } else if (pl->launches++, mma_ok && pl->p.z_x == 0 &&
-             transform_mma_supported(pl->p, pl->std_mats, pl->p.C)) {
-    const CUtensorMap* mx = map_x_sw(pl, x);
-    const CUtensorMap* mv = map_stage(pl, pl->cache_vst, Vq, pl->p.C);
-    if (mx == nullptr || mv == nullptr) return WINO_ERR_CUDA;
-    rc = launch_input_transform_mma(pl->p, opt_of(pl, pdl), *mx, *mv, pl->kron_dev, pl->num_sms,
-                                    pl->status_dev, st);
+  } else if (pl->launches++, tma_ok && pl->xt_images != nullptr && input_tc_supported(pl->p, pl->std_mats) &&
+             (mma || pl->p.z_x != 0 || input_tc_pays(pl->p))) {
+    const CUtensorMap* mx = map_x_tc(pl, x);
+    if (mx == nullptr) return WINO_ERR_CUDA;
+    rc = launch_input_transform_tc(pl->p, opt_with_hint(pl, pdl, stage_mask, Uq), *mx, pl->xt_images, Vq,
+                                   pl->status_dev, st);
   } else if (tma_ok && pl->p.z_x == 0 && tma_chunk(pl->p.C) != 0) {
     const CUtensorMap* mx = map_x(pl, x);
-    const CUtensorMap* mv = map_stage(pl, pl->cache_vst, Vq, pl->p.C);
+    const CUtensorMap* mv = map_stage(pl, pl->cache_vst, Vq, pl->p.C, tma_group(tma_chunk(pl->p.C)));
     if (mx == nullptr || mv == nullptr) return WINO_ERR_CUDA;
-    LaunchOpt o = opt_of(pl, pdl);
-    if ((stage_mask & 2) && !calib) {   // the GEMMs that follow read U_q, which no kernel of this call writes
-      o.l2_hint = Uq;
-      o.l2_hint_bytes = (size_t)pl->p.t * pl->p.t * pl->p.K * pl->p.C;
-    }
-    rc = launch_input_transform_tma(pl->p, o, *mx, *mv, pl->status_dev, st);
+    rc = launch_input_transform_tma(pl->p, opt_with_hint(pl, pdl, stage_mask, Uq), *mx, *mv, pl->status_dev, st);
   } else {
     rc = launch_input_transform(pl->p, opt_of(pl, pdl), x, Vq, calib ? absmax4 + 0 : nullptr, st);
   }
@@ -461,15 +521,13 @@ int forward_impl(wino_plan_t* pl, const int8_t* x, const int8_t* Uq, const float
   }
   if (rc != WINO_OK) return rc;
   if (!(stage_mask & 4)) {
-  } else if (pl->launches++, mma_ok && pl->p.qM_enabled && pl->p.out_dtype == 0 &&
-             transform_mma_supported(pl->p, pl->std_mats, pl->p.K)) {
-    const CUtensorMap* mm = map_m_sw(pl, mbuf);
-    const CUtensorMap* my = map_y(pl, y);
-    if (mm == nullptr || my == nullptr) return WINO_ERR_CUDA;
-    rc = launch_output_transform_mma(pl->p, opt_of(pl, pdl), *mm, *my, pl->kron_dev, bias, pl->s_Y,
-                                     pl->num_sms, pl->status_dev, st);
+  } else if (pl->launches++, tma_ok && pl->xt_images != nullptr && output_tc_supported(pl->p, pl->std_mats) &&
+             (mma || pl->p.out_dtype != 0 || output_tc_pays(pl->p))) {
+    const CUtensorMap* mm = map_m_tc(pl, mbuf);
+    if (mm == nullptr) return WINO_ERR_CUDA;
+    rc = launch_output_transform_tc(pl->p, opt_of(pl, pdl), *mm, pl->xt_images, bias, y, pl->s_Y, pl->status_dev, st);
   } else if (tma_ok && pl->p.qM_enabled && pl->p.out_dtype == 0 && tma_chunk(pl->p.K) != 0) {
-    const CUtensorMap* mm = map_stage(pl, pl->cache_mld, mbuf, pl->p.K);
+    const CUtensorMap* mm = map_stage(pl, pl->cache_mld, mbuf, pl->p.K, tma_group(tma_chunk(pl->p.K)));
     const CUtensorMap* my = map_y(pl, y);
     if (mm == nullptr || my == nullptr) return WINO_ERR_CUDA;
     rc = launch_output_transform_tma(pl->p, opt_of(pl, pdl), *mm, *my, bias, pl->s_Y,
@@ -603,6 +661,7 @@ int wino_plan(const wino_desc_t* desc, wino_plan_t** out) {
       pl->status_dev = nullptr;
     }
   }
+  if (pl->std_mats && pl->status_dev != nullptr) xt_images(pl->device, &pl->xt_images);
   cudaGetLastError();
   pl->small_ok = small_supported(p);
   if (pl->small_ok) pl->small = small_geometry(p, pl->num_sms);
@@ -646,6 +705,7 @@ int wino_plan_set_channel_scales(wino_plan_t* pl, const float* s_w_K, const floa
         if (!std::isfinite(a[k]) || !(a[k] > 0.0f)) return WINO_ERR_INVALID;
   if (pl->status_dev == nullptr) return WINO_ERR_CUDA;
   std::vector<float> tab((size_t)5 * K);
+  float most_M = 0.0f;
   const wino_desc_t& d = pl->d;
   for (int k = 0; k < K; ++k) {
     const double s_w = s_w_K ? (double)s_w_K[k] : (double)d.q_w.scale;
@@ -656,6 +716,7 @@ int wino_plan_set_channel_scales(wino_plan_t* pl, const float* s_w_K, const floa
     const double s_acc = d.q_M.enabled ? s_M : sUV;
     tab[(size_t)kChMultU * K + k] = (float)(s_w / s_U);
     tab[(size_t)kChMultM * K + k] = d.q_M.enabled ? (float)(sUV / s_M) : 1.0f;
+    if (tab[(size_t)kChMultM * K + k] > most_M) most_M = tab[(size_t)kChMultM * K + k];
     tab[(size_t)kChMultY * K + k] = (float)(s_acc / s_Y);
     tab[(size_t)kChSAcc * K + k] = (float)s_acc;
     tab[(size_t)kChSY * K + k] = (float)s_Y;
@@ -672,6 +733,7 @@ int wino_plan_set_channel_scales(wino_plan_t* pl, const float* s_w_K, const floa
     return WINO_ERR_CUDA;
   }
   pl->chan_dev = fresh;
+  pl->chan_m_fits_16 = 16384.0 * pl->d.C * (double)most_M < 32000.0;
   if (!path_supported(pl, pl->path)) {
     pl->path = staged_path_of(pl);
   }
@@ -709,7 +771,11 @@ int wino_conv_forward(wino_plan_t* pl, const int8_t* x, const int8_t* Uq, const 
   if (pl == nullptr || x == nullptr || Uq == nullptr || y == nullptr) return WINO_ERR_INVALID;
   if (!aligned16(x) || !aligned16(Uq) || !aligned16(y) || (bias && !aligned16(bias)))
     return WINO_ERR_ALIGNMENT;
-  if (!pl->forced && pl->small_ok && pl->small.cost < staged_cost(pl)) {
+  // kernel by estimated time, unless a path is forced (a fused-F2 plan needs no workspace, and
+  // runs the staged kernels only where it was given one)
+  const bool f2 = pl->path == WINO_PATH_FUSED_F2;
+  const bool staged = !f2 || (ws != nullptr && aligned16(ws) && staged_cost(pl) < fused_f2_cost(pl));
+  if (!pl->forced && pl->small_ok && pl->small.cost < (staged ? staged_cost(pl) : fused_f2_cost(pl))) {
     const bool scratch = path_uses_scratch(pl);
     if (pl->status_dev == nullptr) return WINO_ERR_CUDA;
     if (scratch && ws == nullptr) return WINO_ERR_WORKSPACE;
@@ -718,6 +784,12 @@ int wino_conv_forward(wino_plan_t* pl, const int8_t* x, const int8_t* Uq, const 
     if (rc == WINO_OK && scratch) {
       pl->last_uq = Uq; pl->last_x = x; pl->last_ws = ws; pl->last_stream = (cudaStream_t)stream;
     }
+    return rc;
+  }
+  if (!pl->forced && f2 && staged) {
+    pl->path = WINO_PATH_STAGED_TC;
+    const int rc = forward_impl(pl, x, Uq, bias, y, ws, nullptr, (cudaStream_t)stream);
+    pl->path = WINO_PATH_FUSED_F2;
     return rc;
   }
   return forward_impl(pl, x, Uq, bias, y, ws, nullptr, (cudaStream_t)stream);

@@ -27,6 +27,7 @@ struct LaunchOpt {
   // for the per-layer values of Params.  Read by the weight transform, the GEMM epilogues
   // and the output transforms.
   const float* chan = nullptr;
+  bool chan_m_fits_16 = false;   // with these multipliers every rounded product of Q_M is below 2^15
 };
 
 // "Done once per device" bookkeeping.  cudaFuncSetAttribute applies to the device
@@ -81,31 +82,39 @@ int launch_gemm_dp4a(const Params& p, const LaunchOpt& o, const int8_t* Vq, cons
 // Q_M on, int8 output and K % 16 == 0).  Channel chunk per block:
 // (128 channels x 1 tile per block measured best on 256-channel layers: twice the
 // blocks of a 256-channel chunk, so the single wave balances over the SMs)
-inline int tma_chunk(int channels) {
+constexpr int tma_chunk(int channels) {
   return channels % 128 == 0 ? 128 : channels % 64 == 0 ? 64 : channels % 32 == 0 ? 32
        : channels % 16 == 0 ? 16 : 0;
 }
-inline int tma_group(int chunk) { return chunk == 128 ? 1 : chunk == 64 ? 4 : chunk == 32 ? 4 : 8; }
+// tiles per block: 128 threads of two channels
+constexpr int tma_group(int chunk) { return 256 / chunk; }
 int launch_input_transform_tma(const Params& p, const LaunchOpt& o, const CUtensorMap& mapX,
                                const CUtensorMap& mapV, int* status, cudaStream_t st);
 int launch_output_transform_tma(const Params& p, const LaunchOpt& o, const CUtensorMap& mapM,
                                 const CUtensorMap& mapY, const float* bias, float s_Y, int* status,
                                 cudaStream_t st);
 
-// Tensor-core transforms (Cook-Toom F2 / F4, channel count a multiple of 128; input
-// needs z_x == 0, output needs Q_M on and an int8 output).  mapX and mapM carry the
-// 128-byte swizzle; mapV and mapY are the plain maps of the kernels above.
-// `kron`: device copy of the plan's Kronecker tables (fill_kronecker_tables).
+// Tensor-core transforms (wino_transforms_tc.cu): Cook-Toom matrices; the input side for m = 2, 4, 6,
+// any input zero point, C a multiple of 16 and products of Q_V that fit 16 bits; the output side for
+// m = 2, 4, Q_M on, K a multiple of 16 (at most 2048).  Channel chunk of a unit: 128 or 64.
+// mapX: x as [N][H][W][C], box input_tc_box; mapM: m_q as [t*t][T][K], box output_tc_box; both with
+// the swizzle of the chunk's width.  `images`: the constant operands (xt_images).
+inline int xt_chunk(int channels) { return channels % 128 == 0 ? 128 : 64; }
+int xt_images(int device, const uint8_t** out);
+bool input_tc_supported(const Params& p, bool std_mats);
+bool output_tc_supported(const Params& p, bool std_mats);
+void input_tc_box(const Params& p, uint32_t box[4]);
+void output_tc_box(const Params& p, uint32_t box[3]);
+int launch_input_transform_tc(const Params& p, const LaunchOpt& o, const CUtensorMap& mapX, const uint8_t* images,
+                              int8_t* Vq, int* status, cudaStream_t st);
+int launch_output_transform_tc(const Params& p, const LaunchOpt& o, const CUtensorMap& mapM, const uint8_t* images,
+                               const float* bias, void* y, float s_Y, int* status, cudaStream_t st);
+
+// Kronecker matrices of the single-launch layer kernel, whose transforms are such products too.
+// `kron`: device copy of the plan's tables (fill_kronecker_tables).
 constexpr int kKronInRows = 48, kKronOutRows = 16;
 constexpr int kKronBytes = (kKronInRows + kKronOutRows) * 64;
-bool transform_mma_supported(const Params& p, bool std_mats, int channels);
 void fill_kronecker_tables(int m, int8_t* dst_host);
-int launch_input_transform_mma(const Params& p, const LaunchOpt& o, const CUtensorMap& mapX,
-                               const CUtensorMap& mapV, const void* kron, int num_sms, int* status,
-                               cudaStream_t st);
-int launch_output_transform_mma(const Params& p, const LaunchOpt& o, const CUtensorMap& mapM,
-                                const CUtensorMap& mapY, const void* kron, const float* bias,
-                                float s_Y, int num_sms, int* status, cudaStream_t st);
 
 // The whole layer in one persistent launch (Cook-Toom F2 / F4, C and K multiples of
 // 128, input zero point 0, Q_M on, int8 output).  `counters`: plan-owned device words,

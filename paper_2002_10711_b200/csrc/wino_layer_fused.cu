@@ -3,7 +3,7 @@
 // counts that are multiples of 128:
 //
 //   phase A  input transform on the tensor cores (patch x Kronecker matrix, see
-//            wino_transforms_mma.cu), Q_V, V_q -> workspace (stays in L2);
+//            wino_transforms_tc.cu), Q_V, V_q -> workspace (stays in L2);
 //   phase B  the t*t Hadamard-stage GEMMs over channels (tcgen05 kind::i8, TMA
 //            operands, int32 accumulators in tensor memory), Q_M, m_q -> workspace;
 //   phase C  output transform on the tensor cores, bias, Q_Y, y.
@@ -39,6 +39,8 @@
 // While the workers are still quantizing phase A, warps 2 and 3 already run the
 // first GEMM item of the CTA into tensor-memory columns 0..255; the transform
 // accumulators live in columns 256..511 until phase A is done.
+#include <cstring>
+
 #include "wino_launch.h"
 #include "wino_ptx.cuh"
 
@@ -223,7 +225,6 @@ k_layer_fused(const __grid_constant__ Params p, const __grid_constant__ CUtensor
   const int per_mb = T2 * a.n_nblk;                     // items per m-block
   const int cbuf = nI & 1;                              // GEMM accumulator buffer phase C borrows
 
-  griddep_launch();
   if (threadIdx.x == 0) {
     WINO_TRACE_AT(0);
     for (int s = 0; s < a.stages; ++s) {
@@ -258,6 +259,9 @@ k_layer_fused(const __grid_constant__ Params p, const __grid_constant__ CUtensor
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  // only now may the next kernel's blocks start: every block of this grid holds its tensor memory,
+  // so none of them can be kept from it by a block that waits for this grid
+  griddep_launch();
   const uint32_t tmem_base = *tmem_slot_p;
 
   if (warp == 0) {
@@ -791,6 +795,22 @@ int launch_layer_fused(const Params& p, const LaunchOpt& o, const FusedGeom& g, 
   if (g.stages < 2) return -2;
   return p.m == 2 ? fused_launch<2>(p, o, g, m, kron, counters, mq, bias, s_Y, status, st)
                   : fused_launch<4>(p, o, g, m, kron, counters, mq, bias, s_Y, status, st);
+}
+
+// Host side: the two Kronecker matrices of the plan's tile size as int8 rows of 64 bytes
+// (kKronInRows rows for the input side, then kKronOutRows for the output side).
+void fill_kronecker_tables(int m, int8_t* dst) {
+  std::memset(dst, 0, kKronBytes);
+  const int t = m + 2, t2 = t * t, mm = m * m;
+  auto bt = [&](int i, int k) { return m == 2 ? (int)std_bt<2>(i, k) : (int)std_bt<4>(i, k); };
+  auto at = [&](int i, int k) { return m == 2 ? (int)std_at<2>(i, k) : (int)std_at<4>(i, k); };
+  for (int xi = 0; xi < t2; ++xi)
+    for (int ab = 0; ab < t2; ++ab)
+      dst[xi * 64 + ab] = (int8_t)(bt(xi / t, ab / t) * bt(xi % t, ab % t));
+  int8_t* out = dst + kKronInRows * 64;
+  for (int pq = 0; pq < mm; ++pq)
+    for (int xi = 0; xi < t2; ++xi)
+      out[pq * 64 + xi] = (int8_t)(at(pq / m, xi / t) * at(pq % m, xi % t));
 }
 
 }  // namespace wino

@@ -23,9 +23,10 @@ struct Params {
   int z_x, z_w, z_Y;
   int qM_enabled;
   int out_dtype;               // 0 int8, 1 float
-  // whatever the data, every rounded product of Q_V (of Q_M) has a magnitude below 2^15, so
+  // whatever the data, every rounded product of Q_V (of Q_M, Q_U) has a magnitude below 2^15, so
   // that its clamp can be done in 16-bit lanes
   int v_fits_16, m_fits_16;
+  int u_fits_16, u_fits_16_chan;   // Q_U, under the per-layer and the per-channel scales
 };
 // Per-output-channel scales travel beside Params as a device array `chan` [5][K] (null: the
 // per-layer values of Params): row kChMultU = s_w[k]/s_U[k], kChMultM = s_U[k]*s_V/s_M[k],

@@ -110,116 +110,217 @@ k_direct_conv(const DirectParams p, const int8_t* __restrict__ x, const int8_t* 
   }
 }
 
-// At most four input channels (a network's first layer, Section 5.1).  The 9 * C codes under a
-// pixel's window fit NW = ceil(9 * C / 4) registers, so a thread takes one output pixel, gathers
-// its window once and walks 32 output channels whose filters, packed the same way, lie in shared
-// memory (every lane reads the same words: broadcasts).  Window and filter pad with zeros.
+// At most four input channels (a network's first layer, Section 5.1): the 9 * C codes under a
+// pixel's window fit one or two K steps of an int8 warp MMA (m16n8k32), so the layer is an
+// implicit GEMM whose A operand is gathered.  A warp takes 32 pixels: every lane gathers the
+// window of one (aligned words, funnel shifts) and leaves it in shared memory, from where it
+// comes back as A fragments; the 64 filters of the block are kept as B fragments in registers.
+// The K order is free as long as windows and filters agree: a row's 3 * C bytes are padded to
+// words (C = 3: the ninth bytes of the three rows share one).  Which filter is which column is free
+// too: lane t of a quad takes channels 16 t .. 16 t + 15, so that it stores 16 bytes and a quad 64.
 // With zero points, sum (x - z_x)(w - z_w) = sum x w - z_w sum x - z_x sum w + 9 C z_x z_w over the
 // whole window, pixels outside the image holding the code z_x.
-// Bound by the ALU pipe: NW dot products and seven quantizer instructions per output.  64 images
-// 32x32, 3 -> 64 channels: 10.0 us, where the byte-wise kernel below took 114.
-constexpr int kNarrowK = 32, kNarrowThreads = 128;
+// Bound by the quantizer's issue slots and the launch.  64 images 32x32, 3 -> 64 channels: 114 us
+// byte by byte, 10.0 with dot products and one pixel per thread, 5.1 like this.
+constexpr int kNarrowK = 64, kNarrowThreads = 128;
+
+// A row of 3 * C bytes at `at` (any alignment), of which bytes [from, to) exist, as three words;
+// bytes that do not exist take the code z (replicated in `fill`).
 template <int C>
+__device__ __forceinline__ void narrow_row(const int8_t* at, int from, int to, uint32_t fill, uint32_t (&r)[3]) {
+  const uint32_t sh = (uint32_t)(reinterpret_cast<uintptr_t>(at) & 3u);
+  const uint32_t* base = reinterpret_cast<const uint32_t*>(at - sh);
+  constexpr int kWords = (3 * C + 3 + 3) / 4;   // words that 3 * C bytes at any alignment touch
+  uint32_t w[4] = {0u, 0u, 0u, 0u};
+#pragma unroll
+  for (int j = 0; j < kWords; ++j) {
+    // only words that hold a byte of the image are read
+    const int lo = 4 * j - (int)sh;
+    if (from < to && lo + 4 > from && lo < to) w[j] = __ldg(base + j);
+  }
+#pragma unroll
+  for (int j = 0; j < 3; ++j) {
+    if (4 * j >= 3 * C) { r[j] = 0u; continue; }
+    uint32_t v = __funnelshift_r(w[j], j + 1 < kWords ? w[j + 1] : 0u, 8u * sh);
+    uint32_t keep = 0u, exist = 0u;
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      const int b = 4 * j + e;
+      if (b < 3 * C) exist |= 0xFFu << (8 * e);
+      if (b < 3 * C && b >= from && b < to) keep |= 0xFFu << (8 * e);
+    }
+    r[j] = (v & keep) | (fill & exist & ~keep);
+  }
+}
+// Three rows in K order: 8 words (one K step), or 16 (C = 4: two).
+template <int C>
+__device__ __forceinline__ void narrow_k(const uint32_t (&r)[3][3], uint32_t (&k)[C == 4 ? 16 : 8]) {
+#pragma unroll
+  for (int i = 0; i < (C == 4 ? 16 : 8); ++i) k[i] = 0u;
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    if (C == 1) {
+      k[a] = r[a][0];
+    } else if (C == 4) {
+      k[3 * a] = r[a][0]; k[3 * a + 1] = r[a][1]; k[3 * a + 2] = r[a][2];
+    } else {
+      k[2 * a] = r[a][0]; k[2 * a + 1] = r[a][1];
+      if (C == 3) k[6] |= (r[a][2] & 0xFFu) << (8 * a);
+    }
+  }
+}
+__device__ __forceinline__ void narrow_mma(int (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0,
+                                           uint32_t b1) {
+  asm volatile("mma.sync.aligned.m16n8k32.row.col.s32.s8.s8.s32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, "
+               "{%0, %1, %2, %3};"
+               : "+r"(d[0]), "+r"(d[1]), "+r"(d[2]), "+r"(d[3])
+               : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+
+template <int C, bool Z>
 __global__ void __launch_bounds__(kNarrowThreads)
 k_direct_conv_narrow(const DirectParams p, const int8_t* __restrict__ x, const int8_t* __restrict__ w,
-                     const float* __restrict__ bias, void* __restrict__ y, int store) {
-  constexpr int NW = (9 * C + 3) / 4, taps = 9 * C, row_bytes = 3 * C;
-  constexpr int WS = (NW + 3) / 4 * 4;     // words between two filters: whole 16-byte reads
-  __shared__ __align__(16) uint32_t s_w[kNarrowK * WS];
-  __shared__ int s_corr[kNarrowK];         // - z_x sum w + 9 C z_x z_w
-  __shared__ float s_mult[kNarrowK], s_b[kNarrowK];
+                     const float* __restrict__ bias, void* __restrict__ y, int wide) {
+  constexpr int KW = C == 4 ? 16 : 8, STEPS = KW / 8;      // words of K, MMA K steps
+  __shared__ __align__(16) uint32_t s_f[kNarrowK * KW];    // filters in K order
+  __shared__ __align__(16) uint32_t s_a[kNarrowThreads * KW];
+  __shared__ __align__(8) float s_mult[kNarrowK], s_b[kNarrowK];
+  __shared__ int s_corr[kNarrowK];
+  const int tid = threadIdx.x, lane = tid & 31, g = lane >> 2, t = lane & 3;
   const int k0 = blockIdx.y * kNarrowK;
   griddep_launch();
-  for (int i = threadIdx.x; i < kNarrowK * WS; i += kNarrowThreads) s_w[i] = 0u;
-  __syncthreads();
-  griddep_wait();
-  const int nk = min(kNarrowK, p.K - k0);
-  for (int i = threadIdx.x; i < nk * taps; i += kNarrowThreads) {
-    const int k = i / taps, j = i - k * taps;
-    reinterpret_cast<int8_t*>(s_w + k * WS)[j] = w[(long)(k0 + k) * taps + j];
-  }
-  const long npix = (long)p.N * p.Ho * p.Wo;
-  const long idx = blockIdx.x * (long)kNarrowThreads + threadIdx.x;
-  uint32_t win[NW];
-#pragma unroll
-  for (int i = 0; i < NW; ++i) win[i] = 0u;
-  if (idx < npix) {
-    const int rest = (int)(idx / p.Wo), wo = (int)(idx - (long)rest * p.Wo);
-    const int n = rest / p.Ho, ho = rest - n * p.Ho;
-    const int h0 = ho * p.stride - 1, w0 = wo * p.stride - 1;
-    const int8_t* xp = x + (((long)n * p.H + h0) * p.W + w0) * p.C;
-    // byte 4 i + j of the window: row (4 i + j) / (3 C); within a row the bytes are contiguous
-#pragma unroll
-    for (int i = 0; i < NW; ++i)
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const int at = 4 * i + j;
-        if (at < taps) {
-          const int a = at / row_bytes, r = at - a * row_bytes, b = r / C;
-          const bool in = (unsigned)(h0 + a) < (unsigned)p.H && (unsigned)(w0 + b) < (unsigned)p.W;
-          const int v = in ? (int)__ldg(xp + (long)a * p.W * C + r) : p.z_x;
-          win[i] |= ((uint32_t)v & 0xFFu) << (8 * j);
-        }
-      }
-  }
-  __syncthreads();
-  if (threadIdx.x < nk) {
-    const int k = threadIdx.x;
-    int sum = 0;
-    for (int j = 0; j < NW; ++j) sum = __dp4a((int)s_w[k * WS + j], 0x01010101, sum);
-    s_corr[k] = -p.z_x * sum + taps * p.z_x * p.z_w;
+  if (tid < kNarrowK) {   // parameters of the layer: no dependency on the preceding kernel
+    const int k = min(k0 + tid, p.K - 1);
     float mult, s_in, s_Y;
-    channel_scales(p, k0 + k, mult, s_in, s_Y);
-    const float b = bias != nullptr ? __ldg(bias + k0 + k) : 0.0f;
-    s_mult[k] = p.out_dtype == 0 ? mult : s_in;
-    s_b[k] = p.out_dtype == 0 && bias != nullptr ? (float)((double)b / (double)s_Y) : b;
+    channel_scales(p, k, mult, s_in, s_Y);
+    const float b = bias != nullptr ? __ldg(bias + k) : 0.0f;
+    s_mult[tid] = p.out_dtype == 0 ? mult : s_in;
+    s_b[tid] = p.out_dtype == 0 && bias != nullptr ? (float)((double)b / (double)s_Y) : b;
+  }
+  griddep_wait();
+  if (tid < kNarrowK) {
+    uint32_t r[3][3], kw[KW];
+    const int k = k0 + tid;
+#pragma unroll
+    for (int a = 0; a < 3; ++a)
+      narrow_row<C>(w + (long)(k < p.K ? k : 0) * 9 * C + a * 3 * C, 0, k < p.K ? 3 * C : 0, 0u, r[a]);
+    narrow_k<C>(r, kw);
+    int sum = 0;
+#pragma unroll
+    for (int i = 0; i < KW; ++i) {
+      s_f[tid * KW + i] = kw[i];
+      sum = __dp4a((int)kw[i], 0x01010101, sum);
+    }
+    s_corr[tid] = -p.z_x * sum + 9 * C * p.z_x * p.z_w;
   }
   __syncthreads();
-  if (idx >= npix) return;
-  int corr = 0;
-  if (p.z_w != 0) {
+  // B fragments: column n = g of product j is channel 16 (g / 2) + 2 j + (g & 1)
+  uint32_t bf[8][STEPS][2];
 #pragma unroll
-    for (int i = 0; i < NW; ++i) corr = __dp4a((int)win[i], 0x01010101, corr);
-    corr *= -p.z_w;
-  }
-  const long o = idx * p.K + k0;
-#pragma unroll 1
-  for (int q = 0; q < nk; q += 16) {
-    uint32_t out[4];
+  for (int j = 0; j < 8; ++j)
 #pragma unroll
-    for (int e4 = 0; e4 < 4; ++e4) {
-      uint32_t word = 0u;
+    for (int q = 0; q < STEPS; ++q) {
+      const uint2 v = *reinterpret_cast<const uint2*>(s_f + (16 * (g >> 1) + 2 * j + (g & 1)) * KW + 8 * q + 2 * t);
+      bf[j][q][0] = v.x;
+      bf[j][q][1] = v.y;
+    }
+  const long npix = (long)p.N * p.Ho * p.Wo;
+  const uint32_t fill = ((uint32_t)p.z_x & 0xFFu) * 0x01010101u;
+  uint32_t* mine = s_a + (tid & ~31) * KW;
+  for (long first = (blockIdx.x * (long)kNarrowThreads + (tid & ~31)); first < npix;
+       first += (long)gridDim.x * kNarrowThreads) {
+    const long idx = first + lane;
+    uint32_t kw[KW];
+    int xsum = 0;
+    {
+      uint32_t r[3][3] = {};
+      if (idx < npix) {
+        const long rest = idx / p.Wo;
+        const int wo = (int)(idx - rest * p.Wo), n = (int)(rest / p.Ho), ho = (int)(rest - (long)n * p.Ho);
+        const int h0 = ho * p.stride - 1, w0 = wo * p.stride - 1;
+        const int from = w0 < 0 ? C : 0, to = min(3, p.W - w0) * C;
+        const int8_t* xp = x + (((long)n * p.H + h0) * p.W + w0) * C;
 #pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const int k = q + 4 * e4 + e;      // (channels past K: zero filters of the padded table)
-        int acc = corr + s_corr[k];
-        const uint4* f = reinterpret_cast<const uint4*>(s_w + k * WS);
-#pragma unroll
-        for (int i = 0; i < WS / 4; ++i) {
-          const uint4 v = f[i];
-          acc = __dp4a((int)win[4 * i], (int)v.x, acc);
-          if (4 * i + 1 < NW) acc = __dp4a((int)win[4 * i + 1 < NW ? 4 * i + 1 : 0], (int)v.y, acc);
-          if (4 * i + 2 < NW) acc = __dp4a((int)win[4 * i + 2 < NW ? 4 * i + 2 : 0], (int)v.z, acc);
-          if (4 * i + 3 < NW) acc = __dp4a((int)win[4 * i + 3 < NW ? 4 * i + 3 : 0], (int)v.w, acc);
-        }
-        const float yf = __fmaf_rn(__int2float_rn(acc), s_mult[k], s_b[k]);
-        if (p.out_dtype == 0) {
-          const float r = __fadd_rn(fminf(fmaxf(yf, p.lo_Y), p.hi_Y), kMagic);
-          word |= ((uint32_t)(magic_to_int(r) + p.z_Y) & 0xFFu) << (8 * e);
-        } else if (k < nk) {
-          reinterpret_cast<float*>(y)[o + k] = yf;
+        for (int a = 0; a < 3; ++a) {
+          const bool in = (unsigned)(h0 + a) < (unsigned)p.H;
+          narrow_row<C>(xp + (long)a * p.W * C, in ? from : 0, in ? to : 0, fill, r[a]);
         }
       }
-      out[e4] = word;
+      narrow_k<C>(r, kw);
     }
-    if (p.out_dtype == 0) {
-      int8_t* yp = reinterpret_cast<int8_t*>(y) + o + q;
-      if (store == 16) {
-        *reinterpret_cast<uint4*>(yp) = make_uint4(out[0], out[1], out[2], out[3]);
-      } else {
+    if constexpr (Z) {
 #pragma unroll
-        for (int j = 0; j < 16; ++j)
-          if (q + j < nk) yp[j] = (int8_t)(out[j >> 2] >> (8 * (j & 3)));
+      for (int i = 0; i < KW; ++i) xsum = __dp4a((int)kw[i], 0x01010101, xsum);
+      xsum *= -p.z_w;
+    }
+    __syncwarp();
+#pragma unroll
+    for (int i = 0; i < KW; i += 4)
+      *reinterpret_cast<uint4*>(mine + lane * KW + i) = make_uint4(kw[i], kw[i + 1], kw[i + 2], kw[i + 3]);
+    __syncwarp();
+#pragma unroll
+    for (int half = 0; half < 2; ++half) {
+      uint2 a0[STEPS], a1[STEPS];
+#pragma unroll
+      for (int q = 0; q < STEPS; ++q) {
+        a0[q] = *reinterpret_cast<const uint2*>(mine + (16 * half + g) * KW + 8 * q + 2 * t);
+        a1[q] = *reinterpret_cast<const uint2*>(mine + (16 * half + g + 8) * KW + 8 * q + 2 * t);
+      }
+      const int c0 = Z ? __shfl_sync(0xffffffffu, xsum, 16 * half + g) : 0;
+      const int c1 = Z ? __shfl_sync(0xffffffffu, xsum, 16 * half + g + 8) : 0;
+      uint32_t o0[4] = {0u, 0u, 0u, 0u}, o1[4] = {0u, 0u, 0u, 0u};   // 16 codes of rows g and g + 8
+      const long p0 = first + 16 * half + g, p1 = p0 + 8;
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        int d[4] = {0, 0, 0, 0};
+#pragma unroll
+        for (int q = 0; q < STEPS; ++q) narrow_mma(d, a0[q].x, a1[q].x, a0[q].y, a1[q].y, bf[j][q][0], bf[j][q][1]);
+        const int kc = 16 * t + 2 * j;
+        if constexpr (Z) {
+          const int s0 = s_corr[kc], s1 = s_corr[kc + 1];
+          d[0] += c0 + s0; d[1] += c0 + s1; d[2] += c1 + s0; d[3] += c1 + s1;
+        }
+        const float2 m = *reinterpret_cast<const float2*>(s_mult + kc), b = *reinterpret_cast<const float2*>(s_b + kc);
+        float f[4];
+        f[0] = __fmaf_rn(__int2float_rn(d[0]), m.x, b.x);
+        f[1] = __fmaf_rn(__int2float_rn(d[1]), m.y, b.y);
+        f[2] = __fmaf_rn(__int2float_rn(d[2]), m.x, b.x);
+        f[3] = __fmaf_rn(__int2float_rn(d[3]), m.y, b.y);
+        if (p.out_dtype == 0) {
+          uint32_t c[4];
+#pragma unroll
+          for (int e = 0; e < 4; ++e)
+            c[e] = (uint32_t)(magic_to_int(__fadd_rn(fminf(fmaxf(f[e], p.lo_Y), p.hi_Y), kMagic)) + p.z_Y);
+          // two codes of each row into half j & 1 of word j / 2
+          const uint32_t h0 = __byte_perm(c[0], c[1], 0x0040u), h1 = __byte_perm(c[2], c[3], 0x0040u);
+          o0[j >> 1] = (j & 1) ? __byte_perm(o0[j >> 1], h0, 0x5410u) : (h0 & 0xFFFFu);
+          o1[j >> 1] = (j & 1) ? __byte_perm(o1[j >> 1], h1, 0x5410u) : (h1 & 0xFFFFu);
+        } else {
+          float* yp = reinterpret_cast<float*>(y);
+#pragma unroll
+          for (int e = 0; e < 2; ++e) {
+            if (k0 + kc + e < p.K && p0 < npix) yp[p0 * p.K + k0 + kc + e] = f[e];
+            if (k0 + kc + e < p.K && p1 < npix) yp[p1 * p.K + k0 + kc + e] = f[2 + e];
+          }
+        }
+      }
+      if (p.out_dtype == 0) {
+        const int kc = k0 + 16 * t;
+#pragma unroll
+        for (int rr = 0; rr < 2; ++rr) {
+          const long px = rr == 0 ? p0 : p1;
+          if (px >= npix || kc >= p.K) continue;
+          int8_t* yp = reinterpret_cast<int8_t*>(y) + px * p.K + kc;
+          const uint32_t q0 = rr == 0 ? o0[0] : o1[0], q1 = rr == 0 ? o0[1] : o1[1], q2 = rr == 0 ? o0[2] : o1[2],
+                         q3 = rr == 0 ? o0[3] : o1[3];
+          if (wide) {
+            *reinterpret_cast<uint4*>(yp) = make_uint4(q0, q1, q2, q3);
+          } else {
+#pragma unroll
+            for (int e = 0; e < 16; ++e)
+              if (kc + e < p.K) yp[e] = (int8_t)((e < 4 ? q0 : e < 8 ? q1 : e < 12 ? q2 : q3) >> (8 * (e & 3)));
+          }
+        }
       }
     }
   }
@@ -278,12 +379,20 @@ int launch_direct_conv(int N, int C, int H, int W, int K, int stride, int z_x, i
   p.mult = mult; p.s_in = s_in; p.s_Y = s_Y; p.lo_Y = lo_Y; p.hi_Y = hi_Y;
   p.out_dtype = out_dtype;
   const long npix = (long)N * p.Ho * p.Wo;
-  if (C <= 4 && (K + kNarrowK - 1) / kNarrowK <= 65535 && (npix + kNarrowThreads - 1) / kNarrowThreads <= 0x7fffffffl) {
-    const dim3 grid((unsigned)((npix + kNarrowThreads - 1) / kNarrowThreads), (unsigned)((K + kNarrowK - 1) / kNarrowK));
-    const int store = K % 16 == 0 ? 16 : 1;   // y is 16-byte aligned
-    auto kernel = C == 1 ? k_direct_conv_narrow<1> : C == 2 ? k_direct_conv_narrow<2>
-                : C == 3 ? k_direct_conv_narrow<3> : k_direct_conv_narrow<4>;
-    return launch_kernel(kernel, grid, dim3(kNarrowThreads), 0, st, true, p, x, w, bias, y, store);
+  if (C <= 4 && (K + kNarrowK - 1) / kNarrowK <= 65535) {
+    // up to four blocks an SM; a warp takes further groups of 32 pixels where there are more
+    const int kb = (K + kNarrowK - 1) / kNarrowK;
+    const long want = (npix + kNarrowThreads - 1) / kNarrowThreads, most = (4l * 148 + kb - 1) / kb;
+    const dim3 grid((unsigned)(want < most ? want : most), (unsigned)kb);
+    const int wide = K % 16 == 0 ? 1 : 0;   // y is 16-byte aligned
+    const bool z = z_x != 0 || z_w != 0;
+    auto go = [&](auto plain, auto with_z) {
+      return launch_kernel(z ? with_z : plain, grid, dim3(kNarrowThreads), 0, st, true, p, x, w, bias, y, wide);
+    };
+    return C == 1 ? go(k_direct_conv_narrow<1, false>, k_direct_conv_narrow<1, true>)
+         : C == 2 ? go(k_direct_conv_narrow<2, false>, k_direct_conv_narrow<2, true>)
+         : C == 3 ? go(k_direct_conv_narrow<3, false>, k_direct_conv_narrow<3, true>)
+                  : go(k_direct_conv_narrow<4, false>, k_direct_conv_narrow<4, true>);
   }
   if (C % 4 != 0 || K % 4 != 0) {
     const long blocks = (npix * K + 127) / 128;

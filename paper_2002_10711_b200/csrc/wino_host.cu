@@ -44,6 +44,7 @@ struct wino_plan {
   wino_desc_t d;
   Params p;
   float s_Y;
+  double u_max;         // bound on |U| in units of the weight codes
   bool std_mats;        // BT and AT equal the built-in Cook-Toom matrices bit for bit
   int path;
   bool forced;          // wino_plan_force_path pinned it
@@ -618,6 +619,13 @@ int wino_plan(const wino_desc_t* desc, wino_plan_t** out) {
     }
     const double v_max = row * row * (128.0 + std::fabs((double)p.z_x));
     p.v_fits_16 = v_max * (double)p.mult_V < 32000.0 ? 1 : 0;
+    double g_row = 0.0;
+    for (int i = 0; i < t; ++i) {
+      const double r = std::fabs((double)p.G[i * 3]) + std::fabs((double)p.G[i * 3 + 1]) + std::fabs((double)p.G[i * 3 + 2]);
+      if (r > g_row) g_row = r;
+    }
+    pl->u_max = g_row * g_row * (128.0 + std::fabs((double)p.z_w));
+    p.u_fits_16 = pl->u_max * (double)p.mult_U < 32000.0 ? 1 : 0;
     p.m_fits_16 = 16384.0 * d.C * (double)p.mult_M < 32000.0 ? 1 : 0;
   }
   pl->std_mats = d.m == 2 ? is_std<2>(p.BT, p.AT) : d.m == 4 ? is_std<4>(p.BT, p.AT)
@@ -705,7 +713,7 @@ int wino_plan_set_channel_scales(wino_plan_t* pl, const float* s_w_K, const floa
         if (!std::isfinite(a[k]) || !(a[k] > 0.0f)) return WINO_ERR_INVALID;
   if (pl->status_dev == nullptr) return WINO_ERR_CUDA;
   std::vector<float> tab((size_t)5 * K);
-  float most_M = 0.0f;
+  float most_M = 0.0f, most_U = 0.0f;
   const wino_desc_t& d = pl->d;
   for (int k = 0; k < K; ++k) {
     const double s_w = s_w_K ? (double)s_w_K[k] : (double)d.q_w.scale;
@@ -716,6 +724,7 @@ int wino_plan_set_channel_scales(wino_plan_t* pl, const float* s_w_K, const floa
     const double s_acc = d.q_M.enabled ? s_M : sUV;
     tab[(size_t)kChMultU * K + k] = (float)(s_w / s_U);
     tab[(size_t)kChMultM * K + k] = d.q_M.enabled ? (float)(sUV / s_M) : 1.0f;
+    if (tab[(size_t)kChMultU * K + k] > most_U) most_U = tab[(size_t)kChMultU * K + k];
     if (tab[(size_t)kChMultM * K + k] > most_M) most_M = tab[(size_t)kChMultM * K + k];
     tab[(size_t)kChMultY * K + k] = (float)(s_acc / s_Y);
     tab[(size_t)kChSAcc * K + k] = (float)s_acc;
@@ -733,6 +742,7 @@ int wino_plan_set_channel_scales(wino_plan_t* pl, const float* s_w_K, const floa
     return WINO_ERR_CUDA;
   }
   pl->chan_dev = fresh;
+  pl->p.u_fits_16_chan = pl->u_max * (double)most_U < 32000.0 ? 1 : 0;
   pl->chan_m_fits_16 = 16384.0 * pl->d.C * (double)most_M < 32000.0;
   if (!path_supported(pl, pl->path)) {
     pl->path = staged_path_of(pl);

@@ -43,3 +43,7 @@ def test_narrow_input(C, shape, stride, zero_points, out_dtype):
                                    (9, 64, 5, 3, 64), (1, 64, 255, 1, 32)])
 def test_odd_sizes_at_stride_two(shape):
     _check(*shape, 2)
+
+
+def test_many_pixels_per_warp():
+    _check(40, 3, 61, 33, 70, 1)     # more groups of 32 pixels than warps, two blocks of channels

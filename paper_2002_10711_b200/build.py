@@ -1,6 +1,6 @@
 """Builds the CUDA library (sm_100a only) in-tree with nvcc: one object per
 translation unit, compiled in parallel, linked into one shared library; and the
-CPython module with the per-pass entry points (csrc/wino_python.c), linked against it."""
+CPython modules with the per-pass entry points (csrc/wino_python*), linked against it."""
 from __future__ import annotations
 
 import os
@@ -14,6 +14,7 @@ CSRC = os.path.join(HERE, "csrc")
 OBJ = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libwino_b200.so")
 NATIVE = os.path.join(HERE, "_native.so")
+NATIVE_TORCH = os.path.join(HERE, "_native_torch.so")
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-O3", "-lineinfo", "-std=c++17",
     "-fmad=false", "--expt-relaxed-constexpr", "-Xcompiler", "-fPIC",
@@ -57,16 +58,33 @@ def build(force: bool = False, verbose: bool = False) -> str:
     return LIB
 
 
+def _stale(target: str, *sources: str) -> bool:
+    return not os.path.exists(target) or os.path.getmtime(target) < max(os.path.getmtime(f) for f in sources)
+
+
 def _build_native(force: bool) -> None:
-    src, header = os.path.join(CSRC, "wino_python.c"), os.path.join(ROOT, "include", "wino.h")
-    if not force and os.path.exists(NATIVE) and os.path.getmtime(NATIVE) >= max(os.path.getmtime(src),
-                                                                               os.path.getmtime(header)):
-        return
-    tmp = NATIVE + f".tmp{os.getpid()}"
-    subprocess.check_call([os.environ.get("CC", "gcc"), "-O2", "-std=c11", "-Wall", "-Wextra", "-fPIC", "-shared",
-                           "-I", sysconfig.get_paths()["include"], "-I", os.path.join(ROOT, "include"), src,
-                           "-L", HERE, "-l:" + os.path.basename(LIB), "-Wl,-rpath,$ORIGIN", "-o", tmp])
-    os.replace(tmp, NATIVE)
+    """The CPython modules: plain C, and the one compiled against torch (layer.py's)."""
+    header = os.path.join(ROOT, "include", "wino.h")
+    common = ["-O2", "-Wall", "-Wextra", "-fPIC", "-shared", "-I", sysconfig.get_paths()["include"],
+              "-I", os.path.join(ROOT, "include")]
+    link = ["-L", HERE, "-l:" + os.path.basename(LIB), "-Wl,-rpath,$ORIGIN"]
+    src = os.path.join(CSRC, "wino_python.c")
+    if force or _stale(NATIVE, src, header):
+        tmp = NATIVE + f".tmp{os.getpid()}"
+        subprocess.check_call([os.environ.get("CC", "gcc"), "-std=c11", *common, src, *link, "-o", tmp])
+        os.replace(tmp, NATIVE)
+    src = os.path.join(CSRC, "wino_python_torch.cpp")
+    if force or _stale(NATIVE_TORCH, src, header):
+        import torch
+        from torch.utils.cpp_extension import include_paths, library_paths
+        tmp = NATIVE_TORCH + f".tmp{os.getpid()}"
+        cuda = os.path.join(os.path.dirname(os.path.dirname(os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc"))), "include")
+        subprocess.check_call(
+            [os.environ.get("CXX", "g++"), "-std=c++17", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+             *common, *[f for d in include_paths() for f in ("-isystem", d)], "-isystem", cuda, src, *link,
+             *[f for d in library_paths() for f in ("-L", d)], "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_cuda",
+             "-ltorch", "-ltorch_python", "-o", tmp])
+        os.replace(tmp, NATIVE_TORCH)
 
 
 if __name__ == "__main__":

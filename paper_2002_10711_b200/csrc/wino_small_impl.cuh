@@ -116,6 +116,8 @@ k_layer_small(const __grid_constant__ Params p, const __grid_constant__ SmallGeo
     }
   }
   __syncthreads();   // barriers and the abort flag are set up
+  if (tma && warp == 7 && lane == 0)   // weights that are not in L2 come in while the preceding kernel runs
+    for (int q = 0; q < nq; ++q) tma_prefetch_l2_3d(&mapU, c0 + 64 * q, k0, 0);
   griddep_wait();
 
   // 1. operands

@@ -10,6 +10,7 @@ import torch
 
 from . import binding
 from .binding import Plan
+from . import _native_torch  # after torch and the library it links against
 
 
 class WinogradConv:
@@ -36,10 +37,13 @@ class WinogradConv:
 
     def forward(self, x_dev: torch.Tensor, y_dev: torch.Tensor | None = None) -> torch.Tensor:
         """x_dev: int8 [N,H,W,C] on the device."""
-        if y_dev is None:
-            y_dev = self.empty_output()
-        self.plan.conv_forward(x_dev, self.Uq, self.bias, y_dev, self.ws)
-        return y_dev
+        y = _native_torch.forward(self.plan._address, x_dev, self.Uq, self.bias, y_dev, self.ws, self._y_like)
+        if type(y) is int:
+            raise binding.WinoError(y, "wino_conv_forward")
+        if y is None:      # addresses instead of tensors
+            y = self.empty_output() if y_dev is None else y_dev
+            self.plan.conv_forward(x_dev, self.Uq, self.bias, y, self.ws)
+        return y
 
     def dump(self, stage: int) -> torch.Tensor:
         p = self.plan

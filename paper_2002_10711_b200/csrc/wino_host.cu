@@ -349,7 +349,7 @@ const CUtensorMap* map_u_small(wino_plan_t* pl, const void* Uq, int KB) {
 }
 
 int launch_gemm(wino_plan_t* pl, const int8_t* Vq, const int8_t* Uq, void* out, int out_mode,
-                unsigned* absmaxM, bool pdl, cudaStream_t st) {
+                unsigned* absmaxM, bool pdl, cudaStream_t st, bool no_tmem_next = false) {
   const Params& p = pl->p;
   const int t2 = p.t * p.t;
   pl->launches++;
@@ -366,7 +366,9 @@ int launch_gemm(wino_plan_t* pl, const int8_t* Vq, const int8_t* Uq, void* out, 
     if (rc != WINO_OK) return rc;
     pl->map_uq_ptr = Uq;
   }
-  return launch_gemm_tc(p, opt_of(pl, pdl), g, pl->mapV, pl->mapU, out, out_mode, absmaxM,
+  LaunchOpt o = opt_of(pl, pdl);
+  o.early_trigger = no_tmem_next;
+  return launch_gemm_tc(p, o, g, pl->mapV, pl->mapU, out, out_mode, absmaxM,
                         pl->status_dev, st);
 }
 
@@ -378,7 +380,10 @@ int launch_gemm(wino_plan_t* pl, const int8_t* Vq, const int8_t* Uq, void* out, 
 //           F6  4.7 M 3.7 / 4.5   8.4 M 6.5 / 6.0   18.9 M 11.4 / 9.2   37.7 M 23 / 16.5
 //   output  F2  8.4 M 4.1 / 4.9   16.8 M 7.4 / 6.3   33.6 M 12.6 / 8.6   67 M 24 / 13
 //           F4  9.4 M 4.6 / 5.2   18.9 M 7.8 / 7.7   37.7 M 13.6 / 11.9
+// With an input zero point the ALU kernel would also have to patch the padding of border tiles
+// (14 -> 19 us on a 160-channel 12 x 22 layer).
 bool input_tc_pays(const Params& p) {
+  if (p.z_x != 0) return true;
   const double codes = (double)p.t * p.t * p.T * p.C;
   return codes > (p.m == 2 ? 12e6 : p.m == 4 ? 14e6 : 7e6);
 }
@@ -400,13 +405,12 @@ LaunchOpt opt_with_hint(const wino_plan_t* pl, bool pdl, int stage_mask, const i
 
 // Estimated times in ns, for the choice between kernels that can run the same layer.  Staged: a
 // start-up latency of three dependent kernels plus a time per code (measured, us: F2 16.8 M codes
-// in and out 14, 134 M 62; F4 9.4 M 12, 75 M 43; F6 9.4 M 14, 75 M 49; with integer dot products
-// 0.6 M 8, 4.9 M 17).  Fused F2: waves of 128 tiles per SM, full or not (28 us at 64 channels).
+// in and out 14, 134 M 62; F4 2.2 M 9.5, 9.4 M 12, 75 M 43; F6 1.5 M 10.9, 9.4 M 14, 75 M 49; with
+// integer dot products 0.6 M 8, 4.9 M 17).  Fused F2: waves of 128 tiles per SM, full or not (28 us at 64 channels).
 long staged_cost(const wino_plan_t* pl) {
   const double codes = (double)pl->p.t * pl->p.t * pl->p.T * (pl->p.C + pl->p.K);
   if (pl->path == WINO_PATH_STAGED_DP4A) return 6500 + (long)(codes * 1.9e-3);
-  const long gpu = (pl->p.m == 6 ? 9500 : 7500) + (long)(codes * (pl->p.m == 2 ? 4.1e-4 : 4.8e-4));
-  return gpu;
+  return (pl->p.m == 6 ? 9800 : 8500) + (long)(codes * (pl->p.m == 2 ? 4.0e-4 : 4.7e-4));
 }
 long fused_f2_cost(const wino_plan_t* pl) {
   const long waves = ((pl->p.T + 127) / 128 + pl->num_sms - 1) / pl->num_sms;
@@ -497,15 +501,17 @@ int forward_impl(wino_plan_t* pl, const int8_t* x, const int8_t* Uq, const float
   if (pl->path == WINO_PATH_FUSED_SMALL) gemm_path = staged_path_of(pl);
   const bool tma_ok = (pl->path == WINO_PATH_STAGED_TC || pl->path == WINO_PATH_STAGED_TC_MMA) && !calib;
   const bool mma = pl->path == WINO_PATH_STAGED_TC_MMA;
+  const bool out_tc = tma_ok && pl->xt_images != nullptr && output_tc_supported(pl->p, pl->std_mats) &&
+                      (mma || output_tc_pays(pl->p));
   int rc = WINO_OK;
   if (!(stage_mask & 1)) {
   } else if (pl->launches++, tma_ok && pl->xt_images != nullptr && input_tc_supported(pl->p, pl->std_mats) &&
-             (mma || pl->p.z_x != 0 || input_tc_pays(pl->p))) {
+             (mma || input_tc_pays(pl->p))) {
     const CUtensorMap* mx = map_x_tc(pl, x);
     if (mx == nullptr) return WINO_ERR_CUDA;
     rc = launch_input_transform_tc(pl->p, opt_with_hint(pl, pdl, stage_mask, Uq), *mx, pl->xt_images, Vq,
                                    pl->status_dev, st);
-  } else if (tma_ok && pl->p.z_x == 0 && tma_chunk(pl->p.C) != 0) {
+  } else if (tma_ok && pl->p.v_fits_16 && tma_chunk(pl->p.C) != 0) {
     const CUtensorMap* mx = map_x(pl, x);
     const CUtensorMap* mv = map_stage(pl, pl->cache_vst, Vq, pl->p.C, tma_group(tma_chunk(pl->p.C)));
     if (mx == nullptr || mv == nullptr) return WINO_ERR_CUDA;
@@ -517,22 +523,22 @@ int forward_impl(wino_plan_t* pl, const int8_t* x, const int8_t* Uq, const float
   if (stage_mask & 2) {
     pl->path = gemm_path;
     rc = launch_gemm(pl, Vq, Uq, mbuf, pl->p.qM_enabled ? kOutMq : kOutI32,
-                     calib ? absmax4 + 1 : nullptr, pdl, st);
+                     calib ? absmax4 + 1 : nullptr, pdl, st, (stage_mask & 4) && !out_tc);
     pl->path = saved_path;
   }
   if (rc != WINO_OK) return rc;
   if (!(stage_mask & 4)) {
-  } else if (pl->launches++, tma_ok && pl->xt_images != nullptr && output_tc_supported(pl->p, pl->std_mats) &&
-             (mma || pl->p.out_dtype != 0 || output_tc_pays(pl->p))) {
+  } else if (pl->launches++, out_tc) {
     const CUtensorMap* mm = map_m_tc(pl, mbuf);
     if (mm == nullptr) return WINO_ERR_CUDA;
     rc = launch_output_transform_tc(pl->p, opt_of(pl, pdl), *mm, pl->xt_images, bias, y, pl->s_Y, pl->status_dev, st);
-  } else if (tma_ok && pl->p.qM_enabled && pl->p.out_dtype == 0 && tma_chunk(pl->p.K) != 0) {
+  } else if (tma_ok && pl->p.qM_enabled && tma_chunk(pl->p.K) != 0) {
     const CUtensorMap* mm = map_stage(pl, pl->cache_mld, mbuf, pl->p.K, tma_group(tma_chunk(pl->p.K)));
-    const CUtensorMap* my = map_y(pl, y);
+    const bool to_float = pl->p.out_dtype != 0;
+    const CUtensorMap* my = to_float ? mm : map_y(pl, y);
     if (mm == nullptr || my == nullptr) return WINO_ERR_CUDA;
-    rc = launch_output_transform_tma(pl->p, opt_of(pl, pdl), *mm, *my, bias, pl->s_Y,
-                                     pl->status_dev, st);
+    rc = launch_output_transform_tma(pl->p, opt_of(pl, pdl), *mm, *my, bias, pl->s_Y, pl->status_dev,
+                                     to_float ? reinterpret_cast<float*>(y) : nullptr, st);
   } else {
     rc = launch_output_transform(pl->p, opt_of(pl, pdl), pl->s_Y, mbuf, bias, y,
                                  calib ? absmax4 + 2 : nullptr, st);

@@ -27,6 +27,8 @@ struct LaunchOpt {
   // for the per-layer values of Params.  Read by the weight transform, the GEMM epilogues
   // and the output transforms.
   const float* chan = nullptr;
+  // The next kernel of the stream's chain uses no tensor memory: it may be started at once.
+  bool early_trigger = false;
   bool chan_m_fits_16 = false;   // with these multipliers every rounded product of Q_M is below 2^15
 };
 
@@ -78,20 +80,20 @@ int launch_output_transform(const Params& p, const LaunchOpt& o, float s_Y, cons
 int launch_gemm_dp4a(const Params& p, const LaunchOpt& o, const int8_t* Vq, const int8_t* Uq,
                      void* out, int out_mode, unsigned* absmaxM, cudaStream_t st);
 
-// TMA-staged transform kernels (input needs z_x == 0 and C % 16 == 0; output needs
-// Q_M on, int8 output and K % 16 == 0).  Channel chunk per block:
-// (128 channels x 1 tile per block measured best on 256-channel layers: twice the
-// blocks of a 256-channel chunk, so the single wave balances over the SMs)
+// TMA-staged transform kernels (input needs C % 16 == 0; output needs Q_M on and K % 16 == 0).
+// Channel chunk per block: the widest that divides the channels (narrow chunks are short rows,
+// which the copy engine delivers no faster than long ones).
 constexpr int tma_chunk(int channels) {
-  return channels % 128 == 0 ? 128 : channels % 64 == 0 ? 64 : channels % 32 == 0 ? 32
-       : channels % 16 == 0 ? 16 : 0;
+  return channels % 128 == 0 ? 128 : channels % 96 == 0 ? 96 : channels % 80 == 0 ? 80 : channels % 64 == 0 ? 64
+       : channels % 48 == 0 ? 48 : channels % 32 == 0 ? 32 : channels % 16 == 0 ? 16 : 0;
 }
-// tiles per block: 128 threads of two channels
+// tiles per block: about 128 threads of two channels
 constexpr int tma_group(int chunk) { return 256 / chunk; }
 int launch_input_transform_tma(const Params& p, const LaunchOpt& o, const CUtensorMap& mapX,
                                const CUtensorMap& mapV, int* status, cudaStream_t st);
+// y_float: the output when it is float (mapY is then not used), else null.
 int launch_output_transform_tma(const Params& p, const LaunchOpt& o, const CUtensorMap& mapM,
-                                const CUtensorMap& mapY, const float* bias, float s_Y, int* status,
+                                const CUtensorMap& mapY, const float* bias, float s_Y, int* status, float* y_float,
                                 cudaStream_t st);
 
 // Tensor-core transforms (wino_transforms_tc.cu): Cook-Toom matrices; the input side for m = 2, 4, 6,

@@ -22,21 +22,18 @@ bool small_supported(const Params& p) {
   return p.C % 4 == 0 && p.v_fits_16 && p.C <= (p.m == 6 ? 512 : 1024);
 }
 
-// Geometry by estimated time.  The kernel's time is a latency (about a block's own time) while
-// the grid fits the SMs once, and grows by a constant per block beyond that.  Measured on B200,
-// back to back in a graph, one chunk per block, no cluster; latency in us, ns per further block:
-//     16*KB channels      16            32            64
-//     F2             3.4 / 10.7    3.6 / 12.9    4.4 / 17.3
-//     F4             4.3 / 16.9    5.3 / 22.7
-//     F6             6.5 / 43.6    8.5 / 58       (one block per SM)
-// A further chunk adds a quarter to the cost per block, and doubles it where the shared memory
-// then holds one block instead of two; a cluster costs 1 us and a third to a half per block, and
-// clusters of four or eight blocks with an SM each leave SMs unused.  The estimate is within
-// 20 % of the measured time from 1 to 2048 blocks.
+// Geometry by estimated time.  The grid runs in rounds of one or two blocks per SM; a round with
+// one block per SM takes `one` (measured on B200, us, one 64-channel chunk per block):
+//     16*KB channels   16    32    64
+//     F2               3.4   3.6   4.4
+//     F4               4.3   5.3
+//     F6               6.5   8.6
+// plus `more` for every further chunk and 1.1 for the exchange in a cluster; two blocks per SM
+// (shared memory permitting, F2 and F4) take 1.1 (F2) to 1.4 times as long as one.  Clusters of four or eight do not
+// fill every SM.  Within 15 % of the measured time from 1 to 2048 blocks.
 SmallGeom small_geometry(const Params& p, int num_sms) {
-  static const double latency[3][3] = {{3.4, 3.6, 4.4}, {4.3, 5.3, 0}, {6.5, 8.5, 0}};
-  static const double per_block[3][3] = {{10.7, 12.9, 17.3}, {16.9, 22.7, 0}, {43.6, 58.0, 0}};
-  static const double per_chunk[3] = {0.35, 1.25, 1.6};    // latency of a further chunk
+  static const double one[3][3] = {{3.4, 3.6, 4.4}, {4.3, 5.3, 0}, {6.5, 8.6, 0}};
+  static const double more[3][3] = {{0.35, 0.6, 0.9}, {1.25, 1.4, 0}, {1.6, 1.6, 0}};
   const int t2 = p.t * p.t, groups = (p.T + 7) / 8, all_chunks = (p.C + 63) / 64;
   const int mi = p.m / 2 - 1;
   SmallGeom best = {};
@@ -55,16 +52,14 @@ SmallGeom small_geometry(const Params& p, int num_sms) {
       const long blocks = (long)groups * g.n_kblk * S;
       if (blocks > 0x7fffffffl) continue;
       g.grid = (int)blocks;
-      const bool one_per_sm = g.smem > 113 * 1024;
-      double each = per_block[mi][ki] * (0.75 + 0.25 * g.chunks);
-      if (one_per_sm && p.m != 6) each *= 1.75;
-      if (S > 1) each *= p.m == 2 ? 1.5 : 1.3;
-      if (S > 2 && one_per_sm) each *= 2.0;
-      const double over = (double)blocks - (S > 2 && one_per_sm ? 0.75 : 1.0) * num_sms;
-      double ns = 1000.0 * (latency[mi][ki] + per_chunk[mi] * (g.chunks - 1) + (S > 1 ? 1.0 : 0.0));
-      if (over > 0) ns += over * each;
-      if (p.C % 16 != 0) ns += 600.0 * p.m * g.chunks;   // operands by 4-byte loads
-      g.cost = (long)ns;
+      const bool two = p.m != 6 && g.smem <= 113 * 1024;
+      const long sms = S == 8 ? num_sms * 3l / 4 : S == 4 ? num_sms * 9l / 10 : num_sms;
+      const long per_round = two ? 2 * sms : sms, rounds = (blocks + per_round - 1) / per_round;
+      double t1 = one[mi][ki] + more[mi][ki] * (g.chunks - 1) + (S > 1 ? 1.1 : 0.0);
+      if (p.C % 16 != 0) t1 += 0.6 * p.m * g.chunks;   // operands by 4-byte loads
+      const double full = two ? t1 * (p.m == 2 ? 1.1 : 1.4) : t1;
+      const bool last_full = blocks - (rounds - 1) * per_round > sms;
+      g.cost = (long)(1000.0 * ((rounds - 1) * full + (last_full ? full : t1)));
       if (best.cost < 0 || g.cost < best.cost) best = g;
     }
   }

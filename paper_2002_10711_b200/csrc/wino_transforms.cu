@@ -13,7 +13,7 @@ namespace wino {
   int launch_input_transform_tma_m##m(const Params&, const LaunchOpt&, const CUtensorMap&,        \
                                       const CUtensorMap&, int*, cudaStream_t);                    \
   int launch_output_transform_tma_m##m(const Params&, const LaunchOpt&, const CUtensorMap&,       \
-                                       const CUtensorMap&, const float*, float, int*, cudaStream_t);
+                                       const CUtensorMap&, const float*, float, int*, float*, cudaStream_t);
 WINO_DECL(2)
 WINO_DECL(4)
 WINO_DECL(6)
@@ -45,11 +45,11 @@ int launch_input_transform_tma(const Params& p, const LaunchOpt& o, const CUtens
                   : launch_input_transform_tma_m6(p, o, mapX, mapV, status, st);
 }
 int launch_output_transform_tma(const Params& p, const LaunchOpt& o, const CUtensorMap& mapM,
-                                const CUtensorMap& mapY, const float* bias, float s_Y, int* status,
+                                const CUtensorMap& mapY, const float* bias, float s_Y, int* status, float* y_float,
                                 cudaStream_t st) {
-  return p.m == 2 ? launch_output_transform_tma_m2(p, o, mapM, mapY, bias, s_Y, status, st)
-       : p.m == 4 ? launch_output_transform_tma_m4(p, o, mapM, mapY, bias, s_Y, status, st)
-                  : launch_output_transform_tma_m6(p, o, mapM, mapY, bias, s_Y, status, st);
+  return p.m == 2 ? launch_output_transform_tma_m2(p, o, mapM, mapY, bias, s_Y, status, y_float, st)
+       : p.m == 4 ? launch_output_transform_tma_m4(p, o, mapM, mapY, bias, s_Y, status, y_float, st)
+                  : launch_output_transform_tma_m6(p, o, mapM, mapY, bias, s_Y, status, y_float, st);
 }
 
 }  // namespace wino

@@ -3,7 +3,8 @@
 //   - the (m+2)x(m+2)xCC input patches (or the t*t x G x CC block of m_q) arrive
 //     in shared memory by TMA; for the input, coordinates may start at -1 and
 //     run past the image: the hardware fills those bytes with zero, which is
-//     the padding (valid when the input zero point is 0);
+//     the padding (with an input zero point every thread then writes the code
+//     of the real value zero over its own channels' bytes there);
 //   - every thread transforms two channels of one tile in packed fp32, reading and
 //     writing shared memory at compile-time offsets;
 //   - the result leaves by one TMA store (rows past the last tile, or pixels past
@@ -28,8 +29,10 @@ __device__ __forceinline__ void sts_u16(uint32_t addr, uint32_t v) {
 }
 // Two signed bytes as floats: the low byte at weight 1 in a float of exponent 2^23, the high
 // byte in one of exponent 2^15, both with the sign bit flipped: one lop3 each, one packed add.
-__device__ __forceinline__ F2 codes_to_f2(uint32_t h) {
-  return v_add(f2_bits((h & 0xFFu) ^ 0x4B000080u, (h & 0xFF00u) ^ 0x47008000u), f2_make(-8388736.0f, -32896.0f));
+// unbias: minus the two offsets, minus the zero point.
+__device__ __forceinline__ F2 codes_unbias(int z) { return f2_make(-(8388736.0f + (float)z), -(32896.0f + (float)z)); }
+__device__ __forceinline__ F2 codes_to_f2(uint32_t h, F2 unbias) {
+  return v_add(f2_bits((h & 0xFFu) ^ 0x4B000080u, (h & 0xFF00u) ^ 0x47008000u), unbias);
 }
 
 #ifdef WINO_TRACE
@@ -40,12 +43,9 @@ WINO_ST_READER(wino_trace_input, g_in_trace)
 WINO_ST_READER(wino_trace_output, g_out_trace)
 #endif
 
-// S16: the plan guarantees that every rounded product of Q_V fits 16 bits (its clamp is then
-// done on two codes at a time); otherwise the clamp is done in fp32.
-// UPB units per block: for grids of several waves the loads of all are issued up front, so that
-// a later unit's load and an earlier unit's store overlap the arithmetic.
+// Plans whose rounded products of Q_V fit 16 bits (the clamp is done on two codes at a time).
 // MINB: blocks per SM asked of the compiler.
-template <int M, int MODE, int CC, int G, bool S16, int UPB, int MINB>
+template <int M, int MODE, int CC, int G, int MINB>
 __global__ void __launch_bounds__((CC / 2) * G, MINB)
 k_input_transform_tma(const __grid_constant__ Params p, const __grid_constant__ CUtensorMap mapX,
                       const __grid_constant__ CUtensorMap mapV, int* __restrict__ status,
@@ -56,15 +56,15 @@ k_input_transform_tma(const __grid_constant__ Params p, const __grid_constant__ 
   constexpr uint32_t kUnitBytes = G * kTileStride;
   extern __shared__ uint8_t smem_raw[];
   const uint32_t base = (smem_u32(smem_raw) + 127u) & ~127u;
-  const uint32_t s_in0 = base;                      // UPB x [G][T2][CC]
-  const uint32_t s_out0 = base + UPB * kUnitBytes;  // UPB x [T2][G][CC]
-  const uint32_t bar0 = s_out0 + UPB * kUnitBytes;  // UPB barriers
+  const uint32_t s_in = base;                 // [G][T2][CC]
+  const uint32_t s_out = base + kUnitBytes;   // [T2][G][CC]
+  const uint32_t bar = s_out + kUnitBytes;
   __shared__ uint32_t abort_flag;
 
   // unit = (tile group, channel chunk)
   const int cchunks = p.C / CC;
-  const int n_units = ((p.T + G - 1) / G) * cchunks;
-  const int u0 = blockIdx.x * UPB;
+  const int group = (int)blockIdx.x / cchunks, c0 = ((int)blockIdx.x - group * cchunks) * CC;
+  const int tau0 = group * G, ntile = min(G, p.T - tau0);
   const int g = threadIdx.x / TPT, c2 = threadIdx.x % TPT;
 
   int trace_step = 0;
@@ -75,7 +75,7 @@ k_input_transform_tma(const __grid_constant__ Params p, const __grid_constant__ 
   }
   griddep_launch();
   if (threadIdx.x == 0) {
-    for (int r = 0; r < UPB; ++r) mbar_init(bar0 + 8u * r, 1);
+    mbar_init(bar, 1);
     abort_flag = 0u;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     tma_prefetch_map(&mapX);
@@ -85,95 +85,76 @@ k_input_transform_tma(const __grid_constant__ Params p, const __grid_constant__ 
   if (threadIdx.x < 32) {
     // the lanes of warp 0 load a tile each; patch coordinates first: nothing but the loads
     // themselves is left for after the wait
-    const int lane = threadIdx.x;
-    int cw[UPB], ch[UPB], cn[UPB], cc[UPB], nt[UPB];
-#pragma unroll
-    for (int r = 0; r < UPB; ++r) {
-      const int unit = u0 + r, group = unit / cchunks, tau = group * G + lane;
-      cc[r] = (unit - group * cchunks) * CC;
-      nt[r] = unit < n_units ? min(G, p.T - group * G) : 0;
-      const int rest = tau / p.TW;
-      cw[r] = (tau - rest * p.TW) * M - 1;
-      cn[r] = rest / p.TH;
-      ch[r] = (rest - cn[r] * p.TH) * M - 1;
-      // ask for the patches to be brought into L2 while the preceding kernel is still running
-      // (a hint only: nothing is read into the SM before the wait below)
-      if (lane < nt[r]) tma_prefetch_l2_4d(&mapX, cc[r], cw[r], ch[r], cn[r]);
-    }
+    const int lane = threadIdx.x, tau = tau0 + lane, rest = tau / p.TW;
+    const int cw = (tau - rest * p.TW) * M - 1, cn = rest / p.TH, ch = (rest - cn * p.TH) * M - 1;
+    // ask for the patches to be brought into L2 while the preceding kernel is still running
+    // (a hint only: nothing is read into the SM before the wait below)
+    if (lane < ntile) tma_prefetch_l2_4d(&mapX, c0, cw, ch, cn);
     if (lane == 0) l2_hint_slice(l2_hint, l2_hint_bytes);   // what the next kernel will want from HBM
     griddep_wait();   // only this warp reads or writes buffers that other kernels touch
-    if (lane == 0) WINO_ST(g_in_trace, trace_step, 1);
-#pragma unroll
-    for (int r = 0; r < UPB; ++r) {
-      if (lane == 0 && nt[r] > 0) mbar_expect_tx(bar0 + 8u * r, (uint32_t)nt[r] * kTileBytes);
-      __syncwarp();
-      if (lane < nt[r])
-        tma_load_4d(s_in0 + (uint32_t)r * kUnitBytes + (uint32_t)lane * kTileStride, &mapX, bar0 + 8u * r, cc[r], cw[r],
-                    ch[r], cn[r]);
+    if (lane == 0) {
+      WINO_ST(g_in_trace, trace_step, 1);
+      mbar_expect_tx(bar, (uint32_t)ntile * kTileBytes);
     }
-  }
-  const F2 mult = f2_both(p.mult_V), mult_n = f2_both(-p.mult_V), magic = f2_both(kMagic);
-  const uint32_t lo = s16x2_both((int)p.lo_V), hi = s16x2_both((int)p.hi_V);
-  const float lo_f = __fadd_rn(p.lo_V, kMagic), hi_f = __fadd_rn(p.hi_V, kMagic);
-#pragma unroll
-  for (int r = 0; r < UPB; ++r) {
-    const int unit = u0 + r;
-    if (unit >= n_units) break;
-    const int group = unit / cchunks, tau0 = group * G, c0 = (unit - group * cchunks) * CC;
-    const uint32_t s_in = s_in0 + (uint32_t)r * kUnitBytes, s_out = s_out0 + (uint32_t)r * kUnitBytes;
+    __syncwarp();
+    if (lane < ntile) tma_load_4d(s_in + (uint32_t)lane * kTileStride, &mapX, bar, c0, cw, ch, cn);
     // one thread polls (bounded); the others sleep in the barrier below
-    if (threadIdx.x == 0 && !mbar_wait(bar0 + 8u * r, 0u, &abort_flag)) {
-      abort_flag = 1u;
-      atomicExch(status, -6);  // WINO_ERR_TIMEOUT
-    }
-    if (threadIdx.x == 0) WINO_ST(g_in_trace, trace_step, 2);
-    __syncthreads();
-    if (*(volatile uint32_t*)&abort_flag != 0u) return;
-    (void)mbar_try_wait(bar0 + 8u * r, 0u);   // every thread observes the completed phase itself
-    if (tau0 + g < p.T) {
-      const uint32_t rd = s_in + (uint32_t)g * kTileStride + (uint32_t)(2 * c2);
-      const uint32_t wr = s_out + (uint32_t)(g * CC + 2 * c2);
-      F2 V[T2];
-      input_transform_2d<M, MODE>(p, [&](int l, F2 (&dcol)[T_]) {
-#pragma unroll
-        for (int a = 0; a < T_; ++a) dcol[a] = codes_to_f2(lds_u16(rd + (uint32_t)((a * T_ + l) * CC)));
-      }, V);
-#pragma unroll
-      for (int xi = 0; xi < T2; ++xi) {
-        const bool neg = MODE == kExact && (pair_negated<T_>(xi / T_) != pair_negated<T_>(xi % T_));
-        uint32_t w;
-        if constexpr (S16) {
-          w = __byte_perm(quant_s16x2(V[xi], neg ? mult_n : mult, magic, lo, hi), 0u, 0x0020u);
-        } else {
-          uint32_t a, b;
-          f2_split(v_fma(V[xi], neg ? mult_n : mult, magic), a, b);
-          a = __float_as_uint(fminf(fmaxf(__uint_as_float(a), lo_f), hi_f));
-          b = __float_as_uint(fminf(fmaxf(__uint_as_float(b), lo_f), hi_f));
-          w = __byte_perm(a, b, 0x0040u);
-        }
-        sts_u16(wr + (uint32_t)(xi * G * CC), w);
+    if (lane == 0) {
+      if (!mbar_wait(bar, 0u, &abort_flag)) {
+        abort_flag = 1u;
+        atomicExch(status, -6);  // WINO_ERR_TIMEOUT
       }
-    }
-    fence_async_smem();
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      WINO_ST(g_in_trace, trace_step, 3);
-      tma_store_3d(&mapV, s_out, c0, tau0, 0);
-      bulk_commit();
+      WINO_ST(g_in_trace, trace_step, 2);
     }
   }
+  __syncthreads();
+  if (*(volatile uint32_t*)&abort_flag != 0u) return;
+  (void)mbar_try_wait(bar, 0u);   // every thread observes the completed phase itself
+  if (g < ntile) {
+    const uint32_t rd = s_in + (uint32_t)g * kTileStride + (uint32_t)(2 * c2);
+    const uint32_t wr = s_out + (uint32_t)(g * CC + 2 * c2);
+    if (p.z_x != 0) {
+      const int tau = tau0 + g, rest = tau / p.TW, w0 = (tau - rest * p.TW) * M - 1, h0 = rest % p.TH * M - 1;
+      const uint32_t pad = ((uint32_t)p.z_x & 0xFFu) * 0x0101u;
+#pragma unroll 1
+      for (int ab = 0; ab < T2; ++ab)
+        if ((unsigned)(h0 + ab / T_) >= (unsigned)p.H || (unsigned)(w0 + ab % T_) >= (unsigned)p.W)
+          sts_u16(rd + (uint32_t)(ab * CC), pad);
+    }
+    const F2 mult = f2_both(p.mult_V), mult_n = f2_both(-p.mult_V), magic = f2_both(kMagic);
+    const uint32_t lo = s16x2_both((int)p.lo_V), hi = s16x2_both((int)p.hi_V);
+    const F2 unbias = codes_unbias(p.z_x);
+    F2 V[T2];
+    input_transform_2d<M, MODE>(p, [&](int l, F2 (&dcol)[T_]) {
+#pragma unroll
+      for (int a = 0; a < T_; ++a) dcol[a] = codes_to_f2(lds_u16(rd + (uint32_t)((a * T_ + l) * CC)), unbias);
+    }, V);
+#pragma unroll
+    for (int xi = 0; xi < T2; ++xi) {
+      const bool neg = MODE == kExact && (pair_negated<T_>(xi / T_) != pair_negated<T_>(xi % T_));
+      sts_u16(wr + (uint32_t)(xi * G * CC),
+              __byte_perm(quant_s16x2(V[xi], neg ? mult_n : mult, magic, lo, hi), 0u, 0x0020u));
+    }
+  }
+  fence_async_smem();
+  __syncthreads();
   if (threadIdx.x == 0) {
+    WINO_ST(g_in_trace, trace_step, 3);
+    tma_store_3d(&mapV, s_out, c0, tau0, 0);
+    bulk_commit();
     bulk_wait_all();    // the bytes are in place before the block leaves
     WINO_ST(g_in_trace, trace_step, 4);
   }
 }
 
-// PK: the output scale varies per output channel (`chan`, rows kChMultY and kChSY).
-template <int M, int MODE, int KC, int G, bool PK>
+// chan: null, or the scales vary per output channel (rows kChMultY and kChSY, or kChSAcc).  Float
+// output goes to y directly, a pair of channels per store.
+template <int M, int MODE, int KC, int G>
 __global__ void __launch_bounds__((KC / 2) * G)
 k_output_transform_tma(const __grid_constant__ Params p, const __grid_constant__ CUtensorMap mapM,
                        const __grid_constant__ CUtensorMap mapY, const float* __restrict__ bias,
-                       float s_Y, int* __restrict__ status, const float* __restrict__ chan) {
+                       float s_Y, int* __restrict__ status, const float* __restrict__ chan,
+                       float* __restrict__ y_float) {
   constexpr int T_ = M + 2, T2 = T_ * T_, TPT = KC / 2;
   constexpr uint32_t kInBytes = T2 * G * KC;          // [T2][G][KC]
   constexpr uint32_t kTileOutBytes = M * M * KC;      // [M][M][KC] per tile
@@ -181,7 +162,7 @@ k_output_transform_tma(const __grid_constant__ Params p, const __grid_constant__
   extern __shared__ uint8_t smem_raw[];
   const uint32_t base = (smem_u32(smem_raw) + 127u) & ~127u;
   const uint32_t s_in = base;
-  const uint32_t s_out = base + kInBytes;             // [G][M][M][KC]
+  const uint32_t s_out = base + ((kInBytes + 127u) & ~127u);   // [G][M][M][KC]
   const uint32_t bar = s_out + G * kTileOut;
   __shared__ uint32_t abort_flag;
 
@@ -203,7 +184,6 @@ k_output_transform_tma(const __grid_constant__ Params p, const __grid_constant__
     abort_flag = 0u;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     tma_prefetch_map(&mapM);
-    tma_prefetch_map(&mapY);
     griddep_wait();
     WINO_ST(g_out_trace, trace_step, 1);
     mbar_expect_tx(bar, kInBytes);   // the full box counts, clipped rows included
@@ -219,17 +199,21 @@ k_output_transform_tma(const __grid_constant__ Params p, const __grid_constant__
     sn = rest / p.TH;
     sh = (rest - sn * p.TH) * M;
   }
-  F2 mult = f2_both(p.mult_Y), b_pre = f2_both(0.0f);
+  F2 mult = f2_both(y_float != nullptr ? p.s_acc : p.mult_Y), b_pre = f2_both(0.0f);
   {
     const int k = k0 + 2 * k2;
     float s0 = s_Y, s1 = s_Y;
-    if constexpr (PK) {
-      mult = f2_make(__ldg(chan + (long)kChMultY * p.K + k), __ldg(chan + (long)kChMultY * p.K + k + 1));
+    if (chan != nullptr) {
+      const float* row = chan + (long)(y_float != nullptr ? kChSAcc : kChMultY) * p.K + k;
+      mult = f2_make(__ldg(row), __ldg(row + 1));
       s0 = __ldg(chan + (long)kChSY * p.K + k);
       s1 = __ldg(chan + (long)kChSY * p.K + k + 1);
     }
-    if (bias != nullptr)
-      b_pre = f2_make((float)((double)__ldg(bias + k) / (double)s0), (float)((double)__ldg(bias + k + 1) / (double)s1));
+    if (bias != nullptr) {
+      b_pre = f2_make(__ldg(bias + k), __ldg(bias + k + 1));
+      if (y_float == nullptr)
+        b_pre = f2_make((float)((double)__ldg(bias + k) / (double)s0), (float)((double)__ldg(bias + k + 1) / (double)s1));
+    }
   }
   griddep_wait();
   if (threadIdx.x == 0) {
@@ -245,11 +229,26 @@ k_output_transform_tma(const __grid_constant__ Params p, const __grid_constant__
   if (g < ntile) {
     const uint32_t rd = s_in + (uint32_t)(g * KC + 2 * k2);
     const uint32_t wr = s_out + (uint32_t)g * kTileOut + (uint32_t)(2 * k2);
+    const F2 unbias = codes_unbias(0);
     F2 Y[M * M];
     output_transform_2d<M, MODE>(p, [&](int i, F2 (&mrow)[T_]) {
 #pragma unroll
-      for (int j = 0; j < T_; ++j) mrow[j] = codes_to_f2(lds_u16(rd + (uint32_t)((i * T_ + j) * G * KC)));
+      for (int j = 0; j < T_; ++j) mrow[j] = codes_to_f2(lds_u16(rd + (uint32_t)((i * T_ + j) * G * KC)), unbias);
     }, Y);
+    if (y_float != nullptr) {
+      const int tau = tau0 + g, rest = tau / p.TW, w0 = (tau - rest * p.TW) * M, n = rest / p.TH;
+      const int h0 = (rest - n * p.TH) * M;
+      float* yp = y_float + (((long)n * p.H + h0) * p.W + w0) * p.K + k0 + 2 * k2;
+#pragma unroll
+      for (int q = 0; q < M * M; ++q) {
+        const int ip = q / M, jp = q % M;
+        uint32_t a, b;
+        f2_split(v_fma(Y[q], mult, b_pre), a, b);
+        if (h0 + ip < p.H && w0 + jp < p.W)
+          *reinterpret_cast<uint2*>(yp + (long)(ip * p.W + jp) * p.K) = make_uint2(a, b);
+      }
+      return;
+    }
     const F2 magic = f2_both(kMagic);
     const uint32_t z = s16x2_both(p.z_Y);
 #pragma unroll
@@ -263,6 +262,7 @@ k_output_transform_tma(const __grid_constant__ Params p, const __grid_constant__
       sts_u16(wr + (uint32_t)(q * KC), __byte_perm(w, 0u, 0x0020u));
     }
   }
+  if (y_float != nullptr) return;
   fence_async_smem();
   __syncthreads();
   if (threadIdx.x < 32) {
@@ -282,70 +282,67 @@ k_output_transform_tma(const __grid_constant__ Params p, const __grid_constant__
 // ---------------------------------------------------------------------------
 namespace {
 
-template <int M, int MODE, int CC, int G, bool S16, int UPB, int MINB>
-int input_tma_launch_u(const Params& p, const LaunchOpt& o, const CUtensorMap& mapX, const CUtensorMap& mapV,
-                       int* status, cudaStream_t st) {
-  constexpr size_t smem =
-      2 * (size_t)UPB * G * ((((M + 2) * (M + 2) * CC) + 127) / 128 * 128) + 128 + 16 * UPB;
-  auto kernel = k_input_transform_tma<M, MODE, CC, G, S16, UPB, MINB>;
+template <int M, int MODE, int CC, int MINB>
+int input_tma_go(const Params& p, const LaunchOpt& o, const CUtensorMap& mapX, const CUtensorMap& mapV, int* status,
+                 cudaStream_t st) {
+  constexpr int G = tma_group(CC);
+  constexpr size_t smem = 2 * (size_t)G * ((((M + 2) * (M + 2) * CC) + 127) / 128 * 128) + 128 + 16;
+  auto kernel = k_input_transform_tma<M, MODE, CC, G, MINB>;
   static DeviceOnce once;   // one per instantiation
   if (int rc = set_max_smem(once, o.device, kernel, smem)) return rc;
   const int units = ((p.T + G - 1) / G) * (p.C / CC);
-  return launch_kernel(kernel, dim3((unsigned)((units + UPB - 1) / UPB)), dim3((CC / 2) * G), smem, st, o.pdl, p, mapX,
-                       mapV, status, static_cast<const uint8_t*>(o.l2_hint), (uint32_t)o.l2_hint_bytes);
+  return launch_kernel(kernel, dim3((unsigned)units), dim3((CC / 2) * G), smem, st, o.pdl, p, mapX, mapV, status,
+                       static_cast<const uint8_t*>(o.l2_hint), (uint32_t)o.l2_hint_bytes);
 }
 template <int M, int MODE, int CC>
 int input_tma_launch(const Params& p, const LaunchOpt& o, const CUtensorMap& mapX, const CUtensorMap& mapV,
                      int* status, cudaStream_t st) {
-  constexpr int G = tma_group(CC);
-  // two units per block once the grid is several waves deep
-  const long units = (long)((p.T + G - 1) / G) * (p.C / CC);
   // F2 at 48 registers, F4 at 80 (F6 is slower within any limit), F4 at 72 with some spilling only
   // where that makes the grid a single wave: the 1024 blocks of a 256-channel, 1024-tile layer
   constexpr int kMin = MODE != kExact ? 1 : M == 2 ? 10 : M == 4 ? 6 : 1;
-  if (!p.v_fits_16) return input_tma_launch_u<M, MODE, CC, G, false, 1, kMin>(p, o, mapX, mapV, status, st);
-  if (units >= 32l * 148) return input_tma_launch_u<M, MODE, CC, G, true, 2, kMin>(p, o, mapX, mapV, status, st);
-  if constexpr (M == 4 && MODE == kExact)
+  if constexpr (M == 4 && MODE == kExact && CC == 128) {
+    const long units = (long)((p.T + 1) / 2) * (p.C / CC);
     if (units > 6l * o.num_sms && units <= 7l * o.num_sms)
-      return input_tma_launch_u<M, MODE, CC, G, true, 1, 7>(p, o, mapX, mapV, status, st);
-  return input_tma_launch_u<M, MODE, CC, G, true, 1, kMin>(p, o, mapX, mapV, status, st);
+      return input_tma_go<M, MODE, CC, 7>(p, o, mapX, mapV, status, st);
+  }
+  return input_tma_go<M, MODE, CC, kMin>(p, o, mapX, mapV, status, st);
 }
 template <int M, int MODE>
 int input_tma_mode(const Params& p, const LaunchOpt& o, const CUtensorMap& mapX, const CUtensorMap& mapV,
                    int* status, cudaStream_t st) {
   const int cc = tma_chunk(p.C);
   return cc == 128 ? input_tma_launch<M, MODE, 128>(p, o, mapX, mapV, status, st)
+       : cc == 96 ? input_tma_launch<M, MODE, 96>(p, o, mapX, mapV, status, st)
+       : cc == 80 ? input_tma_launch<M, MODE, 80>(p, o, mapX, mapV, status, st)
+       : cc == 48 ? input_tma_launch<M, MODE, 48>(p, o, mapX, mapV, status, st)
        : cc == 64 ? input_tma_launch<M, MODE, 64>(p, o, mapX, mapV, status, st)
        : cc == 32 ? input_tma_launch<M, MODE, 32>(p, o, mapX, mapV, status, st)
                   : input_tma_launch<M, MODE, 16>(p, o, mapX, mapV, status, st);
 }
 
-template <int M, int MODE, int KC, bool PK>
+template <int M, int MODE, int KC>
 int output_tma_launch(const Params& p, const LaunchOpt& o, const CUtensorMap& mapM, const CUtensorMap& mapY,
-                      const float* bias, float s_Y, int* status, cudaStream_t st) {
+                      const float* bias, float s_Y, int* status, float* y_float, cudaStream_t st) {
   constexpr int G = tma_group(KC);
-  constexpr size_t smem = (size_t)G * ((M + 2) * (M + 2) * KC + ((M * M * KC + 127) / 128 * 128)) + 128 + 16;
+  constexpr size_t smem = (G * (M + 2) * (M + 2) * KC + 127) / 128 * 128 + (size_t)G * ((M * M * KC + 127) / 128 * 128) + 128 + 16;
   static DeviceOnce once;   // one per instantiation
-  auto kernel = k_output_transform_tma<M, MODE, KC, G, PK>;
+  auto kernel = k_output_transform_tma<M, MODE, KC, G>;
   if (int rc = set_max_smem(once, o.device, kernel, smem)) return rc;
   const int units = ((p.T + G - 1) / G) * (p.K / KC);
   return launch_kernel(kernel, dim3((unsigned)units), dim3((KC / 2) * G), smem, st, o.pdl, p, mapM, mapY, bias, s_Y,
-                       status, PK ? o.chan : nullptr);
-}
-template <int M, int MODE, bool PK>
-int output_tma_pk(const Params& p, const LaunchOpt& o, const CUtensorMap& mapM, const CUtensorMap& mapY,
-                  const float* bias, float s_Y, int* status, cudaStream_t st) {
-  const int kc = tma_chunk(p.K);
-  return kc == 128 ? output_tma_launch<M, MODE, 128, PK>(p, o, mapM, mapY, bias, s_Y, status, st)
-       : kc == 64 ? output_tma_launch<M, MODE, 64, PK>(p, o, mapM, mapY, bias, s_Y, status, st)
-       : kc == 32 ? output_tma_launch<M, MODE, 32, PK>(p, o, mapM, mapY, bias, s_Y, status, st)
-                  : output_tma_launch<M, MODE, 16, PK>(p, o, mapM, mapY, bias, s_Y, status, st);
+                       status, o.chan, y_float);
 }
 template <int M, int MODE>
 int output_tma_mode(const Params& p, const LaunchOpt& o, const CUtensorMap& mapM, const CUtensorMap& mapY,
-                    const float* bias, float s_Y, int* status, cudaStream_t st) {
-  return o.chan != nullptr ? output_tma_pk<M, MODE, true>(p, o, mapM, mapY, bias, s_Y, status, st)
-                           : output_tma_pk<M, MODE, false>(p, o, mapM, mapY, bias, s_Y, status, st);
+                    const float* bias, float s_Y, int* status, float* y_float, cudaStream_t st) {
+  const int kc = tma_chunk(p.K);
+  return kc == 128 ? output_tma_launch<M, MODE, 128>(p, o, mapM, mapY, bias, s_Y, status, y_float, st)
+       : kc == 96 ? output_tma_launch<M, MODE, 96>(p, o, mapM, mapY, bias, s_Y, status, y_float, st)
+       : kc == 80 ? output_tma_launch<M, MODE, 80>(p, o, mapM, mapY, bias, s_Y, status, y_float, st)
+       : kc == 64 ? output_tma_launch<M, MODE, 64>(p, o, mapM, mapY, bias, s_Y, status, y_float, st)
+       : kc == 48 ? output_tma_launch<M, MODE, 48>(p, o, mapM, mapY, bias, s_Y, status, y_float, st)
+       : kc == 32 ? output_tma_launch<M, MODE, 32>(p, o, mapM, mapY, bias, s_Y, status, y_float, st)
+                  : output_tma_launch<M, MODE, 16>(p, o, mapM, mapY, bias, s_Y, status, y_float, st);
 }
 
 }  // namespace
@@ -360,10 +357,9 @@ int WINO_CAT(launch_input_transform_tma_m, WINO_M)(const Params& p, const Launch
 int WINO_CAT(launch_output_transform_tma_m, WINO_M)(const Params& p, const LaunchOpt& o,
                                                      const CUtensorMap& mapM,
                                                      const CUtensorMap& mapY, const float* bias,
-                                                     float s_Y, int* status, cudaStream_t st) {
-  if (!o.std_mats) return output_tma_mode<WINO_M, kDense>(p, o, mapM, mapY, bias, s_Y, status, st);
-  if (WINO_M != 6) return output_tma_mode<WINO_M, kExact>(p, o, mapM, mapY, bias, s_Y, status, st);
-  return output_tma_mode<WINO_M, kSparse>(p, o, mapM, mapY, bias, s_Y, status, st);
+                                                     float s_Y, int* status, float* y_float, cudaStream_t st) {
+  if (!o.std_mats) return output_tma_mode<WINO_M, kDense>(p, o, mapM, mapY, bias, s_Y, status, y_float, st);
+  return output_tma_mode<WINO_M, WINO_M == 6 ? kSparse : kExact>(p, o, mapM, mapY, bias, s_Y, status, y_float, st);
 }
 
 }  // namespace wino

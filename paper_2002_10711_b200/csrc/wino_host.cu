@@ -349,7 +349,7 @@ const CUtensorMap* map_u_small(wino_plan_t* pl, const void* Uq, int KB) {
 }
 
 int launch_gemm(wino_plan_t* pl, const int8_t* Vq, const int8_t* Uq, void* out, int out_mode,
-                unsigned* absmaxM, bool pdl, cudaStream_t st, bool no_tmem_next = false) {
+                unsigned* absmaxM, bool pdl, cudaStream_t st) {
   const Params& p = pl->p;
   const int t2 = p.t * p.t;
   pl->launches++;
@@ -366,9 +366,7 @@ int launch_gemm(wino_plan_t* pl, const int8_t* Vq, const int8_t* Uq, void* out, 
     if (rc != WINO_OK) return rc;
     pl->map_uq_ptr = Uq;
   }
-  LaunchOpt o = opt_of(pl, pdl);
-  o.early_trigger = no_tmem_next;
-  return launch_gemm_tc(p, o, g, pl->mapV, pl->mapU, out, out_mode, absmaxM,
+  return launch_gemm_tc(p, opt_of(pl, pdl), g, pl->mapV, pl->mapU, out, out_mode, absmaxM,
                         pl->status_dev, st);
 }
 
@@ -523,7 +521,7 @@ int forward_impl(wino_plan_t* pl, const int8_t* x, const int8_t* Uq, const float
   if (stage_mask & 2) {
     pl->path = gemm_path;
     rc = launch_gemm(pl, Vq, Uq, mbuf, pl->p.qM_enabled ? kOutMq : kOutI32,
-                     calib ? absmax4 + 1 : nullptr, pdl, st, (stage_mask & 4) && !out_tc);
+                     calib ? absmax4 + 1 : nullptr, pdl, st);
     pl->path = saved_path;
   }
   if (rc != WINO_OK) return rc;

@@ -27,8 +27,6 @@ struct LaunchOpt {
   // for the per-layer values of Params.  Read by the weight transform, the GEMM epilogues
   // and the output transforms.
   const float* chan = nullptr;
-  // The next kernel of the stream's chain uses no tensor memory: it may be started at once.
-  bool early_trigger = false;
   bool chan_m_fits_16 = false;   // with these multipliers every rounded product of Q_M is below 2^15
 };
 

@@ -166,30 +166,33 @@ k_layer_small(const __grid_constant__ Params p, const __grid_constant__ SmallGeo
   if (p.out_dtype == 0 && bias != nullptr && k_on)
     b_scaled = (float)((double)b_real / (double)chan_or(chan, p.K, kChSY, k, s_Y));
 
-  // 2. input transform of the warp's tile, a channel pair per lane and chunk
-  if (on) {
-    if (tma && !mbar_wait<false>(bar_x, 0u, &abort_flag)) {
-      *(volatile uint32_t*)&abort_flag = 1u;
-      atomicExch(status, -6);  // WINO_ERR_TIMEOUT
-    }
-    if (p.z_x != 0) {
-      // padding is the real value zero, i.e. the code z_x
-      const uint32_t pad = ((uint32_t)p.z_x & 0xFFu) * 0x01010101u;
-      for (int q = 0; q < nq; ++q)
-        for (int i = lane; i < T2 * 16; i += 32) {
-          const int pix = i >> 4, h = h0 + pix / T_, wv = w0 + pix % T_;
-          if ((unsigned)h >= (unsigned)p.H || (unsigned)wv >= (unsigned)p.W)
-            sts32(s_x + (uint32_t)(q * 8 + warp) * kPatch + (uint32_t)(pix * 64 + 4 * (i & 15)), pad);
-        }
-      __syncwarp();
-    }
+  // 2. input transform, one chunk of one tile per warp and round (channel pair per lane).  With
+  // fewer than eight tiles the other warps take further chunks
+  const int n_tile = min(8, p.T - group * 8);
+  if (nq > 0) {
     const F2 unbias = f2_make(-(8388736.0f + (float)p.z_x), -(32896.0f + (float)p.z_x));
     const F2 mult = f2_both(p.mult_V), mult_n = f2_both(-p.mult_V), magic = f2_both(kMagic);
     const uint32_t lo = s16x2_both((int)p.lo_V), hi = s16x2_both((int)p.hi_V);
 #pragma unroll 1
-    for (int q = 0; q < nq; ++q) {
-      const uint32_t src = s_x + (uint32_t)(q * 8 + warp) * kPatch + 2u * (uint32_t)lane;
-      const uint32_t dst = s_v + (uint32_t)q * kVChunk + 64u * (uint32_t)warp + 2u * (uint32_t)lane;
+    for (int task = warp; task < n_tile * nq; task += kSmWarps) {
+      const int q = task / n_tile, tile = task - q * n_tile;
+      if (tma && !mbar_wait<false>(smem_u32(bars) + 8u * (uint32_t)tile, 0u, &abort_flag)) {
+        *(volatile uint32_t*)&abort_flag = 1u;
+        if (lane == 0) atomicExch(status, -6);  // WINO_ERR_TIMEOUT
+      }
+      if (p.z_x != 0) {
+        // padding is the real value zero, i.e. the code z_x
+        const uint32_t pad = ((uint32_t)p.z_x & 0xFFu) * 0x01010101u;
+        const int th0 = p.H - tile_left[tile][0] - 1, tw0 = p.W - tile_left[tile][1] - 1;
+        for (int i = lane; i < T2 * 16; i += 32) {
+          const int pix = i >> 4, h = th0 + pix / T_, wv = tw0 + pix % T_;
+          if ((unsigned)h >= (unsigned)p.H || (unsigned)wv >= (unsigned)p.W)
+            sts32(s_x + (uint32_t)(q * 8 + tile) * kPatch + (uint32_t)(pix * 64 + 4 * (i & 15)), pad);
+        }
+        __syncwarp();
+      }
+      const uint32_t src = s_x + (uint32_t)(q * 8 + tile) * kPatch + 2u * (uint32_t)lane;
+      const uint32_t dst = s_v + (uint32_t)q * kVChunk + 64u * (uint32_t)tile + 2u * (uint32_t)lane;
       F2 V[T2];
       input_transform_2d<M, IMODE>(p, [&](int l, F2 (&dcol)[T_]) {
 #pragma unroll

@@ -149,8 +149,10 @@ k_input_transform_tma(const __grid_constant__ Params p, const __grid_constant__ 
 
 // chan: null, or the scales vary per output channel (rows kChMultY and kChSY, or kChSAcc).  Float
 // output goes to y directly, a pair of channels per store.
+// F4 at 64 registers (eight blocks per SM; seven at the compiler's own 72 cost 0.9 us on a layer of
+// 1200 blocks).
 template <int M, int MODE, int KC, int G>
-__global__ void __launch_bounds__((KC / 2) * G)
+__global__ void __launch_bounds__((KC / 2) * G, M == 4 && MODE == kExact ? 8 : 1)
 k_output_transform_tma(const __grid_constant__ Params p, const __grid_constant__ CUtensorMap mapM,
                        const __grid_constant__ CUtensorMap mapY, const float* __restrict__ bias,
                        float s_Y, int* __restrict__ status, const float* __restrict__ chan,

@@ -4,6 +4,7 @@
 // network's strided convolutions, for which no Winograd form exists (Section 5.1).
 // Integer dot products on the ALUs; thread = (output pixel, 4 or 8 output channels).
 #include "wino_launch.h"
+#include "wino_warp_mma.cuh"
 
 namespace wino {
 
@@ -169,14 +170,6 @@ __device__ __forceinline__ void narrow_k(const uint32_t (&r)[3][3], uint32_t (&k
     }
   }
 }
-__device__ __forceinline__ void narrow_mma(int (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0,
-                                           uint32_t b1) {
-  asm volatile("mma.sync.aligned.m16n8k32.row.col.s32.s8.s8.s32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, "
-               "{%0, %1, %2, %3};"
-               : "+r"(d[0]), "+r"(d[1]), "+r"(d[2]), "+r"(d[3])
-               : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
-}
-
 template <int C, bool Z>
 __global__ void __launch_bounds__(kNarrowThreads)
 k_direct_conv_narrow(const DirectParams p, const int8_t* __restrict__ x, const int8_t* __restrict__ w,
@@ -274,7 +267,7 @@ k_direct_conv_narrow(const DirectParams p, const int8_t* __restrict__ x, const i
       for (int j = 0; j < 8; ++j) {
         int d[4] = {0, 0, 0, 0};
 #pragma unroll
-        for (int q = 0; q < STEPS; ++q) narrow_mma(d, a0[q].x, a1[q].x, a0[q].y, a1[q].y, bf[j][q][0], bf[j][q][1]);
+        for (int q = 0; q < STEPS; ++q) mma_s8(d, a0[q].x, a1[q].x, a0[q].y, a1[q].y, bf[j][q][0], bf[j][q][1]);
         const int kc = 16 * t + 2 * j;
         if constexpr (Z) {
           const int s0 = s_corr[kc], s1 = s_corr[kc + 1];

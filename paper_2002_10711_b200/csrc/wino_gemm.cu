@@ -8,64 +8,130 @@
 //                 kind::i8 accumulate in int32 in tensor memory, two accumulator
 //                 buffers let the epilogue of one block overlap the MMAs of the
 //                 next.
-//   k_gemm_dp4a : the same contraction with 4-way integer dot products on the
-//                 ALUs; fallback for channel counts the TMA path cannot take.
+//   k_gemm_warp : the same contraction with int8 warp MMAs; for channel counts
+//                 the TMA path cannot take.
 #include "wino_f32x2.cuh"
 #include "wino_launch.h"
 #include "wino_ptx.cuh"
 #include "wino_trace.cuh"
+#include "wino_warp_mma.cuh"
 
 namespace wino {
 
 // ---------------------------------------------------------------------------
-// ALU fallback.  Thread = (xi, tau, 4 consecutive k).
+// Fallback for channel counts that are multiples of four only, which tensor copies cannot address,
+// and for the narrowest layers: int8 warp MMAs.  A block of eight warps owns 32 * 8 / WN tiles x
+// 32 * WN output channels of one position; 64-channel chunks of both operands arrive by
+// asynchronous copies of 4, 8 or 16 bytes (zeros past C, T and K), two buffers.  A warp's 32 x 32
+// product takes its fragments 16 bytes at a time: both operands' channels are permuted alike inside
+// a chunk, and lane t of a quad is given the columns of channels 8 t .. 8 t + 7, which it stores at
+// once.  128 -> 512 channels, 726 tiles, F4: 20 us; one thread per four sums with dot products, each
+// operand word from global memory, took 1500.
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(128)
-k_gemm_dp4a(const __grid_constant__ Params p, const int8_t* __restrict__ Vq,
-            const int8_t* __restrict__ Uq, void* __restrict__ out, int out_mode,
-            unsigned* __restrict__ absmaxM, const float* __restrict__ chan) {
-  const int C4 = p.C >> 2, K4 = p.K >> 2;
-  const int xi = blockIdx.z;
-  const long idx = blockIdx.x * (long)blockDim.x + threadIdx.x;
-  float vmax = 0.0f;
+template <int WN>
+__global__ void __launch_bounds__(256)
+k_gemm_warp(const __grid_constant__ Params p, const int8_t* __restrict__ Vq, const int8_t* __restrict__ Uq,
+            void* __restrict__ out, int out_mode, unsigned* __restrict__ absmaxM, const float* __restrict__ chan) {
+  constexpr int kRowsA = 32 * 8 / WN, kRowsB = 32 * WN;
+  __shared__ __align__(128) uint8_t s_a[2][kRowsA * 64];
+  __shared__ __align__(128) uint8_t s_b[2][kRowsB * 64];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
+  const int tau0 = blockIdx.x * kRowsA, k0 = blockIdx.y * kRowsB, xi = blockIdx.z;
+  const int8_t* v = Vq + ((long)xi * p.T + tau0) * p.C;
+  const int8_t* u = Uq + ((long)xi * p.K + k0) * p.C;
+  const int lg = (p.C & 15) == 0 ? 2 : (p.C & 7) == 0 ? 3 : 4, per = 64 >> lg;   // 4, 8 or 16 pieces a row
+  const int at = (tid & ((1 << lg) - 1)) * per, row0 = tid >> lg, rows = 256 >> lg;
   griddep_launch();
+  auto load = [&](int ch) {
+    const int c = ch * 64 + at;
+    const uint32_t a = smem_u32(s_a[ch & 1]), b = smem_u32(s_b[ch & 1]);
+    for (int r = row0; r < kRowsA; r += rows) {
+      const bool in = c < p.C && tau0 + r < p.T;
+      cp_async_zfill(a + (uint32_t)(r * 64 + at), v + (in ? (long)r * p.C + c : 0), per, in);
+    }
+    for (int r = row0; r < kRowsB; r += rows) {
+      const bool in = c < p.C && k0 + r < p.K;
+      cp_async_zfill(b + (uint32_t)(r * 64 + at), u + (in ? (long)r * p.C + c : 0), per, in);
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  const int wm = (warp / WN) * 32, wn = (warp % WN) * 32;   // this warp's 32 x 32
+  int acc[2][4][4];
+#pragma unroll
+  for (int i = 0; i < 2; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) acc[i][j][0] = acc[i][j][1] = acc[i][j][2] = acc[i][j][3] = 0;
   griddep_wait();
-  if (idx < (long)p.T * K4) {
-    const int k4 = (int)(idx % K4);
-    const int tau = (int)(idx / K4);
-    const int* v = reinterpret_cast<const int*>(Vq) + ((long)xi * p.T + tau) * C4;
-    const int* u = reinterpret_cast<const int*>(Uq) + ((long)xi * p.K + k4 * 4) * C4;
-    int acc[4] = {0, 0, 0, 0};
-    for (int c4 = 0; c4 < C4; ++c4) {
-      const int vv = __ldg(v + c4);
-#pragma unroll
-      for (int j = 0; j < 4; ++j) acc[j] = __dp4a(vv, __ldg(u + (long)j * C4 + c4), acc[j]);
-    }
-    const long o = ((long)xi * p.T + tau) * p.K + k4 * 4;
-    if (out_mode == kOutI32) {
-      *reinterpret_cast<int4*>(reinterpret_cast<int*>(out) + o) =
-          make_int4(acc[0], acc[1], acc[2], acc[3]);
+  const int n_ch = (p.C + 63) / 64;
+  load(0);
+  for (int ch = 0; ch < n_ch; ++ch) {
+    if (ch + 1 < n_ch) {
+      load(ch + 1);
+      asm volatile("cp.async.wait_group 1;" ::: "memory");
     } else {
-      uint32_t wv = 0;
+      asm volatile("cp.async.wait_group 0;" ::: "memory");
+    }
+    __syncthreads();
+    const uint32_t a = smem_u32(s_a[ch & 1]) + (uint32_t)((wm + g) * 64 + t * 16);
+    const uint32_t b = smem_u32(s_b[ch & 1]) + (uint32_t)(wn * 64 + t * 16);
+    uint4 af[2][2];
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        float r = quant_magic(__int2float_rn(acc[j]), chan_or(chan, p.K, kChMultM, k4 * 4 + j, p.mult_M),
-                              p.lo_M, p.hi_M);
-        wv |= (__float_as_uint(r) & 0xFFu) << (8 * j);
-      }
-      *reinterpret_cast<uint32_t*>(reinterpret_cast<int8_t*>(out) + o) = wv;
+    for (int i = 0; i < 2; ++i) {
+      af[i][0] = lds128(a + (uint32_t)(i * 1024));
+      af[i][1] = lds128(a + (uint32_t)(i * 1024 + 512));
     }
 #pragma unroll
-    for (int j = 0; j < 4; ++j) vmax = fmaxf(vmax, fabsf(__int2float_rn(acc[j])));
+    for (int j = 0; j < 4; ++j) {
+      // column n = g of product j: channel 8 (g / 2) + 2 j + (g & 1)
+      const uint4 bf = lds128(b + (uint32_t)((8 * (g >> 1) + 2 * j + (g & 1)) * 64));
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        mma_s8(acc[i][j], af[i][0].x, af[i][1].x, af[i][0].y, af[i][1].y, bf.x, bf.y);
+        mma_s8(acc[i][j], af[i][0].z, af[i][1].z, af[i][0].w, af[i][1].w, bf.z, bf.w);
+      }
+    }
+    __syncthreads();
   }
+  float vmax = 0.0f;
+  const int k = k0 + wn + 8 * t;
+  float mult[8];
+#pragma unroll
+  for (int e = 0; e < 8; ++e) mult[e] = k + e < p.K ? chan_or(chan, p.K, kChMultM, k + e, p.mult_M) : 0.0f;
+#pragma unroll
+  for (int i = 0; i < 2; ++i)
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {   // rows g and g + 8 of 16-row block i
+      const int tau = tau0 + wm + 16 * i + 8 * h + g;
+      if (tau >= p.T) continue;
+      const long o = ((long)xi * p.T + tau) * p.K + k;
+#pragma unroll
+      for (int half = 0; half < 2; ++half) {
+        if (k + 4 * half >= p.K) continue;
+        const int m0 = acc[i][2 * half][2 * h], m1 = acc[i][2 * half][2 * h + 1];
+        const int m2 = acc[i][2 * half + 1][2 * h], m3 = acc[i][2 * half + 1][2 * h + 1];
+        const float f0 = __int2float_rn(m0), f1 = __int2float_rn(m1), f2 = __int2float_rn(m2), f3 = __int2float_rn(m3);
+        vmax = fmaxf(fmaxf(vmax, fmaxf(fabsf(f0), fabsf(f1))), fmaxf(fabsf(f2), fabsf(f3)));
+        if (out_mode == kOutI32) {
+          *reinterpret_cast<int4*>(reinterpret_cast<int*>(out) + o + 4 * half) = make_int4(m0, m1, m2, m3);
+        } else {
+          const uint32_t r0 = __float_as_uint(quant_magic(f0, mult[4 * half], p.lo_M, p.hi_M));
+          const uint32_t r1 = __float_as_uint(quant_magic(f1, mult[4 * half + 1], p.lo_M, p.hi_M));
+          const uint32_t r2 = __float_as_uint(quant_magic(f2, mult[4 * half + 2], p.lo_M, p.hi_M));
+          const uint32_t r3 = __float_as_uint(quant_magic(f3, mult[4 * half + 3], p.lo_M, p.hi_M));
+          *reinterpret_cast<uint32_t*>(reinterpret_cast<int8_t*>(out) + o + 4 * half) =
+              __byte_perm(__byte_perm(r0, r1, 0x0040u), __byte_perm(r2, r3, 0x0040u), 0x5410u);
+        }
+      }
+    }
   if (absmaxM != nullptr) atomic_absmax(absmaxM, vmax);
 }
 
-int launch_gemm_dp4a(const Params& p, const LaunchOpt& o, const int8_t* Vq, const int8_t* Uq,
-                     void* out, int out_mode, unsigned* absmaxM, cudaStream_t st) {
-  const long total = (long)p.T * (p.K / 4);
-  dim3 grid((unsigned)((total + 127) / 128), 1, (unsigned)(p.t * p.t));
-  return launch_kernel(k_gemm_dp4a, grid, dim3(128), 0, st, o.pdl, p, Vq, Uq, out, out_mode,
+int launch_gemm_warp(const Params& p, const LaunchOpt& o, const int8_t* Vq, const int8_t* Uq, void* out, int out_mode,
+                     unsigned* absmaxM, cudaStream_t st) {
+  const bool wide = p.K > 32;
+  const dim3 grid((unsigned)(wide ? (p.T + 127) / 128 : (p.T + 255) / 256), (unsigned)(wide ? (p.K + 63) / 64 : 1),
+                  (unsigned)(p.t * p.t));
+  return launch_kernel(wide ? k_gemm_warp<2> : k_gemm_warp<1>, grid, dim3(256), 0, st, o.pdl, p, Vq, Uq, out, out_mode,
                        absmaxM, o.chan);
 }
 

@@ -354,7 +354,7 @@ int launch_gemm(wino_plan_t* pl, const int8_t* Vq, const int8_t* Uq, void* out, 
   const int t2 = p.t * p.t;
   pl->launches++;
   if (pl->path == WINO_PATH_STAGED_DP4A)
-    return launch_gemm_dp4a(p, opt_of(pl, pdl), Vq, Uq, out, out_mode, absmaxM, st);
+    return launch_gemm_warp(p, opt_of(pl, pdl), Vq, Uq, out, out_mode, absmaxM, st);
   const TcGeom g = tc_geometry(p, pl->num_sms);
   if (pl->map_vq_ptr != Vq) {
     int rc = encode_map(&pl->mapV, Vq, (uint64_t)p.C, (uint64_t)p.T, (uint64_t)t2, kBM);
@@ -380,12 +380,19 @@ int launch_gemm(wino_plan_t* pl, const int8_t* Vq, const int8_t* Uq, void* out, 
 //           F4  9.4 M 4.6 / 5.2   18.9 M 7.8 / 7.7   37.7 M 13.6 / 11.9
 // With an input zero point the ALU kernel would also have to patch the padding of border tiles
 // (14 -> 19 us on a 160-channel 12 x 22 layer).
+// A quarter of a unit's channels at most may be padding.
+bool xt_fills(int channels) {
+  const int chunk = xt_chunk(channels), padded = (channels + chunk - 1) / chunk * chunk;
+  return 3 * padded <= 4 * channels;
+}
 bool input_tc_pays(const Params& p) {
+  if (!xt_fills(p.C)) return false;
   if (p.z_x != 0) return true;
   const double codes = (double)p.t * p.t * p.T * p.C;
   return codes > (p.m == 2 ? 12e6 : p.m == 4 ? 14e6 : 7e6);
 }
 bool output_tc_pays(const Params& p) {
+  if (!xt_fills(p.K)) return false;
   const double codes = (double)p.t * p.t * p.T * p.K;
   return codes > (p.m == 2 ? 11e6 : 18e6);
 }
@@ -490,14 +497,15 @@ int forward_impl(wino_plan_t* pl, const int8_t* x, const int8_t* Uq, const float
     pl->last_stream = st;
     return WINO_OK;
   }
-  // calibration on a single-kernel plan runs the staged kernels (dp4a or tcgen05 middle stage)
+  // calibration on a single-kernel plan runs the staged kernels (warp-MMA or tcgen05 middle stage)
   const int saved_path = pl->path;
   int gemm_path = pl->path;
   if (pl->path == WINO_PATH_SMALLC) gemm_path = WINO_PATH_STAGED_DP4A;
   if (pl->path == WINO_PATH_FUSED_F2) gemm_path = WINO_PATH_STAGED_TC_PTR;
   if (pl->path == WINO_PATH_FUSED_LAYER) gemm_path = WINO_PATH_STAGED_TC;
   if (pl->path == WINO_PATH_FUSED_SMALL) gemm_path = staged_path_of(pl);
-  const bool tma_ok = (pl->path == WINO_PATH_STAGED_TC || pl->path == WINO_PATH_STAGED_TC_MMA) && !calib;
+  const bool tma_ok = (pl->path == WINO_PATH_STAGED_TC || pl->path == WINO_PATH_STAGED_TC_MMA ||
+                       pl->path == WINO_PATH_STAGED_DP4A) && !calib;
   const bool mma = pl->path == WINO_PATH_STAGED_TC_MMA;
   const bool out_tc = tma_ok && pl->xt_images != nullptr && output_tc_supported(pl->p, pl->std_mats) &&
                       (mma || output_tc_pays(pl->p));
@@ -509,9 +517,10 @@ int forward_impl(wino_plan_t* pl, const int8_t* x, const int8_t* Uq, const float
     if (mx == nullptr) return WINO_ERR_CUDA;
     rc = launch_input_transform_tc(pl->p, opt_with_hint(pl, pdl, stage_mask, Uq), *mx, pl->xt_images, Vq,
                                    pl->status_dev, st);
-  } else if (tma_ok && pl->p.v_fits_16 && tma_chunk(pl->p.C) != 0) {
+  } else if (tma_ok && pl->p.v_fits_16 && tma_chunk(pl->p.C) != 0 &&
+             !(pl->path == WINO_PATH_STAGED_DP4A && pl->p.C == 16)) {   // 16-byte rows: plain loads are faster
     const CUtensorMap* mx = map_x(pl, x);
-    const CUtensorMap* mv = map_stage(pl, pl->cache_vst, Vq, pl->p.C, tma_group(tma_chunk(pl->p.C)));
+    const CUtensorMap* mv = map_stage(pl, pl->cache_vst, Vq, pl->p.C, tma_in_group(pl->p.m, tma_chunk(pl->p.C)));
     if (mx == nullptr || mv == nullptr) return WINO_ERR_CUDA;
     rc = launch_input_transform_tma(pl->p, opt_with_hint(pl, pdl, stage_mask, Uq), *mx, *mv, pl->status_dev, st);
   } else {

@@ -56,7 +56,7 @@ SmallGeom small_geometry(const Params& p, int num_sms) {
       const long sms = S == 8 ? num_sms * 3l / 4 : S == 4 ? num_sms * 9l / 10 : num_sms;
       const long per_round = two ? 2 * sms : sms, rounds = (blocks + per_round - 1) / per_round;
       double t1 = one[mi][ki] + more[mi][ki] * (g.chunks - 1) + (S > 1 ? 1.1 : 0.0);
-      if (p.C % 16 != 0) t1 += 0.6 * p.m * g.chunks;   // operands by 4-byte loads
+      if (p.C % 16 != 0) t1 += 0.6 * p.m * g.chunks * KB;   // operands by small copies
       const double full = two ? t1 * (p.m == 2 ? 1.1 : 1.4) : t1;
       const bool last_full = blocks - (rounds - 1) * per_round > sms;
       g.cost = (long)(1000.0 * ((rounds - 1) * full + (last_full ? full : t1)));

@@ -23,6 +23,7 @@
 #include "wino_launch.h"
 #include "wino_ptx.cuh"
 #include "wino_transform_math.cuh"
+#include "wino_warp_mma.cuh"
 
 #define WINO_CAT_(a, b) a##b
 #define WINO_CAT(a, b) WINO_CAT_(a, b)
@@ -35,19 +36,6 @@ namespace {
 constexpr int kSmThreads = 256;
 constexpr int kSmWarps = kSmThreads / 32;
 
-__device__ __forceinline__ uint4 lds128(uint32_t addr) {
-  uint4 v;
-  asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];"
-               : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr));
-  return v;
-}
-__device__ __forceinline__ void mma_s8(int (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3,
-                                       uint32_t b0, uint32_t b1) {
-  asm volatile("mma.sync.aligned.m16n8k32.row.col.s32.s8.s8.s32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, "
-               "{%8, %9}, {%0, %1, %2, %3};"
-               : "+r"(d[0]), "+r"(d[1]), "+r"(d[2]), "+r"(d[3])
-               : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
-}
 __device__ __forceinline__ uint32_t cluster_addr(uint32_t addr, uint32_t rank) {
   uint32_t r;
   asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
@@ -63,7 +51,7 @@ __device__ __forceinline__ void cluster_sync() {
 }
 
 // IMODE / OMODE: modes of the input and output transform (wino_transform_math.cuh).
-// TMA: operands by tensor copies (C a multiple of 16); otherwise by 4-byte loads.
+// Operands by tensor copies where C is a multiple of 16, otherwise by small asynchronous copies.
 template <int M, int IMODE, int OMODE, int KB>
 __global__ void __launch_bounds__(kSmThreads, M == 6 ? 1 : 2)
 k_layer_small(const __grid_constant__ Params p, const __grid_constant__ SmallGeom a,
@@ -136,21 +124,27 @@ k_layer_small(const __grid_constant__ Params p, const __grid_constant__ SmallGeo
     }
     __syncwarp();
   } else {
-    // the same rows by 4-byte loads, zeros where TMA would have filled them in
-    for (int i = tid; i < nq * T2 * KS * 16; i += kSmThreads) {
-      const int w = i & 15, row = i >> 4, kk = row & (KS - 1), xi = (row / KS) % T2, c = c0 + (row / (KS * T2)) * 64 + 4 * w;
-      const bool in = c < p.C && k0 + kk < p.K;
-      sts32(s_u + 4u * (uint32_t)i,
-            in ? __ldg(reinterpret_cast<const uint32_t*>(Uq + ((long)xi * p.K + k0 + kk) * p.C + c)) : 0u);
-    }
-    if (on)
-      for (int i = lane; i < nq * T2 * 16; i += 32) {
-        const int w = i & 15, pix = (i >> 4) % T2, q = (i >> 4) / T2;
-        const int h = h0 + pix / T_, wv = w0 + pix % T_, c = c0 + q * 64 + 4 * w;
-        const bool in = c < p.C && (unsigned)h < (unsigned)p.H && (unsigned)wv < (unsigned)p.W;
-        sts32(s_x + (uint32_t)(q * 8 + warp) * kPatch + (uint32_t)(pix * 64 + 4 * w),
-              in ? __ldg(reinterpret_cast<const uint32_t*>(x + (((long)n_w * p.H + h) * p.W + wv) * p.C + c)) : 0u);
+    // the same rows by asynchronous copies of 8 or 4 bytes, zeros where TMA would have filled them
+    // in; a thread keeps its column and walks down the rows
+    const int lg = (p.C & 7) == 0 ? 3 : 4, cols = 1 << lg, per = 64 >> lg;   // columns of 8 or 4 bytes
+    const int at = (tid & (cols - 1)) * per;
+    for (int q = 0; q < nq; ++q) {
+      const int c = c0 + q * 64 + at;
+      for (int row = tid >> lg; row < T2 * KS; row += kSmThreads >> lg) {
+        const int xi = row / KS, k = k0 + (row & (KS - 1));
+        const bool in = c < p.C && k < p.K;
+        cp_async_zfill(s_u + (uint32_t)q * kUChunk + (uint32_t)(row * 64 + at),
+                       Uq + (in ? ((long)xi * p.K + k) * p.C + c : 0), per, in);
       }
+      if (on)
+        for (int pix = lane >> lg; pix < T2; pix += 32 >> lg) {
+          const int h = h0 + pix / T_, wv = w0 + pix % T_;
+          const bool in = c < p.C && (unsigned)h < (unsigned)p.H && (unsigned)wv < (unsigned)p.W;
+          cp_async_zfill(s_x + (uint32_t)(q * 8 + warp) * kPatch + (uint32_t)(pix * 64 + at),
+                         x + (in ? (((long)n_w * p.H + h) * p.W + wv) * p.C + c : 0), per, in);
+        }
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
     __syncthreads();
   }
 

@@ -287,7 +287,7 @@ namespace {
 template <int M, int MODE, int CC, int MINB>
 int input_tma_go(const Params& p, const LaunchOpt& o, const CUtensorMap& mapX, const CUtensorMap& mapV, int* status,
                  cudaStream_t st) {
-  constexpr int G = tma_group(CC);
+  constexpr int G = tma_in_group(M, CC);
   constexpr size_t smem = 2 * (size_t)G * ((((M + 2) * (M + 2) * CC) + 127) / 128 * 128) + 128 + 16;
   auto kernel = k_input_transform_tma<M, MODE, CC, G, MINB>;
   static DeviceOnce once;   // one per instantiation
@@ -300,12 +300,13 @@ template <int M, int MODE, int CC>
 int input_tma_launch(const Params& p, const LaunchOpt& o, const CUtensorMap& mapX, const CUtensorMap& mapV,
                      int* status, cudaStream_t st) {
   // F2 at 48 registers, F4 at 80 (F6 is slower within any limit), F4 at 72 with some spilling only
-  // where that makes the grid a single wave: the 1024 blocks of a 256-channel, 1024-tile layer
-  constexpr int kMin = MODE != kExact ? 1 : M == 2 ? 10 : M == 4 ? 6 : 1;
+  // where that makes the grid a single wave: the 2048 blocks of a 256-channel, 1024-tile layer
+  constexpr int kHalf = tma_in_group(M, CC) * CC <= 128 ? 2 : 1;   // blocks of 64 threads
+  constexpr int kMin = MODE != kExact ? 1 : M == 2 ? 10 : M == 4 ? 6 * kHalf : 1;
   if constexpr (M == 4 && MODE == kExact && CC == 128) {
-    const long units = (long)((p.T + 1) / 2) * (p.C / CC);
-    if (units > 6l * o.num_sms && units <= 7l * o.num_sms)
-      return input_tma_go<M, MODE, CC, 7>(p, o, mapX, mapV, status, st);
+    const long units = (long)p.T * (p.C / CC);
+    if (units > 12l * o.num_sms && units <= 14l * o.num_sms)
+      return input_tma_go<M, MODE, CC, 14>(p, o, mapX, mapV, status, st);
   }
   return input_tma_go<M, MODE, CC, kMin>(p, o, mapX, mapV, status, st);
 }

@@ -428,7 +428,7 @@ int forward_small(wino_plan_t* pl, const int8_t* x, const int8_t* Uq, const floa
   const CUtensorMap none = {};
   SmallArgs a;
   a.mapX = a.mapU = &none;
-  if (pl->p.C % 16 == 0) {
+  if (g.tma) {
     a.mapX = map_x_small(pl, x);
     a.mapU = map_u_small(pl, Uq, g.KB);
     if (a.mapX == nullptr || a.mapU == nullptr) return WINO_ERR_CUDA;

@@ -146,7 +146,7 @@ int launch_smallc(const Params& p, const LaunchOpt& o, const int8_t* x, const in
 // `chunks` chunks of 64 channels each.  `cost`: the launcher's estimate of the kernel's time, ns.
 // The maps (C a multiple of 16): x as [N][H][W][C] with box {64, t, t, 1}, U_q as [t*t][K][C]
 // with box {64, 16*KB, t*t}, no swizzle.
-struct SmallGeom { int KB, chunks, S, n_kblk, grid; size_t smem; long cost; };
+struct SmallGeom { int KB, chunks, S, n_kblk, grid, tma; size_t smem; long cost; };
 struct SmallArgs {
   const CUtensorMap *mapX, *mapU;
   const int8_t *x, *Uq;

@@ -34,6 +34,7 @@ bool small_supported(const Params& p) {
 SmallGeom small_geometry(const Params& p, int num_sms) {
   static const double one[3][3] = {{3.4, 3.6, 4.4}, {4.3, 5.3, 0}, {6.5, 8.6, 0}};
   static const double more[3][3] = {{0.35, 0.6, 0.9}, {1.25, 1.4, 0}, {1.6, 1.6, 0}};
+  static const double small_copies[3] = {1.0, 2.2, 3.2};
   const int t2 = p.t * p.t, groups = (p.T + 7) / 8, all_chunks = (p.C + 63) / 64;
   const int mi = p.m / 2 - 1;
   SmallGeom best = {};
@@ -56,7 +57,11 @@ SmallGeom small_geometry(const Params& p, int num_sms) {
       const long sms = S == 8 ? num_sms * 3l / 4 : S == 4 ? num_sms * 9l / 10 : num_sms;
       const long per_round = two ? 2 * sms : sms, rounds = (blocks + per_round - 1) / per_round;
       double t1 = one[mi][ki] + more[mi][ki] * (g.chunks - 1) + (S > 1 ? 1.1 : 0.0);
-      if (p.C % 16 != 0) t1 += 0.6 * p.m * g.chunks * KB;   // operands by small copies
+      // Tensor copies need whole 16-byte pieces; of rows narrower than a chunk they fill in the rest,
+      // which the copy engine does slowly (16 channels, F2: 2.7 us with a block or two, 7.5 with 128,
+      // where small copies take 3.3 and 5.1).
+      g.tma = p.C % 16 == 0 && (p.C >= 64 || blocks <= 48);
+      if (!g.tma) t1 += small_copies[mi] * (KB > 1 ? 1.5 : 1.0) * g.chunks * (p.C % 16 != 0 ? 1.15 : 1.0);
       const double full = two ? t1 * (p.m == 2 ? 1.1 : 1.4) : t1;
       const bool last_full = blocks - (rounds - 1) * per_round > sms;
       g.cost = (long)(1000.0 * ((rounds - 1) * full + (last_full ? full : t1)));

@@ -51,7 +51,7 @@ __device__ __forceinline__ void cluster_sync() {
 }
 
 // IMODE / OMODE: modes of the input and output transform (wino_transform_math.cuh).
-// Operands by tensor copies where C is a multiple of 16, otherwise by small asynchronous copies.
+// Operands by tensor copies (a.tma) or by small asynchronous copies.
 template <int M, int IMODE, int OMODE, int KB>
 __global__ void __launch_bounds__(kSmThreads, M == 6 ? 1 : 2)
 k_layer_small(const __grid_constant__ Params p, const __grid_constant__ SmallGeom a,
@@ -80,7 +80,7 @@ k_layer_small(const __grid_constant__ Params p, const __grid_constant__ SmallGeo
   const int group = blk / a.n_kblk, k0 = (blk - group * a.n_kblk) * KS;
   const int c0 = (int)rank * a.chunks * 64;
   const int nq = min(a.chunks, (p.C - c0 + 63) / 64);          // chunks of this block (0 or less: none)
-  const bool tma = (p.C & 15) == 0;
+  const bool tma = a.tma != 0;
 
   // this warp's tile
   const int tau_w = group * 8 + warp;
@@ -124,9 +124,9 @@ k_layer_small(const __grid_constant__ Params p, const __grid_constant__ SmallGeo
     }
     __syncwarp();
   } else {
-    // the same rows by asynchronous copies of 8 or 4 bytes, zeros where TMA would have filled them
-    // in; a thread keeps its column and walks down the rows
-    const int lg = (p.C & 7) == 0 ? 3 : 4, cols = 1 << lg, per = 64 >> lg;   // columns of 8 or 4 bytes
+    // the same rows by asynchronous copies of 16, 8 or 4 bytes, zeros where TMA would have filled
+    // them in; a thread keeps its column and walks down the rows
+    const int lg = (p.C & 15) == 0 ? 2 : (p.C & 7) == 0 ? 3 : 4, cols = 1 << lg, per = 64 >> lg;
     const int at = (tid & (cols - 1)) * per;
     for (int q = 0; q < nq; ++q) {
       const int c = c0 + q * 64 + at;

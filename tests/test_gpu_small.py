@@ -80,3 +80,11 @@ def test_products_beyond_16_bits_are_refused_and_still_computed():
 def test_automatic_choice_on_both_sides_of_the_line(m, N):
     L, x_q, w_q, bias = build_layer(wi.Workload("sa", 5300 + m, N, 64, 11, 12, 96, m))
     _check(L, x_q, w_q, bias, path=0)
+
+
+@pytest.mark.parametrize("m", [2, 4, 6])
+@pytest.mark.parametrize("C", [16, 48])
+def test_narrow_layers_of_many_tiles(m, C):
+    # beyond 48 blocks the operands of narrow layers come by small copies instead of tensor copies
+    L, x_q, w_q, bias = build_layer(wi.Workload("sn", 5600 + m, 9, C, 9 * m, 7 * m, 32, m))
+    _check(L, x_q, w_q, bias)

@@ -18,6 +18,8 @@ struct Params {
   float BT[kMaxT * kMaxT];     // [t][t]
   float G[kMaxT * 3];          // [t][3]
   float AT[6 * kMaxT];         // [m][t]
+  // every entry of BT and AT twice over: a packed instruction's operand in one load
+  alignas(8) float BT_pair[2 * kMaxT * kMaxT], AT_pair[2 * 6 * kMaxT];
   float mult_V, mult_U, mult_M, mult_Y, s_acc;
   float lo_V, hi_V, lo_U, hi_U, lo_M, hi_M, lo_Y, hi_Y;  // clamp bounds minus zero point
   int z_x, z_w, z_Y;

@@ -605,6 +605,8 @@ int wino_plan(const wino_desc_t* desc, wino_plan_t** out) {
   std::memcpy(p.BT, d.BT, sizeof(float) * t * t);
   std::memcpy(p.G, d.G, sizeof(float) * t * 3);
   std::memcpy(p.AT, d.AT, sizeof(float) * d.m * t);
+  for (int i = 0; i < t * t; ++i) p.BT_pair[2 * i] = p.BT_pair[2 * i + 1] = p.BT[i];
+  for (int i = 0; i < d.m * t; ++i) p.AT_pair[2 * i] = p.AT_pair[2 * i + 1] = p.AT[i];
   pl->d.BT = p.BT; pl->d.G = p.G; pl->d.AT = p.AT;
   const double sUV = (double)d.q_U.scale * (double)d.q_V.scale;
   const double s_acc = d.q_M.enabled ? (double)d.q_M.scale : sUV;

@@ -85,11 +85,11 @@ constexpr int tma_chunk(int channels) {
   return channels % 128 == 0 ? 128 : channels % 96 == 0 ? 96 : channels % 80 == 0 ? 80 : channels % 64 == 0 ? 64
        : channels % 48 == 0 ? 48 : channels % 32 == 0 ? 32 : channels % 16 == 0 ? 16 : 0;
 }
-// Tiles per block: about 128 threads of two channels; half of that for 128-channel chunks in the
-// input transforms of F4 and F6 (smaller blocks balance better over the SMs, 5.3 -> 5.1 us on a
-// 256-channel 8x8 layer at batch 256; F2's shorter blocks do not gain).
+// Tiles per block: about 128 threads of two channels; half of that in the input transforms of F4
+// and F6 (smaller blocks balance better over the SMs, 5.3 -> 5.1 us on a 256-channel 8x8 layer at
+// batch 256, and a narrow layer has more of them; F2's shorter blocks do not gain).
 constexpr int tma_group(int chunk) { return 256 / chunk; }
-constexpr int tma_in_group(int m, int chunk) { return m != 2 && chunk == 128 ? 1 : tma_group(chunk); }
+constexpr int tma_in_group(int m, int chunk) { return m == 2 ? tma_group(chunk) : chunk > 64 ? 1 : 128 / chunk; }
 int launch_input_transform_tma(const Params& p, const LaunchOpt& o, const CUtensorMap& mapX,
                                const CUtensorMap& mapV, int* status, cudaStream_t st);
 // y_float: the output when it is float (mapY is then not used), else null.

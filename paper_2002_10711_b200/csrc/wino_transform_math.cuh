@@ -5,6 +5,7 @@
 //
 // Transform modes:
 //   kDense  : matrices are data (learnt "flex" transforms); every entry is used.
+//   kDensePair: the same for two channels, with the entries read as pairs.
 //   kSparse : the built-in Cook-Toom matrices as compile-time constants.
 //   kExact  : Cook-Toom matrices on integer codes where every intermediate is
 //             exactly representable (input stage for m = 2, 4, 6; output stage for
@@ -16,7 +17,7 @@
 
 namespace wino {
 
-enum { kDense = 0, kSparse = 1, kExact = 2 };
+enum { kDense = 0, kSparse = 1, kExact = 2, kDensePair = 3 };
 
 template <int CPT> struct Pack;
 template <> struct Pack<1> { typedef uint8_t type; };
@@ -126,11 +127,31 @@ __device__ __forceinline__ F2 v_zero(F2) { return f2_both(0.0f); }
 // One step of a fused-multiply-add chain; with a compile-time zero coefficient
 // the step disappears (the chain's value is unchanged by it).
 template <bool STD, typename V>
+__device__ __forceinline__ V chain(F2 coef, V x, V acc) { return v_fma(coef, x, acc); }
+template <bool STD, typename V>
 __device__ __forceinline__ V chain(float coef, V x, V acc) {
   if constexpr (STD) {
     if (coef == 0.0f) return acc;
   }
   return v_fma(coef, x, acc);
+}
+
+// Entries of B^T and A^T: floats, or pairs as they lie in Params.
+template <int M, int MODE>
+__device__ __forceinline__ auto bt_coef(const Params& p, int i, int k) {
+  if constexpr (MODE == kDensePair) {
+    return F2{*reinterpret_cast<const unsigned long long*>(p.BT_pair + 2 * (i * (M + 2) + k))};
+  } else {
+    return Mat<M, MODE != kDense>::bt(p, i, k);
+  }
+}
+template <int M, int MODE>
+__device__ __forceinline__ auto at_coef(const Params& p, int i, int k) {
+  if constexpr (MODE == kDensePair) {
+    return F2{*reinterpret_cast<const unsigned long long*>(p.AT_pair + 2 * (i * (M + 2) + k))};
+  } else {
+    return Mat<M, MODE != kDense>::at(p, i, k);
+  }
 }
 
 // V = (B^T d) B for one channel, or for a pair of channels (VT = F2; kExact: with the signs of
@@ -139,8 +160,7 @@ template <int M, int MODE, typename VT, typename ColFn>
 __device__ __forceinline__ void input_transform_2d(const Params& p, ColFn col,
                                                    VT (&V)[(M + 2) * (M + 2)]) {
   constexpr int T_ = M + 2;
-  constexpr bool STD = MODE != kDense;
-  using MT = Mat<M, STD>;
+  constexpr bool STD = MODE == kSparse || MODE == kExact;
   VT P[T_][T_];
 #pragma unroll
   for (int l = 0; l < T_; ++l) {
@@ -156,7 +176,7 @@ __device__ __forceinline__ void input_transform_2d(const Params& p, ColFn col,
       for (int i = 0; i < T_; ++i) {
         VT acc = v_zero(VT());
 #pragma unroll
-        for (int k = 0; k < T_; ++k) acc = chain<STD>(MT::bt(p, i, k), dcol[k], acc);
+        for (int k = 0; k < T_; ++k) acc = chain<STD>(bt_coef<M, MODE>(p, i, k), dcol[k], acc);
         P[i][l] = acc;
       }
     }
@@ -173,7 +193,7 @@ __device__ __forceinline__ void input_transform_2d(const Params& p, ColFn col,
       for (int j = 0; j < T_; ++j) {
         VT acc = v_zero(VT());
 #pragma unroll
-        for (int l = 0; l < T_; ++l) acc = chain<STD>(MT::bt(p, j, l), P[i][l], acc);
+        for (int l = 0; l < T_; ++l) acc = chain<STD>(bt_coef<M, MODE>(p, j, l), P[i][l], acc);
         V[i * T_ + j] = acc;
       }
     }
@@ -184,7 +204,7 @@ __device__ __forceinline__ void input_transform_2d(const Params& p, ColFn col,
 template <int M, int MODE, typename VT>
 __device__ __forceinline__ void at_pass(const Params& p, const VT (&v)[M + 2], VT (&y)[M]) {
   constexpr int T_ = M + 2;
-  constexpr bool STD = MODE != kDense;
+  constexpr bool STD = MODE == kSparse || MODE == kExact;
   if constexpr (MODE == kExact && M != 6) {
     at_exact(v, y);
   } else {
@@ -192,7 +212,7 @@ __device__ __forceinline__ void at_pass(const Params& p, const VT (&v)[M + 2], V
     for (int r = 0; r < M; ++r) {
       VT acc = v_zero(VT());
 #pragma unroll
-      for (int j = 0; j < T_; ++j) acc = chain<STD>(Mat<M, STD>::at(p, r, j), v[j], acc);
+      for (int j = 0; j < T_; ++j) acc = chain<STD>(at_coef<M, MODE>(p, r, j), v[j], acc);
       y[r] = acc;
     }
   }

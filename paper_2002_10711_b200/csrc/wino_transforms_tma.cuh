@@ -43,6 +43,15 @@ WINO_ST_READER(wino_trace_input, g_in_trace)
 WINO_ST_READER(wino_trace_output, g_out_trace)
 #endif
 
+// Dense F6 (kDensePair), while its threads all are resident at once: entries of the matrices read
+// as pairs spare the two moves that make one of a float, at the price of the registers that hold
+// them (255 and 168).  46 images of 22x22, 64 to 128 channels: 6.1 -> 5.2 us in, 6.2 -> 5.4 us out.
+// From the second wave on more warps hide more than the moves cost (9.1 us with floats, 9.7 with
+// pairs, on 128 such images), so the limits are the threads per SM of one wave.
+constexpr int kPairInThreads = 256, kPairOutThreads = 384;
+// Blocks of `threads` threads (whole warps) that make up so many.
+constexpr int pair_blocks(int limit, int threads) { return limit / ((threads + 31) / 32 * 32); }
+
 // Plans whose rounded products of Q_V fit 16 bits (the clamp is done on two codes at a time).
 // MINB: blocks per SM asked of the compiler.
 template <int M, int MODE, int CC, int G, int MINB>
@@ -152,7 +161,7 @@ k_input_transform_tma(const __grid_constant__ Params p, const __grid_constant__ 
 // F4 at 64 registers (eight blocks per SM; seven at the compiler's own 72 cost 0.9 us on a layer of
 // 1200 blocks).
 template <int M, int MODE, int KC, int G>
-__global__ void __launch_bounds__((KC / 2) * G, M == 4 && MODE == kExact ? 8 : 1)
+__global__ void __launch_bounds__((KC / 2) * G, M == 4 && MODE == kExact ? 8 : MODE == kDensePair ? pair_blocks(kPairOutThreads, (KC / 2) * G) : 1)
 k_output_transform_tma(const __grid_constant__ Params p, const __grid_constant__ CUtensorMap mapM,
                        const __grid_constant__ CUtensorMap mapY, const float* __restrict__ bias,
                        float s_Y, int* __restrict__ status, const float* __restrict__ chan,
@@ -301,12 +310,17 @@ int input_tma_launch(const Params& p, const LaunchOpt& o, const CUtensorMap& map
                      int* status, cudaStream_t st) {
   // F2 at 48 registers, F4 at 80 (F6 is slower within any limit), F4 at 72 with some spilling only
   // where that makes the grid a single wave: the 2048 blocks of a 256-channel, 1024-tile layer
-  constexpr int kHalf = tma_in_group(M, CC) * CC <= 128 ? 2 : 1;   // blocks of 64 threads
+  constexpr int kHalf = tma_in_group(M, CC) * CC <= 128 ? 2 : 1;   // blocks of at most 64 threads
   constexpr int kMin = MODE != kExact ? 1 : M == 2 ? 10 : M == 4 ? 6 * kHalf : 1;
   if constexpr (M == 4 && MODE == kExact && CC == 128) {
     const long units = (long)p.T * (p.C / CC);
     if (units > 12l * o.num_sms && units <= 14l * o.num_sms)
       return input_tma_go<M, MODE, CC, 14>(p, o, mapX, mapV, status, st);
+  }
+  if constexpr (M == 6 && MODE == kDense) {
+    constexpr int G = tma_in_group(M, CC), kPair = pair_blocks(kPairInThreads, (CC / 2) * G);
+    if ((long)((p.T + G - 1) / G) * (p.C / CC) <= (long)kPair * o.num_sms)
+      return input_tma_go<M, kDensePair, CC, kPair>(p, o, mapX, mapV, status, st);
   }
   return input_tma_go<M, MODE, CC, kMin>(p, o, mapX, mapV, status, st);
 }
@@ -324,7 +338,7 @@ int input_tma_mode(const Params& p, const LaunchOpt& o, const CUtensorMap& mapX,
 }
 
 template <int M, int MODE, int KC>
-int output_tma_launch(const Params& p, const LaunchOpt& o, const CUtensorMap& mapM, const CUtensorMap& mapY,
+int output_tma_go(const Params& p, const LaunchOpt& o, const CUtensorMap& mapM, const CUtensorMap& mapY,
                       const float* bias, float s_Y, int* status, float* y_float, cudaStream_t st) {
   constexpr int G = tma_group(KC);
   constexpr size_t smem = (G * (M + 2) * (M + 2) * KC + 127) / 128 * 128 + (size_t)G * ((M * M * KC + 127) / 128 * 128) + 128 + 16;
@@ -334,6 +348,16 @@ int output_tma_launch(const Params& p, const LaunchOpt& o, const CUtensorMap& ma
   const int units = ((p.T + G - 1) / G) * (p.K / KC);
   return launch_kernel(kernel, dim3((unsigned)units), dim3((KC / 2) * G), smem, st, o.pdl, p, mapM, mapY, bias, s_Y,
                        status, o.chan, y_float);
+}
+template <int M, int MODE, int KC>
+int output_tma_launch(const Params& p, const LaunchOpt& o, const CUtensorMap& mapM, const CUtensorMap& mapY,
+                      const float* bias, float s_Y, int* status, float* y_float, cudaStream_t st) {
+  if constexpr (M == 6 && MODE == kDense) {
+    constexpr int G = tma_group(KC), kPair = pair_blocks(kPairOutThreads, (KC / 2) * G);
+    if ((long)((p.T + G - 1) / G) * (p.K / KC) <= (long)kPair * o.num_sms)
+      return output_tma_go<M, kDensePair, KC>(p, o, mapM, mapY, bias, s_Y, status, y_float, st);
+  }
+  return output_tma_go<M, MODE, KC>(p, o, mapM, mapY, bias, s_Y, status, y_float, st);
 }
 template <int M, int MODE>
 int output_tma_mode(const Params& p, const LaunchOpt& o, const CUtensorMap& mapM, const CUtensorMap& mapY,

@@ -40,3 +40,10 @@ def test_several_units_per_block_on_the_tensor_cores(m, N):
     # more units than blocks, so that slots, accumulators and phases come round again
     L, x_q, w_q, bias = build_layer(wi.Workload("ch", 5500 + m, N, 128, 14, 15, 64, m))
     _compare(L, x_q, w_q, bias, 6)
+
+
+@pytest.mark.parametrize("N", [592, 593, 887, 889])
+def test_learnt_f6_around_one_wave_of_blocks(N):
+    # one tile per image: the input and the output transform change kernels at 592 and 888 tiles
+    L, x_q, w_q, bias = build_layer(wi.Workload("ch", 5600, N, 128, 6, 5, 128, 6, flex=True))
+    _compare(L, x_q, w_q, bias, 1)

@@ -438,9 +438,9 @@ def run_ours(args, wl):
         counters = load_counters() if wl.name == "cfg3" else {}
         # the GEMM of the common configuration runs the lean build of the kernel
         gemm_kernel = "k_gemm_tc_lean" if ("k_gemm_tc_lean" in counters or not counters) else "k_gemm_tc"
-        kernel_names = {"input_transform": "k_input_transform_mma" if mma_tr else "k_input_transform_tma",
+        kernel_names = {"input_transform": "k_input_transform_tc" if mma_tr else "k_input_transform_tma",
                         "hadamard_gemm": gemm_kernel,
-                        "output_transform": "k_output_transform_mma" if mma_tr else "k_output_transform_tma"}
+                        "output_transform": "k_output_transform_tc" if mma_tr else "k_output_transform_tma"}
         traffic_of = lambda k: (counters.get(k) or {}).get("dram_bytes")
         if dom == 1:
             peak = 2.0 * peaks["bf16_tflops"]

@@ -83,12 +83,13 @@ enum {
 enum {
   WINO_PATH_AUTO = 0,
   WINO_PATH_STAGED_TC = 1,   /* transform kernels (TMA-staged where the shape allows) + tcgen05 int8 GEMMs */
-  WINO_PATH_STAGED_DP4A = 2, /* transform kernels + integer-dot-product GEMMs on the ALUs */
+  WINO_PATH_STAGED_DP4A = 2, /* transform kernels + GEMMs by warp-level int8 MMAs: C, K multiples of 4 */
   WINO_PATH_SMALLC = 3,      /* one fused warp-shuffle kernel, C <= 32 and K <= 32 (never chosen automatically) */
   WINO_PATH_STAGED_TC_PTR = 4, /* as 1, but always the pointer-based transform kernels */
   WINO_PATH_FUSED_F2 = 5,    /* one fused tcgen05 kernel: m = 2, Cook-Toom matrices, C in {32, 64}, K <= 64 */
-  WINO_PATH_STAGED_TC_MMA = 6, /* as 1, with the transforms themselves on the tensor cores where that is
-                                 exact: Cook-Toom F2 / F4, channel counts multiples of 128 */
+  WINO_PATH_STAGED_TC_MMA = 6, /* as 1, with the transforms themselves on the tensor cores wherever that is
+                                 exact (Cook-Toom matrices; the output transform for m = 2, 4); path 1
+                                 does so for the layers that gain by it */
   WINO_PATH_FUSED_LAYER = 7,  /* the whole layer in one persistent launch (tensor-core transforms and
                                  GEMMs; V_q and m_q pass through the workspace in L2): Cook-Toom F2 / F4,
                                  C and K multiples of 128, input zero point 0, Q_M on, int8 output */
@@ -162,7 +163,7 @@ int wino_plan_force_path(wino_plan_t* plan, int path);
  * stay per layer.  All four NULL returns the plan to per-layer scales.  Call before
  * wino_transform_weights; U_q made under other scales is stale.  The staged paths
  * (WINO_PATH_STAGED_TC, WINO_PATH_STAGED_TC_PTR, WINO_PATH_STAGED_DP4A) and
- * WINO_PATH_FUSED_SMALL implement it: a plan on another path moves to the staged tcgen05 path (or the staged dp4a path), forcing
+ * WINO_PATH_FUSED_SMALL implement it: a plan on another path moves to a staged path; forcing
  * another path afterwards returns WINO_ERR_UNSUPPORTED, and wino_plan_multipliers keeps
  * reporting the per-layer values.  Synchronous (one small host-to-device copy);
  * WINO_ERR_INVALID for a bad scale, WINO_ERR_CUDA without a device. */

@@ -2,7 +2,8 @@
 // with int32 accumulation: the lossless candidate the paper compares the
 // Winograd-aware layers with (Sections 4 and 5.3), and the layer type of the
 // network's strided convolutions, for which no Winograd form exists (Section 5.1).
-// Integer dot products on the ALUs; thread = (output pixel, 4 or 8 output channels).
+// Channel counts the implicit GEMM does not take: integer dot products on the ALUs, thread =
+// (output pixel, 4 or 8 output channels); at most 4 input channels: warp-level MMAs.
 #include "wino_launch.h"
 #include "wino_warp_mma.cuh"
 

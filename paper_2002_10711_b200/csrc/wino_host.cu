@@ -411,7 +411,7 @@ LaunchOpt opt_with_hint(const wino_plan_t* pl, bool pdl, int stage_mask, const i
 // Estimated times in ns, for the choice between kernels that can run the same layer.  Staged: a
 // start-up latency of three dependent kernels plus a time per code (measured, us: F2 16.8 M codes
 // in and out 14, 134 M 62; F4 2.2 M 9.5, 9.4 M 12, 75 M 43; F6 1.5 M 10.9, 9.4 M 14, 75 M 49; with
-// integer dot products 0.6 M 8, 4.9 M 17).  Fused F2: waves of 128 tiles per SM, full or not (28 us at 64 channels).
+// warp-level MMAs 0.7 M 8, 5 M 17, 8.4 M 20, 20 M 37).  Fused F2: waves of 128 tiles per SM, full or not (28 us at 64 channels).
 long staged_cost(const wino_plan_t* pl) {
   const double codes = (double)pl->p.t * pl->p.t * pl->p.T * (pl->p.C + pl->p.K);
   if (pl->path == WINO_PATH_STAGED_DP4A) return 6500 + (long)(codes * 1.9e-3);
@@ -646,10 +646,11 @@ int wino_plan(const wino_desc_t* desc, wino_plan_t** out) {
   pl->std_mats = d.m == 2 ? is_std<2>(p.BT, p.AT) : d.m == 4 ? is_std<4>(p.BT, p.AT)
                                                                : is_std<6>(p.BT, p.AT);
   // Automatic choice, by measurement on B200: the fused F2 kernel where it applies; for
-  // layers of at most 16 channels in and out the staged path with integer dot products on the
-  // ALUs (a 16-wide GEMM leaves the tensor-core pipeline mostly empty: 54 against 73 us at
-  // 16 channels, 32x32, batch 256, F2); else the staged tcgen05 path, else the staged dp4a
-  // path.  The warp-shuffle small-channel kernel stays selectable (wino_plan_force_path) but
+  // layers of at most 16 channels in and out the staged path with warp-level MMAs (a 16-wide GEMM
+  // leaves the tcgen05 pipeline mostly empty: 56 against 72 us at 16 channels, 32x32, batch 256,
+  // F2); else the staged tcgen05 path, else, for channel counts that are not multiples of 16, warp
+  // MMAs again.  A plan made for one of these runs the one-launch kernel instead where its
+  // estimated time is lower (wino_conv_forward).  The warp-shuffle small-channel kernel stays selectable (wino_plan_force_path) but
   // a staged path was faster on every layer size tried, tiny batches included.
   if (path_supported(pl, WINO_PATH_FUSED_F2)) pl->path = WINO_PATH_FUSED_F2;
   else if (d.C <= 16 && d.K <= 16 && path_supported(pl, WINO_PATH_STAGED_DP4A))

@@ -1,5 +1,5 @@
 // Transform kernels of the Winograd-aware quantized layer (paper: Eq. 1, Fig. 2):
-//   k_weight_transform : U_q = Q(G g G^T)          (stage 2, offline)
+//   k_weight_transform, k_weight_transform_packed : U_q = Q(G g G^T)   (stage 2, offline)
 //   k_input_transform  : V_q = Q(B^T d B)          (stage 1)
 //   k_output_transform : y   = Q(A^T m A + bias)   (stage 4)
 // Streaming kernels: a thread owns CPT consecutive channels (1, 2 or 4) of one

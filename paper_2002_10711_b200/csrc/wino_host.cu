@@ -389,7 +389,12 @@ bool input_tc_pays(const Params& p) {
   if (!xt_fills(p.C)) return false;
   if (p.z_x != 0) return true;
   const double codes = (double)p.t * p.t * p.T * p.C;
-  return codes > (p.m == 2 ? 12e6 : p.m == 4 ? 14e6 : 7e6);
+  // F6: from the second wave of the ALU kernel's blocks on (7.2 M codes: ALU 4.8 us, tensor cores
+  // 5.2; 8.4 M: 6.4 and 5.9); later where the next kernel's weights are many and may have to come
+  // from HBM, for which its thousands of blocks ask earlier than 148 can (512 channels, 4x4, batch
+  // 256, weights not in L2: 19.8 us a layer with the ALU kernel, 20.8 with the other)
+  const double weights = (double)p.t * p.t * p.K * p.C;
+  return codes > (p.m == 2 ? 12e6 : p.m == 4 ? 14e6 : weights > 8e6 ? 9.4e6 : 7.5e6);
 }
 bool output_tc_pays(const Params& p) {
   if (!xt_fills(p.K)) return false;

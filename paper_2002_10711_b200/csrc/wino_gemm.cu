@@ -174,9 +174,9 @@ __device__ __forceinline__ float acc_to_float(uint32_t v) {
   else return __int2float_rn((int)v);
 }
 
-// The lean kernels' quantizer of one 32-column chunk: int8 codes, products below 2^15 (clamp on
-// 16-bit lanes).
-template <bool PK>
+// The lean kernels' quantizer of one 32-column chunk: int8 codes, products below 2^15.  SAT: upper
+// bound 127, by the saturating pack; else the clamp on 16-bit lanes (lean_saturates).
+template <bool PK, bool SAT>
 __device__ __forceinline__ void lean_codes(const Params& p, const uint32_t (&r)[32], int k0, const float* mult_k,
                                            uint32_t (&w)[8]) {
   const F2 magic = f2_both(kMagic);
@@ -193,6 +193,13 @@ __device__ __forceinline__ void lean_codes(const Params& p, const uint32_t (&r)[
                                      f2_make(mm.z, mm.w), magic, lo, hi);
       w[q] = __byte_perm(a, b, 0x6420u);
     }
+  } else if constexpr (SAT) {
+    const float lo_m = __fadd_rn(p.lo_M, kMagic);
+#pragma unroll
+    for (int q = 0; q < 8; ++q)
+      w[q] = quant_pack4<true>(__int2float_rn((int)r[4 * q]), __int2float_rn((int)r[4 * q + 1]),
+                               __int2float_rn((int)r[4 * q + 2]), __int2float_rn((int)r[4 * q + 3]), p.mult_M, lo_m,
+                               0.0f);
   } else {
     quant32_fits16(r, f2_both(p.mult_M), magic, lo, hi, w);
   }
@@ -267,7 +274,7 @@ __device__ __forceinline__ void epilogue_chunk(const Params& p, const uint32_t (
 }
 
 // The epilogue warps' loop over their work items.
-template <bool SMALL, bool FULL, bool STATS, bool PK = false, bool LEAN = false>
+template <bool SMALL, bool FULL, bool STATS, bool PK = false, bool LEAN = false, bool SAT = false>
 __device__ __forceinline__ void epilogue_loop(const Params& p, const GemmTcArgs& a, void* out,
                                               unsigned* absmaxM, uint32_t tmem_base,
                                               uint32_t bar_acc_full, uint32_t bar_acc_empty,
@@ -303,7 +310,7 @@ __device__ __forceinline__ void epilogue_loop(const Params& p, const GemmTcArgs&
       const long o = ((long)xi * p.T + tau) * p.K + k0;
       if constexpr (LEAN) {
         uint32_t w[8];
-        lean_codes<PK>(p, r, k0, mult_k, w);
+        lean_codes<PK, SAT>(p, r, k0, mult_k, w);
         store_row32(reinterpret_cast<int8_t*>(out) + o, w, true, 32);
       } else {
         epilogue_chunk<SMALL, FULL, STATS, PK>(p, r, k0, o, a.out_mode, out, vmax, a.wide_store != 0, mult_k);
@@ -327,8 +334,8 @@ __device__ __forceinline__ void epilogue_loop(const Params& p, const GemmTcArgs&
 // per-layer kernel carries none of that code).
 // LEAN: only the epilogue of the common case is compiled in (Q_M to int8 codes whose products
 // stay below 2^15, whole 32-column chunks, 32-byte aligned rows); the kernel's code is a third
-// of the general one's, which shows at every launch.
-template <bool PK, bool LEAN = false>
+// of the general one's, which shows at every launch.  SAT: lean_codes.
+template <bool PK, bool LEAN = false, bool SAT = false>
 __device__ __forceinline__ void gemm_tc_body(const Params& p, const CUtensorMap* mapV,
                                              const CUtensorMap* mapU, const GemmTcArgs& a,
                                              void* __restrict__ out, unsigned* __restrict__ absmaxM,
@@ -388,8 +395,9 @@ __device__ __forceinline__ void gemm_tc_body(const Params& p, const CUtensorMap*
   __syncthreads();
   tc_fence_after();
   // only now may the next kernel's blocks start: every block of this grid holds its tensor memory,
-  // so none of them can be kept from it by a block that waits for this grid.  (Starting an output
-  // transform that uses none earlier still measured 0.4 us slower on a 256-channel 8x8 layer.)
+  // so none of them can be kept from it by a block that waits for this grid.  (Before the
+  // allocation, which is only safe if no kernel that follows uses tensor memory, it measured the same
+  // on layers of 1024 to 2304 tiles: 256 channels, 8x8, batch 256 15.93 us so, 15.98 before.)
   griddep_launch();
   const uint32_t tmem_base = *tmem_slot_p;
 #ifdef WINO_TRACE
@@ -532,7 +540,7 @@ __device__ __forceinline__ void gemm_tc_body(const Params& p, const CUtensorMap*
     griddep_wait();
     if constexpr (LEAN) {
       (void)per_channel; (void)small; (void)full;
-      epilogue_loop<true, true, false, PK, true>(p, a, out, absmaxM, tmem_base, bar_acc_full, bar_acc_empty, abort_p,
+      epilogue_loop<true, true, false, PK, true, SAT>(p, a, out, absmaxM, tmem_base, bar_acc_full, bar_acc_empty, abort_p,
                                                  warp, lane, trace_step, mult_k);
     } else if constexpr (PK) {
       (void)per_channel;
@@ -575,12 +583,12 @@ k_gemm_tc(const __grid_constant__ Params p, const __grid_constant__ CUtensorMap 
           unsigned* __restrict__ absmaxM, int* __restrict__ status) {
   gemm_tc_body<false>(p, &mapV, &mapU, a, out, absmaxM, status);
 }
-template <bool PK>
+template <bool PK, bool SAT>
 __global__ void __launch_bounds__(kGemmThreads, 1)
 k_gemm_tc_lean(const __grid_constant__ Params p, const __grid_constant__ CUtensorMap mapV,
                const __grid_constant__ CUtensorMap mapU, const GemmTcArgs a, void* __restrict__ out,
                unsigned* __restrict__ absmaxM, int* __restrict__ status) {
-  gemm_tc_body<PK, true>(p, &mapV, &mapU, a, out, absmaxM, status);
+  gemm_tc_body<PK, true, SAT>(p, &mapV, &mapU, a, out, absmaxM, status);
 }
 __global__ void __launch_bounds__(kGemmThreads, 1)
 k_gemm_tc_per_channel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMap mapV,
@@ -618,6 +626,23 @@ TcGeom tc_geometry(const Params& p, int num_sms) {
   return g;
 }
 
+// Which of the two lean quantizers (per-layer scales, upper bound 127; else there is only one).  The
+// saturating pack takes more instructions a code, but its kernel fits 64 registers where the other
+// takes 72, and those eight times 576 keep blocks of the output transform from starting beside the
+// GEMM.  Measured on B200, us, GEMM alone and whole layer, 16-bit lanes / saturating pack:
+//   256-column accumulators: 256 ch 8x8 F4 batch 256  5.87, 15.85 / 5.61, 15.59;  128 ch 16x16 F4
+//     batch 200  8.07, 22.97 / 7.82, 22.66;  64 ch 32x32 F4 batch 128  8.77, 26.36 / 8.45, 26.10
+//   narrower, few codes: 128 ch 16x16 F4 batch 32  3.09, 11.10 / 3.08, 10.64, batch 64  3.66, 12.70 /
+//     3.66, 11.86;  64 ch 32x32 F4 batch 32  4.38, 13.77 / 4.41, 12.93
+//   narrower, more codes: 128 ch 16x16 F4 batch 100  4.94, 14.56 / 5.01, 14.77, batch 144  5.79, 17.54
+//     / 6.15, 18.03;  F2 batch 64  4.89, 15.07 / 5.06, 15.41;  32 ch 32x32 F6 batch 128  11.3, 27.0 /
+//     11.8, 27.4.  (One went the other way: 160 ch, 1792 tiles, F4  6.63, 18.48 / 6.07, 18.06.)
+// F6's output transform takes too many registers for blocks of it to fit beside the GEMM either way.
+static bool lean_saturates(const Params& p, const GemmTcArgs& a) {
+  if (p.hi_M != 127.0f) return false;
+  return a.MB * a.BN == 256 || (p.m != 6 && (double)p.t * p.t * p.T * p.K < 5e6);
+}
+
 int launch_gemm_tc(const Params& p, const LaunchOpt& o, const TcGeom& g, const CUtensorMap& mapV,
                    const CUtensorMap& mapU, void* out, int out_mode, unsigned* absmaxM,
                    int* status, cudaStream_t st) {
@@ -636,7 +661,7 @@ int launch_gemm_tc(const Params& p, const LaunchOpt& o, const TcGeom& g, const C
   a.chan_smem = (o.chan != nullptr && (size_t)p.K * 4 <= 24 * 1024) ? 1 : 0;
   const bool lean = absmaxM == nullptr && out_mode == kOutMq && a.wide_store && p.K % a.BN == 0 && a.BN % 32 == 0 &&
                     (o.chan != nullptr ? o.chan_m_fits_16 && a.chan_smem : p.m_fits_16 != 0);
-  static DeviceOnce once_pk, once_lean_pk, once_lean;
+  static DeviceOnce once_pk, once_lean_pk, once_lean, once_lean_sat;
   auto go = [&](auto kernel, DeviceOnce& done, size_t smem) -> int {
     if (int rc = set_max_smem(done, o.device, kernel, 227 * 1024)) return rc;
     return launch_kernel(kernel, dim3((unsigned)g.grid), dim3(kGemmThreads), smem, st, o.pdl, p, mapV, mapU, a, out,
@@ -644,9 +669,11 @@ int launch_gemm_tc(const Params& p, const LaunchOpt& o, const TcGeom& g, const C
   };
   if (o.chan != nullptr) {
     const size_t smem = g.smem + (a.chan_smem ? (size_t)p.K * 4 : 0);
-    return lean ? go(k_gemm_tc_lean<true>, once_lean_pk, smem) : go(k_gemm_tc_per_channel, once_pk, smem);
+    return lean ? go(k_gemm_tc_lean<true, false>, once_lean_pk, smem) : go(k_gemm_tc_per_channel, once_pk, smem);
   }
-  if (lean) return go(k_gemm_tc_lean<false>, once_lean, g.smem);
+  if (lean)
+    return lean_saturates(p, a) ? go(k_gemm_tc_lean<false, true>, once_lean_sat, g.smem)
+                                : go(k_gemm_tc_lean<false, false>, once_lean, g.smem);
   return launch_kernel(k_gemm_tc, dim3((unsigned)g.grid), dim3(kGemmThreads), g.smem, st, o.pdl, p,
                        mapV, mapU, a, out, absmaxM, status);
 }

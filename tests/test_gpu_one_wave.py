@@ -1,0 +1,26 @@
+"""The GEMM's two quantizers of int8 codes (chosen by accumulator width and number of codes), and transform
+builds that are chosen by whether all blocks of a grid are resident at once, on both sides of each line."""
+import pytest
+
+import wino_inputs as wi
+from helpers import build_layer, per_channel
+from test_gpu_parity import _compare
+
+pytestmark = pytest.mark.gpu
+
+
+# 256-column accumulators; fewer and more than 5 M codes in narrower ones; bounds other than 127
+@pytest.mark.parametrize("N,C,K", [(6, 128, 256), (6, 64, 96), (120, 64, 192)])
+@pytest.mark.parametrize("variant", ["plain", "relu", "per_channel", "zero_point_y", "saturating", "bound_100"])
+def test_quantizers_of_the_gemm(N, C, K, variant):
+    L, x_q, w_q, bias = build_layer(wi.Workload("oc", 5720, N, C, 9, 11, K, 4), relu=variant == "relu")
+    if variant == "per_channel":
+        L = per_channel(L, 43, spread=3.0)
+    if variant == "zero_point_y":
+        L.q_Y.zero_point = -11
+    if variant == "saturating":
+        for q in (L.q_V, L.q_U, L.q_M, L.q_Y):
+            q.scale = q.scale / 7.0
+    if variant == "bound_100":
+        L.q_M.qmin, L.q_M.qmax = -100, 100
+    _compare(L, x_q, w_q, bias, 1)

@@ -545,7 +545,7 @@ int forward_impl(wino_plan_t* pl, const int8_t* x, const int8_t* Uq, const float
     if (mm == nullptr) return WINO_ERR_CUDA;
     rc = launch_output_transform_tc(pl->p, opt_of(pl, pdl), *mm, pl->xt_images, bias, y, pl->s_Y, pl->status_dev, st);
   } else if (tma_ok && pl->p.qM_enabled && tma_chunk(pl->p.K) != 0) {
-    const CUtensorMap* mm = map_stage(pl, pl->cache_mld, mbuf, pl->p.K, tma_group(tma_chunk(pl->p.K)));
+    const CUtensorMap* mm = map_stage(pl, pl->cache_mld, mbuf, pl->p.K, tma_out_group(pl->p, pl->std_mats, pl->num_sms));
     const bool to_float = pl->p.out_dtype != 0;
     const CUtensorMap* my = to_float ? mm : map_y(pl, y);
     if (mm == nullptr || my == nullptr) return WINO_ERR_CUDA;

@@ -90,6 +90,16 @@ constexpr int tma_chunk(int channels) {
 // batch 256, and a narrow layer has more of them; F2's shorter blocks do not gain).
 constexpr int tma_group(int chunk) { return 256 / chunk; }
 constexpr int tma_in_group(int m, int chunk) { return m == 2 ? tma_group(chunk) : chunk > 64 ? 1 : 128 / chunk; }
+// Tiles per block of the output transform: one, with one channel per thread and 16 blocks per SM, for
+// F4 in 128-channel chunks while all blocks are resident at once.  Measured on B200, us a layer, two
+// channels per thread / one: 256 ch 8x8 batch 256 15.84 / 15.73, 128 ch 16x16 batch 64 12.68 / 12.43,
+// batch 32 10.93 / 10.58, 384 ch 12x12 batch 32 15.76 / 15.48 (256 ch 8x8 batch 64 11.60 / 11.73);
+// narrower chunks lose (96 ch: 11.80 / 12.45, 64 ch: 13.74 / 13.89).
+inline int tma_out_group(const Params& p, bool std_mats, int num_sms) {
+  const int chunk = tma_chunk(p.K);
+  return p.m == 4 && std_mats && p.out_dtype == 0 && chunk == 128 && (long)p.T * (p.K / 128) <= 16l * num_sms
+             ? 1 : tma_group(chunk);
+}
 int launch_input_transform_tma(const Params& p, const LaunchOpt& o, const CUtensorMap& mapX,
                                const CUtensorMap& mapV, int* status, cudaStream_t st);
 // y_float: the output when it is float (mapY is then not used), else null.

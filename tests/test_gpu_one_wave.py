@@ -24,3 +24,19 @@ def test_quantizers_of_the_gemm(N, C, K, variant):
     if variant == "bound_100":
         L.q_M.qmin, L.q_M.qmax = -100, 100
     _compare(L, x_q, w_q, bias, 1)
+
+
+# blocks per SM x 148: 12, 14 and 16 in F4 (input; 16 also output), 7 in F6
+@pytest.mark.parametrize("m,N", [(4, 1776), (4, 1777), (4, 2072), (4, 2073), (4, 2368), (4, 2369), (6, 1036), (6, 1037)])
+def test_around_one_wave_of_blocks(m, N):
+    # one tile per image and 128 channels: blocks = images
+    L, x_q, w_q, bias = build_layer(wi.Workload("ow", 5700 + m, N, 128, m, m - 1, 128, m))
+    _compare(L, x_q, w_q, bias, 1)
+
+
+# several tiles a block (64, 32 and 16 channels a chunk), one channel per thread and two
+@pytest.mark.parametrize("m,C", [(4, 64), (4, 32), (4, 16), (6, 64), (6, 32)])
+@pytest.mark.parametrize("N", [1, 37, 700])
+def test_narrow_chunks_around_one_wave(m, C, N):
+    L, x_q, w_q, bias = build_layer(wi.Workload("on", 5710 + m, N, C, 2 * m, 2 * m - 1, 32, m))
+    _compare(L, x_q, w_q, bias, 1)

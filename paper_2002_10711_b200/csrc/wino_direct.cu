@@ -5,6 +5,7 @@
 // Channel counts the implicit GEMM does not take: integer dot products on the ALUs, thread =
 // (output pixel, 4 or 8 output channels); at most 4 input channels: warp-level MMAs.
 #include "wino_launch.h"
+#include "wino_narrow_rows.cuh"
 #include "wino_warp_mma.cuh"
 
 namespace wino {
@@ -126,34 +127,6 @@ k_direct_conv(const DirectParams p, const int8_t* __restrict__ x, const int8_t* 
 // byte by byte, 10.0 with dot products and one pixel per thread, 5.1 like this.
 constexpr int kNarrowK = 64, kNarrowThreads = 128;
 
-// A row of 3 * C bytes at `at` (any alignment), of which bytes [from, to) exist, as three words;
-// bytes that do not exist take the code z (replicated in `fill`).
-template <int C>
-__device__ __forceinline__ void narrow_row(const int8_t* at, int from, int to, uint32_t fill, uint32_t (&r)[3]) {
-  const uint32_t sh = (uint32_t)(reinterpret_cast<uintptr_t>(at) & 3u);
-  const uint32_t* base = reinterpret_cast<const uint32_t*>(at - sh);
-  constexpr int kWords = (3 * C + 3 + 3) / 4;   // words that 3 * C bytes at any alignment touch
-  uint32_t w[4] = {0u, 0u, 0u, 0u};
-#pragma unroll
-  for (int j = 0; j < kWords; ++j) {
-    // only words that hold a byte of the image are read
-    const int lo = 4 * j - (int)sh;
-    if (from < to && lo + 4 > from && lo < to) w[j] = __ldg(base + j);
-  }
-#pragma unroll
-  for (int j = 0; j < 3; ++j) {
-    if (4 * j >= 3 * C) { r[j] = 0u; continue; }
-    uint32_t v = __funnelshift_r(w[j], j + 1 < kWords ? w[j + 1] : 0u, 8u * sh);
-    uint32_t keep = 0u, exist = 0u;
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      const int b = 4 * j + e;
-      if (b < 3 * C) exist |= 0xFFu << (8 * e);
-      if (b < 3 * C && b >= from && b < to) keep |= 0xFFu << (8 * e);
-    }
-    r[j] = (v & keep) | (fill & exist & ~keep);
-  }
-}
 // Three rows in K order: 8 words (one K step), or 16 (C = 4: two).
 template <int C>
 __device__ __forceinline__ void narrow_k(const uint32_t (&r)[3][3], uint32_t (&k)[C == 4 ? 16 : 8]) {
@@ -171,7 +144,8 @@ __device__ __forceinline__ void narrow_k(const uint32_t (&r)[3][3], uint32_t (&k
     }
   }
 }
-template <int C, bool Z>
+// TAIL: x or w ends within a word.
+template <int C, bool Z, bool TAIL>
 __global__ void __launch_bounds__(kNarrowThreads)
 k_direct_conv_narrow(const DirectParams p, const int8_t* __restrict__ x, const int8_t* __restrict__ w,
                      const float* __restrict__ bias, void* __restrict__ y, int wide) {
@@ -195,9 +169,9 @@ k_direct_conv_narrow(const DirectParams p, const int8_t* __restrict__ x, const i
   if (tid < kNarrowK) {
     uint32_t r[3][3], kw[KW];
     const int k = k0 + tid;
-#pragma unroll
-    for (int a = 0; a < 3; ++a)
-      narrow_row<C>(w + (long)(k < p.K ? k : 0) * 9 * C + a * 3 * C, 0, k < p.K ? 3 * C : 0, 0u, r[a]);
+    NarrowEnd end = {};
+    if (TAIL) end = narrow_end(w, (long)p.K * 9 * C);
+    narrow_filter<C, TAIL>(w, p.K, k, end, r);
     narrow_k<C>(r, kw);
     int sum = 0;
 #pragma unroll
@@ -219,6 +193,8 @@ k_direct_conv_narrow(const DirectParams p, const int8_t* __restrict__ x, const i
       bf[j][q][1] = v.y;
     }
   const long npix = (long)p.N * p.Ho * p.Wo;
+  NarrowEnd x_end = {};
+  if (TAIL) x_end = narrow_end(x, (long)p.N * p.H * p.W * C);
   const uint32_t fill = ((uint32_t)p.z_x & 0xFFu) * 0x01010101u;
   uint32_t* mine = s_a + (tid & ~31) * KW;
   for (long first = (blockIdx.x * (long)kNarrowThreads + (tid & ~31)); first < npix;
@@ -231,14 +207,7 @@ k_direct_conv_narrow(const DirectParams p, const int8_t* __restrict__ x, const i
       if (idx < npix) {
         const long rest = idx / p.Wo;
         const int wo = (int)(idx - rest * p.Wo), n = (int)(rest / p.Ho), ho = (int)(rest - (long)n * p.Ho);
-        const int h0 = ho * p.stride - 1, w0 = wo * p.stride - 1;
-        const int from = w0 < 0 ? C : 0, to = min(3, p.W - w0) * C;
-        const int8_t* xp = x + (((long)n * p.H + h0) * p.W + w0) * C;
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {
-          const bool in = (unsigned)(h0 + a) < (unsigned)p.H;
-          narrow_row<C>(xp + (long)a * p.W * C, in ? from : 0, in ? to : 0, fill, r[a]);
-        }
+        narrow_window<C, TAIL>(x, p.H, p.W, n, ho * p.stride - 1, wo * p.stride - 1, fill, x_end, r);
       }
       narrow_k<C>(r, kw);
     }
@@ -380,13 +349,19 @@ int launch_direct_conv(int N, int C, int H, int W, int K, int stride, int z_x, i
     const dim3 grid((unsigned)(want < most ? want : most), (unsigned)kb);
     const int wide = K % 16 == 0 ? 1 : 0;   // y is 16-byte aligned
     const bool z = z_x != 0 || z_w != 0;
-    auto go = [&](auto plain, auto with_z) {
-      return launch_kernel(z ? with_z : plain, grid, dim3(kNarrowThreads), 0, st, true, p, x, w, bias, y, wide);
+    const bool tail = narrow_has_tail((long)N * H * W * C) || narrow_has_tail((long)K * 9 * C);
+    auto go = [&](auto plain, auto with_z, auto plain_tail, auto with_z_tail) {
+      return launch_kernel(tail ? (z ? with_z_tail : plain_tail) : z ? with_z : plain, grid, dim3(kNarrowThreads), 0, st,
+                           true, p, x, w, bias, y, wide);
     };
-    return C == 1 ? go(k_direct_conv_narrow<1, false>, k_direct_conv_narrow<1, true>)
-         : C == 2 ? go(k_direct_conv_narrow<2, false>, k_direct_conv_narrow<2, true>)
-         : C == 3 ? go(k_direct_conv_narrow<3, false>, k_direct_conv_narrow<3, true>)
-                  : go(k_direct_conv_narrow<4, false>, k_direct_conv_narrow<4, true>);
+    return C == 1 ? go(k_direct_conv_narrow<1, false, false>, k_direct_conv_narrow<1, true, false>,
+                       k_direct_conv_narrow<1, false, true>, k_direct_conv_narrow<1, true, true>)
+         : C == 2 ? go(k_direct_conv_narrow<2, false, false>, k_direct_conv_narrow<2, true, false>,
+                       k_direct_conv_narrow<2, false, true>, k_direct_conv_narrow<2, true, true>)
+         : C == 3 ? go(k_direct_conv_narrow<3, false, false>, k_direct_conv_narrow<3, true, false>,
+                       k_direct_conv_narrow<3, false, true>, k_direct_conv_narrow<3, true, true>)
+                  : go(k_direct_conv_narrow<4, false, false>, k_direct_conv_narrow<4, true, false>,
+                       k_direct_conv_narrow<4, false, false>, k_direct_conv_narrow<4, true, false>);
   }
   if (C % 4 != 0 || K % 4 != 0) {
     const long blocks = (npix * K + 127) / 128;

@@ -285,12 +285,13 @@ int wino_direct_last_status(void* stream);
  * reads it and clears it, so the next call reports only what happened since. */
 int wino_last_status(wino_plan_t* plan, void* stream);
 
-/* Copies one intermediate of the most recent wino_conv_forward on this plan
- * (staged paths only) into dst_dev: V_q int8 [t*t][T][C], M int32 [t*t][T][K]
- * (recomputed from V_q and U_q with the plan's GEMM kernel), m_q int8
- * [t*t][T][K].  `bytes` must equal the stage size.  Asynchronous on the stream
- * of that forward call, whose x and U_q must still be in place (a one-launch call keeps its
- * intermediates on the SMs; they are then recomputed by the staged kernels). */
+/* Copies one intermediate of the most recent forward call on this plan from that call's
+ * workspace into dst_dev: V_q int8 [t*t][T][C], M int32 [t*t][T][K] (recomputed from that V_q
+ * and U_q with the plan's GEMM kernel), m_q int8 [t*t][T][K].  `bytes` must equal the stage
+ * size.  Asynchronous on the stream of that call, whose workspace (for M also U_q) must still
+ * be in place.  WINO_ERR_UNSUPPORTED if the call left no intermediates: one that ran as a single
+ * kernel, which wino_conv_forward chooses by itself for small layers.  To look at the stages of such
+ * a layer run its staged kernels, wino_debug_run_stages with mask 7, or force a staged path. */
 int wino_debug_dump_stage(wino_plan_t* plan, int stage, void* dst_dev, size_t bytes);
 
 /* The forward pass on a single-kernel path (WINO_PATH_SMALLC, WINO_PATH_FUSED_F2;

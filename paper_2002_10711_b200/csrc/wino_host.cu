@@ -70,8 +70,7 @@ struct wino_plan {
   MapCache cache_x, cache_vst, cache_mld, cache_y, cache_uf, cache_x_sw, cache_m_sw, cache_x_small, cache_u_small, cache_x_tc, cache_m_tc, cache_vst1;
   // last forward call, for wino_debug_dump_stage
   const int8_t* last_uq;
-  const int8_t* last_x;     // non-null: that call left no V_q and m_q in its workspace
-  void* last_ws;
+  void* last_ws;            // null: that call left no V_q and m_q anywhere
   cudaStream_t last_stream;
   long launches;
 };
@@ -449,6 +448,7 @@ int forward_impl(wino_plan_t* pl, const int8_t* x, const int8_t* Uq, const float
                  void* ws, unsigned* absmax4, cudaStream_t st, int stage_mask = 7,
                  int* dbgM = nullptr) {
   if (pl->status_dev == nullptr) return WINO_ERR_CUDA;
+  pl->last_ws = nullptr;   // until the staged kernels of this call have left their stages in `ws`
   const bool calib = absmax4 != nullptr;
   const bool pdl = pl->pdl && !calib;
   if (pl->path == WINO_PATH_FUSED_SMALL && !calib && stage_mask == 7 && dbgM == nullptr)
@@ -497,7 +497,6 @@ int forward_impl(wino_plan_t* pl, const int8_t* x, const int8_t* Uq, const float
                                       pl->status_dev, st);
     if (rc != WINO_OK) return rc;
     pl->last_uq = Uq;
-    pl->last_x = nullptr;
     pl->last_ws = ws;
     pl->last_stream = st;
     return WINO_OK;
@@ -557,7 +556,6 @@ int forward_impl(wino_plan_t* pl, const int8_t* x, const int8_t* Uq, const float
   }
   if (rc != WINO_OK) return rc;
   pl->last_uq = Uq;
-  pl->last_x = nullptr;
   pl->last_ws = ws;
   pl->last_stream = st;
   return WINO_OK;
@@ -811,11 +809,8 @@ int wino_conv_forward(wino_plan_t* pl, const int8_t* x, const int8_t* Uq, const 
     if (pl->status_dev == nullptr) return WINO_ERR_CUDA;
     if (scratch && ws == nullptr) return WINO_ERR_WORKSPACE;
     if (scratch && !aligned16(ws)) return WINO_ERR_ALIGNMENT;
-    const int rc = forward_small(pl, x, Uq, bias, y, (cudaStream_t)stream);
-    if (rc == WINO_OK && scratch) {
-      pl->last_uq = Uq; pl->last_x = x; pl->last_ws = ws; pl->last_stream = (cudaStream_t)stream;
-    }
-    return rc;
+    pl->last_ws = nullptr;   // V_q and m_q stay on the SMs
+    return forward_small(pl, x, Uq, bias, y, (cudaStream_t)stream);
   }
   if (!pl->forced && f2 && staged) {
     pl->path = WINO_PATH_STAGED_TC;
@@ -991,10 +986,6 @@ int wino_debug_dump_stage(wino_plan_t* pl, int stage, void* dst, size_t bytes) {
   if (!aligned16(dst)) return WINO_ERR_ALIGNMENT;
   const uint8_t* ws = reinterpret_cast<const uint8_t*>(pl->last_ws);
   cudaStream_t st = pl->last_stream;
-  if (pl->last_x != nullptr) {   // a one-launch call keeps V_q and m_q on the SMs: make them now
-    const int rc = forward_impl(pl, pl->last_x, pl->last_uq, nullptr, nullptr, pl->last_ws, nullptr, st, 3);
-    if (rc != WINO_OK) return rc;
-  }
   if (stage == WINO_STAGE_VQ) {
     if (bytes != vq_bytes(pl)) return WINO_ERR_INVALID;
     return cudaMemcpyAsync(dst, ws, bytes, cudaMemcpyDeviceToDevice, st) == cudaSuccess ? WINO_OK

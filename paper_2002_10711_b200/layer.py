@@ -46,6 +46,8 @@ class WinogradConv:
         return y
 
     def dump(self, stage: int) -> torch.Tensor:
+        """One intermediate of the last forward call (WinoError ERR_UNSUPPORTED if that ran as one
+        kernel, as small layers do unless the plan's path is forced)."""
         p = self.plan
         t2 = p.t * p.t
         if stage == binding.STAGE_VQ:
@@ -141,7 +143,7 @@ def calibrate_per_channel(make_plan, x_q, w_q, bias, s_x: float, s_w_K, output_p
     conv = WinogradConv(make_plan(s_V, 1.0, 1.0, 1.0, 0), device=device)
     conv.plan.set_channel_scales(s_w_K, s_U_K, None, None)
     conv.load_weights(w, b)
-    conv.forward(x)
+    conv.plan.debug_run_stages(3, x, conv.Uq, conv.bias, conv.empty_output(), conv.ws)   # staged at any size
     M = conv.dump(binding.STAGE_M_I32)
     check(conv.plan)
     m_max = M.abs().amax(dim=(0, 1)).cpu().numpy().astype(np.float64)

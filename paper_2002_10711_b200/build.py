@@ -58,8 +58,23 @@ def build(force: bool = False, verbose: bool = False) -> str:
     return LIB
 
 
-def _stale(target: str, *sources: str) -> bool:
-    return not os.path.exists(target) or os.path.getmtime(target) < max(os.path.getmtime(f) for f in sources)
+def _stale(target: str, abi: str, *sources: str) -> bool:
+    """Missing, older than a source, or built for another interpreter or torch (the note beside it)."""
+    if not os.path.exists(target) or os.path.getmtime(target) < max(os.path.getmtime(f) for f in sources):
+        return True
+    try:
+        with open(target + ".abi") as f:
+            return f.read() != abi
+    except OSError:
+        return True
+
+
+def _install(tmp: str, target: str, abi: str) -> None:
+    if os.path.exists(target + ".abi"):
+        os.remove(target + ".abi")      # no moment at which the note belongs to another file
+    os.replace(tmp, target)
+    with open(target + ".abi", "w") as f:
+        f.write(abi)
 
 
 def _build_native(force: bool) -> None:
@@ -68,14 +83,16 @@ def _build_native(force: bool) -> None:
     common = ["-O2", "-Wall", "-Wextra", "-fPIC", "-shared", "-I", sysconfig.get_paths()["include"],
               "-I", os.path.join(ROOT, "include")]
     link = ["-L", HERE, "-l:" + os.path.basename(LIB), "-Wl,-rpath,$ORIGIN"]
+    python_abi = sysconfig.get_config_var("SOABI")
     src = os.path.join(CSRC, "wino_python.c")
-    if force or _stale(NATIVE, src, header):
+    if force or _stale(NATIVE, python_abi, src, header):
         tmp = NATIVE + f".tmp{os.getpid()}"
         subprocess.check_call([os.environ.get("CC", "gcc"), "-std=c11", *common, src, *link, "-o", tmp])
-        os.replace(tmp, NATIVE)
+        _install(tmp, NATIVE, python_abi)
+    import torch
+    torch_abi = f"{python_abi} torch {torch.__version__} abi {int(torch._C._GLIBCXX_USE_CXX11_ABI)}"
     src = os.path.join(CSRC, "wino_python_torch.cpp")
-    if force or _stale(NATIVE_TORCH, src, header):
-        import torch
+    if force or _stale(NATIVE_TORCH, torch_abi, src, header):
         from torch.utils.cpp_extension import include_paths, library_paths
         tmp = NATIVE_TORCH + f".tmp{os.getpid()}"
         cuda = os.path.join(os.path.dirname(os.path.dirname(os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc"))), "include")
@@ -84,7 +101,7 @@ def _build_native(force: bool) -> None:
              *common, *[f for d in include_paths() for f in ("-isystem", d)], "-isystem", cuda, src, *link,
              *[f for d in library_paths() for f in ("-L", d)], "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_cuda",
              "-ltorch", "-ltorch_python", "-o", tmp])
-        os.replace(tmp, NATIVE_TORCH)
+        _install(tmp, NATIVE_TORCH, torch_abi)
 
 
 if __name__ == "__main__":

@@ -330,7 +330,7 @@ k_direct_conv_bytes(const DirectParams p, const int8_t* __restrict__ x, const in
   }
 }
 
-int launch_direct_conv(int N, int C, int H, int W, int K, int stride, int z_x, int z_w, int z_Y,
+int launch_direct_conv(int num_sms, int N, int C, int H, int W, int K, int stride, int z_x, int z_w, int z_Y,
                        float mult, float s_in, float s_Y, float lo_Y, float hi_Y, int out_dtype,
                        const int8_t* x, const int8_t* w, const float* bias, void* y,
                        const float* s_w_K, const float* s_Y_K, float s_x, float s_w, cudaStream_t st) {
@@ -345,7 +345,7 @@ int launch_direct_conv(int N, int C, int H, int W, int K, int stride, int z_x, i
   if (C <= 4 && (K + kNarrowK - 1) / kNarrowK <= 65535) {
     // up to four blocks an SM; a warp takes further groups of 32 pixels where there are more
     const int kb = (K + kNarrowK - 1) / kNarrowK;
-    const long want = (npix + kNarrowThreads - 1) / kNarrowThreads, most = (4l * 148 + kb - 1) / kb;
+    const long want = (npix + kNarrowThreads - 1) / kNarrowThreads, most = (4l * num_sms + kb - 1) / kb;
     const dim3 grid((unsigned)(want < most ? want : most), (unsigned)kb);
     const int wide = K % 16 == 0 ? 1 : 0;   // y is 16-byte aligned
     const bool z = z_x != 0 || z_w != 0;

@@ -661,7 +661,7 @@ int wino_plan(const wino_desc_t* desc, wino_plan_t** out) {
   else if (path_supported(pl, WINO_PATH_STAGED_TC)) pl->path = WINO_PATH_STAGED_TC;
   else if (path_supported(pl, WINO_PATH_STAGED_DP4A)) pl->path = WINO_PATH_STAGED_DP4A;
   else { delete pl; return WINO_ERR_UNSUPPORTED; }
-  pl->num_sms = 148;
+  pl->num_sms = kDefaultSms;
   pl->pdl = true;
   int ndev = 0;
   if (cudaGetDeviceCount(&ndev) == cudaSuccess && ndev > 0) {
@@ -783,7 +783,7 @@ int wino_transform_weights(wino_plan_t* pl, const int8_t* w, int8_t* Uq, uint32_
   if (!aligned16(w) || !aligned16(Uq)) return WINO_ERR_ALIGNMENT;
   if (pl->status_dev == nullptr) return WINO_ERR_CUDA;
   pl->launches++;
-  return launch_weight_transform(pl->p, pl->chan_dev, w, Uq, absmax, nullptr, (cudaStream_t)stream);
+  return launch_weight_transform(pl->p, opt_of(pl, true), w, Uq, absmax, nullptr, (cudaStream_t)stream);
 }
 
 int wino_transform_weights_channel_stats(wino_plan_t* pl, const int8_t* w, int8_t* Uq,
@@ -792,7 +792,7 @@ int wino_transform_weights_channel_stats(wino_plan_t* pl, const int8_t* w, int8_
   if (!aligned16(w) || !aligned16(Uq)) return WINO_ERR_ALIGNMENT;
   if (pl->status_dev == nullptr) return WINO_ERR_CUDA;
   pl->launches++;
-  return launch_weight_transform(pl->p, pl->chan_dev, w, Uq, nullptr, absmax_K, (cudaStream_t)stream);
+  return launch_weight_transform(pl->p, opt_of(pl, true), w, Uq, nullptr, absmax_K, (cudaStream_t)stream);
 }
 
 int wino_conv_forward(wino_plan_t* pl, const int8_t* x, const int8_t* Uq, const float* bias,
@@ -867,14 +867,14 @@ int wino_direct_conv_forward(const wino_direct_desc_t* d, const int8_t* x, const
   if ((reinterpret_cast<uintptr_t>(d->s_w_K_dev) & 3u) != 0 || (reinterpret_cast<uintptr_t>(d->s_Y_K_dev) & 3u) != 0)
     return WINO_ERR_ALIGNMENT;
   const double s_in = (double)d->q_x.scale * (double)d->q_w.scale;
+  int dev = 0, sms = kDefaultSms;
+  if (cudaGetDevice(&dev) != cudaSuccess) return WINO_ERR_CUDA;
+  if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1)
+    sms = kDefaultSms;
   if (direct_tc_supported(d->C, d->K, d->stride, d->q_x.zero_point, d->q_w.zero_point) &&
       (reinterpret_cast<uintptr_t>(y) & 31u) == 0) {
     // implicit GEMM on the tensor cores: x as [N][H][W][C] boxes of one output tile, w as
     // [K][9][C] slices of one tap
-    int dev = 0, sms = 148;
-    if (cudaGetDevice(&dev) != cudaSuccess) return WINO_ERR_CUDA;
-    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1)
-      sms = 148;
     DirectTcArgs a = direct_tc_geometry(d->N, d->C, d->H, d->W, d->K, d->stride, sms);
     a.mult = (float)(s_in / (double)d->q_Y.scale);
     a.s_in = (float)s_in;
@@ -912,7 +912,7 @@ int wino_direct_conv_forward(const wino_direct_desc_t* d, const int8_t* x, const
     return launch_direct_conv_tc(a, dev, sms, mapX, mapW, bias, y, (cudaStream_t)stream) == 0
                ? WINO_OK : WINO_ERR_CUDA;
   }
-  return launch_direct_conv(d->N, d->C, d->H, d->W, d->K, d->stride, d->q_x.zero_point,
+  return launch_direct_conv(sms, d->N, d->C, d->H, d->W, d->K, d->stride, d->q_x.zero_point,
                             d->q_w.zero_point, d->q_Y.zero_point,
                             (float)(s_in / (double)d->q_Y.scale), (float)s_in, d->q_Y.scale,
                             (float)(d->q_Y.qmin - d->q_Y.zero_point),

@@ -12,12 +12,15 @@
 
 namespace wino {
 
+// SMs of a B200: what is assumed where no device can be asked (plans made without one).
+constexpr int kDefaultSms = 148;
+
 // Launch options shared by all kernels.
 struct LaunchOpt {
   bool std_mats = false;      // B^T and A^T are the built-in Cook-Toom matrices
   bool pdl = false;           // programmatic dependent launch on the stream
   int device = 0;             // the plan's device (current when the launcher runs)
-  int num_sms = 148;          // its SM count
+  int num_sms = kDefaultSms;  // its SM count
   // A buffer a later kernel of the same call will read and that no kernel of the call
   // writes (the transformed weights): the input transform's blocks ask for it to be brought
   // into L2 while they run.  A hint only; null: none.
@@ -69,7 +72,7 @@ int set_max_smem(DeviceOnce& once, int dev, Kern kernel, size_t smem) {
 
 // absmax (nullable): one word, max |U| of the layer; absmax_K (nullable): K words, max |U| of
 // each filter; both as float bits, caller-zeroed.
-int launch_weight_transform(const Params& p, const float* chan, const int8_t* w, int8_t* Uq,
+int launch_weight_transform(const Params& p, const LaunchOpt& o, const int8_t* w, int8_t* Uq,
                             unsigned* absmax, unsigned* absmax_K, cudaStream_t st);
 int launch_input_transform(const Params& p, const LaunchOpt& o, const int8_t* x, int8_t* Vq,
                            unsigned* absmax, cudaStream_t st);
@@ -206,7 +209,7 @@ int launch_direct_conv_tc(const DirectTcArgs& a, int device, int num_sms, const 
                           const CUtensorMap& mapW, const float* bias, void* y, cudaStream_t st);
 // s_w_K, s_Y_K (nullable device arrays of K floats): per-output-channel scales replacing s_w
 // and s_Y; s_x, s_w: the per-layer scales behind mult and s_in.
-int launch_direct_conv(int N, int C, int H, int W, int K, int stride, int z_x, int z_w, int z_Y,
+int launch_direct_conv(int num_sms, int N, int C, int H, int W, int K, int stride, int z_x, int z_w, int z_Y,
                        float mult, float s_in, float s_Y, float lo_Y, float hi_Y, int out_dtype,
                        const int8_t* x, const int8_t* w, const float* bias, void* y,
                        const float* s_w_K, const float* s_Y_K, float s_x, float s_w, cudaStream_t st);

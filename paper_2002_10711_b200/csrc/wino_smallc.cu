@@ -141,7 +141,7 @@ int smallc_launch(const Params& p, const LaunchOpt& o, const int8_t* x, const in
   if (int rc = set_max_smem(once, o.device, k_smallc<M, STD, LPT>, smem)) return rc;
   const int groups = (p.T + (32 / LPT) - 1) / (32 / LPT);
   int blocks = (groups + 3) / 4;
-  if (blocks > 148 * 8) blocks = 148 * 8;
+  if (blocks > o.num_sms * 8) blocks = o.num_sms * 8;
   return launch_kernel(k_smallc<M, STD, LPT>, dim3((unsigned)blocks), dim3(128), smem, st, o.pdl, p, x,
                        Uq, bias, y, s_Y, dbgM);
 }

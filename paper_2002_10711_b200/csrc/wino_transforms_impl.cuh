@@ -327,9 +327,9 @@ k_output_transform(const __grid_constant__ Params p, const void* __restrict__ mb
 namespace {
 
 // Channels per thread: the widest element that still gives every SM several
-// warps of work (148 SMs x 1024 threads as the target).
-int pick_cpt(long items_times_channels) {
-  const long target = 148l * 1024;
+// warps of work (1024 threads an SM as the target).
+int pick_cpt(long items_times_channels, int num_sms) {
+  const long target = 1024l * num_sms;
   if (items_times_channels / 4 >= target) return 4;
   if (items_times_channels / 2 >= target) return 2;
   return 1;
@@ -343,18 +343,19 @@ int weight_cpt(const Params& p, const float* chan, const int8_t* w, int8_t* Uq, 
                        0, st, false, p, chan, w, Uq, absmax, absmax_K);
 }
 template <int M>
-int weight_m(const Params& p, const float* chan, const int8_t* w, int8_t* Uq, unsigned* absmax,
+int weight_m(const Params& p, const LaunchOpt& o, const int8_t* w, int8_t* Uq, unsigned* absmax,
              unsigned* absmax_K, cudaStream_t st) {
+  const float* chan = o.chan;
   const long total = (long)p.K * p.C;
   if (absmax == nullptr && absmax_K == nullptr && (chan != nullptr ? p.u_fits_16_chan : p.u_fits_16) != 0 &&
       total < (1l << 31)) {
     // four channels per thread once that leaves every SM three warps a scheduler
-    const bool wide = total / 4 >= 148l * 384;
+    const bool wide = total / 4 >= 384l * o.num_sms;
     const unsigned threads = (unsigned)(total / (wide ? 4 : 2));
     return launch_kernel(wide ? k_weight_transform_packed<M, 2> : k_weight_transform_packed<M, 1>,
                          dim3((threads + 127) / 128), dim3(128), 0, st, true, p, chan, w, Uq);
   }
-  const int cpt = pick_cpt((long)p.K * p.C);
+  const int cpt = pick_cpt((long)p.K * p.C, o.num_sms);
   return cpt == 4 ? weight_cpt<M, 4>(p, chan, w, Uq, absmax, absmax_K, st)
        : cpt == 2 ? weight_cpt<M, 2>(p, chan, w, Uq, absmax, absmax_K, st)
                   : weight_cpt<M, 1>(p, chan, w, Uq, absmax, absmax_K, st);
@@ -374,19 +375,19 @@ int input_cpt(const Params& p, bool pdl, const int8_t* x, int8_t* Vq, unsigned* 
                        absmax);
 }
 template <int M, int MODE>
-int input_mode(const Params& p, bool pdl, const int8_t* x, int8_t* Vq, unsigned* absmax,
+int input_mode(const Params& p, const LaunchOpt& o, const int8_t* x, int8_t* Vq, unsigned* absmax,
                cudaStream_t st) {
-  const int cpt = absmax != nullptr ? 4 : pick_cpt((long)p.T * p.C);
-  return cpt == 4 ? input_cpt<M, MODE, 4>(p, pdl, x, Vq, absmax, st)
-       : cpt == 2 ? input_cpt<M, MODE, 2>(p, pdl, x, Vq, absmax, st)
-                  : input_cpt<M, MODE, 1>(p, pdl, x, Vq, absmax, st);
+  const int cpt = absmax != nullptr ? 4 : pick_cpt((long)p.T * p.C, o.num_sms);
+  return cpt == 4 ? input_cpt<M, MODE, 4>(p, o.pdl, x, Vq, absmax, st)
+       : cpt == 2 ? input_cpt<M, MODE, 2>(p, o.pdl, x, Vq, absmax, st)
+                  : input_cpt<M, MODE, 1>(p, o.pdl, x, Vq, absmax, st);
 }
 template <int M>
 int input_m(const Params& p, const LaunchOpt& o, const int8_t* x, int8_t* Vq, unsigned* absmax,
             cudaStream_t st) {
-  if (!o.std_mats) return input_mode<M, kDense>(p, o.pdl, x, Vq, absmax, st);
+  if (!o.std_mats) return input_mode<M, kDense>(p, o, x, Vq, absmax, st);
   // Cook-Toom B^T on integer codes is exact for m = 2, 4, 6: factored forms throughout.
-  return input_mode<M, kExact>(p, o.pdl, x, Vq, absmax, st);
+  return input_mode<M, kExact>(p, o, x, Vq, absmax, st);
 }
 
 template <int M, int MODE, bool QM, int CPT>
@@ -403,36 +404,36 @@ int output_cpt(const Params& p, bool pdl, float s_Y, const void* mbuf, const flo
                        mbuf, bias, y, s_Y, absmax2, chan);
 }
 template <int M, int MODE, bool QM>
-int output_mode(const Params& p, bool pdl, float s_Y, const void* mbuf, const float* bias, void* y,
-                unsigned* absmax2, const float* chan, cudaStream_t st) {
-  const int cpt = absmax2 != nullptr ? 4 : pick_cpt((long)p.T * p.K);
-  return cpt == 4 ? output_cpt<M, MODE, QM, 4>(p, pdl, s_Y, mbuf, bias, y, absmax2, chan, st)
-       : cpt == 2 ? output_cpt<M, MODE, QM, 2>(p, pdl, s_Y, mbuf, bias, y, absmax2, chan, st)
-                  : output_cpt<M, MODE, QM, 1>(p, pdl, s_Y, mbuf, bias, y, absmax2, chan, st);
+int output_mode(const Params& p, const LaunchOpt& o, float s_Y, const void* mbuf, const float* bias, void* y,
+                unsigned* absmax2, cudaStream_t st) {
+  const int cpt = absmax2 != nullptr ? 4 : pick_cpt((long)p.T * p.K, o.num_sms);
+  return cpt == 4 ? output_cpt<M, MODE, QM, 4>(p, o.pdl, s_Y, mbuf, bias, y, absmax2, o.chan, st)
+       : cpt == 2 ? output_cpt<M, MODE, QM, 2>(p, o.pdl, s_Y, mbuf, bias, y, absmax2, o.chan, st)
+                  : output_cpt<M, MODE, QM, 1>(p, o.pdl, s_Y, mbuf, bias, y, absmax2, o.chan, st);
 }
 template <int M>
 int output_m(const Params& p, const LaunchOpt& o, float s_Y, const void* mbuf, const float* bias,
              void* y, unsigned* absmax2, cudaStream_t st) {
   const bool qm = p.qM_enabled != 0;
   if (!o.std_mats) {
-    return qm ? output_mode<M, kDense, true>(p, o.pdl, s_Y, mbuf, bias, y, absmax2, o.chan, st)
-              : output_mode<M, kDense, false>(p, o.pdl, s_Y, mbuf, bias, y, absmax2, o.chan, st);
+    return qm ? output_mode<M, kDense, true>(p, o, s_Y, mbuf, bias, y, absmax2, st)
+              : output_mode<M, kDense, false>(p, o, s_Y, mbuf, bias, y, absmax2, st);
   }
   // With Q_M on, the F4 output transform works on integers in [-128, 127]:
   // every intermediate is an integer below 2^24, so the factored form is exact.
-  if (M != 6 && qm) return output_mode<M, kExact, true>(p, o.pdl, s_Y, mbuf, bias, y, absmax2, o.chan, st);
-  return qm ? output_mode<M, kSparse, true>(p, o.pdl, s_Y, mbuf, bias, y, absmax2, o.chan, st)
-            : output_mode<M, kSparse, false>(p, o.pdl, s_Y, mbuf, bias, y, absmax2, o.chan, st);
+  if (M != 6 && qm) return output_mode<M, kExact, true>(p, o, s_Y, mbuf, bias, y, absmax2, st);
+  return qm ? output_mode<M, kSparse, true>(p, o, s_Y, mbuf, bias, y, absmax2, st)
+            : output_mode<M, kSparse, false>(p, o, s_Y, mbuf, bias, y, absmax2, st);
 }
 
 }  // namespace
 
 // Entry points for this translation unit's tile size (one unit per m keeps the
 // build parallel).
-int WINO_CAT(launch_weight_transform_m, WINO_M)(const Params& p, const float* chan, const int8_t* w,
+int WINO_CAT(launch_weight_transform_m, WINO_M)(const Params& p, const LaunchOpt& o, const int8_t* w,
                                                  int8_t* Uq, unsigned* absmax, unsigned* absmax_K,
                                                  cudaStream_t st) {
-  return weight_m<WINO_M>(p, chan, w, Uq, absmax, absmax_K, st);
+  return weight_m<WINO_M>(p, o, w, Uq, absmax, absmax_K, st);
 }
 int WINO_CAT(launch_input_transform_m, WINO_M)(const Params& p, const LaunchOpt& o,
                                                 const int8_t* x, int8_t* Vq, unsigned* absmax,

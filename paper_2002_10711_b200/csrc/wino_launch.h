@@ -82,11 +82,12 @@ int launch_gemm_warp(const Params& p, const LaunchOpt& o, const int8_t* Vq, cons
                      void* out, int out_mode, unsigned* absmaxM, cudaStream_t st);
 
 // TMA-staged transform kernels (input needs C % 16 == 0; output needs Q_M on and K % 16 == 0).
-// Channel chunk per block: the widest that divides the channels (narrow chunks are short rows,
-// which the copy engine delivers no faster than long ones).
+// Channel chunk per block: the widest multiple of 16 up to 128 that divides the channels (narrow chunks
+// are short rows, which the copy engine delivers no faster than long ones).
 constexpr int tma_chunk(int channels) {
-  return channels % 128 == 0 ? 128 : channels % 96 == 0 ? 96 : channels % 80 == 0 ? 80 : channels % 64 == 0 ? 64
-       : channels % 48 == 0 ? 48 : channels % 32 == 0 ? 32 : channels % 16 == 0 ? 16 : 0;
+  for (int chunk = 128; chunk > 0; chunk -= 16)
+    if (channels % chunk == 0) return chunk;
+  return 0;
 }
 // Tiles per block: about 128 threads of two channels; half of that in the input transforms of F4
 // and F6 (smaller blocks balance better over the SMs, 5.3 -> 5.1 us on a 256-channel 8x8 layer at

@@ -381,8 +381,8 @@ int input_tma_go(const Params& p, const LaunchOpt& o, const CUtensorMap& mapX, c
 // then by how many warps share its work; a second, mostly empty wave costs a quarter of the kernel.
 // F4 and F6, Cook-Toom matrices, no zero point (whose padding only the other build patches):
 //   - one channel per thread (twice the warps; 40 registers in F4, 72 in F6, 56 and 96 with several
-//     tiles a block) while that grid is one wave, and for chunks of 96, 80 and 48 channels, which
-//     in pairs do not fill whole warps, always;
+//     tiles a block) while that grid is one wave, and for chunks of 112, 96, 80 and 48 channels,
+//     which in pairs do not fill whole warps, always;
 //   - else two channels per thread at 72 registers (F4, some spilling) where that makes one wave;
 //   - else, F4 in 128-channel chunks, one channel per thread at 32 registers likewise;
 //   - else two channels per thread at 80 registers (F2 48; F6 is slower within any limit).
@@ -422,6 +422,7 @@ int input_tma_mode(const Params& p, const LaunchOpt& o, const CUtensorMap& mapX,
                    int* status, cudaStream_t st) {
   const int cc = tma_chunk(p.C);
   return cc == 128 ? input_tma_launch<M, MODE, 128>(p, o, mapX, mapV, status, st)
+       : cc == 112 ? input_tma_launch<M, MODE, 112>(p, o, mapX, mapV, status, st)
        : cc == 96 ? input_tma_launch<M, MODE, 96>(p, o, mapX, mapV, status, st)
        : cc == 80 ? input_tma_launch<M, MODE, 80>(p, o, mapX, mapV, status, st)
        : cc == 48 ? input_tma_launch<M, MODE, 48>(p, o, mapX, mapV, status, st)
@@ -475,6 +476,7 @@ int output_tma_mode(const Params& p, const LaunchOpt& o, const CUtensorMap& mapM
                     const float* bias, float s_Y, int* status, float* y_float, cudaStream_t st) {
   const int kc = tma_chunk(p.K);
   return kc == 128 ? output_tma_launch<M, MODE, 128>(p, o, mapM, mapY, bias, s_Y, status, y_float, st)
+       : kc == 112 ? output_tma_launch<M, MODE, 112>(p, o, mapM, mapY, bias, s_Y, status, y_float, st)
        : kc == 96 ? output_tma_launch<M, MODE, 96>(p, o, mapM, mapY, bias, s_Y, status, y_float, st)
        : kc == 80 ? output_tma_launch<M, MODE, 80>(p, o, mapM, mapY, bias, s_Y, status, y_float, st)
        : kc == 64 ? output_tma_launch<M, MODE, 64>(p, o, mapM, mapY, bias, s_Y, status, y_float, st)

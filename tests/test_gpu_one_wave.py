@@ -40,3 +40,13 @@ def test_around_one_wave_of_blocks(m, N):
 def test_narrow_chunks_around_one_wave(m, C, N):
     L, x_q, w_q, bias = build_layer(wi.Workload("on", 5710 + m, N, C, 2 * m, 2 * m - 1, 32, m))
     _compare(L, x_q, w_q, bias, 1)
+
+
+@pytest.mark.parametrize("m", [2, 4, 6])
+@pytest.mark.parametrize("variant", ["plain", "zero_points", "flex", "float_out"])
+def test_chunks_of_112_channels(m, variant):
+    L, x_q, w_q, bias = build_layer(wi.Workload("o7", 5730 + m, 3, 112, 7, 9, 224, m, flex=variant == "flex"),
+                                    out_dtype=1 if variant == "float_out" else 0)
+    if variant == "zero_points":
+        L.q_x.zero_point, L.q_w.zero_point, L.q_Y.zero_point = -9, 2, -5
+    _compare(L, x_q, w_q, bias, 1)

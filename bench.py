@@ -45,6 +45,7 @@ if ROOT not in sys.path:
 
 import wino_inputs as wi  # noqa: E402
 
+# ("staged_dp4a": the constant's name; that path's GEMMs are warp-level int8 MMAs)
 PATH_NAMES = {1: "staged_tc", 2: "staged_dp4a", 3: "smallc", 4: "staged_tc_ptr", 5: "fused_f2",
               6: "staged_tc_mma", 7: "fused_layer"}
 

@@ -79,11 +79,14 @@ enum {
  * choice is 5 where it applies, else 2 for layers of at most 16 channels in and out, else 1
  * where C and K are multiples of 16, else 2.  wino_conv_forward on a plan whose path was not
  * forced runs a layer of few tiles by kernel 8 instead, and a layer of path 5 by the kernels of
- * path 1 if it is given a workspace, where that is estimated to be faster (same results). */
+ * path 1 if it is given a workspace, where that is estimated to be faster (same results): with a
+ * workspace, path 5's own kernel is left with layers of C + K up to 64 that are most of one wave
+ * of its blocks.  wino_conv_forward_static makes no such choice: it runs the plan's path as it is. */
 enum {
   WINO_PATH_AUTO = 0,
   WINO_PATH_STAGED_TC = 1,   /* transform kernels (TMA-staged where the shape allows) + tcgen05 int8 GEMMs */
-  WINO_PATH_STAGED_DP4A = 2, /* transform kernels + GEMMs by warp-level int8 MMAs: C, K multiples of 4 */
+  WINO_PATH_STAGED_DP4A = 2, /* transform kernels + GEMMs by warp-level int8 MMAs (the name is that of an
+                                earlier kernel): C, K multiples of 4 */
   WINO_PATH_SMALLC = 3,      /* one fused warp-shuffle kernel, C <= 32 and K <= 32 (never chosen automatically) */
   WINO_PATH_STAGED_TC_PTR = 4, /* as 1, but always the pointer-based transform kernels */
   WINO_PATH_FUSED_F2 = 5,    /* one fused tcgen05 kernel: m = 2, Cook-Toom matrices, C in {32, 64}, K <= 64 */
@@ -212,13 +215,16 @@ int wino_conv_forward(wino_plan_t* plan, const int8_t* x_NHWC_dev, const int8_t*
  * a fixed memory budget; start-up code that runs before the application's
  * allocator exists.
  *
- * Same arguments, results and errors as wino_conv_forward, minus the workspace:
+ * Same arguments, results and errors as wino_conv_forward, minus the workspace, and always the
+ * plan's own path (wino_plan_path) where wino_conv_forward may take a faster kernel for the layer's
+ * size (twice as long on the smallest layers, four times on small ones of path 5; force
+ * WINO_PATH_FUSED_SMALL for those, which needs no scratch).
  * V_q and m_q live in a static device array of WINO_STATIC_SCRATCH_BYTES built
  * into the library (every GPU that loads the library holds those bytes until
  * the process exits).  A plan on a staged path whose wino_workspace_bytes
  * exceeds that size is refused with WINO_ERR_WORKSPACE and nothing is launched;
- * plans on a single-kernel path (WINO_PATH_SMALLC, WINO_PATH_FUSED_F2) need no
- * scratch and are accepted at any size.  The call makes no cudaMalloc /
+ * plans on a single-kernel path (WINO_PATH_SMALLC, WINO_PATH_FUSED_F2,
+ * WINO_PATH_FUSED_SMALL) need no scratch and are accepted at any size.  The call makes no cudaMalloc /
  * cudaFree and uses no allocating library routine.
  *
  * First use on a device: the first call made with a given device current looks
@@ -254,9 +260,8 @@ int wino_calibrate_forward(wino_plan_t* plan, const int8_t* x_NHWC_dev,
  * pointers 16-byte aligned.
  * Stateless: no plan, no workspace.  Without zero points on x and w, with C a
  * multiple of 64, K a multiple of 32 (at most 2048) and y 32-byte aligned, the
- * layer runs as an implicit GEMM on the tensor cores; everything else on the
- * integer ALUs (at most four input channels: one thread per pixel with its window
- * in registers).
+ * layer runs as an implicit GEMM on the tensor cores; with at most four input channels
+ * as one by warp-level int8 MMAs; everything else on the integer ALUs.
  * The results are the same bits either way. */
 typedef struct {
   int32_t N, C, H, W, K, stride;

@@ -372,13 +372,14 @@ int launch_gemm(wino_plan_t* pl, const int8_t* Vq, const int8_t* Uq, void* out, 
 // Whether the tensor-core transforms are the faster ones (both kinds being possible), by the
 // number of codes.  They cost fewer instructions a code but start up more slowly (tensor memory,
 // a constant operand, two hand-overs).  Measured on B200, us, ALU / tensor cores:
-//   input   F2  8.4 M codes 4.7 / 5.1   16.8 M 7.8 / 7.2   33.6 M 14.4 / 11.6   67 M 29 / 24
-//           F4  4.7 M 3.7 / 4.2   9.4 M 5.4 / 5.7   18.9 M 9.6 / 9.0   37.7 M 19.0 / 16.3
-//           F6  4.7 M 3.7 / 4.5   8.4 M 6.5 / 6.0   18.9 M 11.4 / 9.2   37.7 M 23 / 16.5
-//   output  F2  8.4 M 4.1 / 4.9   16.8 M 7.4 / 6.3   33.6 M 12.6 / 8.6   67 M 24 / 13
-//           F4  9.4 M 4.6 / 5.2   18.9 M 7.8 / 7.7   37.7 M 13.6 / 11.9
-// With an input zero point the ALU kernel would also have to patch the padding of border tiles
-// (14 -> 19 us on a 160-channel 12 x 22 layer).
+//   input   F2  8.4 M codes 5.3 / 5.3   10.5 M 5.9 / 5.9   33.6 M 14.4 / 11.6   67 M 29 / 24
+//           F4  7.1 M 4.4 / 5.2   9.4 M 5.3 / 6.0   10.6 M 5.9 / 6.6   13.0 M 7.5 / 7.3   37.7 M 19.0 / 16.3
+//           F6  128 channels 6.3 M 5.2 / 5.3   8.4 M 5.4 / 6.5;  64 channels 6.8 M 5.2 / 5.5   7.3 M 6.9 / 5.8
+//   output  F2  8.4 M 4.5 / 4.5   10.5 M 5.4 / 5.5   33.6 M 12.6 / 8.6   67 M 24 / 13
+//           F4  9.4 M 4.6 / 5.4   14.2 M 6.5 / 6.6   16.5 M 7.1 / 7.4   37.7 M 13.6 / 11.9
+// With an input zero point the ALU kernel also has to patch the padding of border tiles, which makes it
+// the slower one below those lines too:  F4  1.8 M 8.5 / 3.3   4.7 M 9.2 / 6.1   9.4 M 10.5 / 8.8;
+// F6  2.1 M 6.7 / 4.0   4.2 M 7.0 / 6.0.
 // A quarter of a unit's channels at most may be padding.
 bool xt_fills(int channels) {
   const int chunk = xt_chunk(channels), padded = (channels + chunk - 1) / chunk * chunk;
@@ -388,12 +389,14 @@ bool input_tc_pays(const Params& p) {
   if (!xt_fills(p.C)) return false;
   if (p.z_x != 0) return true;
   const double codes = (double)p.t * p.t * p.T * p.C;
-  // F6: from the second wave of the ALU kernel's blocks on (7.2 M codes: ALU 4.8 us, tensor cores
-  // 5.2; 8.4 M: 6.4 and 5.9); later where the next kernel's weights are many and may have to come
-  // from HBM, for which its thousands of blocks ask earlier than 148 can (512 channels, 4x4, batch
-  // 256, weights not in L2: 19.8 us a layer with the ALU kernel, 20.8 with the other)
+  // F6: from the second wave of the ALU kernel's blocks on, which comes at fewer codes with several
+  // tiles a block; later where the next kernel's weights are many and may have to come from HBM, for
+  // which its thousands of blocks ask earlier than one per SM can (512 channels, 4x4, batch 256,
+  // weights not in L2: 19.8 us a layer with the ALU kernel, 20.8 with the other)
   const double weights = (double)p.t * p.t * p.K * p.C;
-  return codes > (p.m == 2 ? 12e6 : p.m == 4 ? 14e6 : weights > 8e6 ? 9.4e6 : 7.5e6);
+  const int chunk = tma_chunk(p.C);
+  const double one_wave = chunk == 128 ? 8.5e6 : chunk > 64 ? 8.2e6 : 7e6;
+  return codes > (p.m == 2 ? 12e6 : p.m == 4 ? 14e6 : weights > 8e6 ? 9.4e6 : one_wave);
 }
 bool output_tc_pays(const Params& p) {
   if (!xt_fills(p.K)) return false;
@@ -648,13 +651,16 @@ int wino_plan(const wino_desc_t* desc, wino_plan_t** out) {
   }
   pl->std_mats = d.m == 2 ? is_std<2>(p.BT, p.AT) : d.m == 4 ? is_std<4>(p.BT, p.AT)
                                                                : is_std<6>(p.BT, p.AT);
-  // Automatic choice, by measurement on B200: the fused F2 kernel where it applies; for
+  // The plan's path, by measurement on B200: the fused F2 kernel where it applies; for
   // layers of at most 16 channels in and out the staged path with warp-level MMAs (a 16-wide GEMM
   // leaves the tcgen05 pipeline mostly empty: 56 against 72 us at 16 channels, 32x32, batch 256,
   // F2); else the staged tcgen05 path, else, for channel counts that are not multiples of 16, warp
-  // MMAs again.  A plan made for one of these runs the one-launch kernel instead where its
-  // estimated time is lower (wino_conv_forward).  The warp-shuffle small-channel kernel stays selectable (wino_plan_force_path) but
-  // a staged path was faster on every layer size tried, tiny batches included.
+  // MMAs again.  wino_conv_forward then takes the one-launch kernel or, for a fused-F2 plan that was
+  // given a workspace, the staged kernels, where their estimated time is lower: by these estimates the
+  // fused F2 kernel runs calls without a workspace and layers of C + K up to 64, of most of a wave.  The
+  // warp-shuffle small-channel kernel stays selectable (wino_plan_force_path) but was the slower one
+  // wherever it was tried (16 channels, 32x32, F2, batch 256 57.1 us against 56.6, batch 64 22.2
+  // against 21.0, F4 batch 256 56 against 38; 32 channels, F2, batch 256 112 against 72).
   if (path_supported(pl, WINO_PATH_FUSED_F2)) pl->path = WINO_PATH_FUSED_F2;
   else if (d.C <= 16 && d.K <= 16 && path_supported(pl, WINO_PATH_STAGED_DP4A))
     pl->path = WINO_PATH_STAGED_DP4A;

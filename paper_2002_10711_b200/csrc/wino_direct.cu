@@ -169,9 +169,7 @@ k_direct_conv_narrow(const DirectParams p, const int8_t* __restrict__ x, const i
   if (tid < kNarrowK) {
     uint32_t r[3][3], kw[KW];
     const int k = k0 + tid;
-    NarrowEnd end = {};
-    if (TAIL) end = narrow_end(w, (long)p.K * 9 * C);
-    narrow_filter<C, TAIL>(w, p.K, k, end, r);
+    narrow_filter<C, TAIL>(w, p.K, k, r);
     narrow_k<C>(r, kw);
     int sum = 0;
 #pragma unroll
@@ -193,8 +191,6 @@ k_direct_conv_narrow(const DirectParams p, const int8_t* __restrict__ x, const i
       bf[j][q][1] = v.y;
     }
   const long npix = (long)p.N * p.Ho * p.Wo;
-  NarrowEnd x_end = {};
-  if (TAIL) x_end = narrow_end(x, (long)p.N * p.H * p.W * C);
   const uint32_t fill = ((uint32_t)p.z_x & 0xFFu) * 0x01010101u;
   uint32_t* mine = s_a + (tid & ~31) * KW;
   for (long first = (blockIdx.x * (long)kNarrowThreads + (tid & ~31)); first < npix;
@@ -207,7 +203,7 @@ k_direct_conv_narrow(const DirectParams p, const int8_t* __restrict__ x, const i
       if (idx < npix) {
         const long rest = idx / p.Wo;
         const int wo = (int)(idx - rest * p.Wo), n = (int)(rest / p.Ho), ho = (int)(rest - (long)n * p.Ho);
-        narrow_window<C, TAIL>(x, p.H, p.W, n, ho * p.stride - 1, wo * p.stride - 1, fill, x_end, r);
+        narrow_window<C, TAIL>(x, p.N, p.H, p.W, n, ho * p.stride - 1, wo * p.stride - 1, fill, r);
       }
       narrow_k<C>(r, kw);
     }

@@ -40,10 +40,9 @@ template <int C, bool TAIL> void windows() {
   for (int N = 1; N <= 2; ++N) for (int H = 1; H <= 4; ++H) for (int W = 1; W <= 7; ++W) for (int st = 1; st <= 2; ++st) {
     if (!TAIL && wino::narrow_has_tail((long)N * H * W * C)) continue;
     int8_t* x = tensor((long)N * H * W * C);
-    const wino::NarrowEnd end = wino::narrow_end(x, g_size);
     for (int n = 0; n < N; ++n) for (int h = 0; h < H; h += st) for (int w = 0; w < W; w += st) {
       uint32_t r[3][3];
-      wino::narrow_window<C, TAIL>(x, H, W, n, h - 1, w - 1, 0x05050505u, end, r);
+      wino::narrow_window<C, TAIL>(x, N, H, W, n, h - 1, w - 1, 0x05050505u, r);
       for (int a = 0; a < 3; ++a) for (int e = 0; e < 3 * C; ++e) {
         const int hh = h - 1 + a, ww = w - 1 + e / C;
         const bool in = hh >= 0 && hh < H && ww >= 0 && ww < W;
@@ -55,10 +54,9 @@ template <int C, bool TAIL> void windows() {
   for (int K = 1; K <= 9; ++K) {
     if (!TAIL && wino::narrow_has_tail((long)K * 9 * C)) continue;
     int8_t* w = tensor((long)K * 9 * C);
-    const wino::NarrowEnd end = wino::narrow_end(w, g_size);
     for (int k = 0; k < K + 2; ++k) {
       uint32_t r[3][3];
-      wino::narrow_filter<C, TAIL>(w, K, k, end, r);
+      wino::narrow_filter<C, TAIL>(w, K, k, r);
       for (int a = 0; a < 3; ++a) for (int e = 0; e < 3 * C; ++e)
         check<C>(r, a, e, k < K ? w[((long)k * 3 + a) * 3 * C + e] : 0);
     }

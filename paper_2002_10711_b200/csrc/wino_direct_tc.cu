@@ -36,13 +36,6 @@ namespace {
 constexpr int kDtEpiWarps = 16;
 constexpr int kDtThreads = 64 + 32 * kDtEpiWarps;
 
-// K-major tile of 64-byte rows with the 64-byte swizzle: start / 16, 8-row group stride
-// 512 B, descriptor version 1, layout 4.
-__device__ __forceinline__ uint64_t desc_sw64(uint32_t smem_addr) {
-  return (uint64_t)((smem_addr & 0x3FFFFu) >> 4) | (1ull << 16) | (32ull << 32) | (1ull << 46) |
-         (4ull << 61);
-}
-
 // PK: the weight and output scales vary per output channel (a build of its own: the per-layer
 // kernel keeps its one multiplier in a register).
 template <bool PK, bool RW>

@@ -143,8 +143,14 @@ int launch_gemm_warp(const Params& p, const LaunchOpt& o, const int8_t* Vq, cons
 //   warp 1   : tensor-memory owner; one lane issues the MMAs
 //   warps 2-17: epilogue.  Warp w reads TMEM lanes 32*(w%4) .. +31 (its hardware
 //              quadrant) and every fourth 32-column chunk, by (w-2)/4.
-// A stage holds 128 channels: A tile 128 x 128 B, B tile BN x 128 B; one MMA
-// consumes 32 channels.
+// A stage holds cB channels (128, or 64 in layers of no more): A tiles of 128 x cB bytes, B tile
+// BN x cB bytes; one MMA consumes 32 channels.
+// What bounds it on narrow layers (64 ch 32x32 batch 256, F4: 17.2 us with 128-byte stages, two of
+// them, and a copy per m-block; 14.4 now): the quantizer takes some 780 cycles per 32 columns and
+// warp with four warps to a scheduler, 6.3 us in all; the rest is the hand-over between the ring, the
+// MMA warp, whose MMAs share the path to shared memory with the epilogue's stores (115 to 230 cycles
+// each, 36 alone), and the two accumulators.  A second MMA warp, waits without back-off and unrolled
+// MMA loops changed nothing.
 // ---------------------------------------------------------------------------
 
 #ifdef WINO_TRACE
@@ -166,6 +172,32 @@ struct GemmTcArgs {
   int wide_store;  // 1: the output rows are 32-byte aligned (one 256-bit store per row piece)
   const float* chan;  // per-output-channel multipliers [5][K], or null
   int chan_smem;      // 1: the block keeps the K multipliers of Q_M in shared memory
+  int bn_log2;        // MB > 1: log2(BN)
+  int cB;             // channels (bytes) per stage: 64 for at most 64 channels, else 128
+  int KB;             // stages per item
+  int box_mb;         // m-blocks one V_q copy brings: boxes have up to 256 rows
+  // gridDim.x items further, in the digits of the item number (m-block fastest, then k-block, then xi)
+  int d_mb, d_nb, d_xi;
+};
+
+// The producer's position in the item list: its lone thread has no other warp's work to hide two
+// divisions an item behind.  (The epilogue warps have: with carries there, which keep six more values
+// alive, the 256-channel GEMM took 0.15 us longer.)
+struct ItemWalk {
+  int mb, nb, xi;
+  __device__ __forceinline__ explicit ItemWalk(const GemmTcArgs& a) {
+    const int per_xi = a.n_mblk * a.n_nblk, rem = (int)blockIdx.x % per_xi;
+    xi = (int)blockIdx.x / per_xi;
+    nb = rem / a.n_mblk;
+    mb = rem - nb * a.n_mblk;
+  }
+  __device__ __forceinline__ void next(const GemmTcArgs& a) {
+    mb += a.d_mb;
+    nb += a.d_nb;
+    xi += a.d_xi;
+    if (mb >= a.n_mblk) { mb -= a.n_mblk; ++nb; }
+    if (nb >= a.n_nblk) { nb -= a.n_nblk; ++xi; }
+  }
 };
 
 template <bool SMALL>
@@ -302,7 +334,7 @@ __device__ __forceinline__ void epilogue_loop(const Params& p, const GemmTcArgs&
     // time per warp, the four warps of a scheduler hide each other's
     // tensor-memory load latency
     auto chunk = [&](const uint32_t (&r)[32], int col) {
-      const int j = a.MB > 1 ? col / a.BN : 0;
+      const int j = a.MB > 1 ? col >> a.bn_log2 : 0;
       const int kcol = col - j * a.BN;
       const int tau = (mb * a.MB + j) * kBM + quad * 32 + lane;
       if (tau >= p.T) return;
@@ -343,7 +375,7 @@ __device__ __forceinline__ void gemm_tc_body(const Params& p, const CUtensorMap*
   extern __shared__ uint8_t smem_raw[];
   // tiles need 1024-byte alignment for the 128-byte swizzle
   const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
-  const uint32_t a_bytes = kBM * kStageK, b_bytes = (uint32_t)a.BN * kStageK;
+  const uint32_t a_bytes = kBM * (uint32_t)a.cB, b_bytes = (uint32_t)(a.BN * a.cB);
   const uint32_t stage_bytes = (uint32_t)a.MB * a_bytes + b_bytes;
   const uint32_t bars = base + (uint32_t)a.stages * stage_bytes;
   const uint32_t bar_full = bars;                           // stages x 8 B
@@ -357,8 +389,7 @@ __device__ __forceinline__ void gemm_tc_body(const Params& p, const CUtensorMap*
   volatile uint32_t* abort_p = reinterpret_cast<volatile uint32_t*>(gen + (abort_slot - base));
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int KB = (p.C + kStageK - 1) / kStageK;
-  const int per_xi = a.n_mblk * a.n_nblk;
+  const int KB = a.KB;
 
   int trace_step = 0;
 #ifdef WINO_TRACE
@@ -413,18 +444,18 @@ __device__ __forceinline__ void gemm_tc_body(const Params& p, const CUtensorMap*
   if (warp == 0) {
     if (lane == 0) {
       int s = 0, issued = 0; uint32_t ph = 0;
-      int xi = blockIdx.x / per_xi, rem = blockIdx.x - xi * per_xi;
-      int nb = rem / a.n_mblk, mb = rem - nb * a.n_mblk;
+      ItemWalk item(a);
       // A lone thread retires an instruction every ten to twenty cycles, and the first loads
       // after the wait are the step's critical path (the generic loop took 0.6 us to get them
       // out).  So the operands of the first item's first one or two stages are computed, and
       // pinned in registers, before the wait; after it only the copy instructions themselves
       // are issued, and the generic loop takes over from there.
+      // (Two only where a stage is 128 channels.)
       const int n_first = (KB >= 2 && a.stages >= 2) ? 2 : 1;
       uint32_t f_bytes = stage_bytes, f_dst = base, f_b_off = (uint32_t)a.MB * a_bytes, f_a_bytes = a_bytes;
-      int f_row_a = (mb * a.MB) * kBM, f_row_b = nb * a.BN, f_xi = xi, f_mb = a.MB, f_n = n_first;
+      int f_row_a = (item.mb * a.MB) * kBM, f_row_b = item.nb * a.BN, f_xi = item.xi, f_mb = a.MB, f_box = a.box_mb, f_n = n_first;
       asm volatile("" : "+r"(f_bytes), "+r"(f_dst), "+r"(f_b_off), "+r"(f_a_bytes), "+r"(f_row_a),
-                        "+r"(f_row_b), "+r"(f_xi), "+r"(f_mb), "+r"(f_n));
+                        "+r"(f_row_b), "+r"(f_xi), "+r"(f_mb), "+r"(f_box), "+r"(f_n));
       griddep_wait();
       WINO_ST(g_gemm_trace, trace_step, 2);
 #pragma unroll
@@ -434,7 +465,7 @@ __device__ __forceinline__ void gemm_tc_body(const Params& p, const CUtensorMap*
           mbar_expect_tx(fb, f_bytes);
           tma_load_3d(fd, mapV, fb, q * kStageK, f_row_a, f_xi);
           tma_load_3d(fd + f_b_off, mapU, fb, q * kStageK, f_row_b, f_xi);
-          for (int j = 1; j < f_mb; ++j)   // rows past T are filled with zeros by the TMA unit
+          for (int j = f_box; j < f_mb; j += f_box)   // rows past T are filled with zeros by the TMA unit
             tma_load_3d(fd + (uint32_t)j * f_a_bytes, mapV, fb, q * kStageK, f_row_a + j * kBM, f_xi);
           if (q == 0) WINO_ST(g_gemm_trace, trace_step, 15);
         }
@@ -442,11 +473,7 @@ __device__ __forceinline__ void gemm_tc_body(const Params& p, const CUtensorMap*
       issued = n_first;
       s = n_first;
       if (s == a.stages) { s = 0; ph ^= 1u; }
-      for (int it = blockIdx.x; it < a.n_items; it += gridDim.x) {
-        if (it != blockIdx.x) {
-          xi = it / per_xi; rem = it - xi * per_xi;
-          nb = rem / a.n_mblk; mb = rem - nb * a.n_mblk;
-        }
+      for (int it = blockIdx.x; it < a.n_items; it += gridDim.x, item.next(a)) {
         bool ok = true;
         for (int kb = (it == (int)blockIdx.x ? n_first : 0); kb < KB; ++kb) {
           // the ring's first pass finds every stage free
@@ -454,11 +481,11 @@ __device__ __forceinline__ void gemm_tc_body(const Params& p, const CUtensorMap*
           ++issued;
           const uint32_t sa = base + (uint32_t)s * stage_bytes;
           mbar_expect_tx(bar_full + 8u * s, stage_bytes);
-          for (int j = 0; j < a.MB; ++j)   // rows past T are filled with zeros by the TMA unit
-            tma_load_3d(sa + (uint32_t)j * a_bytes, mapV, bar_full + 8u * s, kb * kStageK,
-                        (mb * a.MB + j) * kBM, xi);
-          tma_load_3d(sa + (uint32_t)a.MB * a_bytes, mapU, bar_full + 8u * s, kb * kStageK,
-                      nb * a.BN, xi);
+          for (int j = 0; j < a.MB; j += a.box_mb)   // rows past T are filled with zeros by the TMA unit
+            tma_load_3d(sa + (uint32_t)j * a_bytes, mapV, bar_full + 8u * s, kb * a.cB,
+                        (item.mb * a.MB + j) * kBM, item.xi);
+          tma_load_3d(sa + (uint32_t)a.MB * a_bytes, mapU, bar_full + 8u * s, kb * a.cB,
+                      item.nb * a.BN, item.xi);
           if (++s == a.stages) { s = 0; ph ^= 1u; }
         }
         if (!ok) { *abort_p = 1u; break; }
@@ -473,10 +500,10 @@ __device__ __forceinline__ void gemm_tc_body(const Params& p, const CUtensorMap*
     // instruction costs ten to twenty cycles and a stage's MMAs take five hundred.  Descriptors
     // are linear in the tile address (units of 16 bytes), so a stage's are the first stage's
     // plus a multiple of the stage size.
-    const uint64_t da_first = make_desc_sw128(base);
+    const uint64_t da_first = a.cB == 128 ? make_desc_sw128(base) : desc_sw64(base);
     const uint32_t stage_units = stage_bytes >> 4, a_units = a_bytes >> 4;
     const uint32_t b_units = (uint32_t)a.MB * a_units;
-    const int last_ksteps = (p.C - (KB - 1) * kStageK + 31) / 32;   // 1..4
+    const int last_ksteps = (p.C - (KB - 1) * a.cB + 31) / 32;   // 1..4
     uint32_t s_units = 0;   // s * stage_units
     int s = 0; uint32_t ph = 0;
     int li = 0;
@@ -607,13 +634,19 @@ TcGeom tc_geometry(const Params& p, int num_sms) {
   // ... as long as that leaves every CTA at least three items to pipeline
   const int n_nblk0 = (p.K + g.BN - 1) / g.BN;
   while (g.MB > 1 && (p.t * p.t) * ((n_mblk + g.MB - 1) / g.MB) * n_nblk0 < 3 * num_sms) g.MB /= 2;
-  const size_t per_stage = (size_t)g.MB * kBM * kStageK + (size_t)g.BN * kStageK;
+  // At most 64 channels: stages of 64-byte rows with the 64-byte swizzle; 128-byte rows would be half
+  // zero fill, which is written to shared memory and leaves room for half as many stages.
+  g.cB = p.C <= 64 ? 64 : 128;
+  const size_t per_stage = (size_t)(g.MB * kBM + g.BN) * g.cB;
   g.stages = (int)((196 * 1024) / per_stage);
-  const int KB = (p.C + kStageK - 1) / kStageK;
+  const int KB = (p.C + g.cB - 1) / g.cB;
   // one and a half items' worth: with two whole items in the ring the second item's operands
   // compete with the first item's for the path from L2 and delay its accumulator (cfg3: 5.87 us
   // with four stages, 5.74 with three, 6.12 with two)
-  if (g.stages > (3 * KB + 1) / 2) g.stages = (3 * KB + 1) / 2;
+  // ... but four where a stage is an item: its MMAs are over before the next copies, issued when its
+  // slot came free, have landed (64 ch 32x32 batch 256, F4 / F2, two stages 15.4 / 25.3 us, four 14.4 / 23.2)
+  if (KB == 1 && g.stages >= 4) g.stages = 4;
+  else if (g.stages > (3 * KB + 1) / 2) g.stages = (3 * KB + 1) / 2;
   if (g.stages > 8) g.stages = 8;
   if (g.stages < 1) g.stages = 1;
   int acc_stride = 32;
@@ -659,6 +692,13 @@ int launch_gemm_tc(const Params& p, const LaunchOpt& o, const TcGeom& g, const C
   a.chan = o.chan;
   // room for the multipliers behind the ring and the barriers (the ring stops at 196 KB)
   a.chan_smem = (o.chan != nullptr && (size_t)p.K * 4 <= 24 * 1024) ? 1 : 0;
+  a.cB = g.cB;
+  a.KB = (p.C + g.cB - 1) / g.cB;
+  a.box_mb = g.MB > 1 ? 2 : 1;
+  a.bn_log2 = a.BN == 64 ? 6 : 7;
+  a.d_mb = g.grid % a.n_mblk;
+  a.d_nb = g.grid / a.n_mblk % a.n_nblk;
+  a.d_xi = g.grid / a.n_mblk / a.n_nblk;
   const bool lean = absmaxM == nullptr && out_mode == kOutMq && a.wide_store && p.K % a.BN == 0 && a.BN % 32 == 0 &&
                     (o.chan != nullptr ? o.chan_m_fits_16 && a.chan_smem : p.m_fits_16 != 0);
   static DeviceOnce once_pk, once_lean_pk, once_lean, once_lean_sat;

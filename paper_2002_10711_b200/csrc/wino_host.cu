@@ -203,10 +203,10 @@ int encode_tiled(CUtensorMap* map, const void* base, int rank, const uint64_t* d
 }
 
 int encode_map(CUtensorMap* map, const void* base, uint64_t inner, uint64_t rows, uint64_t mats,
-               uint32_t box_rows) {
+               uint32_t box_rows, int stage_k = kStageK) {
   const uint64_t dims[3] = {inner, rows, mats};
-  const uint32_t box[3] = {(uint32_t)kStageK, box_rows, 1};
-  return encode_tiled(map, base, 3, dims, box, CU_TENSOR_MAP_SWIZZLE_128B);
+  const uint32_t box[3] = {(uint32_t)stage_k, box_rows, 1};
+  return encode_tiled(map, base, 3, dims, box, stage_k == 128 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B);
 }
 
 // Tensor maps of the TMA-staged transform kernels (no swizzle).
@@ -356,12 +356,12 @@ int launch_gemm(wino_plan_t* pl, const int8_t* Vq, const int8_t* Uq, void* out, 
     return launch_gemm_warp(p, opt_of(pl, pdl), Vq, Uq, out, out_mode, absmaxM, st);
   const TcGeom g = tc_geometry(p, pl->num_sms);
   if (pl->map_vq_ptr != Vq) {
-    int rc = encode_map(&pl->mapV, Vq, (uint64_t)p.C, (uint64_t)p.T, (uint64_t)t2, kBM);
+    int rc = encode_map(&pl->mapV, Vq, (uint64_t)p.C, (uint64_t)p.T, (uint64_t)t2, g.MB > 1 ? 2 * kBM : kBM, g.cB);
     if (rc != WINO_OK) return rc;
     pl->map_vq_ptr = Vq;
   }
   if (pl->map_uq_ptr != Uq) {
-    int rc = encode_map(&pl->mapU, Uq, (uint64_t)p.C, (uint64_t)p.K, (uint64_t)t2, (uint32_t)g.BN);
+    int rc = encode_map(&pl->mapU, Uq, (uint64_t)p.C, (uint64_t)p.K, (uint64_t)t2, (uint32_t)g.BN, g.cB);
     if (rc != WINO_OK) return rc;
     pl->map_uq_ptr = Uq;
   }

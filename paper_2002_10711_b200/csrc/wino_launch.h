@@ -147,7 +147,7 @@ int launch_layer_fused(const Params& p, const LaunchOpt& o, const FusedGeom& g, 
                        const void* kron, unsigned* counters, int8_t* mq, const float* bias,
                        float s_Y, int* status, cudaStream_t st);
 
-struct TcGeom { int BN, MB, stages, tmem_cols, grid; size_t smem; };
+struct TcGeom { int BN, MB, cB, stages, tmem_cols, grid; size_t smem; };
 TcGeom tc_geometry(const Params& p, int num_sms);
 int launch_gemm_tc(const Params& p, const LaunchOpt& o, const TcGeom& g, const CUtensorMap& mapV,
                    const CUtensorMap& mapU, void* out, int out_mode, unsigned* absmaxM,
@@ -224,7 +224,7 @@ int launch_wait_probe(long long limit_cycles, int* status, cudaStream_t st);
 
 enum { kOutMq = 0, kOutI32 = 1 };
 constexpr int kBM = 128;      // tiles per GEMM block (MMA M)
-constexpr int kStageK = 128;  // channels (bytes) per shared-memory stage
+constexpr int kStageK = 128;  // channels (bytes) per shared-memory stage (TcGeom::cB: 64 in narrow layers)
 
 // Generic launcher: cudaLaunchKernelEx with, where asked for, the programmatic stream
 // serialization attribute (the kernel then calls griddep_wait()) and clusters of `cluster`

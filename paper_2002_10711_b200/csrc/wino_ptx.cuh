@@ -137,6 +137,12 @@ __device__ __forceinline__ uint64_t make_desc_sw128(uint32_t smem_addr) {
   return (uint64_t)((smem_addr & 0x3FFFFu) >> 4) | (1ull << 16) | (64ull << 32) | (1ull << 46) |
          (2ull << 61);
 }
+// K-major tile of 64-byte rows with the 64-byte swizzle: start / 16, 8-row group stride
+// 512 B, descriptor version 1, layout 4.
+__device__ __forceinline__ uint64_t desc_sw64(uint32_t smem_addr) {
+  return (uint64_t)((smem_addr & 0x3FFFFu) >> 4) | (1ull << 16) | (32ull << 32) | (1ull << 46) |
+         (4ull << 61);
+}
 // Instruction descriptor: D = int32, A = B = signed 8-bit, both K-major, M x N.
 __host__ __device__ constexpr uint32_t make_idesc_i8(int M, int N) {
   return (2u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);

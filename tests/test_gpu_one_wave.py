@@ -50,3 +50,12 @@ def test_chunks_of_112_channels(m, variant):
     if variant == "zero_points":
         L.q_x.zero_point, L.q_w.zero_point, L.q_Y.zero_point = -9, 2, -5
     _compare(L, x_q, w_q, bias, 1)
+
+
+# stages of 64 channels, full and not, under accumulators of four, two and one 128-tile blocks; the
+# last group of tiles ragged; more items than blocks, so that every stage comes round again
+@pytest.mark.parametrize("C", [16, 32, 48, 64])
+@pytest.mark.parametrize("K", [64, 96, 128])
+def test_narrow_stages_of_the_gemm(C, K):
+    L, x_q, w_q, bias = build_layer(wi.Workload("ns", 5740 + C, 801, C, 11, 9, K, 6))
+    _compare(L, x_q, w_q, bias, 1)

@@ -22,7 +22,10 @@
 //                bytes per K index, swizzled, "MN-major".
 // F6: 16 B^T (x) B^T has entries up to 441, split as 16 * hi + lo, two products.
 //
-// Persistent blocks, 672 threads: warps 0-3 load, warp 4 issues the products, sixteen epilogue
+// Persistent blocks, 704 threads: warps 0-3 load, warp 4 issues the products, on the input side every
+// other unit's and warp 5 the rest (a unit's waits, products and commits took a single warp 500 cycles,
+// which held up the 64-channel units: 32x32, batch 256, F4 17.4 us with one warp, 15.6 with two, 15.3
+// with four, where 128-channel ones lost 0.1; the output side, of larger units, lost 0 to 0.3), sixteen epilogue
 // warps; warp w reads tensor-memory lanes 32 * (w % 4) and takes every fourth 32-column chunk.
 // Stores go out directly, as 32-byte pieces of lines that other warps complete: exchanging rows
 // between warps to store whole lines cost 6 to 30 % (barriers), a staging tile with TMA stores
@@ -40,8 +43,8 @@ namespace wino {
 
 namespace {
 
-constexpr int kXtThreads = 672;
-constexpr int kXtLoadWarps = 4, kXtMmaWarp = 4, kXtEpi0 = 5;
+constexpr int kXtLoadWarps = 4, kXtMmaWarp = 4, kXtMmaWarps = 2, kXtEpi0 = kXtMmaWarp + kXtMmaWarps;
+constexpr int kXtThreads = 32 * (kXtEpi0 + 16);
 
 __device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
   asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
@@ -111,16 +114,20 @@ __device__ __forceinline__ void xt_setup(const L& s, volatile uint32_t* abort_p,
   if (warp == kXtMmaWarp) tmem_alloc(s.tmem_slot, (uint32_t)columns);
 }
 
-// The MMA warp's loop: for each of `n_my` units one accumulator of NA products of KSTEPS steps.
-template <typename L, int SLOTS, int NBUF, int NA, int KSTEPS, int CH, int A_ONE, int SLOT_BYTES>
-__device__ __forceinline__ void xt_mma_loop(const L& s, int n_my, uint32_t tmem_base, volatile uint32_t* abort_p) {
+// The MMA warps' loop: for each of `n_my` units one accumulator of NA products of KSTEPS steps, the
+// units dealt out in turn (NM divides the numbers of slots and of accumulators, so that each of
+// those always belongs to the same warp and no warp can fall a phase behind on its barrier).
+template <typename L, int SLOTS, int NBUF, int NM, int NA, int KSTEPS, int CH, int A_ONE, int SLOT_BYTES>
+__device__ __forceinline__ void xt_mma_loop(const L& s, int n_my, int which, uint32_t tmem_base,
+                                            volatile uint32_t* abort_p) {
+  static_assert(SLOTS % NM == 0 && NBUF % NM == 0, "a slot and an accumulator belong to one MMA warp");
   const bool leader = elect_one();
   const uint32_t idesc = idesc_i8_b_mn(128, CH);
   const uint64_t da = make_desc_sw128(s.a), db0 = desc_mn<CH>(s.slot);
   bool ok = __all_sync(0xffffffffu, mbar_wait<false>(s.bar_a, 0u, abort_p));
-  int sl = 0, b = 0;
+  int sl = which, b = which;
   uint32_t ph = 0, aph = 0;
-  for (int i = 0; i < n_my && ok; ++i) {
+  for (int i = which; i < n_my && ok; i += NM) {
     ok = __all_sync(0xffffffffu, mbar_wait<false>(s.bar_acc_empty + 8u * b, aph ^ 1u, abort_p)) &&
          __all_sync(0xffffffffu, mbar_wait<false>(s.bar_full + 8u * sl, ph, abort_p));
     if (!ok) break;
@@ -138,8 +145,8 @@ __device__ __forceinline__ void xt_mma_loop(const L& s, int n_my, uint32_t tmem_
       mma_commit(s.bar_acc_full + 8u * b);
     }
     __syncwarp();
-    if (++sl == SLOTS) { sl = 0; ph ^= 1u; }
-    if (++b == NBUF) { b = 0; aph ^= 1u; }
+    if ((sl += NM) >= SLOTS) { sl = which; ph ^= 1u; }
+    if ((b += NM) >= NBUF) { b = which; aph ^= 1u; }
   }
   if (!ok) *abort_p = 1u;
 }
@@ -210,8 +217,8 @@ k_input_transform_tc(const __grid_constant__ Params p, const __grid_constant__ C
       chunk += d_chunk;
       if (chunk >= cchunks) { chunk -= cchunks; ++group; }
     }
-  } else if (warp == kXtMmaWarp) {
-    xt_mma_loop<L, kSlots, kBuf, NA, 4, CH, 16384, kSlot>(s, n_my, tmem_base, abort_p);
+  } else if (warp < kXtEpi0) {
+    xt_mma_loop<L, kSlots, kBuf, kXtMmaWarps, NA, 4, CH, 16384, kSlot>(s, n_my, warp - kXtMmaWarp, tmem_base, abort_p);
   } else {
     const int quad = warp & 3, sub = (warp - kXtEpi0) >> 2;
     const int r = quad * 32 + lane, xi = r / TP, j = r - xi * TP;
@@ -220,10 +227,17 @@ k_input_transform_tc(const __grid_constant__ Params p, const __grid_constant__ C
     const F2 mult = f2_both(M == 6 ? p.mult_V * 0.0625f : p.mult_V), magic = f2_both(kMagic);
     const uint32_t lo = s16x2_both((int)p.lo_V), hi = s16x2_both((int)p.hi_V);
     const bool wide = (p.C & 31) == 0 && (reinterpret_cast<uintptr_t>(Vq) & 31u) == 0;
+    // this warp's units advance by a constant stride: (group, chunk) with carries
+    const int d_u = step * (int)gridDim.x, u0 = (int)blockIdx.x + first * (int)gridDim.x;
+    const int d_group = d_u / cchunks, d_chunk = d_u - d_group * cchunks;
+    int group = u0 / cchunks, chunk = u0 - group * cchunks;
+    int8_t* const row0 = Vq + (long)xi * p.T * p.C;
     griddep_wait();
     for (int i = first; i < n_my; i += step) {
-      const int u = blockIdx.x + i * gridDim.x;
-      const int group = u / cchunks, c = (u - group * cchunks) * CH + col, tau = group * TP + j;
+      const int c = chunk * CH + col, tau = group * TP + j;
+      group += d_group;
+      chunk += d_chunk;
+      if (chunk >= cchunks) { chunk -= cchunks; ++group; }
       int corr = 0;
       if constexpr (Z) {
         const int rest = tau / p.TW, w0 = (tau - rest * p.TW) * M - 1, n = rest / p.TH, h0 = (rest - n * p.TH) * M - 1;
@@ -246,11 +260,16 @@ k_input_transform_tc(const __grid_constant__ Params p, const __grid_constant__ C
       uint32_t v[32];
       tmem_ld32(tacc, v);
       if constexpr (NA == 2) {
-        uint32_t l[32];
-        tmem_ld32(tacc + CH, l);
+        // the low part in two halves: 64 accumulator words at once spill at the 80 registers of a thread
+        uint32_t l[16];
+        tmem_ld16(tacc + CH, l);
         tmem_ld_wait();
 #pragma unroll
-        for (int e = 0; e < 32; ++e) v[e] = v[e] * 16u + l[e];
+        for (int e = 0; e < 16; ++e) v[e] = v[e] * 16u + l[e];
+        tmem_ld16(tacc + CH + 16, l);
+        tmem_ld_wait();
+#pragma unroll
+        for (int e = 0; e < 16; ++e) v[16 + e] = v[16 + e] * 16u + l[e];
       } else {
         tmem_ld_wait();
       }
@@ -264,7 +283,7 @@ k_input_transform_tc(const __grid_constant__ Params p, const __grid_constant__ C
       }
       uint32_t w[8];
       quant32_fits16(v, mult, magic, lo, hi, w);
-      store_row32(Vq + ((long)xi * p.T + tau) * p.C + c, w, wide, p.C - c);
+      store_row32(row0 + (long)tau * p.C + c, w, wide, p.C - c);
     }
   }
   __syncwarp();
@@ -337,8 +356,9 @@ k_output_transform_tc(const __grid_constant__ Params p, const __grid_constant__ 
         if (++sl == kSlots) { sl = 0; ph ^= 1u; }
       }
     }
-  } else if (warp == kXtMmaWarp) {
-    xt_mma_loop<L, kSlots, kBuf, 1, G::K / 32, CH, kA, kSlot>(s, n_my, tmem_base, abort_p);
+  } else if (warp < kXtEpi0) {
+    if (warp == kXtMmaWarp)
+      xt_mma_loop<L, kSlots, kBuf, 1, 1, G::K / 32, CH, kA, kSlot>(s, n_my, 0, tmem_base, abort_p);
   } else {
     const int quad = warp & 3, sub = (warp - kXtEpi0) >> 2;
     const int r = quad * 32 + lane, j = r / G::PX, pix = r - j * G::PX, ip = pix / M, jp = pix - ip * M;

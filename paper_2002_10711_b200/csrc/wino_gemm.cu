@@ -670,7 +670,7 @@ TcGeom tc_geometry(const Params& p, int num_sms) {
 //   narrower, more codes: 128 ch 16x16 F4 batch 100  4.94, 14.56 / 5.01, 14.77, batch 144  5.79, 17.54
 //     / 6.15, 18.03;  F2 batch 64  4.89, 15.07 / 5.06, 15.41;  32 ch 32x32 F6 batch 128  11.3, 27.0 /
 //     11.8, 27.4.  (One went the other way: 160 ch, 1792 tiles, F4  6.63, 18.48 / 6.07, 18.06.)
-// F6's output transform takes too many registers for blocks of it to fit beside the GEMM either way.
+// F6's output transform in pairs takes too many registers for blocks of it to fit beside the GEMM either way.
 static bool lean_saturates(const Params& p, const GemmTcArgs& a) {
   if (p.hi_M != 127.0f) return false;
   return a.MB * a.BN == 256 || (p.m != 6 && (double)p.t * p.t * p.T * p.K < 5e6);

@@ -282,7 +282,7 @@ k_layer_small(const __grid_constant__ Params p, const __grid_constant__ SmallGeo
       const float q = magic_to_float(fminf(fmaxf(__fmaf_rn(m[j], mult_M, kMagic), lo_m), hi_m));
       m[j] = qM ? q : m[j];
     }
-    at_pass<M, OMODE>(p, m, R);
+    at_pass<M, OMODE, -1>(p, m, R);
 #pragma unroll
     for (int jp = 0; jp < M; ++jp)
       sts32(s_r + 4u * (uint32_t)(((row * M + jp) * 8 + tile) * kRowM + kk), __float_as_uint(R[jp]));
@@ -295,7 +295,7 @@ k_layer_small(const __grid_constant__ Params p, const __grid_constant__ SmallGeo
 #pragma unroll
     for (int r = 0; r < T_; ++r)
       c[r] = __uint_as_float(lds32(s_r + 4u * (uint32_t)(((r * M + jp) * 8 + tile) * kRowM + kk)));
-    at_pass<M, OMODE>(p, c, Y);
+    at_pass<M, OMODE, M - 1>(p, c, Y);   // the last column's form of F6 holds for every column
     const long first = tile_at[tile];
     const int rows = tile_left[tile][0];
     if (first < 0 || !k_on || jp >= tile_left[tile][1]) continue;
@@ -338,8 +338,8 @@ int small_kb(const Params& p, const LaunchOpt& o, const SmallGeom& g, const Smal
 int WINO_CAT(launch_small_m, WINO_M)(const Params& p, const LaunchOpt& o, const SmallGeom& g, const SmallArgs& s,
                                      cudaStream_t st) {
   if (!o.std_mats) return small_kb<WINO_M, kDense, kDense>(p, o, g, s, st);
-  // A^T on codes is exact for F2 and F4 only; on un-quantized sums nowhere
-  if (WINO_M != 6 && p.qM_enabled) return small_kb<WINO_M, kExact, WINO_M == 6 ? kSparse : kExact>(p, o, g, s, st);
+  // A^T is exact on codes, on un-quantized sums nowhere
+  if (p.qM_enabled) return small_kb<WINO_M, kExact, kExact>(p, o, g, s, st);
   return small_kb<WINO_M, kExact, kSparse>(p, o, g, s, st);
 }
 

@@ -8,10 +8,10 @@
 //   kDensePair: the same for two channels, with the entries read as pairs.
 //   kSparse : the built-in Cook-Toom matrices as compile-time constants.
 //   kExact  : Cook-Toom matrices on integer codes where every intermediate is
-//             exactly representable (input stage for m = 2, 4, 6; output stage for
-//             m = 2, 4 on int8 codes), so any summation order gives the same bits;
-//             shared sub-expressions are factored out.  The F6 output stage falls
-//             back to the ordered chains.
+//             exactly representable (input stage for m = 2, 4, 6; output stage on
+//             int8 codes for m = 2, 4 and, for m = 6, all of it but six of the 36
+//             pixels), so any summation order gives the same bits; shared
+//             sub-expressions are factored out.
 #pragma once
 #include "wino_f32x2.cuh"
 
@@ -122,6 +122,30 @@ __device__ __forceinline__ void at_exact(const V (&m)[6], V (&y)[4]) {
   y[2] = v_fma(4.0f, c, a);
   y[3] = v_add(v_fma(8.0f, d, b), m[5]);
 }
+// 1-D A^T of F6 for the R = m A pass (COL < 0) and for column COL of the A^T R pass.  On codes of
+// magnitude at most 128 the first pass is exact: multiples of 1/32 below 128 * 67.1.  Column b of R
+// consists of multiples of 2^-b below 128 r_b, and row a of A^T R of multiples of 2^-(a+b) below
+// 128 r_a r_b, with r = 7, 7, 10.5, 18.25, 34.125, 67.0625 the absolute row sums of A^T; that is exact,
+// whatever the order, while 128 r_a r_b 2^(a+b) <= 2^24, i.e. for all (a, b) but (4,4), (3,5), (4,5),
+// (5,5) and their mirror images, whose rows are the ordered chains.
+__device__ constexpr bool at6_ordered(int a, int b) { return (a >= 4 && b >= 4) || (a >= 3 && b >= 5) || (a >= 5 && b >= 3); }
+template <int COL, typename V>
+__device__ __forceinline__ void at6_exact(const V (&m)[8], V (&y)[6]) {
+  const V s1 = v_add(m[1], m[2]), d1 = v_sub(m[1], m[2]);     // the first two links of every chain
+  const V s2 = v_add(m[3], m[4]), d2 = v_sub(m[3], m[4]);
+  const V s3 = v_add(m[5], m[6]), d3 = v_sub(m[5], m[6]);
+  y[0] = v_add(v_add(v_add(m[0], s1), s2), s3);
+  y[1] = v_fma(0.5f, d3, v_fma(2.0f, d2, d1));
+  y[2] = v_fma(0.25f, s3, v_fma(4.0f, s2, s1));
+  if constexpr (at6_ordered(3, COL)) y[3] = v_fma(-0.125f, m[6], v_fma(0.125f, m[5], v_fma(-8.0f, m[4], v_fma(8.0f, m[3], d1))));
+  else y[3] = v_fma(0.125f, d3, v_fma(8.0f, d2, d1));
+  if constexpr (at6_ordered(4, COL)) y[4] = v_fma(0.0625f, m[6], v_fma(0.0625f, m[5], v_fma(16.0f, m[4], v_fma(16.0f, m[3], s1))));
+  else y[4] = v_fma(0.0625f, s3, v_fma(16.0f, s2, s1));
+  if constexpr (at6_ordered(5, COL))
+    y[5] = v_add(v_fma(-0.03125f, m[6], v_fma(0.03125f, m[5], v_fma(-32.0f, m[4], v_fma(32.0f, m[3], d1)))), m[7]);
+  else
+    y[5] = v_add(v_fma(0.03125f, d3, v_fma(32.0f, d2, d1)), m[7]);
+}
 __device__ __forceinline__ float v_zero(float) { return 0.0f; }
 __device__ __forceinline__ F2 v_zero(F2) { return f2_both(0.0f); }
 // One step of a fused-multiply-add chain; with a compile-time zero coefficient
@@ -200,12 +224,14 @@ __device__ __forceinline__ void input_transform_2d(const Params& p, ColFn col,
   }
 }
 
-// y = A^T v, one 1-D pass of the output transform.
-template <int M, int MODE, typename VT>
+// y = A^T v, one 1-D pass of the output transform: COL < 0 the first, else column COL of the second.
+template <int M, int MODE, int COL, typename VT>
 __device__ __forceinline__ void at_pass(const Params& p, const VT (&v)[M + 2], VT (&y)[M]) {
   constexpr int T_ = M + 2;
   constexpr bool STD = MODE == kSparse || MODE == kExact;
-  if constexpr (MODE == kExact && M != 6) {
+  if constexpr (MODE == kExact && M == 6) {
+    at6_exact<COL>(v, y);
+  } else if constexpr (MODE == kExact) {
     at_exact(v, y);
   } else {
 #pragma unroll
@@ -218,6 +244,16 @@ __device__ __forceinline__ void at_pass(const Params& p, const VT (&v)[M + 2], V
   }
 }
 
+template <int M, int MODE, int COL, typename VT>
+__device__ __forceinline__ void output_columns(const Params& p, const VT (&R)[M + 2][M], VT (&Y)[M * M]) {
+  VT c[M + 2], y[M];
+#pragma unroll
+  for (int i = 0; i < M + 2; ++i) c[i] = R[i][COL];
+  at_pass<M, MODE, COL>(p, c, y);
+#pragma unroll
+  for (int ip = 0; ip < M; ++ip) Y[ip * M + COL] = y[ip];
+  if constexpr (COL + 1 < M) output_columns<M, MODE, COL + 1>(p, R, Y);
+}
 // Y = A^T (m A) for one channel or a pair of them: right factor first.  m row-wise via `row(i, out)`.
 template <int M, int MODE, typename VT, typename RowFn>
 __device__ __forceinline__ void output_transform_2d(const Params& p, RowFn row,
@@ -228,17 +264,9 @@ __device__ __forceinline__ void output_transform_2d(const Params& p, RowFn row,
   for (int i = 0; i < T_; ++i) {
     VT mrow[T_];
     row(i, mrow);
-    at_pass<M, MODE>(p, mrow, R[i]);
+    at_pass<M, MODE, -1>(p, mrow, R[i]);
   }
-#pragma unroll
-  for (int jp = 0; jp < M; ++jp) {
-    VT c[T_], y[M];
-#pragma unroll
-    for (int i = 0; i < T_; ++i) c[i] = R[i][jp];
-    at_pass<M, MODE>(p, c, y);
-#pragma unroll
-    for (int ip = 0; ip < M; ++ip) Y[ip * M + jp] = y[ip];
-  }
+  output_columns<M, MODE, 0>(p, R, Y);
 }
 
 }  // namespace wino

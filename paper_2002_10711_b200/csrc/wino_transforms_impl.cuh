@@ -419,10 +419,9 @@ int output_m(const Params& p, const LaunchOpt& o, float s_Y, const void* mbuf, c
     return qm ? output_mode<M, kDense, true>(p, o, s_Y, mbuf, bias, y, absmax2, st)
               : output_mode<M, kDense, false>(p, o, s_Y, mbuf, bias, y, absmax2, st);
   }
-  // With Q_M on, the F4 output transform works on integers in [-128, 127]:
-  // every intermediate is an integer below 2^24, so the factored form is exact.
-  if (M != 6 && qm) return output_mode<M, kExact, true>(p, o, s_Y, mbuf, bias, y, absmax2, st);
-  return qm ? output_mode<M, kSparse, true>(p, o, s_Y, mbuf, bias, y, absmax2, st)
+  // With Q_M on, the output transform works on integers in [-128, 127], where the factored forms are
+  // exact (F6's is not used here: with several channels per thread it spills).
+  return qm ? output_mode<M, M == 6 ? kSparse : kExact, true>(p, o, s_Y, mbuf, bias, y, absmax2, st)
             : output_mode<M, kSparse, false>(p, o, s_Y, mbuf, bias, y, absmax2, st);
 }
 

@@ -455,16 +455,16 @@ int output_tma_go(const Params& p, const LaunchOpt& o, const CUtensorMap& mapM, 
 template <int M, int MODE, int KC>
 int output_tma_launch(const Params& p, const LaunchOpt& o, const CUtensorMap& mapM, const CUtensorMap& mapY,
                       const float* bias, float s_Y, int* status, float* y_float, cudaStream_t st) {
-  if constexpr (M == 4 && MODE == kExact && KC == 128) {
+  if constexpr (MODE == kExact && ((M == 4 && KC == 128) || (M == 6 && KC % 64 == 0))) {
     if (tma_out_group(p, o.std_mats, o.num_sms) == 1)
-      return output_tma_go<M, MODE, KC, 16, 1>(p, o, mapM, mapY, bias, s_Y, status, nullptr, st);
+      return output_tma_go<M, MODE, KC, M == 4 ? 16 : 1024 / KC, 1>(p, o, mapM, mapY, bias, s_Y, status, nullptr, st);
   }
   if constexpr (M == 6 && MODE == kDense) {
     constexpr int G = tma_group(KC), kPair = pair_blocks(kPairOutThreads, (KC / 2) * G);
     if ((long)((p.T + G - 1) / G) * (p.K / KC) <= (long)kPair * o.num_sms)
       return output_tma_go<M, kDensePair, KC, kPair, 2>(p, o, mapM, mapY, bias, s_Y, status, y_float, st);
   }
-  if constexpr (M == 6 && MODE == kSparse) {
+  if constexpr (M == 6 && MODE == kExact) {
     const int rc = output_tma_go<M, MODE, KC, 1, 2>(p, o, mapM, mapY, bias, s_Y, status, y_float, st, true);
     if (rc <= 0) return rc;
   }
@@ -499,7 +499,7 @@ int WINO_CAT(launch_output_transform_tma_m, WINO_M)(const Params& p, const Launc
                                                      const CUtensorMap& mapY, const float* bias,
                                                      float s_Y, int* status, float* y_float, cudaStream_t st) {
   if (!o.std_mats) return output_tma_mode<WINO_M, kDense>(p, o, mapM, mapY, bias, s_Y, status, y_float, st);
-  return output_tma_mode<WINO_M, WINO_M == 6 ? kSparse : kExact>(p, o, mapM, mapY, bias, s_Y, status, y_float, st);
+  return output_tma_mode<WINO_M, kExact>(p, o, mapM, mapY, bias, s_Y, status, y_float, st);
 }
 
 }  // namespace wino

@@ -34,6 +34,19 @@ def test_around_one_wave_of_blocks(m, N):
     _compare(L, x_q, w_q, bias, 1)
 
 
+# F6 output, one tile per image: one channel per thread up to 148 blocks of 128 and 592 of 64 channels, pairs
+# from there on; codes at their bounds, where the factored sums are largest
+@pytest.mark.parametrize("K,N", [(128, 148), (128, 149), (64, 592), (64, 593), (96, 50)])
+@pytest.mark.parametrize("variant", ["plain", "saturating", "float_out"])
+def test_f6_output_transform(K, N, variant):
+    L, x_q, w_q, bias = build_layer(wi.Workload("o6", 5750 + K, N, 64, 6, 5, K, 6),
+                                    out_dtype=1 if variant == "float_out" else 0)
+    if variant == "saturating":
+        L.q_M.scale, L.q_M.qmin = L.q_M.scale / 1000.0, -128
+    _compare(L, x_q, w_q, bias, 1)
+    _compare(L, x_q, w_q, bias, 8, dumps=False)
+
+
 # several tiles a block (64, 32 and 16 channels a chunk), one channel per thread and two
 @pytest.mark.parametrize("m,C", [(4, 64), (4, 32), (4, 16), (6, 64), (6, 32)])
 @pytest.mark.parametrize("N", [1, 37, 700])

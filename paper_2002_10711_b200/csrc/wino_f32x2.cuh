@@ -77,16 +77,46 @@ __device__ __forceinline__ uint32_t quant_s16x2(F2 v, F2 mult, F2 magic, uint32_
   return clamp_s16x2(f2_low_halves(v_fma(v, mult, magic)), lo, hi);
 }
 
-// 32 int32 values of one row -> 32 codes in eight words (|value * mult| < 2^15, |value| < 2^24).
+// The same for the accumulators of a product, where the ALU pipe has nothing else to do and is the
+// limit: the 16-bit lanes are n + 2^15, unsigned, and a multiply-add on the fp32 pipe joins them
+// instead of a prmt.  With the sums
+//   r0 = kMagic + 2^15 + n0:  bits 0x4B400000 + (n0 + 2^15),
+//   r1 = kMagic + (2^15 - 0x4B40) + n1 (both offsets are even, so ties round as without them)
+// the word 2^16 r1 + r0 has n0 + 2^15 below and (r1 mod 2^16) + 0x4B40 = n1 + 2^15 above, without carries
+// for |n| < 2^15.  The clamped lanes' low bytes are the codes.  Sixteen warps, 32 columns each from tensor
+// memory, beside 64-column products: 777 cycles a round with prmt and signed lanes, 675 so.
+__device__ __forceinline__ F2 u16x2_magic() { return f2_make(kMagic + 32768.0f, kMagic + (32768.0f - 19264.0f)); }
+__device__ __forceinline__ uint32_t u16x2_both(int v) { return (uint32_t)(v + 32768) * 0x00010001u; }
+__device__ __forceinline__ uint32_t quant_u16x2(F2 v, F2 mult, F2 magic, uint32_t lo, uint32_t hi) {
+  uint32_t r0, r1, t, r;
+  f2_split(v_fma(v, mult, magic), r0, r1);
+  asm("mad.lo.u32 %0, %1, 65536, %2;" : "=r"(t) : "r"(r1), "r"(r0));
+  asm("max.u16x2 %0, %1, %2;" : "=r"(r) : "r"(t), "r"(lo));
+  asm("min.u16x2 %0, %1, %2;" : "=r"(t) : "r"(r), "r"(hi));
+  return t;
+}
+// Two int32 values as floats; SMALL (|value| <= 2^22): by adding kMagic's bits and taking kMagic off
+// again, which is no conversion on the ALU pipe but more instructions.  Half a quantizer's values
+// that way: 652 cycles in the measurement above; all of them 770.
+template <bool SMALL>
+__device__ __forceinline__ F2 f2_from_ints(uint32_t a, uint32_t b) {
+  if constexpr (SMALL) return v_add(f2_bits(a + kMagicBits, b + kMagicBits), f2_both(-kMagic));
+  else return f2_make(__int2float_rn((int)a), __int2float_rn((int)b));
+}
+// 32 int32 values of one row -> 32 codes in eight words (|value * mult| < 2^15; |value| < 2^24, SMALL:
+// <= 2^22).  U16: unsigned lanes, with magic, lo, hi from u16x2_magic and u16x2_both; else signed ones
+// (f2_both(kMagic), s16x2_both), which are the faster where something else loads the fp32 pipe (F6
+// input transform, whose two products are joined by a multiply-add a value: 14.5 us against 14.7).
+template <bool U16, bool SMALL>
 __device__ __forceinline__ void quant32_fits16(const uint32_t (&v)[32], F2 mult, F2 magic, uint32_t lo, uint32_t hi,
                                                uint32_t (&w)[8]) {
 #pragma unroll
   for (int q = 0; q < 8; ++q) {
-    const uint32_t a = quant_s16x2(f2_make(__int2float_rn((int)v[4 * q]), __int2float_rn((int)v[4 * q + 1])), mult,
-                                   magic, lo, hi);
-    const uint32_t b = quant_s16x2(f2_make(__int2float_rn((int)v[4 * q + 2]), __int2float_rn((int)v[4 * q + 3])), mult,
-                                   magic, lo, hi);
-    w[q] = __byte_perm(a, b, 0x6420u);
+    const F2 v0 = f2_from_ints<SMALL>(v[4 * q], v[4 * q + 1]), v1 = f2_from_ints<false>(v[4 * q + 2], v[4 * q + 3]);
+    if constexpr (U16)
+      w[q] = __byte_perm(quant_u16x2(v0, mult, magic, lo, hi), quant_u16x2(v1, mult, magic, lo, hi), 0x6420u);
+    else
+      w[q] = __byte_perm(quant_s16x2(v0, mult, magic, lo, hi), quant_s16x2(v1, mult, magic, lo, hi), 0x6420u);
   }
 }
 // 32 bytes of a row, of which `left` (a positive multiple of 16) exist; wide: 32-byte aligned.

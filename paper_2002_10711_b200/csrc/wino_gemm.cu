@@ -211,18 +211,16 @@ __device__ __forceinline__ float acc_to_float(uint32_t v) {
 template <bool PK, bool SAT>
 __device__ __forceinline__ void lean_codes(const Params& p, const uint32_t (&r)[32], int k0, const float* mult_k,
                                            uint32_t (&w)[8]) {
-  const F2 magic = f2_both(kMagic);
-  const uint32_t lo = s16x2_both((int)p.lo_M), hi = s16x2_both((int)p.hi_M);
+  const F2 magic = u16x2_magic();
+  const uint32_t lo = u16x2_both((int)p.lo_M), hi = u16x2_both((int)p.hi_M);
   if constexpr (PK) {
     // every lane reads the same 32 multipliers of the block's table (broadcasts)
     const float4* mp = reinterpret_cast<const float4*>(mult_k + k0);
 #pragma unroll
     for (int q = 0; q < 8; ++q) {
       const float4 mm = mp[q];
-      const uint32_t a = quant_s16x2(f2_make(__int2float_rn((int)r[4 * q]), __int2float_rn((int)r[4 * q + 1])),
-                                     f2_make(mm.x, mm.y), magic, lo, hi);
-      const uint32_t b = quant_s16x2(f2_make(__int2float_rn((int)r[4 * q + 2]), __int2float_rn((int)r[4 * q + 3])),
-                                     f2_make(mm.z, mm.w), magic, lo, hi);
+      const uint32_t a = quant_u16x2(f2_from_ints<false>(r[4 * q], r[4 * q + 1]), f2_make(mm.x, mm.y), magic, lo, hi);
+      const uint32_t b = quant_u16x2(f2_from_ints<false>(r[4 * q + 2], r[4 * q + 3]), f2_make(mm.z, mm.w), magic, lo, hi);
       w[q] = __byte_perm(a, b, 0x6420u);
     }
   } else if constexpr (SAT) {
@@ -233,7 +231,7 @@ __device__ __forceinline__ void lean_codes(const Params& p, const uint32_t (&r)[
                                __int2float_rn((int)r[4 * q + 2]), __int2float_rn((int)r[4 * q + 3]), p.mult_M, lo_m,
                                0.0f);
   } else {
-    quant32_fits16(r, f2_both(p.mult_M), magic, lo, hi, w);
+    quant32_fits16<true, false>(r, f2_both(p.mult_M), magic, lo, hi, w);
   }
 }
 
@@ -659,22 +657,15 @@ TcGeom tc_geometry(const Params& p, int num_sms) {
   return g;
 }
 
-// Which of the two lean quantizers (per-layer scales, upper bound 127; else there is only one).  The
-// saturating pack takes more instructions a code, but its kernel fits 64 registers where the other
-// takes 72, and those eight times 576 keep blocks of the output transform from starting beside the
-// GEMM.  Measured on B200, us, GEMM alone and whole layer, 16-bit lanes / saturating pack:
-//   256-column accumulators: 256 ch 8x8 F4 batch 256  5.87, 15.85 / 5.61, 15.59;  128 ch 16x16 F4
-//     batch 200  8.07, 22.97 / 7.82, 22.66;  64 ch 32x32 F4 batch 128  8.77, 26.36 / 8.45, 26.10
-//   narrower, few codes: 128 ch 16x16 F4 batch 32  3.09, 11.10 / 3.08, 10.64, batch 64  3.66, 12.70 /
-//     3.66, 11.86;  64 ch 32x32 F4 batch 32  4.38, 13.77 / 4.41, 12.93
-//   narrower, more codes: 128 ch 16x16 F4 batch 100  4.94, 14.56 / 5.01, 14.77, batch 144  5.79, 17.54
-//     / 6.15, 18.03;  F2 batch 64  4.89, 15.07 / 5.06, 15.41;  32 ch 32x32 F6 batch 128  11.3, 27.0 /
-//     11.8, 27.4.  (One went the other way: 160 ch, 1792 tiles, F4  6.63, 18.48 / 6.07, 18.06.)
-// F6's output transform in pairs takes too many registers for blocks of it to fit beside the GEMM either way.
-static bool lean_saturates(const Params& p, const GemmTcArgs& a) {
-  if (p.hi_M != 127.0f) return false;
-  return a.MB * a.BN == 256 || (p.m != 6 && (double)p.t * p.t * p.T * p.K < 5e6);
-}
+// Which of the two lean quantizers (per-layer scales, upper bound 127; else there is only one): the
+// saturating pack for blocks of 256 output channels, the clamp on 16-bit lanes, of fewer instructions,
+// for narrower ones.  Measured on B200, us, GEMM alone and whole layer, 16-bit lanes / saturating pack:
+//   256 ch 8x8 F4 batch 256  5.99, 15.83 / 5.95, 15.77, batch 64  4.06, 11.56 / 3.98, 11.46;  512 ch 4x4
+//     F4 batch 256  5.99, 14.12 / 5.90, 14.05
+//   64 ch 32x32 batch 256 F4  14.19, 38.36 / 14.63, 39.10, F6  14.07, 42.70 / 14.36, 43.44;  batch 64 F2
+//     9.04, 19.98 / 9.41, 20.36;  128 ch 16x16 F4 batch 32  3.09, 9.87 / 3.09, 9.90, F2 batch 128  8.95,
+//     21.26 / 8.87, 21.22
+static bool lean_saturates(const Params& p, const GemmTcArgs& a) { return p.hi_M == 127.0f && a.BN == 256; }
 
 int launch_gemm_tc(const Params& p, const LaunchOpt& o, const TcGeom& g, const CUtensorMap& mapV,
                    const CUtensorMap& mapU, void* out, int out_mode, unsigned* absmaxM,

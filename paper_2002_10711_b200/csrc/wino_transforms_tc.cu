@@ -224,8 +224,9 @@ k_input_transform_tc(const __grid_constant__ Params p, const __grid_constant__ C
     const int r = quad * 32 + lane, xi = r / TP, j = r - xi * TP;
     const int col = (kColChunks == 4 ? sub : sub & 1) * 32;
     const int first = kColChunks == 4 ? 0 : sub >> 1, step = kColChunks == 4 ? 1 : 2;
-    const F2 mult = f2_both(M == 6 ? p.mult_V * 0.0625f : p.mult_V), magic = f2_both(kMagic);
-    const uint32_t lo = s16x2_both((int)p.lo_V), hi = s16x2_both((int)p.hi_V);
+    const F2 mult = f2_both(M == 6 ? p.mult_V * 0.0625f : p.mult_V), magic = M == 6 ? f2_both(kMagic) : u16x2_magic();
+    const uint32_t lo = M == 6 ? s16x2_both((int)p.lo_V) : u16x2_both((int)p.lo_V);
+    const uint32_t hi = M == 6 ? s16x2_both((int)p.hi_V) : u16x2_both((int)p.hi_V);
     const bool wide = (p.C & 31) == 0 && (reinterpret_cast<uintptr_t>(Vq) & 31u) == 0;
     // this warp's units advance by a constant stride: (group, chunk) with carries
     const int d_u = step * (int)gridDim.x, u0 = (int)blockIdx.x + first * (int)gridDim.x;
@@ -282,7 +283,7 @@ k_input_transform_tc(const __grid_constant__ Params p, const __grid_constant__ C
         for (int e = 0; e < 32; ++e) v[e] -= (uint32_t)corr;
       }
       uint32_t w[8];
-      quant32_fits16(v, mult, magic, lo, hi, w);
+      quant32_fits16<M != 6, M != 6>(v, mult, magic, lo, hi, w);   // |V| <= 100 * 256
       store_row32(row0 + (long)tau * p.C + c, w, wide, p.C - c);
     }
   }

@@ -1,5 +1,6 @@
 """The GEMM's two quantizers of int8 codes (chosen by accumulator width and number of codes), and transform
 builds that are chosen by whether all blocks of a grid are resident at once, on both sides of each line."""
+import numpy as np
 import pytest
 
 import wino_inputs as wi
@@ -24,6 +25,20 @@ def test_quantizers_of_the_gemm(N, C, K, variant):
     if variant == "bound_100":
         L.q_M.qmin, L.q_M.qmax = -100, 100
     _compare(L, x_q, w_q, bias, 1)
+
+
+# rounded products up to the limit of the 16-bit lanes: inputs and weights of +-127, V and U codes nearly all
+# at their bounds, scales just inside the bounds that the plan checks (|B^T| row sums 2, 10; |V| <= 128 row^2)
+@pytest.mark.parametrize("m,row", [(2, 2), (4, 10)])
+def test_products_at_the_limit_of_16_bits(m, row):
+    L, x_q, w_q, bias = build_layer(wi.Workload("lim", 5760 + m, 9, 16, 13, 15, 64, m))
+    x_q = np.where(x_q > np.median(x_q), 127, -127).astype(np.int8)
+    w_q = np.where(w_q > 0, 127, -127).astype(np.int8)
+    L.q_V.scale = L.q_x.scale * (128.0 * row * row) / 31990.0
+    L.q_U.scale = L.q_w.scale / 100.0
+    L.q_M.scale = L.q_U.scale * L.q_V.scale * (16384.0 * 16) / 31990.0
+    for path in (1, 6):
+        _compare(L, x_q, w_q, bias, path)
 
 
 # blocks per SM x 148: 12, 14 and 16 in F4 (input; 16 also output), 7 in F6

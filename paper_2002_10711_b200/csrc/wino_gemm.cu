@@ -161,23 +161,27 @@ WINO_ST_READER(wino_trace_gemm, g_gemm_trace)
 constexpr int kEpiWarps = 16;
 constexpr int kGemmThreads = 64 + 32 * kEpiWarps;
 
+// Channels (bytes) per stage and stages per item, from what every launch reads anyway: a further
+// argument is a further line of the constant cache, which is empty when a kernel starts.
+__host__ __device__ __forceinline__ constexpr int stage_channels(int C) { return C <= 64 ? 64 : 128; }
+__host__ __device__ __forceinline__ constexpr int stages_per_item(int C) { return C <= 64 ? 1 : (C + 127) >> 7; }
+// m-blocks that one copy of V_q brings (boxes have up to 256 rows).
+__host__ __device__ __forceinline__ constexpr int box_blocks(int MB) { return MB > 1 ? 2 : 1; }
+
 struct GemmTcArgs {
+  // in the order of need: what every launch reads before its first copy comes first
   int BN;          // multiple of 16, <= 256
   int stages;
-  int tmem_cols;   // power of two >= 32, >= 2 * acc_stride
-  int acc_stride;  // columns between the two accumulator buffers
-  int out_mode;
   int MB;          // m-blocks (128 tiles each) per work item, sharing one U_q tile
   int n_mblk, n_nblk, n_items;   // n_mblk counts groups of MB m-blocks
-  int wide_store;  // 1: the output rows are 32-byte aligned (one 256-bit store per row piece)
-  const float* chan;  // per-output-channel multipliers [5][K], or null
-  int chan_smem;      // 1: the block keeps the K multipliers of Q_M in shared memory
-  int bn_log2;        // MB > 1: log2(BN)
-  int cB;             // channels (bytes) per stage: 64 for at most 64 channels, else 128
-  int KB;             // stages per item
-  int box_mb;         // m-blocks one V_q copy brings: boxes have up to 256 rows
+  int tmem_cols;   // power of two >= 32, >= 2 * acc_stride
+  int acc_stride;  // columns between the two accumulator buffers
   // gridDim.x items further, in the digits of the item number (m-block fastest, then k-block, then xi)
   int d_mb, d_nb, d_xi;
+  int out_mode;
+  int wide_store;  // 1: the output rows are 32-byte aligned (one 256-bit store per row piece)
+  int chan_smem;   // 1: the block keeps the K multipliers of Q_M in shared memory
+  const float* chan;  // per-output-channel multipliers [5][K], or null
 };
 
 // The producer's position in the item list: its lone thread has no other warp's work to hide two
@@ -332,7 +336,7 @@ __device__ __forceinline__ void epilogue_loop(const Params& p, const GemmTcArgs&
     // time per warp, the four warps of a scheduler hide each other's
     // tensor-memory load latency
     auto chunk = [&](const uint32_t (&r)[32], int col) {
-      const int j = a.MB > 1 ? col >> a.bn_log2 : 0;
+      const int j = a.MB > 1 ? col >> (a.BN == 64 ? 6 : 7) : 0;
       const int kcol = col - j * a.BN;
       const int tau = (mb * a.MB + j) * kBM + quad * 32 + lane;
       if (tau >= p.T) return;
@@ -373,7 +377,8 @@ __device__ __forceinline__ void gemm_tc_body(const Params& p, const CUtensorMap*
   extern __shared__ uint8_t smem_raw[];
   // tiles need 1024-byte alignment for the 128-byte swizzle
   const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
-  const uint32_t a_bytes = kBM * (uint32_t)a.cB, b_bytes = (uint32_t)(a.BN * a.cB);
+  const int KB = stages_per_item(p.C), cB = stage_channels(p.C), box_mb = box_blocks(a.MB);
+  const uint32_t a_bytes = kBM * (uint32_t)cB, b_bytes = (uint32_t)(a.BN * cB);
   const uint32_t stage_bytes = (uint32_t)a.MB * a_bytes + b_bytes;
   const uint32_t bars = base + (uint32_t)a.stages * stage_bytes;
   const uint32_t bar_full = bars;                           // stages x 8 B
@@ -387,7 +392,6 @@ __device__ __forceinline__ void gemm_tc_body(const Params& p, const CUtensorMap*
   volatile uint32_t* abort_p = reinterpret_cast<volatile uint32_t*>(gen + (abort_slot - base));
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int KB = a.KB;
 
   int trace_step = 0;
 #ifdef WINO_TRACE
@@ -451,7 +455,7 @@ __device__ __forceinline__ void gemm_tc_body(const Params& p, const CUtensorMap*
       // (Two only where a stage is 128 channels.)
       const int n_first = (KB >= 2 && a.stages >= 2) ? 2 : 1;
       uint32_t f_bytes = stage_bytes, f_dst = base, f_b_off = (uint32_t)a.MB * a_bytes, f_a_bytes = a_bytes;
-      int f_row_a = (item.mb * a.MB) * kBM, f_row_b = item.nb * a.BN, f_xi = item.xi, f_mb = a.MB, f_box = a.box_mb, f_n = n_first;
+      int f_row_a = (item.mb * a.MB) * kBM, f_row_b = item.nb * a.BN, f_xi = item.xi, f_mb = a.MB, f_box = box_mb, f_n = n_first;
       asm volatile("" : "+r"(f_bytes), "+r"(f_dst), "+r"(f_b_off), "+r"(f_a_bytes), "+r"(f_row_a),
                         "+r"(f_row_b), "+r"(f_xi), "+r"(f_mb), "+r"(f_box), "+r"(f_n));
       griddep_wait();
@@ -479,10 +483,10 @@ __device__ __forceinline__ void gemm_tc_body(const Params& p, const CUtensorMap*
           ++issued;
           const uint32_t sa = base + (uint32_t)s * stage_bytes;
           mbar_expect_tx(bar_full + 8u * s, stage_bytes);
-          for (int j = 0; j < a.MB; j += a.box_mb)   // rows past T are filled with zeros by the TMA unit
-            tma_load_3d(sa + (uint32_t)j * a_bytes, mapV, bar_full + 8u * s, kb * a.cB,
+          for (int j = 0; j < a.MB; j += box_mb)   // rows past T are filled with zeros by the TMA unit
+            tma_load_3d(sa + (uint32_t)j * a_bytes, mapV, bar_full + 8u * s, kb * cB,
                         (item.mb * a.MB + j) * kBM, item.xi);
-          tma_load_3d(sa + (uint32_t)a.MB * a_bytes, mapU, bar_full + 8u * s, kb * a.cB,
+          tma_load_3d(sa + (uint32_t)a.MB * a_bytes, mapU, bar_full + 8u * s, kb * cB,
                       item.nb * a.BN, item.xi);
           if (++s == a.stages) { s = 0; ph ^= 1u; }
         }
@@ -498,10 +502,10 @@ __device__ __forceinline__ void gemm_tc_body(const Params& p, const CUtensorMap*
     // instruction costs ten to twenty cycles and a stage's MMAs take five hundred.  Descriptors
     // are linear in the tile address (units of 16 bytes), so a stage's are the first stage's
     // plus a multiple of the stage size.
-    const uint64_t da_first = a.cB == 128 ? make_desc_sw128(base) : desc_sw64(base);
+    const uint64_t da_first = cB == 128 ? make_desc_sw128(base) : desc_sw64(base);
     const uint32_t stage_units = stage_bytes >> 4, a_units = a_bytes >> 4;
     const uint32_t b_units = (uint32_t)a.MB * a_units;
-    const int last_ksteps = (p.C - (KB - 1) * a.cB + 31) / 32;   // 1..4
+    const int last_ksteps = (p.C - (KB - 1) * cB + 31) / 32;   // 1..4
     uint32_t s_units = 0;   // s * stage_units
     int s = 0; uint32_t ph = 0;
     int li = 0;
@@ -634,16 +638,20 @@ TcGeom tc_geometry(const Params& p, int num_sms) {
   while (g.MB > 1 && (p.t * p.t) * ((n_mblk + g.MB - 1) / g.MB) * n_nblk0 < 3 * num_sms) g.MB /= 2;
   // At most 64 channels: stages of 64-byte rows with the 64-byte swizzle; 128-byte rows would be half
   // zero fill, which is written to shared memory and leaves room for half as many stages.
-  g.cB = p.C <= 64 ? 64 : 128;
+  g.cB = stage_channels(p.C);
   const size_t per_stage = (size_t)(g.MB * kBM + g.BN) * g.cB;
   g.stages = (int)((196 * 1024) / per_stage);
-  const int KB = (p.C + g.cB - 1) / g.cB;
+  const int KB = stages_per_item(p.C);
   // one and a half items' worth: with two whole items in the ring the second item's operands
   // compete with the first item's for the path from L2 and delay its accumulator (cfg3: 5.87 us
   // with four stages, 5.74 with three, 6.12 with two)
   // ... but four where a stage is an item: its MMAs are over before the next copies, issued when its
-  // slot came free, have landed (64 ch 32x32 batch 256, F4 / F2, two stages 15.4 / 25.3 us, four 14.4 / 23.2)
-  if (KB == 1 && g.stages >= 4) g.stages = 4;
+  // slot came free, have landed (64 ch 32x32 batch 256, F4 / F2, two stages 15.4 / 25.3 us, four 14.4 / 23.2).
+  // Not with less than three items a block or for blocks of 256 channels, where that only takes shared
+  // memory from the output transform's early blocks (128 ch 28x28 batch 16, F4: layer 9.6 us with two, 11.1
+  // with four; 128 -> 256 ch 14x14 batch 64 14.49 and 14.64).
+  const long n_items = (long)(p.t * p.t) * ((n_mblk + g.MB - 1) / g.MB) * n_nblk0;
+  if (KB == 1 && g.BN < 256 && g.stages >= 4 && n_items >= 3l * num_sms) g.stages = 4;
   else if (g.stages > (3 * KB + 1) / 2) g.stages = (3 * KB + 1) / 2;
   if (g.stages > 8) g.stages = 8;
   if (g.stages < 1) g.stages = 1;
@@ -683,10 +691,6 @@ int launch_gemm_tc(const Params& p, const LaunchOpt& o, const TcGeom& g, const C
   a.chan = o.chan;
   // room for the multipliers behind the ring and the barriers (the ring stops at 196 KB)
   a.chan_smem = (o.chan != nullptr && (size_t)p.K * 4 <= 24 * 1024) ? 1 : 0;
-  a.cB = g.cB;
-  a.KB = (p.C + g.cB - 1) / g.cB;
-  a.box_mb = g.MB > 1 ? 2 : 1;
-  a.bn_log2 = a.BN == 64 ? 6 : 7;
   a.d_mb = g.grid % a.n_mblk;
   a.d_nb = g.grid / a.n_mblk % a.n_nblk;
   a.d_xi = g.grid / a.n_mblk / a.n_nblk;

@@ -49,6 +49,15 @@ def test_around_one_wave_of_blocks(m, N):
     _compare(L, x_q, w_q, bias, 1)
 
 
+# one to nine blocks of a transform per SM: from two to eight the grid asks for the shared memory that
+# spreads it over the SMs, the output's only where the GEMM's items are level
+@pytest.mark.parametrize("m", [2, 4, 6])
+@pytest.mark.parametrize("N", [148, 149, 296, 512, 1184, 1185])
+def test_few_blocks_per_sm(m, N):
+    L, x_q, w_q, bias = build_layer(wi.Workload("fb", 5770 + m, N, 128, m, m - 1, 128, m))
+    _compare(L, x_q, w_q, bias, 1)
+
+
 # F6 output, one tile per image: one channel per thread up to 148 blocks of 128 and 592 of 64 channels, pairs
 # from there on; codes at their bounds, where the factored sums are largest
 @pytest.mark.parametrize("K,N", [(128, 148), (128, 149), (64, 592), (64, 593), (96, 50)])

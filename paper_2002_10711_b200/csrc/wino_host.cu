@@ -416,13 +416,18 @@ LaunchOpt opt_with_hint(const wino_plan_t* pl, bool pdl, int stage_mask, const i
 }
 
 // Estimated times in ns, for the choice between kernels that can run the same layer.  Staged: a
-// start-up latency of three dependent kernels plus a time per code (measured, us: F2 16.8 M codes
-// in and out 14, 134 M 62; F4 2.2 M 9.5, 9.4 M 12, 75 M 43; F6 1.5 M 10.9, 9.4 M 14, 75 M 49; with
-// warp-level MMAs 0.7 M 8, 5 M 17, 8.4 M 20, 20 M 37).  Fused F2: waves of 128 tiles per SM, full or not (28 us at 64 channels).
+// start-up latency of three dependent kernels (and of their three launches, which the one-launch kernel
+// saves two of) plus a time per code and per byte of weights (measured, us: F2 1 M codes in and out 6.3,
+// 33.5 M 20, 134 M 52; F4 0.6 M 6.6, 2.4 M 7.0 to 8.1, 9.4 M 9.5, 75 M 38; F4, 0.6 M codes, 2.4 MB of
+// weights 7.1, 9.4 MB 8.0; F6 0.6 M 8.0, 1.2 M 8.7, 75 M 43; with warp-level MMAs 0.7 M 8, 5 M 17, 8.4 M
+// 20, 20 M 37).  Where the one-launch kernel's estimate is the higher one so is its time: F4 256 ch 8x8
+// batch 8 8.5 against 7.1, batch 16 9.5 and 7.2; 512 ch 4x4 batch 16 9.6 and 8.0; 128 ch 16x16 batch 16 8.0
+// and 7.0, batch 8 6.3 and 7.0.  Fused F2: waves of 128 tiles per SM, full or not (28 us at 64 channels).
 long staged_cost(const wino_plan_t* pl) {
-  const double codes = (double)pl->p.t * pl->p.t * pl->p.T * (pl->p.C + pl->p.K);
+  const Params& p = pl->p;
+  const double codes = (double)p.t * p.t * p.T * (p.C + p.K), weights = (double)p.t * p.t * p.K * p.C;
   if (pl->path == WINO_PATH_STAGED_DP4A) return 6500 + (long)(codes * 1.9e-3);
-  return (pl->p.m == 6 ? 9800 : 8500) + (long)(codes * (pl->p.m == 2 ? 4.0e-4 : 4.7e-4));
+  return (p.m == 2 ? 6700 : p.m == 4 ? 6900 : 8000) + (long)(codes * (p.m == 2 ? 3.7e-4 : 4.0e-4) + weights * 1.0e-4);
 }
 long fused_f2_cost(const wino_plan_t* pl) {
   const long waves = ((pl->p.T + 127) / 128 + pl->num_sms - 1) / pl->num_sms;

@@ -59,3 +59,30 @@ def small(wl: wi.Workload, **kw) -> wi.Workload:
     d = copy.copy(wl.__dict__)
     d.update(kw)
     return wi.Workload(**d)
+
+
+def f6_order_sensitive(N: int, K: int, C: int = 64, H: int = 6, W: int = 6, out_dtype: int = 1):
+    """An F6 layer whose output shows in which order A^T m A was summed: the codes of U, V and M are nearly
+    all at or near their bounds, so that the sums of the six pixels that are not exact in fp32 exceed 24 bits.
+    out_dtype 0 (whole 6x6 images, all alike): the output scale is 1/128 of the accumulators', a unit in the
+    last place of a sum of 2^16 to 2^17, and channel k's bias takes its sum at pixel F6_ORDERED[k % 6] away."""
+    L, x_q, w_q, bias = build_layer(wi.Workload("f6o", 5750 + K, N, C, H, W, K, 6), out_dtype=1)
+    L.q_U.scale /= 3000.0
+    L.q_V.scale /= 20.0
+    # powers of two: nothing is lost in taking a bias to output codes
+    L.q_M.scale = float(np.exp2(np.rint(np.log2(L.q_U.scale * L.q_V.scale * 127.0 * 127.0 * C ** 0.5 * 3e-3))))
+    L.q_M.qmin = -128
+    L.out_dtype = out_dtype
+    if out_dtype == 0:
+        assert (H, W) == (6, 6)
+        x_q[:] = x_q[:1]
+        L.q_Y.scale, L.q_Y.qmin = L.q_M.scale / 128.0, -128
+        one = copy.deepcopy(L)
+        one.N, one.out_dtype = 1, 1
+        y = oracle.forward(one, x_q[:1], w_q, bias=None)[0]
+        bias = np.array([-y[(*F6_ORDERED[k % 6], k)] for k in range(K)], np.float32)
+    return L, x_q, w_q, bias
+
+
+# (row, column) of the output pixels of an F6 tile whose sums need more than 24 bits
+F6_ORDERED = [(4, 4), (3, 5), (5, 3), (4, 5), (5, 4), (5, 5)]

@@ -4,7 +4,7 @@ import numpy as np
 import pytest
 
 import wino_inputs as wi
-from helpers import build_layer, per_channel
+from helpers import build_layer, f6_order_sensitive, per_channel
 from test_gpu_parity import _compare
 
 pytestmark = pytest.mark.gpu
@@ -67,6 +67,19 @@ def test_f6_output_transform(K, N, variant):
                                     out_dtype=1 if variant == "float_out" else 0)
     if variant == "saturating":
         L.q_M.scale, L.q_M.qmin = L.q_M.scale / 1000.0, -128
+    _compare(L, x_q, w_q, bias, 1)
+    _compare(L, x_q, w_q, bias, 8, dumps=False)
+
+
+# the same builds, and the one-launch kernel, on sums that show the order of their terms: as floats, and as codes
+# of a unit in the last place each (the one-channel builds write codes only)
+@pytest.mark.parametrize("K,N", [(128, 148), (128, 149), (64, 592), (64, 593), (96, 50)])
+@pytest.mark.parametrize("out", ["codes", "float", "float_ragged"])
+def test_f6_output_transform_sums_in_order(K, N, out):
+    if out == "float_ragged":
+        L, x_q, w_q, bias = f6_order_sensitive((N + 3) // 4, K, H=11, W=12)
+    else:
+        L, x_q, w_q, bias = f6_order_sensitive(N, K, out_dtype=0 if out == "codes" else 1)
     _compare(L, x_q, w_q, bias, 1)
     _compare(L, x_q, w_q, bias, 8, dumps=False)
 

@@ -1,4 +1,4 @@
-"""The GEMM's two quantizers of int8 codes (chosen by accumulator width and number of codes), and transform
+"""The GEMM's two quantizers of int8 codes (chosen by the width of a block's columns), and transform
 builds that are chosen by whether all blocks of a grid are resident at once, on both sides of each line."""
 import numpy as np
 import pytest
@@ -10,8 +10,10 @@ from test_gpu_parity import _compare
 pytestmark = pytest.mark.gpu
 
 
-# 256-column accumulators; fewer and more than 5 M codes in narrower ones; bounds other than 127
-@pytest.mark.parametrize("N,C,K", [(6, 128, 256), (6, 64, 96), (120, 64, 192)])
+# blocks of 256 output channels (saturating pack) and narrower ones (clamp on 16-bit lanes), these with one, two
+# and four 128-tile blocks to an accumulator; bounds other than 127
+@pytest.mark.parametrize("N,C,K", [(6, 128, 256), (6, 64, 96), (120, 64, 192), (360, 64, 64), (720, 32, 64),
+                                   (360, 64, 128)])
 @pytest.mark.parametrize("variant", ["plain", "relu", "per_channel", "zero_point_y", "saturating", "bound_100"])
 def test_quantizers_of_the_gemm(N, C, K, variant):
     L, x_q, w_q, bias = build_layer(wi.Workload("oc", 5720, N, C, 9, 11, K, 4), relu=variant == "relu")
@@ -103,9 +105,10 @@ def test_chunks_of_112_channels(m, variant):
 
 
 # stages of 64 channels, full and not, under accumulators of four, two and one 128-tile blocks; the
-# last group of tiles ragged; more items than blocks, so that every stage comes round again
+# last group of tiles ragged; at least five items to each of 148 blocks, so that the four stages come round again
 @pytest.mark.parametrize("C", [16, 32, 48, 64])
-@pytest.mark.parametrize("K", [64, 96, 128])
-def test_narrow_stages_of_the_gemm(C, K):
-    L, x_q, w_q, bias = build_layer(wi.Workload("ns", 5740 + C, 801, C, 11, 9, K, 6))
+@pytest.mark.parametrize("K,N,blocks", [(64, 1793, 4), (96, 801, 1), (128, 801, 2)])
+def test_narrow_stages_of_the_gemm(C, K, N, blocks):
+    L, x_q, w_q, bias = build_layer(wi.Workload("ns", 5740 + C, N, C, 11, 9, K, 6))
+    assert 64 * -(-4 * N // (128 * blocks)) >= 5 * 148
     _compare(L, x_q, w_q, bias, 1)

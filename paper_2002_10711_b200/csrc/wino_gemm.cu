@@ -660,8 +660,8 @@ TcGeom tc_geometry(const Params& p, int num_sms) {
   g.tmem_cols = 2 * acc_stride;
   g.smem = 1024 + g.stages * per_stage + 16 * g.stages + 64;
   const int n_mgrp = (n_mblk + g.MB - 1) / g.MB;
-  const int items = (p.t * p.t) * n_mgrp * ((p.K + g.BN - 1) / g.BN);
-  g.grid = items < num_sms ? items : num_sms;
+  g.items = (p.t * p.t) * n_mgrp * n_nblk0;
+  g.grid = g.items < num_sms ? g.items : num_sms;
   return g;
 }
 
@@ -686,7 +686,7 @@ int launch_gemm_tc(const Params& p, const LaunchOpt& o, const TcGeom& g, const C
   a.MB = g.MB;
   a.n_mblk = ((p.T + kBM - 1) / kBM + g.MB - 1) / g.MB;
   a.n_nblk = (p.K + g.BN - 1) / g.BN;
-  a.n_items = p.t * p.t * a.n_mblk * a.n_nblk;
+  a.n_items = g.items;
   a.wide_store = (reinterpret_cast<uintptr_t>(out) & 31u) == 0 ? 1 : 0;
   a.chan = o.chan;
   // room for the multipliers behind the ring and the barriers (the ring stops at 196 KB)

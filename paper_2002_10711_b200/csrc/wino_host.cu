@@ -556,7 +556,9 @@ int forward_impl(wino_plan_t* pl, const int8_t* x, const int8_t* Uq, const float
     const bool to_float = pl->p.out_dtype != 0;
     const CUtensorMap* my = to_float ? mm : map_y(pl, y);
     if (mm == nullptr || my == nullptr) return WINO_ERR_CUDA;
-    rc = launch_output_transform_tma(pl->p, opt_of(pl, pdl), *mm, *my, bias, pl->s_Y, pl->status_dev,
+    LaunchOpt o = opt_of(pl, pdl);
+    if (gemm_path != WINO_PATH_STAGED_DP4A) o.gemm_items = tc_geometry(pl->p, pl->num_sms).items;
+    rc = launch_output_transform_tma(pl->p, o, *mm, *my, bias, pl->s_Y, pl->status_dev,
                                      to_float ? reinterpret_cast<float*>(y) : nullptr, st);
   } else {
     rc = launch_output_transform(pl->p, opt_of(pl, pdl), pl->s_Y, mbuf, bias, y,

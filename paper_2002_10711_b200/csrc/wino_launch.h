@@ -31,6 +31,8 @@ struct LaunchOpt {
   // and the output transforms.
   const float* chan = nullptr;
   bool chan_m_fits_16 = false;   // with these multipliers every rounded product of Q_M is below 2^15
+  // Work items of the tensor-core GEMM in front of an output transform, 0 if it is another GEMM.
+  long gemm_items = 0;
 };
 
 // "Done once per device" bookkeeping.  cudaFuncSetAttribute applies to the device
@@ -153,7 +155,7 @@ int launch_layer_fused(const Params& p, const LaunchOpt& o, const FusedGeom& g, 
                        const void* kron, unsigned* counters, int8_t* mq, const float* bias,
                        float s_Y, int* status, cudaStream_t st);
 
-struct TcGeom { int BN, MB, cB, stages, tmem_cols, grid; size_t smem; };
+struct TcGeom { int BN, MB, cB, stages, tmem_cols, items, grid; size_t smem; };
 TcGeom tc_geometry(const Params& p, int num_sms);
 int launch_gemm_tc(const Params& p, const LaunchOpt& o, const TcGeom& g, const CUtensorMap& mapV,
                    const CUtensorMap& mapU, void* out, int out_mode, unsigned* absmaxM,

@@ -14,9 +14,8 @@
 // two waves a layer is, then issue slots.  One channel per thread spends a shared-memory
 // wavefront on every 32 codes read or written and two clamp instructions on every code.
 #pragma once
-#include <algorithm>
-
 #include "wino_ptx.cuh"
+#include "wino_spread.h"
 #include "wino_trace.cuh"
 #include "wino_transform_math.cuh"
 
@@ -361,23 +360,6 @@ class Resident {
   int n_[DeviceOnce::kMaxDevices + 1] = {};
 };
 
-// Dynamic shared memory with which a grid of two to eight blocks per SM, on average, cannot have more
-// than that on any.  These blocks are launched while the preceding kernel runs and gather on whatever
-// SMs it leaves free, up to sixteen on each of a few SMs, and the kernel then takes as long as those.
-// Larger grids even out by themselves.  Measured on B200, us, without / with it:
-//   input transform alone  128 ch 16x16 F4 batch 30 3.43 / 2.32, batch 40 3.72 / 2.57;  512 ch 4x4 F4 batch
-//     100 3.11 / 2.06, F6 batch 140 4.81 / 3.54;  64 ch 16x16 F2 batch 30 2.50 / 2.16
-//   output transform alone  256 ch 8x8 F4 batch 128 3.55 / 2.82;  96 ch 20x20 F4 batch 20 3.06 / 2.21;  128
-//     ch 8x8 F2 batch 64 2.60 / 2.08
-//   whole layers, with both  256 ch 8x8 F4 batch 128 12.67 / 10.29, batch 56 11.55 / 8.77, batch 32 8.04 /
-//     8.09;  128 ch 28x28 F4 batch 8 9.06 / 7.23;  160 -> 192 ch 14x14 F4 batch 16 11.23 / 8.05;  512 ch 4x4
-//     F4 batch 128 11.41 / 10.11;  128 ch 12x12 F6 batch 64 11.58 / 9.77
-constexpr size_t kSpreadSmem = 220 * 1024;
-inline size_t spread_smem(size_t smem, long units, int num_sms) {
-  const long per = (units + num_sms - 1) / num_sms;
-  return per >= 2 && per <= 8 ? std::max(smem, kSpreadSmem / (size_t)per - 1024) : smem;
-}
-
 // Launches the input transform; with one_wave only if its blocks are all resident at once, else it
 // returns 1.
 template <int M, int MODE, int CC, int MINB, int CPT>
@@ -387,9 +369,9 @@ int input_tma_go(const Params& p, const LaunchOpt& o, const CUtensorMap& mapX, c
   constexpr size_t smem = 2 * (size_t)G * ((((M + 2) * (M + 2) * CC) + 127) / 128 * 128) + 128 + 16;
   auto kernel = k_input_transform_tma<M, MODE, CC, G, MINB, CPT>;
   static DeviceOnce once;   // one per instantiation
-  if (int rc = set_max_smem(once, o.device, kernel, std::max(smem, spread_smem(0, 2, 1)))) return rc;
+  if (int rc = set_max_smem(once, o.device, kernel, spread_smem(smem, 2))) return rc;
   const long units = (long)((p.T + G - 1) / G) * (p.C / CC);
-  const size_t ask = spread_smem(smem, units, o.num_sms);
+  const size_t ask = spread_smem(smem, in_blocks_per_sm(units, o.num_sms));
   if (one_wave) {
     static Resident resident;
     if (units > (long)o.num_sms * resident.blocks(o.device, kernel, (CC / CPT) * G, smem)) return 1;
@@ -459,14 +441,9 @@ int output_tma_go(const Params& p, const LaunchOpt& o, const CUtensorMap& mapM, 
   constexpr size_t smem = (G * (M + 2) * (M + 2) * KC + 127) / 128 * 128 + (size_t)G * ((M * M * KC + 127) / 128 * 128) + 128 + 16;
   static DeviceOnce once;   // one per instantiation
   auto kernel = k_output_transform_tma<M, MODE, KC, G, MINB, CPT>;
-  if (int rc = set_max_smem(once, o.device, kernel, std::max(smem, spread_smem(0, 2, 1)))) return rc;
+  if (int rc = set_max_smem(once, o.device, kernel, spread_smem(smem, 2))) return rc;
   const long units = (long)((p.T + G - 1) / G) * (p.K / KC);
-  // spread unless some of the GEMM's blocks have an item more than others: the SMs that the others
-  // leave early are then the place for the excess (128 ch 16x16 F4 batch 48, 216 items, 9.4 us without,
-  // 10.3 with; batch 64, 288 items, 11.1 and 9.5)
-  const long items = (long)p.t * p.t * ((p.T + kBM - 1) / kBM) * ((p.K + 255) / 256);
-  const bool level = items <= o.num_sms || (items <= 2l * o.num_sms && 10 * items >= 19l * o.num_sms);
-  const size_t ask = level ? spread_smem(smem, units, o.num_sms) : smem;
+  const size_t ask = spread_smem(smem, out_blocks_per_sm(units, o.gemm_items, p.C, o.num_sms));
   if (one_wave) {
     static Resident resident;
     if (units > (long)o.num_sms * resident.blocks(o.device, kernel, (KC / CPT) * G, smem)) return 1;

@@ -23,9 +23,16 @@ inline size_t spread_smem(size_t smem, int per) {
 //   whole layers, with both  256 ch 8x8 F4 batch 128 12.67 / 10.29, batch 56 11.55 / 8.77, batch 32 8.04 /
 //     8.09;  128 ch 28x28 F4 batch 8 9.06 / 7.23;  160 -> 192 ch 14x14 F4 batch 16 11.23 / 8.05;  512 ch 4x4
 //     F4 batch 128 11.41 / 10.11;  128 ch 12x12 F6 batch 64 11.58 / 9.77
-inline int in_blocks_per_sm(long units, int num_sms) {
+// The input transform's limit.  None in a layer of more than 64 output channels and many un-quantized sums
+// (`sums` of them, 0 if they are quantized): what runs before it is as a rule another such layer's long
+// pointer-based output transform, on whose last SMs the whole grid would then wait.  Layers, us, without /
+// with the limit: 128 ch 8x8 F6 batch 150 (4.9 M sums) 25.0 / 26.6;  256 ch 8x8 F6 batch 75 (4.9 M) 27.6 /
+// 30.0;  128 -> 256 ch 8x8 F4 batch 150 (5.5 M) 23.1 / 24.7;  256 ch 4x4 F2 batch 150 (2.5 M) 16.5 / 17.1;
+// below  256 ch 8x8 F4 batch 50 (1.8 M) 18.2 / 16.6;  128 ch 4x4 F2 batch 150 (1.2 M) 13.4 / 11.4;  64 output
+// channels  256 ch 8x8 F4 batch 100 (0.9 M) 14.0 / 13.3, 64 ch 8x8 F4 batch 400 (3.7 M) 18.3 / 17.4.
+inline int in_blocks_per_sm(long units, int K, long sums, int num_sms) {
   const long per = (units + num_sms - 1) / num_sms;
-  return per >= 2 && per <= 8 ? (int)per : 0;
+  return per >= 2 && per <= 8 && (K <= 64 || sums <= 2200000) ? (int)per : 0;
 }
 
 // The output transform, behind a tensor-core GEMM of `items` work items and C input channels (items 0:

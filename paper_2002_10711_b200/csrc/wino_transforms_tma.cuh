@@ -371,7 +371,8 @@ int input_tma_go(const Params& p, const LaunchOpt& o, const CUtensorMap& mapX, c
   static DeviceOnce once;   // one per instantiation
   if (int rc = set_max_smem(once, o.device, kernel, spread_smem(smem, 2))) return rc;
   const long units = (long)((p.T + G - 1) / G) * (p.C / CC);
-  const size_t ask = spread_smem(smem, in_blocks_per_sm(units, o.num_sms));
+  const long sums = p.qM_enabled ? 0 : (long)p.t * p.t * p.T * p.K;
+  const size_t ask = spread_smem(smem, in_blocks_per_sm(units, p.K, sums, o.num_sms));
   if (one_wave) {
     static Resident resident;
     if (units > (long)o.num_sms * resident.blocks(o.device, kernel, (CC / CPT) * G, smem)) return 1;

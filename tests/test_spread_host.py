@@ -21,8 +21,11 @@ int main(int argc, char** argv) {
   bad += spread_smem(5000, 0) != 5000 || spread_smem(200000, 3) != 200000;
   // whatever the choice, no block has to wait for another's place
   for (int sms : {1, 132, 148}) for (long units = 1; units < 3000; ++units) {
-    const int in = in_blocks_per_sm(units, sms);
-    bad += in != 0 && (in < 2 || in > 8 || (long)in * sms < units);
+    for (int K : {64, 128}) for (long sums : {0l, 2200000l, 2200001l}) {
+      const int in = in_blocks_per_sm(units, K, sums, sms);
+      const bool limit = units > sms && units <= 8l * sms && (K == 64 || sums <= 2200000l);
+      bad += limit ? in < 2 || in > 8 || (long)in * sms < units : in != 0;
+    }
     for (long items = 0; items < 700; items += 3) for (int C : {64, 128, 144, 512}) {
       const int out = out_blocks_per_sm(units, items, C, sms);
       bad += out != 0 && (out < 2 || out > 8 || (long)out * sms < units);

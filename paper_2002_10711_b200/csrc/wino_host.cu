@@ -415,19 +415,32 @@ LaunchOpt opt_with_hint(const wino_plan_t* pl, bool pdl, int stage_mask, const i
   return o;
 }
 
-// Estimated times in ns, for the choice between kernels that can run the same layer.  Staged: a
-// start-up latency of three dependent kernels (and of their three launches, which the one-launch kernel
-// saves two of) plus a time per code and per byte of weights (measured, us: F2 1 M codes in and out 6.3,
-// 33.5 M 20, 134 M 52; F4 0.6 M 6.6, 2.4 M 7.0 to 8.1, 9.4 M 9.5, 75 M 38; F4, 0.6 M codes, 2.4 MB of
-// weights 7.1, 9.4 MB 8.0; F6 0.6 M 8.0, 1.2 M 8.7, 75 M 43; with warp-level MMAs 0.7 M 8, 5 M 17, 8.4 M
-// 20, 20 M 37).  Where the one-launch kernel's estimate is the higher one so is its time: F4 256 ch 8x8
-// batch 8 8.5 against 7.1, batch 16 9.5 and 7.2; 512 ch 4x4 batch 16 9.6 and 8.0; 128 ch 16x16 batch 16 8.0
-// and 7.0, batch 8 6.3 and 7.0.  Fused F2: waves of 128 tiles per SM, full or not (28 us at 64 channels).
+// Estimated times in ns, for the choice between kernels that can run the same layer.  Staged: a start-up
+// latency of three dependent kernels and of their launches, a time per code, per byte of weights and per
+// un-quantized sum (four bytes, through the pointer-based output transform), and what learnt matrices, an
+// input zero point and rows of less than 64 channels add to the transforms; F6's output transform has a quick
+// build for small grids in chunks of 64 and 128 channels only.  Fitted on B200 to the layers of small_geometry,
+// forced onto this path (5 to 10 % standard deviation).  Of 4800 layers either kernel can run, the choice
+// costs 0.3 % on average and more than 7 % on one in sixty.  Us, one launch / staged, times (of a loop of calls
+// and a graph, averaged) and estimates:
+//   F4  512 ch 4x4 batch 16  9.9 / 8.8 and 9.6 / 8.9;  256 ch 8x8 batch 16  10.1 / 7.9 and 9.4 / 8.1, batch 8
+//     7.9 / 7.8 and 7.8 / 7.9, batch 4  7.3 / 7.8 and 7.1 / 7.8;  128 ch 16x16 batch 16  8.3 / 7.6 and 8.5 /
+//     8.4, batch 8  6.5 / 7.5 and 7.2 / 7.9;  un-quantized 256 ch 8x8 batch 16  9.8 / 11.5 and 9.4 / 10.5
+//   F2  un-quantized 128 ch 14x14 batch 16  10.1 / 14.2 and 11.0 / 14.7, learnt  11.5 / 8.0 and 12.7 / 8.6
+//   F6  128 ch 16x16 batch 16  11.4 / 9.1 and 10.8 / 9.8, un-quantized  11.1 / 15.7 and 10.8 / 14.5
+// Fused F2: waves of 128 tiles per SM, full or not (28 us at 64 channels).
 long staged_cost(const wino_plan_t* pl) {
+  static const double start[3] = {7000, 7300, 8100}, per_code[3] = {4.0e-4, 4.3e-4, 6.5e-4};
+  static const double start_warp[3] = {7000, 7500, 9300};   // GEMM by warp-level MMAs
+  static const double learnt[3] = {300, 900, 3100}, zero[3] = {1000, 1100, 600};
   const Params& p = pl->p;
-  const double codes = (double)p.t * p.t * p.T * (p.C + p.K), weights = (double)p.t * p.t * p.K * p.C;
-  if (pl->path == WINO_PATH_STAGED_DP4A) return 6500 + (long)(codes * 1.9e-3);
-  return (p.m == 2 ? 6700 : p.m == 4 ? 6900 : 8000) + (long)(codes * (p.m == 2 ? 3.7e-4 : 4.0e-4) + weights * 1.0e-4);
+  const int mi = p.m / 2 - 1;
+  const double v = (double)p.t * p.t * p.T * p.C, sums = (double)p.t * p.t * p.T * p.K;
+  double ns = (p.qM_enabled ? 0.0 : 4.0e-3 * sums) + (pl->std_mats ? 0.0 : learnt[mi]) + (p.z_x == 0 ? 0.0 : zero[mi]);
+  if (pl->path == WINO_PATH_STAGED_DP4A) return (long)(ns + start_warp[mi] + 1.5e-3 * (v + sums));
+  if (p.m == 6 && tma_chunk(p.K) % 64 != 0) ns += 700;
+  if (p.m != 2) ns += 700 * ((tma_chunk(p.C) < 64) + (tma_chunk(p.K) < 64));
+  return (long)(ns + start[mi] + per_code[mi] * (v + sums) + 1.4e-4 * p.t * p.t * p.K * p.C);
 }
 long fused_f2_cost(const wino_plan_t* pl) {
   const long waves = ((pl->p.T + 127) / 128 + pl->num_sms - 1) / pl->num_sms;
@@ -704,7 +717,7 @@ int wino_plan(const wino_desc_t* desc, wino_plan_t** out) {
   if (pl->std_mats && pl->status_dev != nullptr) xt_images(pl->device, &pl->xt_images);
   cudaGetLastError();
   pl->small_ok = small_supported(p);
-  if (pl->small_ok) pl->small = small_geometry(p, pl->num_sms);
+  if (pl->small_ok) pl->small = small_geometry(p, pl->std_mats, pl->num_sms);
   *out = pl;
   return WINO_OK;
 }

@@ -178,7 +178,7 @@ struct SmallArgs {
   int* status;
 };
 bool small_supported(const Params& p);
-SmallGeom small_geometry(const Params& p, int num_sms);
+SmallGeom small_geometry(const Params& p, bool std_mats, int num_sms);
 int launch_small(const Params& p, const LaunchOpt& o, const SmallGeom& g, const SmallArgs& s, cudaStream_t st);
 
 // Fully fused F2 kernel for narrow layers (C in {32, 64}, K <= 64, Cook-Toom matrices).

@@ -102,13 +102,14 @@ constexpr int tma_in_group(int m, int chunk) { return m == 2 ? tma_group(chunk) 
 // batch 32 10.93 / 10.58, 384 ch 12x12 batch 32 15.76 / 15.48 (256 ch 8x8 batch 64 11.60 / 11.73);
 // narrower chunks lose (96 ch: 11.80 / 12.45, 64 ch: 13.74 / 13.89).
 // F6 likewise while a handful of blocks per SM is all there is: at 64 registers they start beside the
-// GEMM, and a block is over sooner.  Layer, us, two channels per thread / one: 128 ch 12x12 batch 32
-// (128 blocks) 9.63 / 7.89, batch 64 (256) 9.97 / 10.65; 64 ch 32x32 batch 8 (288) 8.92 / 8.43, batch 16
-// (576) 11.16 / 9.73, batch 32 (1152) 12.91 / 13.62.
+// GEMM, and a block is over sooner.  Layer, us, two channels per thread / one, blocks per SM in brackets: 128
+// channels a block  128 ch 12x12 batch 64 (2) 9.9 / 9.2, batch 100 (3) 11.0 / 9.8, 512 ch 8x8 batch 32 (4) 12.7
+// / 12.2, 128 ch 12x12 batch 150 (5) 12.6 / 13.1, 256 ch 12x12 batch 75 (5) 13.6 / 14.1;  64 channels  64 ch
+// 12x12 batch 64 (2) 9.1 / 8.2, batch 150 (5) 10.4 / 9.7, batch 200 (6) 11.4 / 10.4, batch 275 (8) 12.4 / 13.1.
 inline int tma_out_group(const Params& p, bool std_mats, int num_sms) {
   const int chunk = tma_chunk(p.K);
   if (p.m == 6 && std_mats && p.out_dtype == 0 && (chunk == 128 || chunk == 64))
-    return (long)p.T * (p.K / chunk) <= (chunk == 128 ? 1l : 4l) * num_sms ? 1 : tma_group(chunk);
+    return (long)p.T * (p.K / chunk) <= (chunk == 128 ? 4l : 6l) * num_sms ? 1 : tma_group(chunk);
   return p.m == 4 && std_mats && p.out_dtype == 0 && chunk == 128 && (long)p.T * (p.K / 128) <= 16l * num_sms
              ? 1 : tma_group(chunk);
 }

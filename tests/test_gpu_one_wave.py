@@ -60,9 +60,10 @@ def test_few_blocks_per_sm(m, N):
     _compare(L, x_q, w_q, bias, 1)
 
 
-# F6 output, one tile per image: one channel per thread up to 148 blocks of 128 and 592 of 64 channels, pairs
-# from there on; codes at their bounds, where the factored sums are largest
-@pytest.mark.parametrize("K,N", [(128, 148), (128, 149), (64, 592), (64, 593), (96, 50)])
+# F6 output, one tile per image: one channel per thread up to 592 blocks of 128 and 888 of 64 channels, pairs
+# from there on; blocks at most one, and more, to an SM; codes at their bounds, where the factored sums are largest
+@pytest.mark.parametrize("K,N", [(128, 148), (128, 149), (128, 592), (128, 593), (64, 592), (64, 593), (64, 888),
+                                 (64, 889), (96, 50)])
 @pytest.mark.parametrize("variant", ["plain", "saturating", "float_out"])
 def test_f6_output_transform(K, N, variant):
     L, x_q, w_q, bias = build_layer(wi.Workload("o6", 5750 + K, N, 64, 6, 5, K, 6),
@@ -75,7 +76,8 @@ def test_f6_output_transform(K, N, variant):
 
 # the same builds, and the one-launch kernel, on sums that show the order of their terms: as floats, and as codes
 # of a unit in the last place each (the one-channel builds write codes only)
-@pytest.mark.parametrize("K,N", [(128, 148), (128, 149), (64, 592), (64, 593), (96, 50)])
+@pytest.mark.parametrize("K,N", [(128, 148), (128, 149), (128, 592), (128, 593), (64, 592), (64, 593), (64, 888),
+                                 (64, 889), (96, 50)])
 @pytest.mark.parametrize("out", ["codes", "float", "float_ragged"])
 def test_f6_output_transform_sums_in_order(K, N, out):
     if out == "float_ragged":

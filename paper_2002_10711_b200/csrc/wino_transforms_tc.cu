@@ -11,7 +11,8 @@
 // What bounds a transform of a large layer is the number of issue slots a code costs.
 // Transforming on the ALUs takes 10 to 14 for F4; here the product leaves the tensor cores as
 // int32 and a code costs 4.2: conversion 1, half a packed fma (two slots), the clamp on 16-bit
-// lanes 1, packing 0.75, its share of a 32-column tensor-memory load and of a 32-byte store.  To
+// lanes 1, packing 0.75 (on the input side of F2 and F4 half of it as multiply-adds, off the ALU
+// pipe), its share of a 32-column tensor-memory load and of a 32-byte store.  To
 // have it so, the product is laid out with (tile, position) as its rows and channels as its
 // columns: a thread then holds 32 consecutive channels of one row of V_q (of one pixel of y).
 //     A operand  constant, K-major: the Kronecker matrix of several tiles, block diagonal,
@@ -22,15 +23,16 @@
 //                bytes per K index, swizzled, "MN-major".
 // F6: 16 B^T (x) B^T has entries up to 441, split as 16 * hi + lo, two products.
 //
-// Persistent blocks, 704 threads: warps 0-3 load, warp 4 issues the products, on the input side every
-// other unit's and warp 5 the rest (a unit's waits, products and commits took a single warp 500 cycles,
-// which held up the 64-channel units: 32x32, batch 256, F4 17.4 us with one warp, 15.6 with two, 15.3
-// with four, where 128-channel ones lost 0.1; the output side, of larger units, lost 0 to 0.3), sixteen epilogue
+// Persistent blocks, 704 threads on the input side and 672 on the output side: warps 0-3 load, warp 4
+// issues the products, on the input side every other unit's and warp 5 the rest (a unit's waits, products
+// and commits took a single warp 500 cycles, which held up the 64-channel units: 32x32, batch 256, F4 17.4 us
+// with one warp, 15.6 with two, 15.3 with four, where 128-channel ones lost 0.1; the output side, of larger
+// units, lost 0 to 0.3 with a second one, 0.05 to 0.1 with an idle warp), sixteen epilogue
 // warps; warp w reads tensor-memory lanes 32 * (w % 4) and takes every fourth 32-column chunk.
 // Stores go out directly, as 32-byte pieces of lines that other warps complete: exchanging rows
 // between warps to store whole lines cost 6 to 30 % (barriers), a staging tile with TMA stores
-// 0 to 16 %; the ALU pipe, 60 % busy (64 channels, 32x32, F4, batch 256: 9.98 M warp instructions for
-// 75.5 M codes, 53 % of the issue slots), and the latency of the few warps are what is left.
+// 0 to 16 %; the ALU pipe (60 % busy before packing left it in part: 64 channels, 32x32, F4, batch 256, 9.98 M
+// warp instructions for 75.5 M codes, 53 % of the issue slots) and the latency of the few warps are what is left.
 // Four load warps for the input side: a unit is two to eight boxes of short rows, and one warp
 // issuing them (1200 cycles a unit) held everything else up.
 #include <vector>
@@ -43,8 +45,10 @@ namespace wino {
 
 namespace {
 
-constexpr int kXtLoadWarps = 4, kXtMmaWarp = 4, kXtMmaWarps = 2, kXtEpi0 = kXtMmaWarp + kXtMmaWarps;
-constexpr int kXtThreads = 32 * (kXtEpi0 + 16);
+// Warps of the two kernels: loads, products (two warps on the input side), epilogue.
+constexpr int kXtLoadWarps = 4, kXtMmaWarp = 4, kXtEpiWarps = 16;
+constexpr int kXiEpi0 = kXtMmaWarp + 2, kXiThreads = 32 * (kXiEpi0 + kXtEpiWarps);
+constexpr int kXoEpi0 = kXtMmaWarp + 1, kXoThreads = 32 * (kXoEpi0 + kXtEpiWarps);
 
 __device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
   asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
@@ -159,7 +163,7 @@ __device__ __forceinline__ void xt_mma_loop(const L& s, int n_my, int which, uin
 // off it.
 // ---------------------------------------------------------------------------
 template <int M, int CH, bool Z>
-__global__ void __launch_bounds__(kXtThreads, 1)
+__global__ void __launch_bounds__(kXiThreads, 1)
 k_input_transform_tc(const __grid_constant__ Params p, const __grid_constant__ CUtensorMap mapX,
                      const uint8_t* __restrict__ a_image, int8_t* __restrict__ Vq, int* __restrict__ status,
                      const uint8_t* __restrict__ l2_hint, uint32_t l2_hint_bytes) {
@@ -217,10 +221,10 @@ k_input_transform_tc(const __grid_constant__ Params p, const __grid_constant__ C
       chunk += d_chunk;
       if (chunk >= cchunks) { chunk -= cchunks; ++group; }
     }
-  } else if (warp < kXtEpi0) {
-    xt_mma_loop<L, kSlots, kBuf, kXtMmaWarps, NA, 4, CH, 16384, kSlot>(s, n_my, warp - kXtMmaWarp, tmem_base, abort_p);
+  } else if (warp < kXiEpi0) {
+    xt_mma_loop<L, kSlots, kBuf, kXiEpi0 - kXtMmaWarp, NA, 4, CH, 16384, kSlot>(s, n_my, warp - kXtMmaWarp, tmem_base, abort_p);
   } else {
-    const int quad = warp & 3, sub = (warp - kXtEpi0) >> 2;
+    const int quad = warp & 3, sub = (warp - kXiEpi0) >> 2;
     const int r = quad * 32 + lane, xi = r / TP, j = r - xi * TP;
     const int col = (kColChunks == 4 ? sub : sub & 1) * 32;
     const int first = kColChunks == 4 ? 0 : sub >> 1, step = kColChunks == 4 ? 1 : 2;
@@ -304,7 +308,7 @@ k_input_transform_tc(const __grid_constant__ Params p, const __grid_constant__ C
 // once per block into shared memory.
 // ---------------------------------------------------------------------------
 template <int M, int CH, bool PK>
-__global__ void __launch_bounds__(kXtThreads, 1)
+__global__ void __launch_bounds__(kXoThreads, 1)
 k_output_transform_tc(const __grid_constant__ Params p, const __grid_constant__ CUtensorMap mapM,
                       const uint8_t* __restrict__ a_image, const float* __restrict__ bias, void* __restrict__ y,
                       float s_Y, int* __restrict__ status, const float* __restrict__ chan) {
@@ -325,7 +329,7 @@ k_output_transform_tc(const __grid_constant__ Params p, const __grid_constant__ 
   const int n_my = (int)blockIdx.x < units ? (units - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
 
   xt_setup<L, kSlots, kBuf>(s, abort_p, warp, kBuf * CH, 4 * kColChunks);
-  for (int k = threadIdx.x; k < p.K; k += kXtThreads) {
+  for (int k = threadIdx.x; k < p.K; k += kXoThreads) {
     float b = bias != nullptr ? __ldg(bias + k) : 0.0f;
     if (p.out_dtype == 0 && bias != nullptr)
       b = (float)((double)b / (double)(PK ? __ldg(chan + (long)kChSY * p.K + k) : s_Y));
@@ -357,11 +361,10 @@ k_output_transform_tc(const __grid_constant__ Params p, const __grid_constant__ 
         if (++sl == kSlots) { sl = 0; ph ^= 1u; }
       }
     }
-  } else if (warp < kXtEpi0) {
-    if (warp == kXtMmaWarp)
-      xt_mma_loop<L, kSlots, kBuf, 1, 1, G::K / 32, CH, kA, kSlot>(s, n_my, 0, tmem_base, abort_p);
+  } else if (warp < kXoEpi0) {
+    xt_mma_loop<L, kSlots, kBuf, 1, 1, G::K / 32, CH, kA, kSlot>(s, n_my, 0, tmem_base, abort_p);
   } else {
-    const int quad = warp & 3, sub = (warp - kXtEpi0) >> 2;
+    const int quad = warp & 3, sub = (warp - kXoEpi0) >> 2;
     const int r = quad * 32 + lane, j = r / G::PX, pix = r - j * G::PX, ip = pix / M, jp = pix - ip * M;
     const int col = (kColChunks == 4 ? sub : sub & 1) * 32;
     const int first = kColChunks == 4 ? 0 : sub >> 1, step = kColChunks == 4 ? 1 : 2;
@@ -492,7 +495,7 @@ int input_go(const Params& p, const LaunchOpt& o, const CUtensorMap& mapX, const
   if (int rc = set_max_smem(once, o.device, k_input_transform_tc<M, CH, Z>, smem)) return rc;
   const long units = (long)((p.T + G::TP - 1) / G::TP) * ((p.C + CH - 1) / CH);
   const int grid = units < o.num_sms ? (int)units : o.num_sms;
-  return launch_kernel(k_input_transform_tc<M, CH, Z>, dim3((unsigned)grid), dim3(kXtThreads), smem, st, o.pdl, p, mapX,
+  return launch_kernel(k_input_transform_tc<M, CH, Z>, dim3((unsigned)grid), dim3(kXiThreads), smem, st, o.pdl, p, mapX,
                        img, Vq, status, static_cast<const uint8_t*>(o.l2_hint), (uint32_t)o.l2_hint_bytes);
 }
 template <int M>
@@ -515,7 +518,7 @@ int output_go(const Params& p, const LaunchOpt& o, const CUtensorMap& mapM, cons
   if (int rc = set_max_smem(once, o.device, k_output_transform_tc<M, CH, PK>, 227 * 1024)) return rc;
   const long units = (long)((p.T + G::TP - 1) / G::TP) * ((p.K + CH - 1) / CH);
   const int grid = units < o.num_sms ? (int)units : o.num_sms;
-  return launch_kernel(k_output_transform_tc<M, CH, PK>, dim3((unsigned)grid), dim3(kXtThreads), smem, st, o.pdl, p,
+  return launch_kernel(k_output_transform_tc<M, CH, PK>, dim3((unsigned)grid), dim3(kXoThreads), smem, st, o.pdl, p,
                        mapM, img, bias, y, s_Y, status, o.chan);
 }
 template <int M>

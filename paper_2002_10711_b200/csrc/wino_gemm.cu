@@ -4,10 +4,10 @@
 // followed by the quantizer of the Hadamard output (paper: Fig. 2).
 //
 //   k_gemm_tc   : persistent, warp-specialised tcgen05 kernel.  int8 operands are
-//                 staged in shared memory by TMA (128-byte swizzle), MMAs of
-//                 kind::i8 accumulate in int32 in tensor memory, two accumulator
-//                 buffers let the epilogue of one block overlap the MMAs of the
-//                 next.
+//                 staged in shared memory by TMA (128-byte swizzle, 64-byte with
+//                 at most 64 channels), MMAs of kind::i8 accumulate in int32 in
+//                 tensor memory, two accumulator buffers let the epilogue of one
+//                 block overlap the MMAs of the next.
 //   k_gemm_warp : the same contraction with int8 warp MMAs; for channel counts
 //                 the TMA path cannot take.
 #include "wino_f32x2.cuh"
@@ -146,8 +146,8 @@ int launch_gemm_warp(const Params& p, const LaunchOpt& o, const int8_t* Vq, cons
 // A stage holds cB channels (128, or 64 in layers of no more): A tiles of 128 x cB bytes, B tile
 // BN x cB bytes; one MMA consumes 32 channels.
 // What bounds it on narrow layers (64 ch 32x32 batch 256, F4: 17.2 us with 128-byte stages, two of
-// them, and a copy per m-block; 14.4 now): the quantizer takes some 780 cycles per 32 columns and
-// warp with four warps to a scheduler, 6.3 us in all; the rest is the hand-over between the ring, the
+// them, and a copy per m-block; 14.2 now): the quantizer takes some 675 cycles per 32 columns and
+// warp with four warps to a scheduler, 5.4 us in all; the rest is the hand-over between the ring, the
 // MMA warp, whose MMAs share the path to shared memory with the epilogue's stores (115 to 230 cycles
 // each, 36 alone), and the two accumulators.  A second MMA warp, waits without back-off and unrolled
 // MMA loops changed nothing.
@@ -668,8 +668,10 @@ TcGeom tc_geometry(const Params& p, int num_sms) {
 // Which of the two lean quantizers (per-layer scales, upper bound 127; else there is only one): the
 // saturating pack for blocks of 256 output channels, the clamp on 16-bit lanes, of fewer instructions,
 // for narrower ones.  Measured on B200, us, GEMM alone and whole layer, 16-bit lanes / saturating pack:
-//   256 ch 8x8 F4 batch 256  5.99, 15.83 / 5.95, 15.77, batch 64  4.06, 11.56 / 3.98, 11.46;  512 ch 4x4
-//     F4 batch 256  5.99, 14.12 / 5.90, 14.05
+//   256 ch 8x8 F4 batch 256  5.72, 15.35 / 5.60, 15.28, batch 64  4.28, 9.21 / 4.15, 9.02, batch 32  4.21,
+//     8.42 / 4.08, 8.28;  512 ch 4x4 F4 batch 256  5.31, 11.06 / 5.21, 10.98;  64 -> 256 ch 14x14 F2 batch 32
+//     4.96, 10.94 / 4.89, 10.84 (the other way: 256 ch 8x8 F2 batch 256  8.12, 21.30 / 8.30, 21.40);  295 layers
+//     of 16 to 2400 tiles 1.009
 //   64 ch 32x32 batch 256 F4  14.19, 38.36 / 14.63, 39.10, F6  14.07, 42.70 / 14.36, 43.44;  batch 64 F2
 //     9.04, 19.98 / 9.41, 20.36;  128 ch 16x16 F4 batch 32  3.09, 9.87 / 3.09, 9.90, F2 batch 128  8.95,
 //     21.26 / 8.87, 21.22

@@ -12,9 +12,12 @@
 //             fused-multiply-add chains in the contract's order.
 //   kSparse : the built-in Cook-Toom matrices as compile-time constants; zero
 //             entries vanish (the chain's value does not change).
-//   kExact  : Cook-Toom F4 with every intermediate an integer below 2^24, so
-//             any summation order gives the same bits; shared sub-expressions
-//             are factored out (12 instead of 22 operations per 1-D transform).
+//   kExact  : Cook-Toom matrices on integer codes, every intermediate exactly
+//             representable, so any summation order gives the same bits; shared
+//             sub-expressions are factored out (F4 input: 12 instead of 22
+//             operations per 1-D transform).  Here the input transforms and the
+//             output transforms of F2 and F4; F6's spills with several channels
+//             per thread.
 #pragma once
 #include <cstdlib>
 #include "wino_launch.h"

@@ -420,24 +420,27 @@ LaunchOpt opt_with_hint(const wino_plan_t* pl, bool pdl, int stage_mask, const i
 // un-quantized sum (four bytes, through the pointer-based output transform), and what learnt matrices, an
 // input zero point and rows of less than 64 channels add to the transforms; F6's output transform has a quick
 // build for small grids in chunks of 64 and 128 channels only.  Fitted on B200 to the layers of small_geometry,
-// forced onto this path (5 to 10 % standard deviation).  Of 4800 layers either kernel can run, the choice
-// costs 0.3 % on average and more than 7 % on one in sixty.  Us, one launch / staged, times (of a loop of calls
+// forced onto this path (5 to 10 % standard deviation).  Of 5700 layers either kernel can run, the choice
+// costs 0.3 % on average and more than 7 % on one in seventy.  Us, one launch / staged, times (of a loop of calls
 // and a graph, averaged) and estimates:
 //   F4  512 ch 4x4 batch 16  9.9 / 8.8 and 9.6 / 8.9;  256 ch 8x8 batch 16  10.1 / 7.9 and 9.4 / 8.1, batch 8
 //     7.9 / 7.8 and 7.8 / 7.9, batch 4  7.3 / 7.8 and 7.1 / 7.8;  128 ch 16x16 batch 16  8.3 / 7.6 and 8.5 /
 //     8.4, batch 8  6.5 / 7.5 and 7.2 / 7.9;  un-quantized 256 ch 8x8 batch 16  9.8 / 11.5 and 9.4 / 10.5
-//   F2  un-quantized 128 ch 14x14 batch 16  10.1 / 14.2 and 11.0 / 14.7, learnt  11.5 / 8.0 and 12.7 / 8.6
+//   F2  un-quantized 128 ch 14x14 batch 16  10.1 / 14.2 and 11.0 / 14.0, learnt  11.5 / 8.0 and 12.7 / 8.6
 //   F6  128 ch 16x16 batch 16  11.4 / 9.1 and 10.8 / 9.8, un-quantized  11.1 / 15.7 and 10.8 / 14.5
 // Fused F2: waves of 128 tiles per SM, full or not (28 us at 64 channels).
 long staged_cost(const wino_plan_t* pl) {
   static const double start[3] = {7000, 7300, 8100}, per_code[3] = {4.0e-4, 4.3e-4, 6.5e-4};
-  static const double start_warp[3] = {7000, 7500, 9300};   // GEMM by warp-level MMAs
+  static const double start_warp[3] = {7000, 7500, 9300}, learnt_warp[3] = {300, 900, 2000};   // warp-level MMAs
   static const double learnt[3] = {300, 900, 3100}, zero[3] = {1000, 1100, 600};
   const Params& p = pl->p;
   const int mi = p.m / 2 - 1;
   const double v = (double)p.t * p.t * p.T * p.C, sums = (double)p.t * p.t * p.T * p.K;
-  double ns = (p.qM_enabled ? 0.0 : 4.0e-3 * sums) + (pl->std_mats ? 0.0 : learnt[mi]) + (p.z_x == 0 ? 0.0 : zero[mi]);
-  if (pl->path == WINO_PATH_STAGED_DP4A) return (long)(ns + start_warp[mi] + 1.5e-3 * (v + sums));
+  const double many = 1.3e6;   // un-quantized sums, from which on they keep the output transform busy
+  double ns = p.qM_enabled ? 0.0 : sums < many ? 4.0e-3 * sums : 4.0e-3 * many + 1.7e-3 * (sums - many);
+  if (pl->path == WINO_PATH_STAGED_DP4A)
+    return (long)(ns + start_warp[mi] + 1.5e-3 * (v + sums) + (pl->std_mats ? 0.0 : learnt_warp[mi]));
+  ns += (pl->std_mats ? 0.0 : learnt[mi]) + (p.z_x == 0 ? 0.0 : zero[mi]);
   if (p.m == 6 && tma_chunk(p.K) % 64 != 0) ns += 700;
   if (p.m != 2) ns += 700 * ((tma_chunk(p.C) < 64) + (tma_chunk(p.K) < 64));
   return (long)(ns + start[mi] + per_code[mi] * (v + sums) + 1.4e-4 * p.t * p.t * p.K * p.C);
@@ -565,7 +568,8 @@ int forward_impl(wino_plan_t* pl, const int8_t* x, const int8_t* Uq, const float
     if (mm == nullptr) return WINO_ERR_CUDA;
     rc = launch_output_transform_tc(pl->p, opt_of(pl, pdl), *mm, pl->xt_images, bias, y, pl->s_Y, pl->status_dev, st);
   } else if (tma_ok && pl->p.qM_enabled && tma_chunk(pl->p.K) != 0) {
-    const CUtensorMap* mm = map_stage(pl, pl->cache_mld, mbuf, pl->p.K, tma_out_group(pl->p, pl->std_mats, pl->num_sms));
+    const int group = tma_out_group(pl->p, pl->std_mats, pl->chan_dev != nullptr, pl->num_sms);
+    const CUtensorMap* mm = map_stage(pl, pl->cache_mld, mbuf, pl->p.K, group);
     const bool to_float = pl->p.out_dtype != 0;
     const CUtensorMap* my = to_float ? mm : map_y(pl, y);
     if (mm == nullptr || my == nullptr) return WINO_ERR_CUDA;
@@ -747,6 +751,7 @@ int wino_plan_set_channel_scales(wino_plan_t* pl, const float* s_w_K, const floa
                                  const float* s_M_K, const float* s_Y_K) {
   if (pl == nullptr) return WINO_ERR_INVALID;
   const int K = pl->d.K;
+  pl->cache_mld = MapCache{};   // the boxes of m_q depend on whether there are such scales (tma_out_group)
   if (s_w_K == nullptr && s_U_K == nullptr && s_M_K == nullptr && s_Y_K == nullptr) {   // per-layer scales again
     if (pl->chan_dev) cudaFree(pl->chan_dev);
     pl->chan_dev = nullptr;

@@ -106,10 +106,12 @@ constexpr int tma_in_group(int m, int chunk) { return m == 2 ? tma_group(chunk) 
 // channels a block  128 ch 12x12 batch 64 (2) 9.9 / 9.2, batch 100 (3) 11.0 / 9.8, 512 ch 8x8 batch 32 (4) 12.7
 // / 12.2, 128 ch 12x12 batch 150 (5) 12.6 / 13.1, 256 ch 12x12 batch 75 (5) 13.6 / 14.1;  64 channels  64 ch
 // 12x12 batch 64 (2) 9.1 / 8.2, batch 150 (5) 10.4 / 9.7, batch 200 (6) 11.4 / 10.4, batch 275 (8) 12.4 / 13.1.
-inline int tma_out_group(const Params& p, bool std_mats, int num_sms) {
+// With scales per output channel, of which a block reads three, up to two:  128 ch 12x12 batch 75 (3) 11.0 /
+// 11.7, 512 ch 8x8 batch 37 (4) 16.3 / 16.9;  64 ch 12x12 batch 75 (3) 10.1 / 10.7, batch 150 (5) 10.9 / 12.1.
+inline int tma_out_group(const Params& p, bool std_mats, bool per_channel, int num_sms) {
   const int chunk = tma_chunk(p.K);
   if (p.m == 6 && std_mats && p.out_dtype == 0 && (chunk == 128 || chunk == 64))
-    return (long)p.T * (p.K / chunk) <= (chunk == 128 ? 4l : 6l) * num_sms ? 1 : tma_group(chunk);
+    return (long)p.T * (p.K / chunk) <= (per_channel ? 2l : chunk == 128 ? 4l : 6l) * num_sms ? 1 : tma_group(chunk);
   return p.m == 4 && std_mats && p.out_dtype == 0 && chunk == 128 && (long)p.T * (p.K / 128) <= 16l * num_sms
              ? 1 : tma_group(chunk);
 }

@@ -27,7 +27,8 @@ bool small_supported(const Params& p) {
 // block, `exchange` in a cluster, `copies` a chunk without tensor copies, and as much of `load` as the round
 // fills SMs: U_q and the patches then come through L2 to all of them at once.  Two blocks per SM (shared
 // memory permitting, F2 and F4) take `two` times as long as one.  Clusters of four or eight do not fill every
-// SM.  Learnt matrices and an input zero point, whose padding is patched, lengthen the input transform.
+// SM.  Learnt matrices and an input zero point, whose padding is patched, lengthen the input transform; at
+// most four tiles leave half of a block's warps idle and take 0.92 of the time.
 // Fitted on B200 to 8000 times of layers of 1 to 2048 blocks with every option and most geometries, per call,
 // averaged over a loop of calls and a CUDA graph of them: 5.6 (F6) to 7.4 % (F2) standard deviation.  Where
 // the geometry differs from that of an earlier fit without `load` (700 layers), 0.95 of the time.
@@ -67,7 +68,7 @@ SmallGeom small_geometry(const Params& p, bool std_mats, int num_sms) {
       const double full = (t1 + load[mi]) * (two ? twice[mi] : 1.0);
       const long last = blocks - (rounds - 1) * per_round;
       const double us = (rounds - 1) * full + (last > sms ? full : t1 + load[mi] * last / sms);
-      g.cost = (long)(1000.0 * us * (std_mats ? 1.0 : learnt[mi]) * (p.z_x == 0 ? 1.0 : zero[mi]));
+      g.cost = (long)(1000.0 * us * (std_mats ? 1.0 : learnt[mi]) * (p.z_x == 0 ? 1.0 : zero[mi]) * (p.T <= 4 ? 0.92 : 1.0));
       if (best.cost < 0 || g.cost < best.cost) best = g;
     }
   }

@@ -460,7 +460,7 @@ template <int M, int MODE, int KC>
 int output_tma_launch(const Params& p, const LaunchOpt& o, const CUtensorMap& mapM, const CUtensorMap& mapY,
                       const float* bias, float s_Y, int* status, float* y_float, cudaStream_t st) {
   if constexpr (MODE == kExact && ((M == 4 && KC == 128) || (M == 6 && KC % 64 == 0))) {
-    if (tma_out_group(p, o.std_mats, o.num_sms) == 1)
+    if (tma_out_group(p, o.std_mats, o.chan != nullptr, o.num_sms) == 1)
       return output_tma_go<M, MODE, KC, M == 4 ? 16 : 1024 / KC, 1>(p, o, mapM, mapY, bias, s_Y, status, nullptr, st);
   }
   if constexpr (M == 6 && MODE == kDense) {

@@ -19,6 +19,8 @@ pytestmark = pytest.mark.gpu
     (16, 256, 8, 8, 256, 4, dict(q_M=False), 1),         # 9.8 / 11.5
     (32, 128, 8, 8, 128, 6, dict(q_M=False), 1),         # 10.7 / 15.0
     (16, 128, 14, 14, 128, 2, dict(flex=True), 3),       # 11.5 / 8.0
+    (34, 128, 17, 17, 128, 2, dict(q_M=False), 3),       # 27.1 / 21.7
+    (1, 512, 7, 4, 512, 4, dict(flex=True), 1),          # 7.1 / 9.8
     (16, 48, 16, 16, 80, 6, {}, 1),                      # 9.2 / 12.1
 ])
 def test_one_launch_or_three(N, C, H, W, K, m, options, launches):

@@ -2,9 +2,13 @@
 builds that are chosen by whether all blocks of a grid are resident at once, on both sides of each line."""
 import numpy as np
 import pytest
+import torch
 
+import oracle
 import wino_inputs as wi
 from helpers import build_layer, f6_order_sensitive, per_channel
+from paper_2002_10711_b200 import binding
+from paper_2002_10711_b200.layer import WinogradConv
 from test_gpu_parity import _compare
 
 pytestmark = pytest.mark.gpu
@@ -86,6 +90,23 @@ def test_f6_output_transform_sums_in_order(K, N, out):
         L, x_q, w_q, bias = f6_order_sensitive(N, K, out_dtype=0 if out == "codes" else 1)
     _compare(L, x_q, w_q, bias, 1)
     _compare(L, x_q, w_q, bias, 8, dumps=False)
+
+
+# F6 output: the line between its two builds is another with scales per output channel; a plan that has run
+# takes them, and loses them again, with tensor maps of the build that it then runs
+@pytest.mark.parametrize("K,N", [(128, 296), (128, 297), (64, 400)])
+def test_f6_channel_scales_on_a_plan_that_has_run(K, N):
+    L, x_q, w_q, bias = build_layer(wi.Workload("o6c", 5780 + K, N, 64, 6, 5, K, 6))
+    P = per_channel(L, 47)
+    conv = WinogradConv(binding.Plan.from_layer(L, path=1))
+    x = torch.from_numpy(x_q).cuda()
+    for layer, scales in ((L, None), (P, (P.s_w_K, P.s_U_K, P.s_M_K, P.s_Y_K)), (L, (None,) * 4)):
+        if scales is not None:
+            conv.plan.set_channel_scales(*scales)
+        conv.load_weights(w_q, bias)
+        y = conv.forward(x)
+        assert conv.plan.last_status() == 0
+        assert (y.cpu().numpy() == oracle.forward(layer, x_q, w_q, bias=bias)).all()
 
 
 # several tiles a block (64, 32 and 16 channels a chunk), one channel per thread and two
